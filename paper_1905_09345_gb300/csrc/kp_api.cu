@@ -844,7 +844,7 @@ KM_API int kmeans_init(kmeans_ctx **out, const float *X, int64_t N, int32_t D, i
             const int kp = dense_tcb_kp(p);
             INIT_CUDA(dalloc(c, &p.Ch, (size_t)kp * Dt));
             INIT_CUDA(dalloc(c, &p.Cl, (size_t)kp * Dt));
-            INIT_CUDA(dalloc(c, &p.cnorm, (size_t)K));
+            INIT_CUDA(dalloc(c, &p.cnorm, (size_t)kp));
         }
     }
 

@@ -124,7 +124,7 @@ struct Params {
     struct SettleReq *sreq;  // N, indexed by row: rows the tensor-core pass left to the exact settle
     uint32_t *sbits;     // ceil(N / 128) * 4 words: bit n set = row n has a settle request
     uint16_t *Ch, *Cl;   // Kp x D bfloat16 halves of C (tensor-core pass with K > 256)
-    float *cnorm;        // K: ||c||^2 of that pass
+    float *cnorm;        // Kp: ||c - mu||^2 of that pass (padding: +inf)
     int32_t *squeue;     // N: the rows with a request, compacted from the bitmap
     int32_t *perm;       // N: point ids sorted by label (full recompute of the cluster sums)
     int32_t *slab;       // N: their labels

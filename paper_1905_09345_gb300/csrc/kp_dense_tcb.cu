@@ -7,15 +7,29 @@
 // centroids stream through shared memory in blocks of 128 (both bfloat16
 // halves, loaded by TMA from a split copy made at the start of each pass),
 // and each row's scan -- group minima, winner, runner-up -- carries across
-// the blocks.  Group minima are converted to lower bounds and written to lb
-// after every 64 columns, so shared memory holds only the groups those
-// columns close.
+// the blocks.
 //
-// Persistent CTA per SM, 320 threads: warp 0 issues TMA, one thread of warp 1
-// the MMAs, warps 2..9 are two epilogue groups of four.  Tiles of 128 points
-// go in pairs to the two groups; both tiles of a pair use each centroid block
-// while it is in shared memory.  Each group owns two TMEM buffers of 128
-// columns, so the MMAs of block j+1 run while the group scans block j.
+// Persistent CTA per SM, 576 threads: warp 0 issues TMA, one thread of warp 1
+// the MMAs, warps 2..17 read the accumulators.  Tiles of 128 points go in
+// pairs; both tiles of a pair use each centroid block while it is in shared
+// memory.  The scan bounds the kernel (about 12 instructions per row and
+// column at half of the issue rate; the tensor pipe is active 25-40% of the
+// time), so every tile has eight warps:
+// two per TMEM lane quadrant, one for the blocks of the first half of the
+// centroids, one for those of the second half (each warp's columns stay one
+// ascending run, so its group minima close in order).  The blocks are issued
+// alternately from the two halves, and each (tile, half) owns one of the four
+// TMEM buffers of 128 columns, so three buffers are scanned or waiting while
+// the fourth is multiplied.
+// The bfloat16 halves of a block have shared-memory slots of their own and
+// the products with the high half come first (x_h c_h, x_l c_h of both
+// tiles, then x_h c_l), so that one half loads while the other is multiplied.
+//
+// Measured on GB300 (one pass): 4,194,304 x 128, K = 1024, G = 103: 5.2 ms with
+// four scanning warps per tile and a column-by-column scan, 3.5 ms now;
+// 1,048,576 x 32, K = 4096, G = 410: 4.9 -> 2.7 ms.  Blocks of 64 columns with
+// two buffers per (tile, half) measured 5.9 and 4.2 ms, a sixteen-column
+// tournament 5.5 and 3.7 (spills, and the code outgrows the instruction cache).
 #include "kp_tc.cuh"
 
 namespace kp {
@@ -23,24 +37,115 @@ namespace {
 
 constexpr int kNB = 128;                       // centroids per block (MMA N)
 constexpr int kBAtom = kNB * 128;              // one 64-element column block of a centroid block
-constexpr int kEpiWarps = 4;
-constexpr int kPairs = 2;                      // epilogue groups = tiles in flight
-constexpr int kThreads = 64 + kPairs * kEpiWarps * 32;
+constexpr int kQuadWarps = 4;                  // warps of a (tile, half): the TMEM lane quadrants
+constexpr int kEpi = 4 * kQuadWarps;           // two tiles x two halves
+constexpr int kThreads = 64 + kEpi * 32;
 constexpr int kMaxKp = 4096;
+constexpr int kSlots = 7;                      // staged group minima per row: 3 left over + those that
+                                               // four columns can close, whatever the groups' sizes
+constexpr int kCnSlots = 4;                    // blocks of norms per half
 
 struct TcbCfg {
     int Kp;          // K padded to a multiple of kNB
-    int nb;          // centroid blocks
-    int bst;         // centroid-block stages (1 or 2)
-    int srow;        // staging floats per row (odd, >= groups 64 columns can close + 1)
-    uint32_t off_A, off_B, off_cn, off_bm, off_stage, off_bar;
+    int nb, hb;      // centroid blocks; blocks of the first half
+    int hs;          // slots of half a centroid block (even, 2 or 4)
+    uint32_t off_B, off_cn, off_bm, off_stage, off_t4, off_mrg, off_bar;
     int num_tiles;
     float e_lin, e_c2, xn_lo, xn_hi;
 };
 
-// uses of accumulator buffer `buf` (blocks j with j % 2 == buf) before block j of pair pr
-__device__ __forceinline__ uint32_t acc_uses(int pr, int j, int buf, int nb) {
-    return (uint32_t)(pr * ((nb + 1 - buf) >> 1) + (j >> 1));
+__device__ __forceinline__ unsigned long long pack_f2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Running scan of one row over an ascending run of accumulator columns, four
+// at a time: the smallest value and the runner-up from the sorted pairs of the
+// four, the winner as the index of its group of four (whose values the lane
+// keeps in shared memory, from which the column is read off at the end), and
+// the open group's minimum.  A group boundary among the four columns (the
+// same for every row) closes the minimum into the row's next staging slot.
+// The stores carry no memory clobber, so that the scan's loads may move
+// across them; what they wrote is read back by volatile accesses only.
+struct Scan4 {
+    float b1, b2, gm;
+    int c4;        // first column of the four that hold b1
+    uint32_t row;  // staging slots of the row
+    uint32_t t4;   // the lane's four values
+    int pend;      // closed minima staged (warp-uniform)
+
+    __device__ __forceinline__ void four(const uint32_t *acc, const float4 &cn, uint32_t nib, int c) {
+        unsigned long long t01, t23;
+        const unsigned long long m2 = 0xc0000000c0000000ull;  // (-2, -2)
+        asm("fma.rn.f32x2 %0, %1, %2, %3;"
+            : "=l"(t01)
+            : "l"(pack_f2(__uint_as_float(acc[0]), __uint_as_float(acc[1]))), "l"(m2), "l"(pack_f2(cn.x, cn.y)));
+        asm("fma.rn.f32x2 %0, %1, %2, %3;"
+            : "=l"(t23)
+            : "l"(pack_f2(__uint_as_float(acc[2]), __uint_as_float(acc[3]))), "l"(m2), "l"(pack_f2(cn.z, cn.w)));
+        float t[4];
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[0]), "=f"(t[1]) : "l"(t01));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[2]), "=f"(t[3]) : "l"(t23));
+        const float l0 = fminf(t[0], t[1]), h0 = fmaxf(t[0], t[1]);
+        const float l1 = fminf(t[2], t[3]), h1 = fmaxf(t[2], t[3]);
+        const float m = fminf(l0, l1);
+        const float s = min3(fmaxf(l0, l1), h0, h1);  // the second smallest of the four
+        b2 = min3(b2, s, fmaxf(b1, m));
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %6, %7;\n\t@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t"
+            "selp.s32 %0, %8, %0, p;\n\t}"
+            : "+r"(c4)
+            : "r"(t4), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(m), "f"(b1), "r"(c));
+        b1 = fminf(b1, m);
+        if (nib == 0) {
+            gm = fminf(gm, m);
+        } else {  // (branches on nib are warp-uniform)
+            auto close = [&](float v) {
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + 4u * (uint32_t)pend), "f"(v));
+                ++pend;
+            };
+            if (nib & 1u) {
+                close(gm);
+                gm = INFINITY;
+            }
+            if (nib & 2u) {
+                close(fminf(gm, t[0]));
+                gm = t[1];
+            } else {
+                gm = fminf(gm, l0);
+            }
+            if (nib & 4u) {
+                close(gm);
+                gm = INFINITY;
+            }
+            if (nib & 8u) {
+                close(fminf(gm, t[2]));
+                gm = t[3];
+            } else {
+                gm = fminf(gm, l1);
+            }
+        }
+    }
+    // the winner's column (lowest among equal values)
+    __device__ __forceinline__ int winner() const {
+        float t0, t1, t2, t3;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t0), "=f"(t1), "=f"(t2), "=f"(t3) : "r"(t4));
+        if (b1 == INFINITY) return c4;
+        return c4 + (t0 == b1 ? 0 : (t1 == b1 ? 1 : (t2 == b1 ? 2 : 3)));
+    }
+};
+
+__device__ __forceinline__ float lds_f(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
 }
 
 template <int D>
@@ -56,25 +161,28 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->path = KM_PATH_DENSE_TC;
     constexpr int NA = D / 64;
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
-    const int Kp = cfg.Kp, nb = cfg.nb, BS = cfg.bst;
-    uint8_t *sA = sm + cfg.off_A;  // 2 stages: [NA atoms x_h][NA atoms x_l]
-    uint8_t *sB = sm + cfg.off_B;  // BS stages: [NA atoms c_h][NA atoms c_l]
-    float *cn = reinterpret_cast<float *>(sm + cfg.off_cn);  // [Kp] ||c||^2 (+inf: padding)
-    float *pen = cn + Kp;                                    // [Kp] +inf where a group opens
+    const int nb = cfg.nb, hb = cfg.hb, HS = cfg.hs;
+    uint8_t *sA = sm;               // 2 tiles: [NA atoms x_h][NA atoms x_l]
+    uint8_t *sB = sm + cfg.off_B;   // HS slots of NA atoms: c_h, c_l of successive blocks
+    float *cnr = reinterpret_cast<float *>(sm + cfg.off_cn);  // [2 halves][kCnSlots][kNB] ||c||^2 (+inf: padding)
     uint32_t *bm = reinterpret_cast<uint32_t *>(sm + cfg.off_bm);  // [Kp / 32] group-start masks
-    float *stage = reinterpret_cast<float *>(sm + cfg.off_stage);  // [8 warps x 32 rows][srow]
+    float4 *mrg = reinterpret_cast<float4 *>(sm + cfg.off_mrg);    // [2 tiles][128 rows] the second half's result
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + cfg.off_bar);
-    uint64_t *full_a = bars;                 // [2]
-    uint64_t *empty_a = bars + 2;            // [2]
-    uint64_t *full_b = bars + 4;             // [BS]
-    uint64_t *empty_b = bars + 4 + BS;       // [BS]
-    uint64_t *acc_full = bars + 4 + 2 * BS;  // [2 groups][2 buffers]
-    uint64_t *acc_empty = acc_full + 4;      // [2][2]
-    uint64_t *mma_done = acc_empty + 4;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
+    uint64_t *full_a = bars;               // [2]
+    uint64_t *empty_a = bars + 2;          // [2]
+    uint64_t *acc_full = bars + 4;         // [2 tiles][2 halves]
+    uint64_t *acc_empty = bars + 8;        // [2][2]
+    uint64_t *mfull = bars + 12;           // [2 tiles][4 quadrants]
+    uint64_t *mempty = bars + 20;          // [2][4]
+    uint64_t *cn_full = bars + 28;         // [2 halves][kCnSlots]
+    uint64_t *mma_done = bars + 36;
+    uint64_t *full_b = bars + 37;          // [HS]
+    uint64_t *empty_b = full_b + HS;       // [HS]
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(empty_b + HS);
     float *c2max_s = reinterpret_cast<float *>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the broadcast tells the compiler that the warp index is warp-uniform)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int v = ctrl->v;
     const int K = p.K, G = p.G;
     // this CTA's tiles: blockIdx.x + i * gridDim.x; pairs (2pr, 2pr + 1)
@@ -86,15 +194,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) {
             bar_init(&full_a[i], 1);
-            bar_init(&empty_a[i], 1 + kEpiWarps);  // the MMAs' commit and the norm reads
-        }
-        for (int i = 0; i < BS; ++i) {
-            bar_init(&full_b[i], 1);
-            bar_init(&empty_b[i], 1);
+            bar_init(&empty_a[i], 1);
         }
         for (int i = 0; i < 4; ++i) {
             bar_init(&acc_full[i], 1);
-            bar_init(&acc_empty[i], kEpiWarps);
+            bar_init(&acc_empty[i], kQuadWarps);
+        }
+        for (int i = 0; i < 8; ++i) {
+            bar_init(&mfull[i], 1);
+            bar_init(&mempty[i], 1);
+            bar_init(&cn_full[i], 1);
+        }
+        for (int i = 0; i < HS; ++i) {
+            bar_init(&full_b[i], 1);
+            bar_init(&empty_b[i], 1);
         }
         bar_init(mma_done, 1);
         *c2max_s = 0.f;
@@ -106,31 +219,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // norms (from the pass's split copy), penalties, group-start masks
-    for (int c = threadIdx.x; c < Kp / 32; c += blockDim.x) bm[c] = 0u;
+    // largest norm, group-start masks
+    for (int c = threadIdx.x; c < cfg.Kp / 32; c += blockDim.x) bm[c] = 0u;
     {
         float cm = 0.f;
-        for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
-            const float s2 = k < K ? p.cnorm[k] : INFINITY;
-            if (k < K) cm = fmaxf(cm, s2);
-            cn[k] = s2;
-            pen[k] = 0.f;
-        }
+        for (int k = threadIdx.x; k < K; k += blockDim.x) cm = fmaxf(cm, p.cnorm[k]);
         cm = warp_max(cm);
-        __syncthreads();  // c2max_s, the masks and the penalties initialised
+        __syncthreads();  // c2max_s and the masks initialised
         if (lane == 0 && cm > 0.f) atomicMax(reinterpret_cast<int *>(c2max_s), __float_as_int(cm));
         for (int g = 1 + threadIdx.x; g < G; g += blockDim.x) {
             const int col = p.gstart[g];
-            if ((unsigned)col < (unsigned)Kp) {
-                atomicOr(&bm[col >> 5], 1u << (col & 31));
-                pen[col] = INFINITY;
-            }
+            if ((unsigned)col < (unsigned)cfg.Kp) atomicOr(&bm[col >> 5], 1u << (col & 31));
         }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+
+    // step k of a tile pair takes block blk(k): alternately from the two halves
+    // (the first half has the odd block)
+    auto blk = [&](int k) { return (k & 1) ? hb + (k >> 1) : (k >> 1); };
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA
@@ -140,8 +249,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmch) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmcl) : "memory");
             bool ok = true;
-            int nbl = 0;           // centroid blocks issued
+            int nl = 0;            // half blocks issued
             int ia[2] = {0, 0};    // tiles issued into each A stage
+            int uh[2] = {0, 0};    // blocks of norms issued per half
             for (int pr = 0; pr < npair && ok; ++pr) {
                 for (int g = 0; g < 2 && ok; ++g) {
                     const int i = 2 * pr + g;
@@ -156,25 +266,42 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tma_2d(st + (NA + a) * kAtomBytes, &tml, 64 * a, tile * kTM, &full_a[g]);
                     }
                 }
-                for (int j = 0; j < nb && ok; ++j) {
-                    const int bs = nbl % BS, fb = nbl / BS;
-                    if (fb > 0 && !(ok = bar_wait(&empty_b[bs], (fb - 1) & 1, ctrl))) break;
-                    ++nbl;
-                    uint8_t *sb = sB + (size_t)bs * 2 * NA * kBAtom;
-                    mbar_arrive_expect_tx(&full_b[bs], (uint32_t)(2 * NA * kBAtom));
-                    for (int a = 0; a < NA; ++a) {
-                        tma_2d(sb + a * kBAtom, &tmch, 64 * a, j * kNB, &full_b[bs]);
-                        tma_2d(sb + (NA + a) * kBAtom, &tmcl, 64 * a, j * kNB, &full_b[bs]);
+                for (int k = 0; k < nb && ok; ++k) {
+                    const int j = blk(k), h = k & 1;
+                    for (int part = 0; part < 2; ++part) {
+                        const int bs = nl % HS, fb = nl / HS;
+                        if (fb > 0 && !(ok = bar_wait(&empty_b[bs], (fb - 1) & 1, ctrl))) break;
+                        ++nl;
+                        uint8_t *sb = sB + (size_t)bs * NA * kBAtom;
+                        mbar_arrive_expect_tx(&full_b[bs], (uint32_t)(NA * kBAtom));
+                        for (int a = 0; a < NA; ++a)
+                            tma_2d(sb + a * kBAtom, part ? &tmcl : &tmch, 64 * a, j * kNB, &full_b[bs]);
+                        if (part == 0) {
+                            // the block's norms.  Their slot was last read for this half's
+                            // block four uses ago; the slot of c_h just waited for (at most
+                            // two blocks back) was multiplied after the scan of this half's
+                            // block three uses ago had released its accumulators.
+                            uint64_t *cb = &cn_full[h * kCnSlots + (uh[h] & (kCnSlots - 1))];
+                            mbar_arrive_expect_tx(cb, kNB * 4);
+                            tma_bulk_g2s(cnr + (h * kCnSlots + (uh[h] & (kCnSlots - 1))) * kNB, p.cnorm + j * kNB,
+                                         kNB * 4, cb);
+                            ++uh[h];
+                        }
                     }
                 }
             }
             // drain: the last loads of each barrier have landed before the block exits
             for (int g = 0; g < 2; ++g)
                 if (ia[g] > 0) bar_wait(&full_a[g], (ia[g] - 1) & 1, ctrl);
-            for (int b = 0; b < BS; ++b) {
-                const int uses = nbl > b ? (nbl - b + BS - 1) / BS : 0;
+            for (int b = 0; b < HS; ++b) {
+                const int uses = nl > b ? (nl - b + HS - 1) / HS : 0;
                 if (uses > 0) bar_wait(&full_b[b], (uses - 1) & 1, ctrl);
             }
+            for (int h = 0; h < 2; ++h)
+                for (int b = 0; b < kCnSlots; ++b) {
+                    const int uses = uh[h] > b ? (uh[h] - b + kCnSlots - 1) / kCnSlots : 0;
+                    if (uses > 0) bar_wait(&cn_full[h * kCnSlots + b], (uses - 1) & 1, ctrl);
+                }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA
@@ -183,68 +310,77 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kNB >> 3) << 17) |
                                    ((uint32_t)(kTM >> 4) << 24);
             bool ok = true;
-            int nbl = 0;
+            int nl = 0;
+            // [d_tmem] (+)= A atom rows at sa . B atom rows at sb, over the D coordinates
+            auto product = [&](uint32_t d_tmem, const uint8_t *sa, const uint8_t *sb, bool fresh) {
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ++ks) {
+                    const int a = ks >> 2, jj = ks & 3;
+                    const uint64_t da = desc_sw128(smem_u32(sa + a * kAtomBytes + jj * 32));
+                    const uint64_t db = desc_sw128(smem_u32(sb + a * kBAtom + jj * 32));
+                    const uint32_t acc = !(fresh && ks == 0);
+                    asm volatile(
+                        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+                        "l"(da), "l"(db), "r"(idesc), "r"(acc)
+                        : "memory");
+                }
+            };
+            auto commit = [&](uint64_t *b) {
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 smem_u32(b))
+                             : "memory");
+            };
             for (int pr = 0; pr < npair && ok; ++pr) {
                 const int ng = 2 * pr + 1 < ntile ? 2 : 1;
                 for (int g = 0; g < ng && ok; ++g) ok = bar_wait(&full_a[g], pr & 1, ctrl);
                 if (!ok) break;
                 tc_fence_after();
-                for (int j = 0; j < nb && ok; ++j, ++nbl) {
-                    const int bs = nbl % BS, fb = nbl / BS;
-                    if (!(ok = bar_wait(&full_b[bs], fb & 1, ctrl))) break;
-                    tc_fence_after();
-                    const uint8_t *sb = sB + (size_t)bs * 2 * NA * kBAtom;
-                    const int buf = j & 1;
-                    for (int g = 0; g < ng; ++g) {
-                        const uint32_t uses = acc_uses(pr, j, buf, nb);
-                        if (uses > 0 && !(ok = bar_wait(&acc_empty[g * 2 + buf], (uses - 1) & 1, ctrl))) break;
+                for (int k = 0; k < nb && ok; ++k) {
+                    const int h = k & 1;
+                    const uint32_t uses = (uint32_t)(pr * (h ? nb - hb : hb) + (k >> 1));
+                    for (int part = 0; part < 2 && ok; ++part, ++nl) {
+                        const int bs = nl % HS, fb = nl / HS;
+                        if (!(ok = bar_wait(&full_b[bs], fb & 1, ctrl))) break;
                         tc_fence_after();
-                        const uint32_t d_tmem = tmem + (uint32_t)(g * 2 * kNB + buf * kNB);
-                        const uint8_t *st = sA + (size_t)g * 2 * NA * kAtomBytes;
-#pragma unroll
-                        for (int ks = 0; ks < D / 16; ++ks) {
-                            const int a = ks >> 2, jj = ks & 3;
-                            const uint64_t dah = desc_sw128(smem_u32(st + a * kAtomBytes + jj * 32));
-                            const uint64_t dal = desc_sw128(smem_u32(st + (NA + a) * kAtomBytes + jj * 32));
-                            const uint64_t dbh = desc_sw128(smem_u32(sb + a * kBAtom + jj * 32));
-                            const uint64_t dbl = desc_sw128(smem_u32(sb + (NA + a) * kBAtom + jj * 32));
-                            const uint32_t acc = ks > 0;
-                            asm volatile(
-                                "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %4, %4;\n\t"
-                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %3, q;\n\t"
-                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %6, %2, %3, q;\n\t}" ::"r"(d_tmem),
-                                "l"(dah), "l"(dbh), "r"(idesc), "r"(acc), "l"(dbl), "l"(dal)
-                                : "memory");
+                        const uint8_t *sb = sB + (size_t)bs * NA * kBAtom;
+                        if (part == 0 && uses > 0) {
+                            // the (tile, half) buffers are scanned; at a pair's start also a
+                            // missing second tile's, whose last scan may still read the norms
+                            for (int g = 0; g < (k < 2 ? 2 : ng) && ok; ++g)
+                                ok = bar_wait(&acc_empty[g * 2 + h], (uses - 1) & 1, ctrl);
+                            if (!ok) break;
+                            tc_fence_after();
                         }
-                        asm volatile(
-                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                smem_u32(&acc_full[g * 2 + buf]))
-                            : "memory");
+                        for (int g = 0; g < ng; ++g) {
+                            const uint32_t d_tmem = tmem + (uint32_t)((g * 2 + h) * kNB);
+                            const uint8_t *st = sA + (size_t)g * 2 * NA * kAtomBytes;
+                            if (part == 0) {
+                                product(d_tmem, st, sb, true);                      // x_h c_h
+                                product(d_tmem, st + NA * kAtomBytes, sb, false);   // x_l c_h
+                            } else {
+                                product(d_tmem, st, sb, false);                     // x_h c_l
+                                commit(&acc_full[g * 2 + h]);
+                            }
+                        }
+                        commit(&empty_b[bs]);  // the slot is free once these MMAs have read it
                     }
-                    if (!ok) break;
-                    // the block's stage is free once these MMAs have read it
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                     smem_u32(&empty_b[bs]))
-                                 : "memory");
                 }
                 if (!ok) break;
-                for (int g = 0; g < ng; ++g)
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                     smem_u32(&empty_a[g]))
-                                 : "memory");
+                for (int g = 0; g < ng; ++g) commit(&empty_a[g]);
             }
             // every MMA of this thread is complete before TMEM is freed
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(mma_done))
-                         : "memory");
+            commit(mma_done);
             bar_wait(mma_done, 0, ctrl);
         }
     } else {
         // ------------------------------------------------------- epilogue
-        const int g = (warp - 2) / kEpiWarps;  // epilogue group = tile of the pair
-        const int q = warp & 3;                // TMEM lane quadrant of this warp
+        const int e = warp - 2;
+        const int h = e >> 3;          // half of the centroids
+        const int g = (e >> 2) & 1;    // tile of the pair
+        const int q = warp & 3;        // TMEM lane quadrant of this warp
         const int r = q * 32 + lane;
+        const int pair = g * 4 + q;    // the two warps of a quadrant meet at mfull / mempty
         const float c2max = __fmul_ru(*c2max_s, 1.0f + 1.0f / 1024);
         const float cmax = sqrt_hi(c2max);
         const float ec2 = __fmul_ru(cfg.e_c2, c2max);
@@ -252,88 +388,140 @@ __global__ void __launch_bounds__(kThreads, 1)
         // group bounds, for the exact settle's candidate groups
         const bool bounds = p.algo == KM_ALGO_FILTERED;
         const bool has_lb = p.lb != nullptr;
-        const int wrow = (warp - 2) * 32;      // this warp's rows in the staging area
-        float *row = stage + (size_t)(wrow + lane) * cfg.srow;
-        const uint32_t row_addr = smem_u32(row);
+        const int j0 = h ? hb : 0, nblk = h ? nb - hb : hb;
+        // the group open across the two halves' border: both halves hold a part
+        // of it, and the second half starts in its slot
+        const int gsplit = __shfl_sync(0xffffffffu, p.grp[kNB * hb - 1], 0);
+        Scan4 sc;
+        sc.row = smem_u32(sm + cfg.off_stage) + (uint32_t)((e * 32 + lane) * kSlots) * 4u;
+        sc.t4 = smem_u32(sm + cfg.off_t4) + (uint32_t)(e * 32 + lane) * 16u;
+        const float4 *cnh = reinterpret_cast<const float4 *>(cnr + h * kCnSlots * kNB);
         unsigned long long c_changed = 0, c_dist = 0;
         for (int pr = 0; pr < npair; ++pr) {
             const int i = 2 * pr + g;
             if (i >= ntile) break;
             const int tile = (int)blockIdx.x + i * (int)gridDim.x;
-            if (!__all_sync(0xffffffffu, bar_wait(&full_a[g], pr & 1, ctrl))) break;
-            const uint8_t *st = sA + (size_t)g * 2 * NA * kAtomBytes;
             const int64_t n = (int64_t)tile * kTM + r;
             const bool valid = n < p.N;
-            const int old = valid ? (first ? -1 : p.label[n]) : -1;
             const float xn = valid ? p.xnorm[n] : 0.f;
-            __syncwarp();
-            if (lane == 0) bar_arrive(&empty_a[g]);
             const float xlo = __fmul_rd(xn, cfg.xn_lo), xup = __fmul_ru(xn, cfg.xn_hi);
             const float R = __fadd_ru(sqrt_hi(xup), cmax);  // bounds ||x - mu|| + ||c - mu||
             const float E = __fmaf_ru(p.e_cen, __fmul_ru(R, R), __fmaf_ru(cfg.e_lin, __fmul_ru(sqrt_hi(xup), cmax), ec2));
-            const float twoE = __fmul_ru(2.f, E);
-            const int64_t n0 = (int64_t)tile * kTM + q * 32;
-            const int rows = (int)max((int64_t)0, min((int64_t)32, p.N - n0));
+            float *lbrow = p.lb + n * p.Gp;
+            const bool store = has_lb && valid;
+            auto bound_of = [&](float t) { return t == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xlo, t), E)); };
 
-            // converts this thread's staged minima [0, cnt) in place, then the
-            // warp writes them to lb as groups gfirst.. of its 32 rows
-            int gfirst = 0;
-            auto flush = [&](int cnt) {
-                for (int s = 0; s < cnt; ++s) {
-                    const float tg = row[s];
-                    row[s] = tg == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xlo, tg), E));
+            sc.b1 = sc.b2 = sc.gm = INFINITY;
+            sc.c4 = kNB * j0;
+            sc.pend = h ? (gsplit & 3) : 0;
+            int gq = h ? (gsplit & ~3) : 0;  // group of slot 0 (a multiple of four)
+            float gsp = INFINITY;            // second half: its part of group gsplit
+            bool head = h != 0;              // its slots still start with that group's four
+            // slots [0, cnt) of the four that group gsplit lies in (second half)
+            auto head_slots = [&](int cnt) {
+                const int s0 = gsplit & 3;
+                gsp = lds_f(sc.row + 4u * (uint32_t)s0);
+                for (int s = s0 + 1; s < cnt; ++s) {
+                    const float b = bound_of(lds_f(sc.row + 4u * (uint32_t)s));
+                    if (store) lbrow[gq + s] = b;
                 }
-                __syncwarp();
-                const float *st0 = stage + (size_t)wrow * cfg.srow;
-                for (int e = lane; e < rows * cnt; e += 32) {
-                    const int rw = e / cnt, s = e - rw * cnt;
-                    if (has_lb && gfirst + s < G) p.lb[(n0 + rw) * p.Gp + gfirst + s] = st0[rw * cfg.srow + s];
-                }
-                __syncwarp();
-                gfirst += cnt;
+                head = false;
             };
-
-            RowScan sc;
-            sc.init(row);
-            for (int j = 0; j < nb; ++j) {
-                const int buf = j & 1;
-                const uint32_t uses = acc_uses(pr, j, buf, nb);
-                if (!__all_sync(0xffffffffu, bar_wait(&acc_full[g * 2 + buf], uses & 1, ctrl))) {
-                    gfirst = -1;
-                    break;
-                }
+            bool ok = true;
+            for (int b = 0; b < nblk; ++b) {
+                const uint32_t u = (uint32_t)(pr * nblk + b);
+                ok = __all_sync(0xffffffffu, bar_wait(&acc_full[g * 2 + h], u & 1, ctrl) &&
+                                                 bar_wait(&cn_full[h * kCnSlots + (u & (kCnSlots - 1))],
+                                                          (u / kCnSlots) & 1, ctrl));
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t tb = tmem + (uint32_t)(g * 2 * kNB + buf * kNB) + ((uint32_t)(q * 32) << 16);
-                {
-                    uint32_t ra[32], rb[32];
-                    tmem_ld32_async(tb, ra);
-#pragma unroll 1
-                    for (int c0 = 0; c0 < kNB; c0 += 64) {
-                        tmem_wait32(ra);
-                        tmem_ld32_async(tb + c0 + 32, rb);
-                        scan_one(sc, ra, j * kNB + c0, cn, pen);
-                        tmem_wait32(rb);
-                        if (c0 + 64 < kNB) {
-                            tmem_ld32_async(tb + c0 + 64, ra);
-                        } else {  // the accumulators are read: release them
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) bar_arrive(&acc_empty[g * 2 + buf]);
+                const uint32_t tb = tmem + (uint32_t)((g * 2 + h) * kNB) + ((uint32_t)(q * 32) << 16);
+                const float4 *cn4 = cnh + (u & (kCnSlots - 1)) * (kNB / 4);
+                const int cb = kNB * (j0 + b);
+                // four columns, then -- when four groups have closed -- their bounds to lb
+                auto sixteen = [&](const uint32_t(&acc)[16], int c0) {
+                    // (a broadcast, so that the compiler knows the mask to be warp-uniform)
+                    const uint32_t m16 = __shfl_sync(0xffffffffu, bm[(cb + c0) >> 5], 0) >> ((cb + c0) & 31);
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        const uint32_t nib = (m16 >> j) & 15u;
+                        sc.four(&acc[j], cn4[(c0 + j) >> 2], nib, cb + c0 + j);
+                        if (nib && sc.pend >= 4) {  // warp-uniform
+                            if (head) {
+                                head_slots(4);
+                            } else {  // whole groups, never empty: a finite minimum
+                                float4 o;
+                                o.x = sqrt_lo(__fsub_rd(__fadd_rd(xlo, lds_f(sc.row)), E));
+                                o.y = sqrt_lo(__fsub_rd(__fadd_rd(xlo, lds_f(sc.row + 4)), E));
+                                o.z = sqrt_lo(__fsub_rd(__fadd_rd(xlo, lds_f(sc.row + 8)), E));
+                                o.w = sqrt_lo(__fsub_rd(__fadd_rd(xlo, lds_f(sc.row + 12)), E));
+                                if (store) *reinterpret_cast<float4 *>(lbrow + gq) = o;
+                            }
+                            gq += 4;
+                            sc.pend -= 4;
+                            for (int s = 0; s < sc.pend; ++s) {
+                                const float t = lds_f(sc.row + 16u + 4u * (uint32_t)s);
+                                asm volatile("st.shared.f32 [%0], %1;" ::"r"(sc.row + 4u * (uint32_t)s), "f"(t));
+                            }
                         }
-                        scan_one(sc, rb, j * kNB + c0 + 32, cn, pen);
-                        // groups closed in these 64 columns: slots [0, (rp - row) / 4)
-                        flush((int)((sc.rp - row_addr) >> 2));
-                        sc.rp = row_addr;
                     }
+                };
+                uint32_t ra[16], rb[16];
+                tmem_ld16_async(tb, ra);
+#pragma unroll 1
+                for (int c0 = 0; c0 < kNB; c0 += 32) {
+                    tmem_wait16(ra);
+                    tmem_ld16_async(tb + c0 + 16, rb);
+                    sixteen(ra, c0);
+                    tmem_wait16(rb);
+                    if (c0 + 32 < kNB) {
+                        tmem_ld16_async(tb + c0 + 32, ra);
+                    } else {  // the accumulators are read: release them
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) bar_arrive(&acc_empty[g * 2 + h]);
+                    }
+                    sixteen(rb, c0 + 16);
                 }
             }
-            if (gfirst < 0) break;  // a wait timed out (error recorded)
-            sc.close();
-            flush(1);  // the last group
-            float b1, b2;
-            int i1;
-            sc.result(b1, i1, b2);
-            const float thr = __fadd_ru(b1, twoE);
+            if (!ok) break;  // a wait timed out (error recorded)
+            // the open group's minimum
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(sc.row + 4u * (uint32_t)sc.pend), "f"(sc.gm) : "memory");
+            ++sc.pend;
+            if (h) {
+                if (head) {
+                    head_slots(sc.pend);
+                } else {
+                    for (int s = 0; s < sc.pend; ++s) {
+                        const float b = bound_of(lds_f(sc.row + 4u * (uint32_t)s));
+                        if (store) lbrow[gq + s] = b;
+                    }
+                }
+                const int ci = sc.winner();
+                if (pr > 0 && !__all_sync(0xffffffffu, bar_wait(&mempty[pair], (pr - 1) & 1, ctrl))) break;
+                mrg[g * kTM + r] = make_float4(sc.b1, sc.b2, __int_as_float(ci), gsp);
+                __syncwarp();
+                if (lane == 0) bar_arrive(&mfull[pair]);  // with the bounds stored above
+                continue;
+            }
+            const int old = valid ? (first ? -1 : p.label[n]) : -1;
+            const int ai = sc.winner();
+            if (!__all_sync(0xffffffffu, bar_wait(&mfull[pair], pr & 1, ctrl))) break;
+            const float4 mg = mrg[g * kTM + r];
+            __syncwarp();
+            if (lane == 0) bar_arrive(&mempty[pair]);
+            for (int s = 0; s < sc.pend; ++s) {  // the last of them is gsplit
+                float t = lds_f(sc.row + 4u * (uint32_t)s);
+                if (s == sc.pend - 1) t = fminf(t, mg.w);
+                const float b = bound_of(t);
+                if (store) lbrow[gq + s] = b;
+            }
+            // the first half holds the lower indices: it wins ties
+            const bool bw = mg.x < sc.b1;
+            const float b1 = bw ? mg.x : sc.b1;
+            const int i1 = bw ? __float_as_int(mg.z) : ai;
+            const float b2 = fminf(fminf(sc.b2, mg.y), fmaxf(sc.b1, mg.x));
+            const float thr = __fadd_ru(b1, __fmul_ru(2.f, E));
             const bool need = valid && b2 <= thr;
             const unsigned nm = __ballot_sync(0xffffffffu, need);
             if (need) {
@@ -355,8 +543,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!need) p.label[n] = best;
                 // the winner's group excludes the winner: every other column is
                 // at least the runner-up; the smallest group bound is that bound
-                const float lw = b2 == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xlo, b2), E));
-                if (has_lb) p.lb[n * p.Gp + group_of(bm, best)] = lw;
+                const float lw = bound_of(b2);
+                if (has_lb) lbrow[p.grp[best]] = lw;
                 if (bounds) {
                     p.lbg[n] = lw;
                     p.u[n] = sqrt_hi(__fadd_ru(__fadd_ru(xup, b1), E));
@@ -398,40 +586,30 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // C -> (c_h, c_l) bfloat16 copies (K padded to Kp with zero rows) and the
-// FP32 norms, as the kernel above reads them; gated like the dense pass
+// FP32 norms (padding: +inf), as the kernel above reads them; gated like the
+// dense pass.  A warp per centroid.
 __global__ void k_split_c(Params p, int Kp, int respect_done, int if_dense) {
     Ctrl *ctrl = p.ctrl;
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;
     if (if_dense && !*(volatile int *)&ctrl->dense_mode) return;
     const int D = p.D, Dt = tc_dim(p.D);
-    const int64_t total = (int64_t)Kp * Dt;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(i / Dt), d = (int)(i - (int64_t)k * Dt);
-        float x = (k < p.K && d < D) ? p.C[(size_t)k * p.Dp + d] : 0.f;  // zero padding
-        if (p.mu && k < p.K && d < D) x = __fsub_rn(x, p.mu[d]);  // c - mu
-        const __nv_bfloat16 h = __float2bfloat16_rn(x);
-        const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
-        p.Ch[i] = __bfloat16_as_ushort(h);
-        p.Cl[i] = __bfloat16_as_ushort(l);
-    }
-    // norms: one warp per centroid, the same two-accumulator FP32 sum as the
-    // single-block kernel (even / odd coordinates, then added)
     const int lane = threadIdx.x & 31;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t k = wid; k < p.K; k += nw) {
-        if (lane == 0) {
-            const float *c = p.C + (size_t)k * p.Dp;
-            float a0 = 0.f, a1 = 0.f;
-            for (int d = 0; d + 1 < D; d += 2) {  // ||c - mu||^2, the values split above
-                const float v0 = p.mu ? __fsub_rn(c[d], p.mu[d]) : c[d];
-                const float v1 = p.mu ? __fsub_rn(c[d + 1], p.mu[d + 1]) : c[d + 1];
-                a0 = fmaf(v0, v0, a0);
-                a1 = fmaf(v1, v1, a1);
-            }
-            p.cnorm[k] = a0 + a1;
+    const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int k = wid; k < Kp; k += nw) {
+        float s2 = 0.f;
+        for (int d = lane; d < Dt; d += 32) {
+            float x = (k < p.K && d < D) ? p.C[(size_t)k * p.Dp + d] : 0.f;  // zero padding
+            if (p.mu && k < p.K && d < D) x = __fsub_rn(x, p.mu[d]);  // c - mu
+            const __nv_bfloat16 h = __float2bfloat16_rn(x);
+            const __nv_bfloat16 l = __float2bfloat16_rn(x - __bfloat162float(h));
+            p.Ch[(size_t)k * Dt + d] = __bfloat16_as_ushort(h);
+            p.Cl[(size_t)k * Dt + d] = __bfloat16_as_ushort(l);
+            s2 = fmaf(x, x, s2);  // ||c - mu||^2 of the values split
         }
+        s2 = warp_sum(s2);
+        if (lane == 0) p.cnorm[k] = k < p.K ? s2 : INFINITY;
     }
 }
 
@@ -441,6 +619,7 @@ bool plan_b(const Params &p, size_t smem_limit, TcbCfg &cfg, size_t &smem) {
     cfg.Kp = ((p.K + kNB - 1) / kNB) * kNB;
     if (cfg.Kp > kMaxKp) return false;
     cfg.nb = cfg.Kp / kNB;
+    cfg.hb = (cfg.nb + 1) / 2;
     // groups that 64 columns (the span between two flushes of the staged
     // minima) can close under the contiguous grouping j -> j G / K, plus the
     // one still open
@@ -451,30 +630,34 @@ bool plan_b(const Params &p, size_t smem_limit, TcbCfg &cfg, size_t &smem) {
         const int g0 = (int)(c0 * p.G / p.K), g1 = (int)(c1 * p.G / p.K);
         most = std::max(most, g1 - g0 + 1);
     }
-    cfg.srow = (most + 2) | 1;
+    const int srow = (most + 2) | 1;
     const size_t NA = Dt / 64;
-    const size_t a_stage = 2 * NA * (size_t)kAtomBytes;
-    const size_t b_stage = 2 * NA * (size_t)kBAtom;
-    const size_t tables = (size_t)cfg.Kp * 8 + (size_t)cfg.Kp / 32 * 4;
-    const size_t stage_bytes = (size_t)kPairs * kEpiWarps * 32 * cfg.srow * 4;
-    const size_t bars = (4 + 2 * 2 + 8 + 1) * 8 + 16;
-    auto need = [&](int bst) { return 1024 + 2 * a_stage + bst * b_stage + tables + 16 + stage_bytes + bars + 16; };
-    cfg.bst = need(2) <= smem_limit ? 2 : 1;
-    if (need(cfg.bst) > smem_limit) return false;
-    size_t off = 0;
-    cfg.off_A = (uint32_t)off;
-    off += 2 * a_stage;
+    const size_t a_bytes = 2 * 2 * NA * (size_t)kAtomBytes;
+    const size_t half = NA * (size_t)kBAtom;
+    // the shapes this engine takes: a bound on Kp and on the groups that 64
+    // columns hold (beyond it the FP32 engine runs)
+    if (1024 + a_bytes + 2 * half + (size_t)cfg.Kp * 8 + (size_t)cfg.Kp / 32 * 4 + 256 * (size_t)srow * 4 + 184 >
+        smem_limit)
+        return false;
+    size_t off = a_bytes;
     cfg.off_B = (uint32_t)off;
-    off += cfg.bst * b_stage;
+    cfg.hs = 4;
+    const size_t fixed = 2 * kCnSlots * kNB * 4 + ((size_t)cfg.Kp / 32 * 4 + 15) / 16 * 16 +
+                         (size_t)kEpi * 32 * (kSlots * 4 + 16) + 2 * kTM * 16 + (37 + 2 * 4) * 8 + 16;
+    if (1024 + off + 4 * half + fixed > smem_limit) cfg.hs = 2;
+    off += cfg.hs * half;
     cfg.off_cn = (uint32_t)off;
-    off += (size_t)cfg.Kp * 8;
+    off += 2 * kCnSlots * kNB * 4;
     cfg.off_bm = (uint32_t)off;
-    off += ((size_t)cfg.Kp / 32 * 4 + 15) & ~size_t(15);
+    off += ((size_t)cfg.Kp / 32 * 4 + 15) / 16 * 16;
+    cfg.off_t4 = (uint32_t)off;
+    off += (size_t)kEpi * 32 * 16;
+    cfg.off_mrg = (uint32_t)off;
+    off += 2 * kTM * 16;
     cfg.off_stage = (uint32_t)off;
-    off += stage_bytes;
-    off = (off + 7) & ~size_t(7);
-    cfg.off_bar = (uint32_t)off;
-    off += (4 + 2 * cfg.bst + 8 + 1) * 8 + 16;
+    off += (size_t)kEpi * 32 * kSlots * 4;
+    cfg.off_bar = (uint32_t)off;  // a multiple of 8: every part above is a multiple of 16
+    off += (37 + 2 * cfg.hs) * 8 + 16;
     smem = 1024 + off;
     if (smem > smem_limit) return false;
     cfg.num_tiles = (int)((p.N + kTM - 1) / kTM);
@@ -516,8 +699,7 @@ cudaError_t launch_b(const Params &p, cudaStream_t s, int first, int respect_don
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     {
-        const int64_t total = (int64_t)cfg.Kp * Dt;
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, (int64_t)num_sms * 4));
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((cfg.Kp + 7) / 8, (int64_t)num_sms * 4));
         count_launch();
         k_split_c<<<(unsigned)grid, 256, 0, s>>>(p, cfg.Kp, respect_done, if_dense);
         cudaError_t e = cudaGetLastError();

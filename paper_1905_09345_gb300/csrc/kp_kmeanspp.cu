@@ -16,22 +16,60 @@
 //            to W); the centre is the first point (in index order) whose
 //            running sum of q exceeds T; W = 0: floor(u_j * N); first: floor(u_0 * N).
 //
-// Per centre: k_pp_update (the new centre's FP64 distances, the running
-// minimum and its maximum), k_pp_blocksum (integer weights summed per chunk of
-// 1024 points), k_pp_pick (one block: the chunk holding T, then the point in
-// it; copies the point to the output centroids).
+// FP64 runs at 1/64 of the FP32 rate, so D(x)^2 is kept in FP64 but evaluated
+// only where it can change: per centre an FP32 distance with a rigorous error
+// bound settles, for all but about N / j of the points after j centres, that
+// the new centre is not nearer.  The others are collected per block (FP64
+// costs a warp the same for one lane as for 32) and get their FP64 distance;
+// the conversions of x to FP64, which share that pipe, are made on the integer
+// one.  What is left is one read of X per centre.
+//
+// The weights need no FP64 either: Q(x) = floor(D(x)^2 2^(64 - e0)), 64 bits
+// with 2^e0 > max D^2 at the time e0 was set, is made from the bits of D^2
+// when that changes, and for max D^2 in [2^(e-1), 2^e), e = e0 - k <= e0,
+// q(x) = Q(x) >> (32 - k) exactly (a floor of a floor).  k, the leading zeros
+// of max Q, is the first occupied bin of a histogram of leading zeros.  The
+// histogram and the chunk sums of q change only with the points that change;
+// a second set of sums is kept for k + 1, so that the usual step of k costs a
+// re-summation during the next sweep only.
+//
+// One launch per centre (k_pp_step): the distances to the centre drawn last,
+// the sums, and -- in the last block to finish -- the next draw: the chunk
+// holding T, then the point in it, copied to the output centroids.  Every
+// block owns a run of chunks.
+// Measured on GB300 (1,048,576 x 32, K = 128): 337 us per centre and 43.9 ms in
+// all with FP64 distances to every point; now 46 us once half a dozen centres
+// stand (21 the read of X, at 6.4 TB/s; 8 the FP64 distances; 8 the draw; 5
+// the launch) and 7.0 ms in all.  3,878 x 100: 45 -> 22 us per centre.
+#include <cmath>
+
 #include "kp_common.cuh"
 
 namespace kp {
 namespace {
 
-constexpr int kPPChunk = 1024;  // points per block sum
 constexpr int kPPThreads = 256;
+constexpr int kPPWarps = kPPThreads / 32;
+// blocks per SM of the sweep and row groups a warp has in flight: 96 KB of rows
+// per SM either way; 4 blocks with 4 or 6 groups measured 7.3 ms for the job
+// above, 3 with 8 groups 7.0 ms (fewer spills)
+constexpr int kPPBlocks = 3, kPPU = 8;
+constexpr int kPPSegment = 2048;   // points filtered between two looks at the list
+constexpr int kPPList = 2 * kPPSegment;
+constexpr int kPPMaxChunks = 4096; // chunk size: the power of two >= 32 that gives at most so many
+constexpr int kPPBins = 65;        // leading zeros of Q (64: zero)
+constexpr unsigned long long kPPNaN = ~0ull;  // Q of a point whose D^2 is NaN: weight 0
 
 struct PPState {
-    unsigned long long wmax;  // bit pattern of max D^2 (non-negative doubles order as their bits)
+    unsigned long long wmax;  // after the first centre: bit pattern of max D^2 (doubles >= 0 order as their bits)
     long long pick;           // the centre chosen last
     long long err;            // nonzero: an index out of range was produced
+    int e0;                   // scale of Q
+    int k;                    // leading zeros of max Q when the last draw was made
+    int cur;                  // sums[cur]: of the weights at k; sums[cur ^ 1]: at k + 1
+    int resum;                // sums[cur ^ 1] must be made anew
+    unsigned ticket;          // blocks done
+    int hist[kPPBins];        // points by leading zeros of Q
 };
 
 __device__ __forceinline__ long long uniform_index(double u, long long N) {
@@ -39,72 +77,82 @@ __device__ __forceinline__ long long uniform_index(double u, long long N) {
     return i < 0 ? 0 : (i >= N ? N - 1 : i);
 }
 
-// 2^(32 - e) for wmax = m 2^e, m in [0.5, 1) (wmax normal: a nonzero squared
-// distance between FP32 points is at least 2^-298)
-__device__ __forceinline__ double weight_scale(unsigned long long wbits) {
-    const int e = (int)((wbits >> 52) & 0x7ff) - 1022;
-    return __longlong_as_double((long long)(1023 + 32 - e) << 52);
+// e with d = m 2^e, m in [0.5, 1) (d normal: a nonzero squared distance between
+// FP32 points is at least 2^-298)
+__device__ __forceinline__ int exponent_of(unsigned long long bits) { return (int)((bits >> 52) & 0x7ff) - 1022; }
+
+// floor(d 2^(64 - e0)) for 0 <= d < 2^e0, from the bits of d
+__device__ __forceinline__ unsigned long long quant(double d, int e0) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+    const int ex = (int)(bits >> 52);
+    if (ex >= 0x7ff && d != d) return kPPNaN;
+    if (ex == 0) return 0ull;  // zero (or below every weight)
+    const unsigned long long m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int sh = ex - 1011 - e0;  // d = m 2^(ex - 1075)
+    return sh >= 0 ? m << min(sh, 11) : (sh > -64 ? m >> -sh : 0ull);
+}
+// the weight at e = e0 - k; k > 32 only when every Q is zero
+__device__ __forceinline__ unsigned long long weight(unsigned long long q, int k) {
+    return q == kPPNaN ? 0ull : q >> (32 - min(k, 32));
+}
+__device__ __forceinline__ int bin_of(unsigned long long q) { return q ? __clzll((long long)q) : 64; }
+
+// float to double on the integer pipe, exact for zero and normal numbers;
+// others set `odd` (no branch, so that several conversions and products are in
+// flight at once)
+__device__ __forceinline__ double widen(float x, bool &odd) {
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    odd |= m != 0u && m - 0x00800000u >= 0x7f000000u;
+    const unsigned h = m == 0u ? 0u : (m >> 3) + 0x38000000u;
+    return __hiloint2double((int)((u & 0x80000000u) | h), (int)(u << 29));
 }
 
-__device__ __forceinline__ unsigned long long weight(double d, double scale) {
-    return (unsigned long long)floor(__dmul_rn(d, scale));  // exact: a power-of-two scaling
-}
-
-__global__ void k_pp_first(const double *u, long long N, PPState *st) {
-    st->pick = uniform_index(u[0], N);
-    st->wmax = 0ull;
-    st->err = 0;
-}
-
-
-// dmin[n] = min(dmin[n], D(x_n, X[pick])^2); wmax = max over n (one atomic per warp)
-__global__ void __launch_bounds__(kPPThreads) k_pp_update(const float *X, long long N, int D, double *dmin,
-                                                         PPState *st, int first) {
-    const long long pick = st->pick;
-    const float *c = X + pick * D;
-    double m = 0.0;
-    for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < N;
-         n += (long long)gridDim.x * blockDim.x) {
-        const float *x = X + n * D;
-        double s = 0.0;
-        for (int i = 0; i < D; ++i) {
-            const double t = __dsub_rn((double)x[i], (double)c[i]);
+// FP64 squared distance, i ascending, no fused multiply-add (VEC: D a multiple
+// of 4, rows 16-byte aligned); c in FP64
+template <bool VEC>
+__device__ __forceinline__ double dist2(const float *x, const double *c, int D) {
+    constexpr int B = 8;  // coordinates whose squares are formed before they are summed
+    double s = 0.0;
+    bool odd = false;
+    int i = 0;
+    for (; i + B <= D; i += B) {
+        float xv[B];
+        if constexpr (VEC) {
+#pragma unroll
+            for (int k = 0; k < B; k += 4) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(x + i + k));
+                xv[k] = v.x;
+                xv[k + 1] = v.y;
+                xv[k + 2] = v.z;
+                xv[k + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < B; ++k) xv[k] = __ldg(x + i + k);
+        }
+        double t[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) t[k] = __dsub_rn(widen(xv[k], odd), c[i + k]);
+#pragma unroll
+        for (int k = 0; k < B; ++k) t[k] = __dmul_rn(t[k], t[k]);
+#pragma unroll
+        for (int k = 0; k < B; ++k) s = __dadd_rn(s, t[k]);
+    }
+    for (; i < D; ++i) {
+        const double t = __dsub_rn(widen(__ldg(x + i), odd), c[i]);
+        s = __dadd_rn(s, __dmul_rn(t, t));
+    }
+    if (odd) {  // a subnormal, infinite or NaN coordinate
+        s = 0.0;
+        for (i = 0; i < D; ++i) {
+            const double t = __dsub_rn((double)__ldg(x + i), c[i]);
             s = __dadd_rn(s, __dmul_rn(t, t));
         }
-        const double d = first ? s : fmin(dmin[n], s);
-        dmin[n] = d;
-        m = fmax(m, d);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(&st->wmax, (unsigned long long)__double_as_longlong(m));
+    return s;
 }
 
-// bsum[b] = sum of q over points [b * 1024, (b + 1) * 1024)
-__global__ void __launch_bounds__(kPPThreads) k_pp_blocksum(const double *dmin, long long N, const PPState *st,
-                                                           unsigned long long *bsum) {
-    __shared__ unsigned long long ws[kPPThreads / 32];
-    const unsigned long long wbits = st->wmax;
-    const double scale = wbits ? weight_scale(wbits) : 0.0;
-    const long long n0 = (long long)blockIdx.x * kPPChunk;
-    unsigned long long acc = 0;
-    if (wbits)
-        for (int k = threadIdx.x; k < kPPChunk; k += blockDim.x) {
-            const long long n = n0 + k;
-            if (n < N) acc += weight(dmin[n], scale);
-        }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int w = 0; w < kPPThreads / 32; ++w) t += ws[w];
-        bsum[blockIdx.x] = t;
-    }
-}
-
-// inclusive scan of one value per thread across a block of 1024 threads
+// inclusive scan of one value per thread across the block
 __device__ __forceinline__ unsigned long long block_scan_incl(unsigned long long v, unsigned long long *sh,
                                                               unsigned long long *total) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -115,114 +163,476 @@ __device__ __forceinline__ unsigned long long block_scan_incl(unsigned long long
     }
     if (lane == 31) sh[w] = v;
     __syncthreads();
-    if (w == 0) {
-        unsigned long long s = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0ull;
+    unsigned long long before = 0, all = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long t = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += t;
-        }
-        sh[lane] = s;  // inclusive sums of the warp totals
+    for (int i = 0; i < kPPWarps; ++i) {
+        if (i < w) before += sh[i];
+        all += sh[i];
     }
+    if (total) *total = all;
     __syncthreads();
-    const unsigned long long out = v + (w > 0 ? sh[w - 1] : 0ull);
-    if (total) *total = sh[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return out;
+    return v + before;
+}
+__device__ __forceinline__ unsigned long long warp_sum_u(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ unsigned long long warp_max_u(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
-// one block of 1024 threads: the draw of centre j
-__global__ void __launch_bounds__(1024) k_pp_pick(const float *X, long long N, int D, const double *dmin,
-                                                 const unsigned long long *bsum, long long nb, const double *u,
-                                                 int j, PPState *st, float *C, long long *idx) {
-    __shared__ unsigned long long sh[32];
-    __shared__ long long s_block;
+struct PPArgs {
+    const float *X;
+    long long N;
+    int D;
+    double *dmin;                 // N: D(x)^2
+    unsigned long long *Q;        // N
+    float *ub;                    // N: D(x)^2 rounded up to FP32 (the filter's bound)
+    unsigned long long *sums[2];  // chunk sums of the weights
+    int csh;                      // log2 of the chunk size
+    long long nb;                 // chunks
+    const double *u;
+    PPState *st;
+    float *C;
+    long long *idx;
+};
+
+// the chunks of this block: [first, last)
+__device__ __forceinline__ long long chunk0(const PPArgs &a, unsigned blk) {
+    return (long long)blk * a.nb / gridDim.x;
+}
+
+// centre j is point `pick`: its row to C, its index to idx
+__device__ __forceinline__ void take_centre(const PPArgs &a, int j, long long pick) {
+    for (int i = threadIdx.x; i < a.D; i += kPPThreads) a.C[(long long)j * a.D + i] = a.X[pick * a.D + i];
+    if (threadIdx.x == 0) {
+        a.idx[j] = pick;
+        a.st->pick = pick;
+    }
+}
+
+// The last block to finish (whole block): the draw of centre j from the chunk
+// sums.  Every other block's results are visible (fence and ticket).
+__device__ void draw(const PPArgs &a, int j) {
+    __shared__ unsigned long long sh[kPPWarps];
     __shared__ unsigned long long s_before;
-    __shared__ long long s_pick;
-    const int tid = threadIdx.x;
-    // per-thread run of chunk sums, scanned across the block
-    const long long per = (nb + 1023) / 1024;
-    const long long b0 = tid * per, b1 = min(b0 + per, nb);
-    unsigned long long run = 0;
-    for (long long b = b0; b < b1; ++b) run += bsum[b];
-    unsigned long long W = 0;
-    const unsigned long long incl = block_scan_incl(run, sh, &W);
+    __shared__ long long s_block, s_pick;
+    __shared__ int s_k;
+    __shared__ unsigned long long s_sum[kPPMaxChunks + kPPMaxChunks / 16];
+    constexpr int kPer = kPPMaxChunks / kPPThreads;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    PPState *st = a.st;
+    int cur = st->cur;
+    const int kg = st->k;
+    // the sums at k, read before k is known to stand
+    unsigned long long v[kPer];
+    auto load_sums = [&](const unsigned long long *bs) {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const long long b = i * kPPThreads + tid;
+            v[i] = b < a.nb ? __ldcg(bs + b) : 0ull;
+        }
+    };
+    load_sums(a.sums[cur]);
+    if (warp == 0) {  // the first occupied bin
+        const int h0 = __ldcg(&st->hist[lane]), h1 = __ldcg(&st->hist[32 + lane]);
+        const unsigned b0 = __ballot_sync(0xffffffffu, h0 != 0), b1 = __ballot_sync(0xffffffffu, h1 != 0);
+        if (lane == 0) s_k = b0 ? __ffs(b0) - 1 : (b1 ? 31 + __ffs(b1) : 64);
+    }
     if (tid == 0) {
         s_block = -1;
-        s_pick = N;
+        s_pick = a.N;
     }
     __syncthreads();
-    if (W == 0) {  // every weight is zero: a uniform draw
-        if (tid == 0) s_pick = uniform_index(u[j], N);
-    } else {
-        unsigned long long T = (unsigned long long)floor(__dmul_rn(u[j], (double)W));
-        if (T >= W) T = W - 1;
-        const unsigned long long excl = incl - run;
-        if (excl <= T && T < incl) {  // exactly one thread: its run holds T
-            unsigned long long acc = excl;
-            for (long long b = b0; b < b1; ++b) {
-                if (acc + bsum[b] > T) {
-                    s_block = b;
-                    s_before = acc;
-                    break;
+    int kt = s_k, resum = 0;
+    if (kt == kg + 1 && kt <= 32) {
+        cur ^= 1;
+        resum = 1;
+    } else if (kt != kg) {
+        // the maximum fell by more than a factor of two: both sums are made anew
+        // (with a new Q when max Q has lost its leading bits)
+        int e0 = st->e0;
+        const bool requant = kt > 32;
+        if (requant) {
+            unsigned long long m = 0;
+            for (long long n = tid; n < a.N; n += kPPThreads) {
+                const double d = __ldcg(a.dmin + n);
+                if (d == d) m = max(m, (unsigned long long)__double_as_longlong(d));
+            }
+            m = warp_max_u(m);
+            if (lane == 0) sh[warp] = m;
+            if (tid < kPPBins) st->hist[tid] = 0;
+            __syncthreads();
+            m = 0;
+            for (int w = 0; w < kPPWarps; ++w) m = max(m, sh[w]);
+            kt = m ? 0 : 64;  // all zero: it stays so
+            e0 = m ? exponent_of(m) : e0;
+            __syncthreads();
+        }
+        for (long long b = warp; b < a.nb; b += kPPWarps) {
+            unsigned long long s0 = 0, s1 = 0;
+            const long long n1 = min(a.N, (b + 1) << a.csh);
+            for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
+                unsigned long long q;
+                if (requant) {
+                    q = quant(__ldcg(a.dmin + n), e0);
+                    a.Q[n] = q;
+                    if (q != kPPNaN) atomicAdd(&st->hist[bin_of(q)], 1);
+                } else {
+                    q = __ldcg(a.Q + n);
                 }
-                acc += bsum[b];
+                s0 += weight(q, kt);
+                s1 += weight(q, kt + 1);
+            }
+            s0 = warp_sum_u(s0);
+            s1 = warp_sum_u(s1);
+            if (lane == 0) {
+                a.sums[cur][b] = s0;
+                a.sums[cur ^ 1][b] = s1;
+            }
+        }
+        if (tid == 0) st->e0 = e0;
+        __threadfence();
+        __syncthreads();
+    }
+    if (kt != kg) load_sums(a.sums[cur]);
+    // per-thread run of consecutive chunk sums, scanned across the block
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int b = i * kPPThreads + tid;
+        s_sum[b + (b >> 4)] = v[i];
+    }
+    __syncthreads();
+    const int per = (int)((a.nb + kPPThreads - 1) / kPPThreads);  // at most kPer
+    const int b0 = tid * per;
+    unsigned long long run = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int b = b0 + i;
+        v[i] = i < per && b < a.nb ? s_sum[b + (b >> 4)] : 0ull;
+        run += v[i];
+    }
+    unsigned long long W = 0;
+    const unsigned long long incl = block_scan_incl(run, sh, &W);
+    if (W == 0) {  // every weight is zero: a uniform draw
+        if (tid == 0) s_pick = uniform_index(a.u[j], a.N);
+    } else {
+        unsigned long long T = (unsigned long long)floor(__dmul_rn(a.u[j], (double)W));
+        if (T >= W) T = W - 1;
+        unsigned long long acc = incl - run;
+        if (acc <= T && T < incl) {  // exactly one thread: its run holds T
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                if (acc <= T && acc + v[i] > T) {
+                    s_block = b0 + i;
+                    s_before = acc;
+                }
+                acc += v[i];
             }
         }
         __syncthreads();
         const long long b = s_block;
         if (b >= 0) {
-            const double scale = weight_scale(st->wmax);
-            const long long n = b * kPPChunk + tid;
-            const unsigned long long q = n < N ? weight(dmin[n], scale) : 0ull;
-            const unsigned long long in = block_scan_incl(q, sh, nullptr);
-            if (n < N && s_before + in > T && s_before + in - q <= T) s_pick = n;  // the first run above T
+            // the chunk, 256 points at a time, until the running sum exceeds T
+            unsigned long long before = s_before;
+            const long long n1 = min(a.N, (b + 1) << a.csh);
+            for (long long n0 = b << a.csh; n0 < n1; n0 += kPPThreads) {
+                const long long n = n0 + tid;
+                const unsigned long long q = n < n1 ? weight(__ldcg(a.Q + n), kt) : 0ull;
+                unsigned long long tot;
+                const unsigned long long in = before + block_scan_incl(q, sh, &tot);
+                if (in > T && in - q <= T) s_pick = n;  // the first run above T
+                before += tot;
+                if (before > T) break;  // block-uniform
+            }
         }
     }
     __syncthreads();
     long long pick = s_pick;
-    if (pick < 0 || pick >= N) {  // cannot happen: the chunk sums and the scan agree
+    if (pick < 0 || pick >= a.N) {  // cannot happen: the chunk sums and the scan agree
         if (tid == 0) st->err = 1;
         pick = 0;
     }
-    for (int i = tid; i < D; i += blockDim.x) C[(long long)j * D + i] = X[pick * D + i];
+    take_centre(a, j, pick);
     if (tid == 0) {
-        idx[j] = pick;
-        st->pick = pick;
-        st->wmax = 0ull;  // the update of this centre recomputes it
+        st->k = kt;
+        st->cur = cur;
+        st->resum = resum;
+        st->ticket = 0u;
     }
+}
+
+// true in every thread of the last block to get here
+__device__ __forceinline__ bool last_block(PPState *st) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Centre 0, drawn uniformly: every point's FP64 distance, and the scale of Q
+// (k_pp_quant then makes Q).
+template <bool VEC>
+__global__ void __launch_bounds__(kPPThreads) k_pp_first(PPArgs a) {
+    extern __shared__ double sd[];  // the centre (D)
+    const long long pick = uniform_index(a.u[0], a.N);
+    for (int i = threadIdx.x; i < a.D; i += kPPThreads) sd[i] = (double)a.X[pick * a.D + i];
+    __syncthreads();
+    unsigned long long m = 0;
+    for (long long n = (long long)blockIdx.x * kPPThreads + threadIdx.x; n < a.N; n += (long long)gridDim.x * kPPThreads) {
+        const double d = dist2<VEC>(a.X + n * a.D, sd, a.D);
+        a.dmin[n] = d;
+        if (d == d) m = max(m, (unsigned long long)__double_as_longlong(d));
+    }
+    m = warp_max_u(m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(&a.st->wmax, m);
+    if (blockIdx.x == 0) take_centre(a, 0, pick);
+    if (!last_block(a.st)) return;
+    if (threadIdx.x == 0) {
+        const unsigned long long w = __ldcg(&a.st->wmax);
+        a.st->e0 = w ? exponent_of(w) : 0;
+        a.st->k = w ? 0 : 64;
+        a.st->ticket = 0u;
+    }
+}
+
+// Q and the filter's bound of every point, the chunk sums and the histogram,
+// the draw of centre 1
+__global__ void __launch_bounds__(kPPThreads) k_pp_quant(PPArgs a) {
+    __shared__ int hist[kPPBins];
+    if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
+    __syncthreads();
+    const int e0 = a.st->e0, k = a.st->k, lane = threadIdx.x & 31;
+    const long long c1 = chunk0(a, blockIdx.x + 1);
+    for (long long b = chunk0(a, blockIdx.x) + (threadIdx.x >> 5); b < c1; b += kPPWarps) {
+        unsigned long long s0 = 0, s1 = 0;
+        const long long n1 = min(a.N, (b + 1) << a.csh);
+        for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
+            const double d = a.dmin[n];
+            const unsigned long long q = quant(d, e0);
+            a.Q[n] = q;
+            a.ub[n] = d == d ? __double2float_ru(d) : INFINITY;
+            s0 += weight(q, k);
+            s1 += weight(q, k + 1);
+            if (q != kPPNaN) atomicAdd(&hist[bin_of(q)], 1);
+        }
+        s0 = warp_sum_u(s0);
+        s1 = warp_sum_u(s1);
+        if (lane == 0) {
+            a.sums[0][b] = s0;
+            a.sums[1][b] = s1;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < kPPBins && hist[threadIdx.x]) atomicAdd(&a.st->hist[threadIdx.x], hist[threadIdx.x]);
+    if (last_block(a.st)) draw(a, 1);
+}
+
+// Centre j - 1 (drawn last): the distances it shortens, the sums, the draw of
+// centre j.  A row is read by LPR = 2^lprl lanes, 16 bytes each (VEC: D a
+// multiple of 4 and 16-byte aligned rows) or one coordinate each, so that a
+// warp's loads are contiguous; successive centres sweep a block's points in
+// opposite directions, so that the end of one sweep is found in L2 by the
+// next.
+template <bool VEC>
+__global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int j, int lprl, float eps_lo, float tiny) {
+    extern __shared__ double sd[];  // the centre: FP64 (D), then FP32 padded to a multiple of LPR vectors with zeros
+    __shared__ unsigned list[kPPList];
+    __shared__ int hist[kPPBins];
+    __shared__ int nlist;
+    const int D = a.D, LPR = 1 << lprl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *sc = reinterpret_cast<float *>(sd + ((D + 1) & ~1));
+    constexpr int W = VEC ? 4 : 1;
+    const int nv = D / W;                      // vectors of a row
+    const int steps = (nv + LPR - 1) >> lprl;  // vectors per lane
+    {
+        const float *c = a.X + a.st->pick * D;
+        for (int i = threadIdx.x; i < steps * LPR * W; i += kPPThreads) {
+            const float v = i < D ? c[i] : 0.f;
+            sc[i] = v;
+            if (i < D) sd[i] = (double)v;
+        }
+    }
+    if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) nlist = 0;
+    const int e0 = a.st->e0, k = a.st->k;
+    unsigned long long *sums0 = a.sums[a.st->cur], *sums1 = a.sums[a.st->cur ^ 1];
+    const long long c0 = chunk0(a, blockIdx.x), c1 = chunk0(a, blockIdx.x + 1);
+    const long long p0 = c0 << a.csh, p1 = min(a.N, c1 << a.csh);  // this block's points
+    if (a.st->resum)
+        for (long long b = c0 + warp; b < c1; b += kPPWarps) {
+            unsigned long long s = 0;
+            const long long n1 = min(a.N, (b + 1) << a.csh);
+            for (long long n = (b << a.csh) + lane; n < n1; n += 32) s += weight(a.Q[n], k + 1);
+            s = warp_sum_u(s);
+            if (lane == 0) sums1[b] = s;
+        }
+    __syncthreads();
+
+    const int sub = lane >> lprl, l = lane & (LPR - 1), rows = 32 >> lprl;
+    constexpr int U = kPPU;  // row groups in flight
+    for (long long q0 = p0; q0 < p1; q0 += kPPSegment) {
+        // the filter, on a segment of this block's points
+        const int cnt = (int)min((long long)kPPSegment, p1 - q0);
+        // (odd centres: the segments and their rows from the end)
+        const long long s0 = (j & 1) ? p1 - (q0 - p0) - cnt : q0;
+        for (int g0 = warp * U * rows; g0 < cnt; g0 += kPPWarps * U * rows) {
+            float s[U], ub[U];
+            int r[U];
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+                s[v] = 0.f;
+                r[v] = g0 + v * rows + sub;
+                if (j & 1) r[v] = cnt - 1 - r[v];  // below zero past the end
+                if (r[v] >= cnt) r[v] = -1;
+                ub[v] = l == 0 && r[v] >= 0 ? a.ub[s0 + r[v]] : 0.f;
+            }
+            for (int t = 0; t < steps; ++t) {
+                const int q = l + (t << lprl);
+                if constexpr (VEC) {
+                    float4 x[U];
+#pragma unroll
+                    for (int v = 0; v < U; ++v)
+                        x[v] = r[v] >= 0 && q < nv ? __ldg(reinterpret_cast<const float4 *>(a.X + (s0 + r[v]) * D) + q)
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 cc = *reinterpret_cast<const float4 *>(sc + 4 * q);
+#pragma unroll
+                    for (int v = 0; v < U; ++v) {
+                        const float d0 = x[v].x - cc.x, d1 = x[v].y - cc.y, d2 = x[v].z - cc.z, d3 = x[v].w - cc.w;
+                        s[v] = fmaf(d3, d3, fmaf(d2, d2, fmaf(d1, d1, fmaf(d0, d0, s[v]))));
+                    }
+                } else {
+                    float x[U];
+#pragma unroll
+                    for (int v = 0; v < U; ++v) x[v] = r[v] >= 0 && q < nv ? __ldg(a.X + (s0 + r[v]) * D + q) : 0.f;
+                    const float cc = sc[q];
+#pragma unroll
+                    for (int v = 0; v < U; ++v) {
+                        const float d = x[v] - cc;
+                        s[v] = fmaf(d, d, s[v]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < U; ++v)
+                for (int o = LPR >> 1; o > 0; o >>= 1) s[v] += __shfl_xor_sync(0xffffffffu, s[v], o);
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+                bool pass = false;
+                if (l == 0 && r[v] >= 0) {
+                    // not nearer when the distance is certainly at least D^2 (an
+                    // overflowed one settles nothing)
+                    const float lo = __fsub_rd(__fmul_rd(s[v], eps_lo), tiny);
+                    pass = !(lo >= ub[v] && s[v] < INFINITY);
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, pass);
+                if (m) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&nlist, __popc(m));
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (pass) list[base + __popc(m & ((1u << lane) - 1u))] = (unsigned)(s0 + r[v] - p0);
+                }
+            }
+        }
+        __syncthreads();
+        // the FP64 distances of the points it kept, when they fill the block or
+        // the points end
+        const int n = nlist;
+        if (n < kPPSegment / 2 && q0 + kPPSegment < p1) continue;  // (room for a whole segment is left)
+        for (int i = threadIdx.x; i < n; i += kPPThreads) {
+            const long long pt = p0 + list[i];
+            const double s = dist2<VEC>(a.X + pt * D, sd, D);
+            const double d = a.dmin[pt], m = fmin(d, s);
+            if (m < d || (d != d && m == m)) {
+                const unsigned long long qo = a.Q[pt], qn = quant(m, e0);
+                a.dmin[pt] = m;
+                a.ub[pt] = __double2float_ru(m);
+                a.Q[pt] = qn;
+                const long long b = pt >> a.csh;
+                atomicAdd(&sums0[b], weight(qn, k) - weight(qo, k));  // modulo 2^64
+                atomicAdd(&sums1[b], weight(qn, k + 1) - weight(qo, k + 1));
+                if (qo != kPPNaN) atomicAdd(&hist[bin_of(qo)], -1);
+                atomicAdd(&hist[bin_of(qn)], 1);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) nlist = 0;
+        __syncthreads();
+    }
+    if (threadIdx.x < kPPBins && hist[threadIdx.x]) atomicAdd(&a.st->hist[threadIdx.x], hist[threadIdx.x]);
+    if (last_block(a.st)) draw(a, j);
 }
 
 }  // namespace
 
 cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const double *u, float *C, long long *idx,
-                            double *dmin, unsigned long long *bsum, void *state, cudaStream_t s, int num_sms,
-                            long long *err_out) {
-    PPState *st = static_cast<PPState *>(state);
-    const long long nb = (N + kPPChunk - 1) / kPPChunk;
-    const unsigned ug = (unsigned)std::min<int64_t>((N + kPPThreads - 1) / kPPThreads, (int64_t)num_sms * 16);
+                            double *dmin, unsigned long long *Q, float *ub, unsigned long long *sums, void *state,
+                            cudaStream_t s, int num_sms, long long *err_out) {
+    PPArgs a;
+    a.X = X;
+    a.N = N;
+    a.D = D;
+    a.dmin = dmin;
+    a.Q = Q;
+    a.ub = ub;
+    a.csh = kmeanspp_chunk_log2(N);
+    a.nb = (N + ((int64_t)1 << a.csh) - 1) >> a.csh;
+    a.sums[0] = sums;
+    a.sums[1] = sums + a.nb;
+    a.u = u;
+    a.st = static_cast<PPState *>(state);
+    a.C = C;
+    a.idx = idx;
     cudaError_t e;
+    if ((e = cudaMemsetAsync(state, 0, sizeof(PPState), s)) != cudaSuccess) return e;
+    // 16-byte loads where the rows allow; lanes per row: its vectors rounded up
+    // to a power of two, at most a warp
+    const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    const int nv = vec ? D / 4 : D;
+    int lprl = 0;
+    while ((1 << lprl) < nv && lprl < 5) ++lprl;
+    const int steps = (nv + (1 << lprl) - 1) >> lprl;
+    const size_t smem = (size_t)((D + 1) & ~1) * 8 + (size_t)steps * (4u << lprl) * (vec ? 4 : 1);
+    auto step = vec ? k_pp_step<true> : k_pp_step<false>;
+    if ((e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    // FP32 error of a D-term sum of squared differences (any order), with room
+    // for the FP64 sum's own (2^-53 relative): true >= computed (1 - eps) - tiny
+    const double eps = (D + 8) * std::ldexp(1.0, -24) * (1.0 + 1.0 / 1024);
+    float eps_lo = (float)(1.0 - eps);
+    if ((double)eps_lo > 1.0 - eps) eps_lo = std::nextafter(eps_lo, 0.0f);
+    const float tiny = std::ldexp((float)(D + 8), -149);
+    // one wave of blocks that own whole chunks
+    const unsigned grid = (unsigned)std::min<int64_t>(a.nb, (int64_t)num_sms * kPPBlocks);
+    const unsigned fg = (unsigned)std::min<int64_t>((N + kPPThreads - 1) / kPPThreads, (int64_t)num_sms * 8);
     count_launch();
-    k_pp_first<<<1, 1, 0, s>>>(u, N, st);
+    if (vec) k_pp_first<true><<<fg, kPPThreads, (size_t)D * 8, s>>>(a);
+    else k_pp_first<false><<<fg, kPPThreads, (size_t)D * 8, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // centre 0 is drawn by a pick over all-zero chunk sums (the uniform draw
-    // floor(u_0 N)), which also copies its row out
-    if ((e = cudaMemsetAsync(bsum, 0, (size_t)nb * 8, s)) != cudaSuccess) return e;
-    for (int j = 0; j < K; ++j) {
-        if (j > 0) {
-            count_launch();
-            k_pp_blocksum<<<(unsigned)nb, kPPThreads, 0, s>>>(dmin, N, st, bsum);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        }
+    if (K > 1) {
         count_launch();
-        k_pp_pick<<<1, 1024, 0, s>>>(X, N, D, dmin, bsum, nb, u, j, st, C, idx);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        count_launch();
-        k_pp_update<<<ug, kPPThreads, 0, s>>>(X, N, D, dmin, st, j == 0 ? 1 : 0);
+        k_pp_quant<<<grid, kPPThreads, 0, s>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if (err_out) return cudaMemcpyAsync(err_out, &st->err, 8, cudaMemcpyDeviceToHost, s);
+    for (int j = 2; j < K; ++j) {
+        count_launch();
+        step<<<grid, kPPThreads, smem, s>>>(a, j, lprl, eps_lo, tiny);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (err_out) return cudaMemcpyAsync(err_out, &a.st->err, 8, cudaMemcpyDeviceToHost, s);
     return cudaSuccess;
+}
+
+int kmeanspp_chunk_log2(int64_t N) {
+    int c = 5;
+    while (((N - 1) >> c) >= kPPMaxChunks) ++c;
+    return c;
 }
 
 size_t kmeanspp_state_bytes() { return sizeof(PPState); }
@@ -253,24 +663,27 @@ KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K,
                                                   cudaSuccess)
         return fail(KM_ECUDA, "device query failed");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int64_t nb = (N + 1023) / 1024;
+    const int64_t nb = ((N - 1) >> kmeanspp_chunk_log2(N)) + 1;
+    float *ub = nullptr;
     double *dmin = nullptr, *ud = nullptr;
-    unsigned long long *bsum = nullptr;
+    unsigned long long *bsum = nullptr, *Q = nullptr;
     void *st = nullptr;
     float *Cd = nullptr;
     long long *idx = nullptr;
     long long err = 0;
     cudaError_t e = pool_alloc(dev, reinterpret_cast<void **>(&dmin), (size_t)N * 8, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&bsum), (size_t)nb * 8, s);
+    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&Q), (size_t)N * 8, s);
+    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ub), (size_t)N * 4, s);
+    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&bsum), (size_t)nb * 16, s);
     if (e == cudaSuccess) e = pool_alloc(dev, &st, kmeanspp_state_bytes(), s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ud), (size_t)K * 8, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&Cd), (size_t)K * D * 4, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&idx), (size_t)K * 8, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ud, u, (size_t)K * 8, cudaMemcpyDefault, s);
-    if (e == cudaSuccess) e = launch_kmeanspp(X, N, D, K, ud, Cd, idx, dmin, bsum, st, s, sms, &err);
+    if (e == cudaSuccess) e = launch_kmeanspp(X, N, D, K, ud, Cd, idx, dmin, Q, ub, bsum, st, s, sms, &err);
     if (e == cudaSuccess) e = cudaMemcpyAsync(centroids, Cd, (size_t)K * D * 4, cudaMemcpyDefault, s);
     if (e == cudaSuccess && indices) e = cudaMemcpyAsync(indices, idx, (size_t)K * 8, cudaMemcpyDefault, s);
-    for (void *p : {(void *)dmin, (void *)bsum, st, (void *)ud, (void *)Cd, (void *)idx})
+    for (void *p : {(void *)dmin, (void *)Q, (void *)ub, (void *)bsum, st, (void *)ud, (void *)Cd, (void *)idx})
         if (p) cudaFreeAsync(p, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {

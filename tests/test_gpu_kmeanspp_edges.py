@@ -1,0 +1,71 @@
+"""k-means++ seeding at the edges of its filter, lists and weights: chunk and
+warp remainders, odd and long rows, misaligned points, distances over many
+binary orders of magnitude (the weights' scale then falls by more than one
+step at a time, and past the stored bits), subnormal coordinates, points far
+from the origin.  The indices must equal O4's bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kp():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1905_09345_gb300 import build, kpynq
+    build.build()
+    oracle.build()
+    return kpynq
+
+
+def check(kp, X, K, seed, shift=0):
+    """shift: floats by which the device copy of X is misaligned."""
+    N, D = X.shape
+    u = np.random.default_rng(seed).uniform(size=K)
+    buf = torch.empty(N * D + shift, dtype=torch.float32, device="cuda")
+    buf[shift:] = torch.from_numpy(np.ascontiguousarray(X, np.float32)).cuda().reshape(-1)
+    C = torch.empty(K, D, dtype=torch.float32, device="cuda")
+    idx = torch.empty(K, dtype=torch.int64, device="cuda")
+    kp.kmeans_init_kmeanspp(buf[shift:].reshape(N, D), N, D, K, u, C, idx)
+    ref, _ = oracle.kmeanspp(X.astype(np.float64), K, u)
+    got = idx.cpu().numpy()
+    assert np.array_equal(got, ref), np.flatnonzero(got != ref)[:5]
+    assert np.array_equal(C.cpu().numpy(), X[ref])
+
+
+SHAPES = [(1, 1, 1), (2, 5, 2), (31, 4, 31), (33, 8, 20), (1000, 1, 30), (4097, 12, 40), (131073, 3, 20),
+          (131072, 8, 25), (20000, 129, 30), (9000, 260, 25), (300, 4096, 12), (600000, 4, 12)]
+
+
+@pytest.mark.parametrize("N,D,K", SHAPES, ids=[f"N{s[0]}_D{s[1]}_K{s[2]}" for s in SHAPES])
+def test_shapes(kp, N, D, K):
+    rng = np.random.default_rng(N + D)
+    X = (rng.normal(size=(N, D)) * rng.uniform(0.1, 10.0, size=(1, D))).astype(np.float32)
+    check(kp, X, K, seed=D)
+    if N < 50000:
+        check(kp, X, K, seed=D + 1, shift=1)
+
+
+@pytest.mark.parametrize("span", [6, 40, 120])
+def test_scales(kp, span):
+    """Points at distances 2^0 .. 2^-span: each centre removes the largest."""
+    rng = np.random.default_rng(span)
+    N, D = 3000, 6
+    X = rng.normal(size=(N, D)) * np.exp2(-rng.uniform(0, span, size=(N, 1)))
+    check(kp, X.astype(np.float32), 120, seed=1)
+
+
+def test_far_from_origin_and_subnormal(kp):
+    rng = np.random.default_rng(5)
+    X = (rng.normal(size=(5000, 16)) * 1e-2 + 1e4).astype(np.float32)
+    X[rng.integers(0, 5000, size=1500)] = X[7]  # many duplicates
+    check(kp, X, 60, seed=2)
+    Y = rng.normal(size=(2000, 5)).astype(np.float32)
+    Y[:, 2] = (rng.integers(0, 50, size=2000) * 2.0 ** -149).astype(np.float32)  # subnormal coordinates
+    Y[::3, 0] = 0.0
+    check(kp, Y, 50, seed=3)
+    check(kp, np.zeros((500, 3), np.float32), 20, seed=4)  # every weight zero

@@ -482,7 +482,7 @@ KM_API int kmeans_mlp_train(kmeans_mlp *m, const float *X, int64_t N, const int3
                             double *accuracy);
 
 /* pred[n] = the class with the largest logit (the first on ties) for N rows
- * of X (N x D FP32; X and pred device memory), in chunks of up to 2^17 rows. */
+ * of X (N x D FP32; X and pred device memory), in one launch. */
 KM_API int kmeans_mlp_predict_net(kmeans_mlp *m, const float *X, int64_t N, int32_t *pred);
 
 KM_API void kmeans_mlp_destroy(kmeans_mlp *m);
@@ -506,7 +506,7 @@ KM_API const char *kmeans_mlp_last_error(const kmeans_mlp *m);
  * and point filters, distance calculator; Sec. I), so labels are exactly
  * those without a proposal -- a wrong prediction only costs work.  All six
  * pointers NULL: remove the proposal.  Allocates the network, N int32
- * predictions, its chunk buffers and the K x G table.  Errors: KM_EINVAL
+ * predictions and the K x G table.  Errors: KM_EINVAL
  * (Lloyd context, hidden outside [1, 256], D > 256 or G > 512, some pointers
  * NULL), KM_ENOMEM, KM_ECUDA. */
 KM_API int kmeans_set_proposal(kmeans_ctx *c, const float *W1, const float *b1, const float *W2, const float *b2,

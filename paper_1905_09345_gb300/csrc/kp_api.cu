@@ -1165,7 +1165,7 @@ KM_API int kmeans_set_proposal(kmeans_ctx *c, const float *W1, const float *b1, 
         if ((rc = kmeans_mlp_create(&net, p.D, hidden, p.G, 0, c->stream)))
             return set_err(c, rc, "proposal network: %s", kmeans_last_error(nullptr));
         c->net = net;
-        if ((rc = kmeans_mlp_set_params(net, W1, b1, W2, b2, W3, b3)) || (rc = mlp_prepare(net, p.N)))
+        if ((rc = kmeans_mlp_set_params(net, W1, b1, W2, b2, W3, b3)))
             return set_err(c, rc, "proposal network: %s", mlp_message(net));
         if (!c->pred) KP_CUDA(c, dalloc(c, &c->pred, (size_t)p.N));
         if (!c->cc_table) KP_CUDA(c, dalloc(c, &c->cc_table, (size_t)p.K * p.G));

@@ -363,9 +363,8 @@ cudaError_t launch_dense_assign(const Params &p, cudaStream_t s, int first, int 
 __host__ __device__ inline int tc_dim(int D) { return D == 32 || D == 64 ? 64 : (D == 128 ? 128 : 0); }
 bool dense_tc_eligible(const Params &p, size_t smem_limit);
 bool dense_tcb_eligible(const Params &p, size_t smem_limit);
-// the proposal network on the tensor cores (kp_mlp.cu): buffers for N rows,
-// then the predicted class of every row, ordered on s (KM_* status)
-int mlp_prepare(kmeans_mlp *m, int64_t N);
+// the proposal network on the tensor cores (kp_mlp.cu): the predicted class
+// of every row, ordered on s (KM_* status)
 int mlp_predict_enqueue(kmeans_mlp *m, const float *X, int64_t N, int32_t *pred, cudaStream_t s);
 int mlp_error_flag(kmeans_mlp *m);  // synchronises; KM_ETIMEOUT if a bounded wait gave up
 const char *mlp_message(const kmeans_mlp *m);

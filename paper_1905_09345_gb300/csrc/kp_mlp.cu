@@ -8,7 +8,8 @@
 // exact erf form), trained with softmax cross-entropy (mean over the batch)
 // and Adam, FP32 master weights and bfloat16 compute weights.
 //
-// Every matrix product is one kernel, k_mlp_gemm:
+// Inference is one kernel for the three layers, k_mlp_infer (below).  In
+// training every matrix product is one kernel, k_mlp_gemm:
 //     C[M x N] = A[M x K] . B[N x K]^T
 // with both operands bfloat16 and K-major in global memory, staged into shared
 // memory by TMA (128-byte swizzle, one 64-element K slice per stage, a ring of
@@ -22,7 +23,6 @@
 //     SOFTMAX  bias + softmax cross-entropy: the loss, and the logit gradient
 //              (p - onehot(y)) / B as bfloat16 (row-major and transposed), with
 //              its per-warp column sums (the bias gradient);
-//     ARGMAX   bias + the first largest logit (inference);
 //     MUL      the backpropagated gradient times GELU'(z) (row-major and/or
 //              transposed bfloat16, per-warp column sums);
 //     F32      the FP32 tile itself (split-K partial products of a weight
@@ -53,7 +53,7 @@ constexpr int kMK = 64;        // K per stage: one 128-byte row of bfloat16
 constexpr int kMThreads = 192; // warp 0 TMA, warp 1 MMA (and TMEM allocation), warps 2..5 epilogue
 constexpr uint32_t kMPolls = 1u << 22;
 
-enum Epi : int { E_GELU = 0, E_SOFTMAX = 1, E_ARGMAX = 2, E_MUL = 3, E_F32 = 4 };
+enum Epi : int { E_GELU = 0, E_SOFTMAX = 1, E_MUL = 3, E_F32 = 4 };
 
 struct GemmCfg {
     int M, N;          // valid output rows / columns
@@ -62,7 +62,7 @@ struct GemmCfg {
     int tmem_cols;     // power of two >= nch * bn
     int stages;
     int mode;          // Epi
-    const float *bias; // N (GELU, SOFTMAX, ARGMAX)
+    const float *bias; // N (GELU, SOFTMAX)
     uint16_t *out;     // row-major bfloat16 M x ldo (nullable)
     int ldo;
     uint16_t *outT;    // transposed bfloat16 N x ldt (nullable)
@@ -77,7 +77,6 @@ struct GemmCfg {
     const int32_t *y;  // SOFTMAX: class of each row
     float scale;       // SOFTMAX: 1 / batch
     double *loss;      // SOFTMAX: [0] += cross-entropy, [1] += correct predictions, [2] += rows
-    int32_t *pred;     // ARGMAX
     int *err;          // KM_ETIMEOUT when a bounded wait gave up
 };
 
@@ -277,26 +276,6 @@ __global__ void __launch_bounds__(kMThreads, 1)
                         for (int j = 0; j < 16; ++j) g.outT[(size_t)(n0 + j) * g.ldt + row] = bf16_bits(a[j]);
                     }
                 }
-            } else if (g.mode == E_ARGMAX) {
-                float best = -INFINITY;
-                int bi = 0;
-                for (int c0 = 0; c0 < TC; c0 += 16) {
-                    uint32_t v[16];
-                    tmem_ld16_async(tb_ + c0, v);
-                    tmem_wait16(v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int n = c0 + j;  // one N tile: nb == 0
-                        if (n < g.N) {
-                            const float l = __uint_as_float(v[j]) + g.bias[n];
-                            if (l > best) {
-                                best = l;
-                                bi = n;
-                            }
-                        }
-                    }
-                }
-                if (valid) g.pred[row] = bi;
             } else {  // E_SOFTMAX (one N tile: nb == 0)
                 float mx = -INFINITY;
                 for (int c0 = 0; c0 < TC; c0 += 16) {
@@ -373,6 +352,317 @@ __global__ void __launch_bounds__(kMThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
+// inference: the three layers and the largest logit in one kernel
+// ---------------------------------------------------------------------------
+// Persistent CTA per SM; tiles of 128 rows go alternately to two groups of
+// eight epilogue warps (two per TMEM lane quadrant, one per half of the
+// columns).  A tile's activations never leave the SM: its group stages the
+// rows as bfloat16 into its A buffer, the tensor cores multiply it by W1, the
+// group turns the accumulators into GELU(z + b) in the same A buffer, and so
+// on for W2; the logits (in chunks of at most 256 columns) only pass through
+// registers for the running maximum.  The weights stream from L2 through a
+// ring of 64-element K slices; while one group works on its accumulators (256
+// TMEM columns each), the other's product runs.
+// The GELU (an erff per activation) bounds it.  Measured on GB300, 1,048,576 x
+// 32 -> 256 -> 256 -> 410: 2.69 ms as a cast and three products per 131,072
+// rows with the activations through memory, 0.86 ms now (436 TFLOP/s); 2,090 x
+// 64 -> 256 -> 256 -> 33: 66 -> 42 us.
+constexpr int kInGroupWarps = 8;
+constexpr int kInThreads = 64 + 2 * kInGroupWarps * 32;
+
+struct InferCfg {
+    const float *X;
+    int64_t N;
+    int D, Dk, Hp, C;   // row width, padded; padded hidden width; classes
+    int nch, bn;        // logit chunks and columns per chunk
+    int x_vec;          // rows allow 16-byte loads
+    int stages;         // weight ring
+    int64_t tiles;
+    uint32_t a_bytes, w_bytes;  // an A buffer; a ring stage
+    const float *b1, *b2, *b3;
+    int32_t *pred;
+    int *err;
+};
+
+// the two warps of a quadrant (named barrier `id`, 64 threads): every thread
+// contributes v, every thread gets the AND
+__device__ __forceinline__ bool pair_all(bool v, int id) {
+    int out;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.and.pred q, %2, 64, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(out)
+        : "r"((int)v), "r"(id)
+        : "memory");
+    return out != 0;
+}
+
+__global__ void __launch_bounds__(kInThreads, 1)
+    k_mlp_infer(const __grid_constant__ CUtensorMap t1, const __grid_constant__ CUtensorMap t2,
+                const __grid_constant__ CUtensorMap t3, InferCfg c) {
+    extern __shared__ uint8_t raw[];
+    uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+    const int S = c.stages;
+    uint8_t *ring = sm + 2 * (size_t)c.a_bytes;
+    float *sb1 = reinterpret_cast<float *>(ring + (size_t)S * c.w_bytes);
+    float *sb2 = sb1 + c.Hp;
+    float *sb3 = sb2 + c.Hp;  // nch * bn; -inf past the classes, so that they are never the largest
+    float2 *mrg = reinterpret_cast<float2 *>(sb3 + c.nch * c.bn);  // [2][128]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(mrg + 2 * kMM);
+    uint64_t *a_ready = bars, *acc_full = bars + 2, *done = bars + 4, *full = bars + 5, *empty = full + S;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(empty + S);
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int phases = 2 + c.nch;
+    // this CTA's tiles: blockIdx.x + i * gridDim.x; group g takes i = g, g + 2, ...
+    const int64_t mine = c.tiles > (int64_t)blockIdx.x
+                             ? (c.tiles - (int64_t)blockIdx.x + (int64_t)gridDim.x - 1) / (int64_t)gridDim.x
+                             : 0;
+
+    if (threadIdx.x == 0) {
+        for (int g = 0; g < 2; ++g) {
+            bar_init(&a_ready[g], kInGroupWarps);
+            bar_init(&acc_full[g], 1);
+        }
+        bar_init(done, 1);
+        for (int i = 0; i < S; ++i) {
+            bar_init(&full[i], 1);
+            bar_init(&empty[i], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int i = threadIdx.x; i < c.Hp; i += blockDim.x) {
+        sb1[i] = c.b1[i];
+        sb2[i] = c.b2[i];
+    }
+    for (int i = threadIdx.x; i < c.nch * c.bn; i += blockDim.x) sb3[i] = i < c.C ? c.b3[i] : -INFINITY;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&t1) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&t2) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&t3) : "memory");
+            uint32_t nl = 0;  // slices issued
+            bool ok = true;
+            for (int64_t i0 = 0; i0 < mine && ok; i0 += 2)
+                for (int ph = 0; ph < phases && ok; ++ph)
+                    for (int g = 0; g < 2 && i0 + g < mine && ok; ++g) {
+                        const CUtensorMap *t = ph == 0 ? &t1 : (ph == 1 ? &t2 : &t3);
+                        const int ks = (ph == 0 ? c.Dk : c.Hp) / kMK;
+                        const uint32_t rows = (uint32_t)(ph < 2 ? c.Hp : c.bn);
+                        const int r0 = ph < 2 ? 0 : (ph - 2) * c.bn;
+                        for (int k = 0; k < ks; ++k, ++nl) {
+                            const uint32_t st = nl % S, f = nl / S;
+                            if (f > 0 && !(ok = mwait(&empty[st], (f - 1) & 1, c.err))) break;
+                            mbar_arrive_expect_tx(&full[st], rows * 128u);
+                            tma_2d(ring + (size_t)st * c.w_bytes, t, k * kMK, r0, &full[st]);
+                        }
+                    }
+            // every issued copy has landed before the block can exit
+            for (uint32_t j = nl > (uint32_t)S ? nl - S : 0; j < nl; ++j) mwait(&full[j % S], (j / S) & 1, c.err);
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA
+        if (lane == 0) {
+            uint32_t nl = 0;
+            uint32_t na[2] = {0, 0};  // phases issued per group
+            bool ok = true;
+            for (int64_t i0 = 0; i0 < mine && ok; i0 += 2)
+                for (int ph = 0; ph < phases && ok; ++ph)
+                    for (int g = 0; g < 2 && i0 + g < mine && ok; ++g) {
+                        const int ks = (ph == 0 ? c.Dk : c.Hp) / kMK;
+                        const int nn = ph < 2 ? c.Hp : c.bn;
+                        // kind::f16: F32 accumulate, BF16 A and B, both K-major, M = 128
+                        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nn >> 3) << 17) |
+                                               ((uint32_t)(kMM >> 4) << 24);
+                        // the group's A operand is in place and its accumulators are read
+                        if (!(ok = mwait(&a_ready[g], na[g] & 1, c.err))) break;
+                        ++na[g];
+                        tc_fence_after();
+                        const uint8_t *A = sm + (size_t)g * c.a_bytes;
+                        for (int k = 0; k < ks; ++k, ++nl) {
+                            const uint32_t st = nl % S;
+                            if (!(ok = mwait(&full[st], (nl / S) & 1, c.err))) break;
+                            tc_fence_after();
+                            const uint8_t *B = ring + (size_t)st * c.w_bytes;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {  // four K = 16 steps inside the 128-byte row
+                                const uint64_t da = desc_sw128(smem_u32(A + k * (kMM * 128) + j * 32));
+                                const uint64_t db = desc_sw128(smem_u32(B + j * 32));
+                                const uint32_t acc = (k > 0 || j > 0) ? 1u : 0u;
+                                asm volatile(
+                                    "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
+                                        tmem + (uint32_t)(g * 256)),
+                                    "l"(da), "l"(db), "r"(idesc), "r"(acc)
+                                    : "memory");
+                            }
+                            asm volatile(
+                                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                    smem_u32(&empty[st]))
+                                : "memory");
+                        }
+                        if (!ok) break;
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                         smem_u32(&acc_full[g]))
+                                     : "memory");
+                    }
+            // every MMA of this thread is complete before TMEM is freed
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             smem_u32(done))
+                         : "memory");
+            mwait(done, 0, c.err);
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------------- epilogue
+        const int e = warp - 2;
+        const int g = e >> 3, half = (e >> 2) & 1;
+        const int q = warp & 3;  // TMEM lane quadrant of this warp
+        const int r = q * 32 + lane;
+        const int pid = 1 + g * 4 + q;
+        const int gt = (e & 7) * 32 + lane;  // thread of the group
+        uint8_t *A = sm + (size_t)g * c.a_bytes;
+        const uint32_t tb = tmem + (uint32_t)(g * 256) + ((uint32_t)(q * 32) << 16);
+        uint32_t na = 0;  // accumulators awaited
+        auto release = [&]() {  // A written (generic proxy) and TMEM read: the next product may run
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) bar_arrive(&a_ready[g]);
+        };
+        auto await = [&]() {  // pair-uniform: a named barrier needs both warps
+            const bool ok = __all_sync(0xffffffffu, mwait(&acc_full[g], na & 1, c.err));
+            ++na;
+            const bool both = pair_all(ok, pid);
+            tc_fence_after();
+            return both;
+        };
+        for (int64_t i = g; i < mine; i += 2) {
+            const int64_t m0 = ((int64_t)blockIdx.x + i * (int64_t)gridDim.x) * kMM;
+            // the rows as bfloat16, zero-padded to Dk, in 16-byte chunks
+            const int cq = c.Dk >> 3;
+            for (int idx = gt; idx < kMM * cq; idx += kInGroupWarps * 32) {
+                const int rr = idx / cq, ch = idx - rr * cq, d0 = ch * 8;
+                const int64_t n = m0 + rr;
+                float v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = 0.f;
+                if (n < c.N) {
+                    const float *x = c.X + n * c.D;
+                    if (c.x_vec) {
+#pragma unroll
+                        for (int k = 0; k < 8; k += 4)
+                            if (d0 + k < c.D) {
+                                const float4 t = __ldg(reinterpret_cast<const float4 *>(x + d0 + k));
+                                v[k] = t.x;
+                                v[k + 1] = t.y;
+                                v[k + 2] = t.z;
+                                v[k + 3] = t.w;
+                            }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (d0 + k < c.D) v[k] = __ldg(x + d0 + k);
+                    }
+                }
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    w[k] = (uint32_t)bf16_bits(v[2 * k]) | ((uint32_t)bf16_bits(v[2 * k + 1]) << 16);
+                *reinterpret_cast<uint4 *>(A + swz_chunk(rr, ch, kMM * 128)) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            release();
+            bool ok = true;
+            // the hidden layers: this warp's half of the columns, 16 at a time
+            for (int layer = 0; layer < 2; ++layer) {
+                if (!(ok = await())) break;
+                const float *bias = layer ? sb2 : sb1;
+                const int c1 = (half + 1) * (c.Hp >> 1);
+#pragma unroll 1
+                for (int c0 = half * (c.Hp >> 1); c0 < c1; c0 += 16) {
+                    uint32_t v[16];
+                    tmem_ld16_async(tb + c0, v);
+                    float b[16];
+#pragma unroll
+                    for (int k = 0; k < 16; k += 4) {
+                        const float4 t = *reinterpret_cast<const float4 *>(bias + c0 + k);
+                        b[k] = t.x;
+                        b[k + 1] = t.y;
+                        b[k + 2] = t.z;
+                        b[k + 3] = t.w;
+                    }
+                    tmem_wait16(v);
+                    uint32_t w[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float a0 = gelu(__uint_as_float(v[2 * k]) + b[2 * k]);
+                        const float a1 = gelu(__uint_as_float(v[2 * k + 1]) + b[2 * k + 1]);
+                        w[k] = (uint32_t)bf16_bits(a0) | ((uint32_t)bf16_bits(a1) << 16);
+                    }
+                    *reinterpret_cast<uint4 *>(A + swz_chunk(r, c0 >> 3, kMM * 128)) =
+                        make_uint4(w[0], w[1], w[2], w[3]);
+                    *reinterpret_cast<uint4 *>(A + swz_chunk(r, (c0 >> 3) + 1, kMM * 128)) =
+                        make_uint4(w[4], w[5], w[6], w[7]);
+                }
+                release();
+            }
+            if (!ok) break;  // a wait timed out (error recorded)
+            // the logits: the first largest over this warp's half of every chunk
+            float best = -INFINITY;
+            int bi = 0;
+            for (int h = 0; h < c.nch; ++h) {
+                if (!(ok = await())) break;
+                const int nu = c.bn >> 4, hu = (nu + 1) >> 1;
+                const int u1 = half ? nu : hu;
+#pragma unroll 1
+                for (int u = half ? hu : 0; u < u1; ++u) {
+                    uint32_t v[16];
+                    tmem_ld16_async(tb + u * 16, v);
+                    tmem_wait16(v);
+                    const int n0 = h * c.bn + u * 16;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const float l = __uint_as_float(v[k]) + sb3[n0 + k];
+                        if (l > best) {
+                            best = l;
+                            bi = n0 + k;
+                        }
+                    }
+                }
+                if (h + 1 < c.nch) release();
+            }
+            if (!ok) break;
+            if (half) mrg[g * kMM + r] = make_float2(best, __int_as_float(bi));
+            pair_all(true, pid);
+            if (!half) {
+                // (the next write of the slot follows this warp's next a_ready arrival)
+                const float2 o = mrg[g * kMM + r];
+                const int oi = __float_as_int(o.y);
+                if (o.x > best || (o.x == best && oi < bi)) bi = oi;
+                if (m0 + r < c.N) c.pred[m0 + r] = bi;
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------
 // data movement and the update
 // ---------------------------------------------------------------------------
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014): a counter-based generator
@@ -409,16 +699,6 @@ __global__ void k_mlp_gather(const float *X, int64_t N, int D, const int32_t *la
         int y = labels[src];
         if (K > 0) y = (int)(((int64_t)y * G) / K);
         yb[i] = (y >= 0 && y < G) ? y : 0;
-    }
-}
-
-// X (rows r0.., m of them) -> bfloat16 m x Dk, zero padding
-__global__ void k_mlp_cast_x(const float *X, int64_t m, int D, int Dk, uint16_t *Xc) {
-    const int64_t total = m * Dk;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / Dk;
-        const int d = (int)(e - r * Dk);
-        Xc[e] = bf16_bits(d < D ? X[r * D + d] : 0.f);
     }
 }
 
@@ -548,9 +828,6 @@ struct kmeans_mlp {
     int32_t *yb = nullptr;
     int s1 = 1, s2 = 1, s3 = 1;
     std::vector<void *> batch_allocs;
-    // inference buffers (chunk of Mc rows)
-    int64_t Mc = 0;
-    uint16_t *Xc = nullptr, *A1c = nullptr, *A2c = nullptr;
     std::vector<void *> allocs;
     char errmsg[512] = "";
 };
@@ -812,46 +1089,42 @@ bool dev_ptr(const void *p) {
 
 }  // namespace
 
-// inference buffers for chunks of up to 2^17 rows (made once, before any
-// capture of the inference launches)
-int mlp_prepare(kmeans_mlp *m, int64_t N) {
-    if (m->Mc) return KM_OK;
-    const MlpDims &d = m->d;
-    int64_t mc = std::min<int64_t>(std::max<int64_t>(N, 1), (int64_t)1 << 17);
-    mc = (mc + kMM - 1) / kMM * kMM;
-    MLP_CUDA(m, mlp_alloc(m, &m->Xc, (size_t)mc * d.Dk, m->allocs));
-    MLP_CUDA(m, mlp_alloc(m, &m->A1c, (size_t)mc * d.Hp, m->allocs));
-    MLP_CUDA(m, mlp_alloc(m, &m->A2c, (size_t)mc * d.Hp, m->allocs));
-    m->Mc = mc;
-    return KM_OK;
-}
-
 // pred[n] = the class with the largest logit (first maximum), on stream s
 // (used by the context's seeded iteration 0 and by kmeans_mlp_predict_net)
 int mlp_predict_enqueue(kmeans_mlp *m, const float *X, int64_t N, int32_t *pred, cudaStream_t s) {
     const MlpDims &d = m->d;
+    InferCfg c;
+    c.X = X;
+    c.N = N;
+    c.D = d.D;
+    c.Dk = d.Dk;
+    c.Hp = d.Hp;
+    c.C = d.G;
+    c.nch = m->nch3;
+    c.bn = m->bn3;
+    c.x_vec = d.D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    c.tiles = (N + kMM - 1) / kMM;
+    c.a_bytes = (uint32_t)(std::max(d.Dk, d.Hp) / 64) * (kMM * 128);
+    c.w_bytes = (uint32_t)std::max(d.Hp, m->bn3) * 128u;
+    c.b1 = m->b1p;
+    c.b2 = m->b2p;
+    c.b3 = m->b3p;
+    c.pred = pred;
+    c.err = m->err;
+    const size_t fixed = 1024 + 2 * (size_t)c.a_bytes + (size_t)(2 * d.Hp + c.nch * c.bn) * 4 + 2 * kMM * 8 + 256;
+    c.stages = (int)std::min<size_t>(6, (m->smem_optin - fixed) / c.w_bytes);
+    if (fixed > m->smem_optin || c.stages < 2)
+        return mlp_fail(m, KM_EINVAL, "the network's tiles do not fit in shared memory");
+    const size_t smem = fixed + (size_t)c.stages * c.w_bytes;
+    CUtensorMap t1, t2, t3;
     int rc;
-    if ((rc = mlp_prepare(m, N))) return rc;
-    for (int64_t r0 = 0; r0 < N; r0 += m->Mc) {
-        const int rows = (int)std::min<int64_t>(m->Mc, N - r0);
-        count_launch();
-        k_mlp_cast_x<<<(unsigned)std::min<int64_t>(((int64_t)rows * d.Dk + 255) / 256, (int64_t)m->num_sms * 8), 256,
-                       0, s>>>(X + r0 * d.D, rows, d.D, d.Dk, m->Xc);
-        MLP_CUDA(m, cudaGetLastError());
-        GemmCfg g = cfg0(E_GELU);
-        g.bias = m->b1p; g.out = m->A1c; g.ldo = d.Hp;
-        if ((rc = launch_gemm(m, {m->Xc, m->Mc, d.Dk, m->W1b, d.Hp, d.Dk, d.Dk, rows, d.Hp, 1, d.Hp, 1, 1}, g, s)))
-            return rc;
-        g = cfg0(E_GELU);
-        g.bias = m->b2p; g.out = m->A2c; g.ldo = d.Hp;
-        if ((rc = launch_gemm(m, {m->A1c, m->Mc, d.Hp, m->W2b, d.Hp, d.Hp, d.Hp, rows, d.Hp, 1, d.Hp, 1, 1}, g, s)))
-            return rc;
-        g = cfg0(E_ARGMAX);
-        g.bias = m->b3p; g.pred = pred + r0;
-        if ((rc = launch_gemm(m, {m->A2c, m->Mc, d.Hp, m->W3b, d.G, d.Hp, d.Hp, rows, d.G, m->nch3, m->bn3, 1, 1},
-                              g, s)))
-            return rc;
-    }
+    if ((rc = make_map(m, &t1, m->W1b, d.Hp, d.Dk, d.Dk, d.Hp))) return rc;
+    if ((rc = make_map(m, &t2, m->W2b, d.Hp, d.Hp, d.Hp, d.Hp))) return rc;
+    if ((rc = make_map(m, &t3, m->W3b, d.G, d.Hp, d.Hp, m->bn3))) return rc;
+    MLP_CUDA(m, cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    count_launch();
+    k_mlp_infer<<<(unsigned)std::min<int64_t>(c.tiles, m->num_sms), kInThreads, smem, s>>>(t1, t2, t3, c);
+    MLP_CUDA(m, cudaGetLastError());
     return KM_OK;
 }
 

@@ -15,8 +15,8 @@
 // memory by TMA (128-byte swizzle, one 64-element K slice per stage, a ring of
 // stages), multiplied by tcgen05.mma (kind::f16, M = 128 rows per CTA, up to
 // two N chunks of <= 256 columns) into FP32 accumulators in TMEM, and read back
-// by four epilogue warps (one TMEM lane quadrant each, one row per thread)
-// that apply the layer's fused epilogue:
+// by sixteen epilogue warps (four per TMEM lane quadrant, each a quarter of the
+// columns, one row per thread) that apply the layer's fused epilogue:
 //     GELU     bias + GELU -> bfloat16 activations (row-major and/or
 //              transposed) and the FP32 derivative GELU'(z) for the backward
 //              pass;
@@ -30,6 +30,13 @@
 // The weight-gradient products contract over the batch, so the forward and
 // backward epilogues also write the transposed copies those products read
 // K-major; every operand stays in the layout the tensor cores take directly.
+// A step's products are small (B = 8192 gives 64 to 128 CTAs of a few K
+// slices), so latency bounds them: sixteen epilogue warps share a tile, the
+// three weight gradients are one launch, the launches (tensor maps included)
+// are planned once per batch size and each may start its set-up while the one
+// ahead ends.  Measured on GB300, B = 8192, 32 -> 256 -> 256 -> 410: a
+// gradient 249 us with four epilogue warps and eight separate launches, 119
+// now; a training step 201 -> 107 us.
 //
 // Shapes are padded once: D to Dk (a multiple of 64, the K slice), the hidden
 // width H to Hp (a multiple of 64) with zero weights and biases (a padded unit
@@ -38,6 +45,7 @@
 // that contract over the classes.
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -50,14 +58,16 @@ namespace {
 
 constexpr int kMM = 128;       // rows per tile (TMEM lanes)
 constexpr int kMK = 64;        // K per stage: one 128-byte row of bfloat16
-constexpr int kMThreads = 192; // warp 0 TMA, warp 1 MMA (and TMEM allocation), warps 2..5 epilogue
+constexpr int kMParts = 4;     // epilogue warps per TMEM lane quadrant
+constexpr int kMThreads = 64 + kMParts * 128; // warp 0 TMA, warp 1 MMA (and TMEM allocation), warps 2..17 epilogue
 constexpr uint32_t kMPolls = 1u << 22;
 
 enum Epi : int { E_GELU = 0, E_SOFTMAX = 1, E_MUL = 3, E_F32 = 4 };
 
 struct GemmCfg {
     int M, N;          // valid output rows / columns
-    int k_steps;       // K slices of 64 per CTA (split-K: blockIdx.z selects the slice range)
+    int mt, nt;        // CTAs along M and N (the rest of a product's CTAs split K)
+    int k_steps;       // K slices of 64 per CTA (split-K: the CTA's split selects the slice range)
     int nch, bn;       // N chunks per CTA and columns per chunk (multiple of 16, <= 256)
     int tmem_cols;     // power of two >= nch * bn
     int stages;
@@ -111,21 +121,80 @@ __device__ __forceinline__ float lane_sum(float v) {
     return v;
 }
 
-__global__ void __launch_bounds__(kMThreads, 1)
-    k_mlp_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, GemmCfg g) {
+// Sums over the lanes of sixteen columns, each by lane_sum's tree, in 16
+// shuffles instead of 80: at every step a lane passes on the half of its
+// columns that the partner keeps.  Even lanes return their column's sum (*col).
+__device__ __forceinline__ float lane_sums16(const float (&v)[16], int lane, int &col) {
+    float a[8];
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4, h2 = lane & 2;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float got = __shfl_xor_sync(0xffffffffu, h16 ? v[k] : v[k + 8], 16);
+        a[k] = (h16 ? v[k + 8] : v[k]) + got;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float got = __shfl_xor_sync(0xffffffffu, h8 ? a[k] : a[k + 4], 8);
+        a[k] = (h8 ? a[k + 4] : a[k]) + got;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float got = __shfl_xor_sync(0xffffffffu, h4 ? a[k] : a[k + 2], 4);
+        a[k] = (h4 ? a[k + 2] : a[k]) + got;
+    }
+    const float got = __shfl_xor_sync(0xffffffffu, h2 ? a[0] : a[1], 2);
+    a[0] = (h2 ? a[1] : a[0]) + got;
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    col = (h16 ? 8 : 0) + (h8 ? 4 : 0) + (h4 ? 2 : 0) + (h2 ? 1 : 0);
+    return a[0];
+}
+
+// Up to three products in one launch: CTAs [first[p], first[p + 1]) are product p's.
+struct GemmBatch {
+    CUtensorMap ta[3], tb[3];
+    GemmCfg g[3];
+    int first[4];
+    int stages;         // of the largest product
+    uint32_t st_bytes;  // stage size of the largest
+    int tmem_cols;
+};
+
+// The epilogue warps' named barrier (1): every thread contributes v, gets the AND.
+__device__ __forceinline__ bool epi_all(bool v) {
+    int out;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(out)
+        : "r"((int)v), "n"(kMParts * 128)
+        : "memory");
+    return out != 0;
+}
+
+// Programmatic dependent launch: the next kernel of the chain may start its
+// set-up on idle SMs (trigger); it touches nothing that earlier kernels write
+// or read before they have finished (wait).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__global__ void __launch_bounds__(kMThreads, 1) k_mlp_gemm(const __grid_constant__ GemmBatch gb) {
     extern __shared__ uint8_t raw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
-    const int S = g.stages;
+    const int pb = (int)blockIdx.x >= gb.first[2] ? 2 : ((int)blockIdx.x >= gb.first[1] ? 1 : 0);
+    const GemmCfg &g = gb.g[pb];
+    const int S = gb.stages;
     constexpr uint32_t a_bytes = kMM * 128;
-    const uint32_t b_bytes = (uint32_t)(g.nch * g.bn) * 128u;
-    const uint32_t st_bytes = a_bytes + b_bytes;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + (size_t)S * st_bytes);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + (size_t)S * gb.st_bytes);
     uint64_t *full = bars, *empty = bars + S, *accb = bars + 2 * S;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * S + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * kMM;
-    const int nb = blockIdx.y * g.nch * g.bn;  // first output column of this CTA
-    const int ks0 = blockIdx.z * g.k_steps;
+    float4 *red = reinterpret_cast<float4 *>(bars + 2 * S + 2);  // [kMParts][128] (softmax)
+    float *sbias = reinterpret_cast<float *>(red + kMParts * kMM);  // [512]
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int cta = (int)blockIdx.x - gb.first[pb];
+    const int bx = cta % g.mt, by = cta / g.mt % g.nt, bz = cta / (g.mt * g.nt);
+    const int m0 = bx * kMM;
+    const int nb = by * g.nch * g.bn;  // first output column of this CTA
+    const int ks0 = bz * g.k_steps;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < S; ++i) {
@@ -137,10 +206,14 @@ __global__ void __launch_bounds__(kMThreads, 1)
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(g.tmem_cols)
+                     "r"(gb.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_trigger();
+    pdl_wait();
+    if (g.bias)  // this CTA's columns, zero past the output
+        for (int i = threadIdx.x; i < g.nch * g.bn; i += kMThreads) sbias[i] = nb + i < g.N ? g.bias[nb + i] : 0.f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -149,17 +222,19 @@ __global__ void __launch_bounds__(kMThreads, 1)
     if (warp == 0) {
         // ------------------------------------------------------------ TMA
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&ta) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tb) : "memory");
+            const CUtensorMap *ta = &gb.ta[pb], *tb = &gb.tb[pb];
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)ta) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)tb) : "memory");
+            const uint32_t bytes = a_bytes + (uint32_t)(g.nch * g.bn) * 128u;
             int i = 0;
             for (; i < g.k_steps; ++i) {
                 const int s = i % S, f = i / S;
                 if (f > 0 && !mwait(&empty[s], (f - 1) & 1, g.err)) break;
-                uint8_t *st = sm + (size_t)s * st_bytes;
-                mbar_arrive_expect_tx(&full[s], st_bytes);
+                uint8_t *st = sm + (size_t)s * gb.st_bytes;
+                mbar_arrive_expect_tx(&full[s], bytes);
                 const int kc = (ks0 + i) * kMK;
-                tma_2d(st, &ta, kc, m0, &full[s]);
-                for (int c = 0; c < g.nch; ++c) tma_2d(st + a_bytes + c * g.bn * 128, &tb, kc, nb + c * g.bn, &full[s]);
+                tma_2d(st, ta, kc, m0, &full[s]);
+                for (int c = 0; c < g.nch; ++c) tma_2d(st + a_bytes + c * g.bn * 128, tb, kc, nb + c * g.bn, &full[s]);
             }
             // every issued copy has landed before the block can exit
             for (int j = i - S < 0 ? 0 : i - S; j < i; ++j) mwait(&full[j % S], (j / S) & 1, g.err);
@@ -174,7 +249,7 @@ __global__ void __launch_bounds__(kMThreads, 1)
                 const int s = i % S;
                 if (!mwait(&full[s], (i / S) & 1, g.err)) break;
                 tc_fence_after();
-                const uint8_t *st = sm + (size_t)s * st_bytes;
+                const uint8_t *st = sm + (size_t)s * gb.st_bytes;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {  // four K = 16 steps inside the 128-byte row
                     const uint64_t da = desc_sw128(smem_u32(st + j * 32));
@@ -203,134 +278,168 @@ __global__ void __launch_bounds__(kMThreads, 1)
         __syncwarp();
     } else {
         // ------------------------------------------------------- epilogue
-        const int q = warp & 3;  // TMEM lane quadrant of this warp
+        const int part = (warp - 2) >> 2;  // quarter of the columns
+        const int q = warp & 3;            // TMEM lane quadrant of this warp
         const int r = q * 32 + lane;
         const int row = m0 + r;
         const bool valid = row < g.M;
-        const bool ok = __all_sync(0xffffffffu, mwait(accb, 0, g.err));
+        const bool ok = epi_all(mwait(accb, 0, g.err));
         tc_fence_after();
         const uint32_t tb_ = tmem + ((uint32_t)(q * 32) << 16);
-        const int TC = g.nch * g.bn;
+        const int units = g.nch * g.bn >> 4;  // of 16 columns
+        const int u0 = part * units / kMParts, u1 = (part + 1) * units / kMParts;
         const int rw = (m0 + q * 32) >> 5;  // row warp (for the per-warp column sums)
-        if (ok) {
-            if (g.mode == E_GELU || g.mode == E_MUL || g.mode == E_F32) {
-                for (int c0 = 0; c0 < TC; c0 += 16) {
-                    uint32_t v[16];
-                    tmem_ld16_async(tb_ + c0, v);
-                    tmem_wait16(v);
-                    const int n0 = nb + c0;
-                    if (n0 >= g.N) break;  // warp-uniform; N is a multiple of 16
-                    float a[16];
-                    if (g.mode == E_GELU) {
-                        float d[16];
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const float z = __uint_as_float(v[j]) + g.bias[n0 + j];
-                            a[j] = gelu(z);
-                            d[j] = gelu_d(z);
-                        }
-                        if (valid) {
-                            if (g.out) store_bf16x16(g.out + (size_t)row * g.ldo + n0, a);
-                            if (g.aux) {
-                                float4 *ap = reinterpret_cast<float4 *>(g.aux + (size_t)row * g.lda + n0);
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) ap[j] = make_float4(d[4 * j], d[4 * j + 1], d[4 * j + 2], d[4 * j + 3]);
-                            }
-                        }
-                    } else if (g.mode == E_MUL) {
-                        if (valid) {
-                            const float4 *ap = reinterpret_cast<const float4 *>(g.aux + (size_t)row * g.lda + n0);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const float4 dd = ap[j];
-                                a[4 * j] = __uint_as_float(v[4 * j]) * dd.x;
-                                a[4 * j + 1] = __uint_as_float(v[4 * j + 1]) * dd.y;
-                                a[4 * j + 2] = __uint_as_float(v[4 * j + 2]) * dd.z;
-                                a[4 * j + 3] = __uint_as_float(v[4 * j + 3]) * dd.w;
-                            }
-                            if (g.out) store_bf16x16(g.out + (size_t)row * g.ldo + n0, a);
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) a[j] = 0.f;
-                        }
-                        if (g.colsum) {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                const float cs = lane_sum(a[j]);
-                                if (lane == 0) g.colsum[(size_t)rw * g.ldc + n0 + j] = cs;
-                            }
-                        }
-                    } else {  // E_F32
-                        if (valid) {
-                            float4 *pp = reinterpret_cast<float4 *>(g.part + (size_t)blockIdx.z * g.part_split +
-                                                                    (size_t)row * g.ldp + n0);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                pp[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                    __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-                        }
-                        continue;
-                    }
-                    if (g.outT && valid) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) g.outT[(size_t)(n0 + j) * g.ldt + row] = bf16_bits(a[j]);
-                    }
-                }
-            } else {  // E_SOFTMAX (one N tile: nb == 0)
-                float mx = -INFINITY;
-                for (int c0 = 0; c0 < TC; c0 += 16) {
-                    uint32_t v[16];
-                    tmem_ld16_async(tb_ + c0, v);
-                    tmem_wait16(v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (c0 + j < g.N) mx = fmaxf(mx, __uint_as_float(v[j]) + g.bias[c0 + j]);
-                }
-                const int y = valid ? g.y[row] : -1;
-                float s = 0.f, ly = 0.f, best = -INFINITY;
-                int bi = 0;
-                for (int c0 = 0; c0 < TC; c0 += 16) {
-                    uint32_t v[16];
-                    tmem_ld16_async(tb_ + c0, v);
-                    tmem_wait16(v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int n = c0 + j;
-                        if (n < g.N) {
-                            const float l = __uint_as_float(v[j]) + g.bias[n];
-                            s += expf(l - mx);
-                            if (n == y) ly = l;
-                            if (l > best) {
-                                best = l;
-                                bi = n;
-                            }
-                        }
-                    }
-                }
-                const float inv_s = 1.0f / s;
-                for (int c0 = 0; c0 < TC; c0 += 16) {
-                    uint32_t v[16];
-                    tmem_ld16_async(tb_ + c0, v);
-                    tmem_wait16(v);
+        if (ok && g.mode != E_SOFTMAX) {
+            for (int u = u0; u < u1; ++u) {
+                const int c0 = u * 16, n0 = nb + c0;
+                if (n0 >= g.N) break;  // warp-uniform; N is a multiple of 16
+                uint32_t v[16];
+                tmem_ld16_async(tb_ + c0, v);
+                tmem_wait16(v);
+                float a[16];
+                if (g.mode == E_GELU) {
                     float d[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
-                        const int n = c0 + j;
-                        const float l = __uint_as_float(v[j]) + (n < g.N ? g.bias[n] : 0.f);
-                        d[j] = (valid && n < g.N) ? (expf(l - mx) * inv_s - (n == y ? 1.f : 0.f)) * g.scale : 0.f;
+                        const float z = __uint_as_float(v[j]) + sbias[c0 + j];
+                        a[j] = gelu(z);
+                        d[j] = gelu_d(z);
                     }
                     if (valid) {
-                        store_bf16x16(g.out + (size_t)row * g.ldo + c0, d);
+                        store_bf16x16(g.out + (size_t)row * g.ldo + n0, a);
+                        float4 *ap = reinterpret_cast<float4 *>(g.aux + (size_t)row * g.lda + n0);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (c0 + j < g.N) g.outT[(size_t)(c0 + j) * g.ldt + row] = bf16_bits(d[j]);
+                        for (int j = 0; j < 4; ++j)
+                            ap[j] = make_float4(d[4 * j], d[4 * j + 1], d[4 * j + 2], d[4 * j + 3]);
                     }
+                } else if (g.mode == E_MUL) {
+                    if (valid) {
+                        const float4 *ap = reinterpret_cast<const float4 *>(g.aux + (size_t)row * g.lda + n0);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float cs = lane_sum(d[j]);
-                        if (lane == 0 && c0 + j < g.N) g.colsum[(size_t)rw * g.ldc + c0 + j] = cs;
+                        for (int j = 0; j < 4; ++j) {
+                            const float4 dd = ap[j];
+                            a[4 * j] = __uint_as_float(v[4 * j]) * dd.x;
+                            a[4 * j + 1] = __uint_as_float(v[4 * j + 1]) * dd.y;
+                            a[4 * j + 2] = __uint_as_float(v[4 * j + 2]) * dd.z;
+                            a[4 * j + 3] = __uint_as_float(v[4 * j + 3]) * dd.w;
+                        }
+                        if (g.out) store_bf16x16(g.out + (size_t)row * g.ldo + n0, a);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) a[j] = 0.f;
+                    }
+                    int col;
+                    const float cs = lane_sums16(a, lane, col);
+                    if (!(lane & 1)) g.colsum[(size_t)rw * g.ldc + n0 + col] = cs;
+                } else {  // E_F32
+                    if (valid) {
+                        float4 *pp = reinterpret_cast<float4 *>(g.part + (size_t)bz * g.part_split +
+                                                                (size_t)row * g.ldp + n0);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            pp[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                                __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+                    }
+                    continue;
+                }
+                if (g.outT && valid) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) g.outT[(size_t)(n0 + j) * g.ldt + row] = bf16_bits(a[j]);
+                }
+            }
+        } else if (ok) {  // E_SOFTMAX (one N tile: nb == 0); a row's four warps meet in shared memory
+            float mx = -INFINITY;
+            int bi = 0;
+            for (int u = u0; u < u1; ++u) {
+                uint32_t v[16];
+                tmem_ld16_async(tb_ + u * 16, v);
+                tmem_wait16(v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int n = u * 16 + j;
+                    if (n < g.N) {
+                        const float l = __uint_as_float(v[j]) + sbias[n];
+                        if (l > mx) {
+                            mx = l;
+                            bi = n;
+                        }
                     }
                 }
+            }
+            red[part * kMM + r] = make_float4(mx, __int_as_float(bi), 0.f, 0.f);
+            epi_all(true);
+            mx = -INFINITY;
+            bi = 0;
+#pragma unroll
+            for (int k = 0; k < kMParts; ++k) {  // ascending columns: the first largest
+                const float4 o = red[k * kMM + r];
+                if (o.x > mx) {
+                    mx = o.x;
+                    bi = __float_as_int(o.y);
+                }
+            }
+            epi_all(true);  // read before it is written again
+            const int y = valid ? g.y[row] : -1;
+            // exp(l - max) takes the logits' place in TMEM
+            float ly = 0.f;
+            for (int u = u0; u < u1; ++u) {
+                uint32_t v[16];
+                tmem_ld16_async(tb_ + u * 16, v);
+                tmem_wait16(v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int n = u * 16 + j;
+                    const float l = __uint_as_float(v[j]) + sbias[n];
+                    if (n == y) ly = l;
+                    v[j] = __float_as_uint(n < g.N ? expf(l - mx) : 0.f);
+                }
+                tmem_st16(tb_ + u * 16, v);
+            }
+            // their sum in ascending columns (one running sum per row, handed from
+            // quarter to quarter: the rounding of a plain loop over the classes)
+            float s = 0.f;
+#pragma unroll 1
+            for (int k = 0; k < kMParts; ++k) {
+                if (part == k) {
+                    if (k > 0) s = red[(k - 1) * kMM + r].x;
+                    for (int u = u0; u < u1; ++u) {
+                        uint32_t v[16];
+                        tmem_ld16_async(tb_ + u * 16, v);
+                        tmem_wait16(v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) s += __uint_as_float(v[j]);  // zero past the classes
+                    }
+                    red[k * kMM + r] = make_float4(s, ly, 0.f, 0.f);
+                }
+                asm volatile("bar.sync %0, %1;" ::"r"(2 + q), "n"(kMParts * 32) : "memory");
+            }
+            s = red[(kMParts - 1) * kMM + r].x;
+            ly = 0.f;
+#pragma unroll
+            for (int k = 0; k < kMParts; ++k) ly += red[k * kMM + r].y;  // the other quarters hold zero
+            const float inv_s = 1.0f / s;
+            for (int u = u0; u < u1; ++u) {
+                const int c0 = u * 16;
+                uint32_t v[16];
+                tmem_ld16_async(tb_ + c0, v);
+                tmem_wait16(v);
+                float d[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int n = c0 + j;
+                    d[j] = (valid && n < g.N) ? (__uint_as_float(v[j]) * inv_s - (n == y ? 1.f : 0.f)) * g.scale : 0.f;
+                }
+                if (valid) {
+                    store_bf16x16(g.out + (size_t)row * g.ldo + c0, d);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (c0 + j < g.N) g.outT[(size_t)(c0 + j) * g.ldt + row] = bf16_bits(d[j]);
+                }
+                int col;
+                const float cs = lane_sums16(d, lane, col);
+                if (!(lane & 1) && c0 + col < g.N) g.colsum[(size_t)rw * g.ldc + c0 + col] = cs;
+            }
+            if (part == 0) {
                 const float ce = valid ? (logf(s) + mx - ly) : 0.f;
                 const float hit = (valid && bi == y) ? 1.f : 0.f;
                 const float ces = lane_sum(ce), hits = lane_sum(hit), rows = lane_sum(valid ? 1.f : 0.f);
@@ -346,7 +455,7 @@ __global__ void __launch_bounds__(kMThreads, 1)
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.tmem_cols)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(gb.tmem_cols)
                      : "memory");
     }
 }
@@ -675,7 +784,7 @@ __device__ __host__ __forceinline__ uint64_t splitmix64(uint64_t z) {
 
 struct MlpState {
     int32_t t;      // Adam steps taken
-    int32_t pad;
+    int32_t err;    // KM_ETIMEOUT when a bounded wait gave up
     double loss[3]; // cross-entropy sum, correct predictions, rows (since the last read)
 };
 
@@ -683,23 +792,34 @@ struct MlpState {
 // counter-based draw per (seed, step, row)), or rows 0..B-1 when seed is
 // ~0ull.  Writes Xb (B x Dk bfloat16, zero padding), XbT (Dn x B, rows >= D
 // zero) and the classes yb (labels mapped to contiguous groups when K > 0).
-__global__ void k_mlp_gather(const float *X, int64_t N, int D, const int32_t *labels, int K, int G, int B, int Dk,
-                             int Dn, uint64_t seed, const MlpState *st, uint16_t *Xb, uint16_t *XbT, int32_t *yb) {
-    const int i = blockIdx.x;  // one block per row
-    if (i >= B) return;
-    int64_t src = i;
-    if (seed != ~0ull) src = (int64_t)(splitmix64(seed ^ splitmix64(((uint64_t)st->t << 32) | (uint32_t)i)) % (uint64_t)N);
-    for (int d = threadIdx.x; d < Dk; d += blockDim.x) {
-        const float v = d < D ? X[src * D + d] : 0.f;
-        const uint16_t b = bf16_bits(v);
-        Xb[(size_t)i * Dk + d] = b;
-        if (d < Dn) XbT[(size_t)d * B + i] = b;
+// A block per 32 rows: the rows pass through shared memory, so that both copies
+// are written in runs of consecutive elements.
+constexpr int kGatherRows = 32, kGatherThreads = 256;
+__global__ void __launch_bounds__(kGatherThreads)
+    k_mlp_gather(const float *X, int64_t N, int D, const int32_t *labels, int K, int G, int B, int Dk, int Dn,
+                 uint64_t seed, const MlpState *st, uint16_t *Xb, uint16_t *XbT, int32_t *yb) {
+    __shared__ uint16_t tile[kGatherRows][256 + 2];  // Dk <= 256
+    pdl_trigger();
+    const int i0 = blockIdx.x * kGatherRows;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = warp; k < kGatherRows && i0 + k < B; k += kGatherThreads / 32) {
+        const int i = i0 + k;
+        int64_t src = i;
+        if (seed != ~0ull) src = (int64_t)(splitmix64(seed ^ splitmix64(((uint64_t)st->t << 32) | (uint32_t)i)) % (uint64_t)N);
+        for (int d = lane; d < Dk; d += 32) {
+            const uint16_t b = bf16_bits(d < D ? X[src * D + d] : 0.f);
+            Xb[(size_t)i * Dk + d] = b;
+            tile[k][d] = b;
+        }
+        if (lane == 0) {
+            int y = labels[src];
+            if (K > 0) y = (int)(((int64_t)y * G) / K);
+            yb[i] = (y >= 0 && y < G) ? y : 0;
+        }
     }
-    if (threadIdx.x == 0) {
-        int y = labels[src];
-        if (K > 0) y = (int)(((int64_t)y * G) / K);
-        yb[i] = (y >= 0 && y < G) ? y : 0;
-    }
+    __syncthreads();
+    if (i0 + lane < B)
+        for (int d = warp; d < Dn; d += kGatherThreads / 32) XbT[(size_t)d * B + i0 + lane] = tile[lane][d];
 }
 
 struct MlpDims {
@@ -710,6 +830,7 @@ struct MlpDims {
 
 struct ApplyArgs {
     int mode;           // 0: gradient out, 1: Adam step, 2: copy the masters to the compute weights
+    int wblocks;        // blocks for the weights (the others take the biases)
     float *master, *m1, *m2;
     const float *pW1, *pW2, *pW3;  // split-K partials
     int s1, s2, s3;
@@ -725,54 +846,88 @@ struct ApplyArgs {
 
 // One thread per parameter: its gradient (sum of the split-K partials or of
 // the per-warp column sums), then the requested action; the compute copies
-// (bfloat16 weights, padded FP32 biases) are rewritten from the masters.
-__global__ void k_mlp_apply(MlpDims d, ApplyArgs a) {
+// (bfloat16 weights, padded FP32 biases) are rewritten from the masters.  The
+// last blocks take the biases, 32 a block: eight warps sum an eighth of the
+// row warps each (one thread over all of them took 20 us).
+constexpr int kApplyThreads = 256;
+__device__ __forceinline__ void apply_one(const MlpDims &d, const ApplyArgs &a, int64_t i, float gsum, float bc1,
+                                          float bc2) {
+    // Adam (Kingma and Ba): bias-corrected first and second moments
+    const float m = a.b1 * a.m1[i] + (1.0f - a.b1) * gsum;
+    const float v = a.b2 * a.m2[i] + (1.0f - a.b2) * gsum * gsum;
+    a.m1[i] = m;
+    a.m2[i] = v;
+    a.master[i] -= a.lr * (m / bc1) / (sqrtf(v / bc2) + a.eps);
+}
+__global__ void __launch_bounds__(kApplyThreads) k_mlp_apply(MlpDims d, ApplyArgs a) {
+    __shared__ float part[kApplyThreads];
+    pdl_trigger();
+    pdl_wait();
     const int t1 = a.mode == 1 ? a.st->t + 1 : 0;
     const float bc1 = a.mode == 1 ? 1.0f - powf(a.b1, (float)t1) : 1.f;
     const float bc2 = a.mode == 1 ? 1.0f - powf(a.b2, (float)t1) : 1.f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d.P; i += (int64_t)gridDim.x * blockDim.x) {
-        int seg;
-        int64_t o;
-        if (i < d.ob1) { seg = 0; o = i - d.oW1; }
-        else if (i < d.oW2) { seg = 1; o = i - d.ob1; }
-        else if (i < d.ob2) { seg = 2; o = i - d.oW2; }
-        else if (i < d.oW3) { seg = 3; o = i - d.ob2; }
-        else if (i < d.ob3) { seg = 4; o = i - d.oW3; }
-        else { seg = 5; o = i - d.ob3; }
-        int r = 0, c = 0;  // (row, column) of a weight
-        if (seg == 0) { r = (int)(o / d.D); c = (int)(o % d.D); }
-        else if (seg == 2) { r = (int)(o / d.H); c = (int)(o % d.H); }
-        else if (seg == 4) { r = (int)(o / d.H); c = (int)(o % d.H); }
+    if ((int)blockIdx.x >= a.wblocks) {
+        // biases: b1, b2 (H each), b3 (G) as one run
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int o = ((int)blockIdx.x - a.wblocks) * 32 + lane;
+        const bool in = o < 2 * d.H + d.G;
+        const int seg = o < d.H ? 0 : (o < 2 * d.H ? 1 : 2);
+        const int c = seg == 0 ? o : (seg == 1 ? o - d.H : o - 2 * d.H);
+        const int64_t i = (seg == 0 ? d.ob1 : (seg == 1 ? d.ob2 : d.ob3)) + c;
+        float gsum = 0.f;
         if (a.mode != 2) {
-            float gsum = 0.f;
-            switch (seg) {
-                case 0: for (int z = 0; z < a.s1; ++z) gsum += a.pW1[z * a.ps1 + (int64_t)r * d.Dn + c]; break;
-                case 1: for (int w = 0; w < a.nrw; ++w) gsum += a.cs1[(int64_t)w * d.Hp + o]; break;
-                case 2: for (int z = 0; z < a.s2; ++z) gsum += a.pW2[z * a.ps2 + (int64_t)r * d.Hp + c]; break;
-                case 3: for (int w = 0; w < a.nrw; ++w) gsum += a.cs2[(int64_t)w * d.Hp + o]; break;
-                case 4: for (int z = 0; z < a.s3; ++z) gsum += a.pW3[z * a.ps3 + (int64_t)r * d.Hp + c]; break;
-                default: for (int w = 0; w < a.nrw; ++w) gsum += a.cs3[(int64_t)w * d.G + o]; break;
+            const float *cs = seg == 0 ? a.cs1 : (seg == 1 ? a.cs2 : a.cs3);
+            const int ld = seg == 2 ? d.G : d.Hp;
+            float sum = 0.f;
+            if (in) {
+#pragma unroll 8
+                for (int w = warp; w < a.nrw; w += kApplyThreads / 32) sum += cs[(int64_t)w * ld + c];
             }
+            part[threadIdx.x] = sum;
+            __syncthreads();
+            if (warp == 0)
+                for (int w = 0; w < kApplyThreads / 32; ++w) gsum += part[w * 32 + lane];
+        }
+        if (warp != 0 || !in) return;
+        if (a.mode == 0) {
+            a.grad[i] = gsum;
+            return;
+        }
+        if (a.mode == 1) apply_one(d, a, i, gsum, bc1, bc2);
+        (seg == 0 ? a.b1p : (seg == 1 ? a.b2p : a.b3p))[c] = a.master[i];
+        return;
+    }
+    // weights: W1, W2, W3 as one run
+    const int64_t n1 = (int64_t)d.H * d.D, n2 = (int64_t)d.H * d.H, nw = n1 + n2 + (int64_t)d.G * d.H;
+    for (int64_t o = (int64_t)blockIdx.x * kApplyThreads + threadIdx.x; o < nw; o += (int64_t)a.wblocks * kApplyThreads) {
+        const int seg = o < n1 ? 0 : (o < n1 + n2 ? 1 : 2);
+        const int64_t w = seg == 0 ? o : (seg == 1 ? o - n1 : o - n1 - n2);
+        const int64_t i = (seg == 0 ? d.oW1 : (seg == 1 ? d.oW2 : d.oW3)) + w;
+        const int ld = seg == 0 ? d.D : d.H;
+        const int r = (int)(w / ld), c = (int)(w - (int64_t)r * ld);  // (row, column) of the weight
+        if (a.mode != 2) {
+            const float *pw = seg == 0 ? a.pW1 : (seg == 1 ? a.pW2 : a.pW3);
+            const int sn = seg == 0 ? a.s1 : (seg == 1 ? a.s2 : a.s3);
+            const int64_t ps = seg == 0 ? a.ps1 : (seg == 1 ? a.ps2 : a.ps3);
+            pw += (int64_t)r * (seg == 0 ? d.Dn : d.Hp) + c;
+            float gsum = 0.f;
+#pragma unroll 8
+            for (int z = 0; z < sn; ++z) gsum += pw[z * ps];
             if (a.mode == 0) {
                 a.grad[i] = gsum;
                 continue;
             }
-            // Adam (Kingma and Ba): bias-corrected first and second moments
-            const float m = a.b1 * a.m1[i] + (1.0f - a.b1) * gsum;
-            const float v = a.b2 * a.m2[i] + (1.0f - a.b2) * gsum * gsum;
-            a.m1[i] = m;
-            a.m2[i] = v;
-            a.master[i] -= a.lr * (m / bc1) / (sqrtf(v / bc2) + a.eps);
+            apply_one(d, a, i, gsum, bc1, bc2);
         }
-        const float w = a.master[i];
-        const uint16_t wb = bf16_bits(w);
-        switch (seg) {
-            case 0: a.W1b[(size_t)r * d.Dk + c] = wb; break;
-            case 1: a.b1p[o] = w; break;
-            case 2: a.W2b[(size_t)r * d.Hp + c] = wb; a.W2T[(size_t)c * d.Hp + r] = wb; break;
-            case 3: a.b2p[o] = w; break;
-            case 4: a.W3b[(size_t)r * d.Hp + c] = wb; a.W3T[(size_t)c * d.Gk + r] = wb; break;
-            default: a.b3p[o] = w; break;
+        const uint16_t wb = bf16_bits(a.master[i]);
+        if (seg == 0) {
+            a.W1b[(size_t)r * d.Dk + c] = wb;
+        } else if (seg == 1) {
+            a.W2b[(size_t)r * d.Hp + c] = wb;
+            a.W2T[(size_t)c * d.Hp + r] = wb;
+        } else {
+            a.W3b[(size_t)r * d.Hp + c] = wb;
+            a.W3T[(size_t)c * d.Gk + r] = wb;
         }
     }
 }
@@ -818,7 +973,7 @@ struct kmeans_mlp {
     uint16_t *W1b = nullptr, *W2b = nullptr, *W2T = nullptr, *W3b = nullptr, *W3T = nullptr;
     float *b1p = nullptr, *b2p = nullptr, *b3p = nullptr;
     MlpState *st = nullptr;
-    int *err = nullptr;
+    int *err = nullptr;  // &st->err
     // training buffers (batch B)
     int B = 0;
     uint16_t *Xb = nullptr, *XbT = nullptr, *A1 = nullptr, *A1T = nullptr, *A2 = nullptr, *A2T = nullptr,
@@ -827,6 +982,12 @@ struct kmeans_mlp {
           *cs2 = nullptr, *cs3 = nullptr;
     int32_t *yb = nullptr;
     int s1 = 1, s2 = 1, s3 = 1;
+    // the training products of a batch of B rows, as launched: layers 1, 2, 3, dZ2,
+    // dZ1, and the three weight gradients together
+    static constexpr int kPlans = 6;
+    GemmBatch plan[kPlans];
+    int grid[kPlans] = {};
+    size_t smem[kPlans] = {};
     std::vector<void *> batch_allocs;
     std::vector<void *> allocs;
     char errmsg[512] = "";
@@ -896,33 +1057,61 @@ struct GemmSpec {
     int splits;
 };
 
-int launch_gemm(kmeans_mlp *m, const GemmSpec &sp, GemmCfg g, cudaStream_t s) {
-    CUtensorMap ta, tb;
+// adds a product to launch `k` of the network's plan
+int plan_add(kmeans_mlp *m, int k, int idx, const GemmSpec &sp, GemmCfg g) {
+    GemmBatch &b = m->plan[k];
+    if (idx == 0) {
+        memset(&b, 0, sizeof(b));
+        m->grid[k] = 0;
+    }
     int rc;
-    if ((rc = make_map(m, &ta, sp.A, sp.a_rows, sp.K, sp.a_ld, kMM))) return rc;
-    if ((rc = make_map(m, &tb, sp.Bm, sp.b_rows, sp.K, sp.b_ld, sp.bn))) return rc;
+    if ((rc = make_map(m, &b.ta[idx], sp.A, sp.a_rows, sp.K, sp.a_ld, kMM))) return rc;
+    if ((rc = make_map(m, &b.tb[idx], sp.Bm, sp.b_rows, sp.K, sp.b_ld, sp.bn))) return rc;
     g.M = sp.M;
     g.N = sp.N;
+    g.mt = (sp.M + kMM - 1) / kMM;
+    g.nt = sp.ntiles;
     g.nch = sp.nch;
     g.bn = sp.bn;
     g.k_steps = (int)(sp.K / kMK / sp.splits);
-    g.tmem_cols = pow2_at_least(sp.nch * sp.bn);
     g.err = m->err;
-    const size_t st_bytes = (size_t)kMM * 128 + (size_t)sp.nch * sp.bn * 128;
+    b.g[idx] = g;
+    b.first[idx] = m->grid[k];
+    m->grid[k] += g.mt * g.nt * sp.splits;
+    for (int i = idx + 1; i < 4; ++i) b.first[i] = m->grid[k];
+    b.st_bytes = std::max<uint32_t>(b.st_bytes, (uint32_t)kMM * 128u + (uint32_t)(sp.nch * sp.bn) * 128u);
+    b.tmem_cols = std::max(b.tmem_cols, pow2_at_least(sp.nch * sp.bn));
+    const size_t fixed = 1024 + 256 + (size_t)kMParts * kMM * 16 + 512 * 4;  // alignment, barriers, row reductions, bias
     int stages = 4;
-    while (stages > 2 && 1024 + stages * st_bytes + 256 > m->smem_optin) --stages;
-    g.stages = stages;
-    size_t smem = 1024 + stages * st_bytes + 256;
-    // CTAs resident on one SM must not ask for more than its 512 TMEM columns
-    const size_t sm_smem = 233472;  // shared memory per SM
-    while ((sm_smem / smem) * (size_t)g.tmem_cols > 512) smem += 4096;
-    if (smem > m->smem_optin) return mlp_fail(m, KM_EINVAL, "product tile does not fit in shared memory");
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return mlp_fail(m, KM_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    dim3 grid((unsigned)((sp.M + kMM - 1) / kMM), (unsigned)sp.ntiles, (unsigned)sp.splits);
+    while (stages > 2 && fixed + stages * (size_t)b.st_bytes > m->smem_optin) --stages;
+    b.stages = stages;
+    // (the 576 threads' registers let one CTA reside on an SM, so the TMEM columns always suffice)
+    m->smem[k] = fixed + stages * (size_t)b.st_bytes;
+    if (m->smem[k] > m->smem_optin) return mlp_fail(m, KM_EINVAL, "product tile does not fit in shared memory");
+    return KM_OK;
+}
+
+// a launch that may begin before the kernel ahead of it on the stream ends
+// (the kernel waits for it itself: pdl_wait)
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+                       const A &...args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
     count_launch();
-    k_mlp_gemm<<<grid, kMThreads, smem, s>>>(ta, tb, g);
-    e = cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+int launch_plan(kmeans_mlp *m, int k, cudaStream_t s) {
+    const cudaError_t e = launch_pdl(k_mlp_gemm, (unsigned)m->grid[k], kMThreads, m->smem[k], s, m->plan[k]);
     if (e != cudaSuccess) return mlp_fail(m, KM_ECUDA, "k_mlp_gemm launch: %s", cudaGetErrorString(e));
     return KM_OK;
 }
@@ -947,6 +1136,46 @@ void hidden_tiles(const kmeans_mlp *m, int M, int &bn, int &ntiles) {
     }
 }
 
+// the launches of one batch's forward and backward pass
+int plan_batch(kmeans_mlp *m, int B) {
+    const MlpDims &d = m->d;
+    int rc, bnh, nth;
+    hidden_tiles(m, B, bnh, nth);
+    // layer 1: A1 = GELU(Xb W1^T + b1), with A1^T and GELU'(z1)
+    GemmCfg g = cfg0(E_GELU);
+    g.bias = m->b1p; g.out = m->A1; g.ldo = d.Hp; g.outT = m->A1T; g.ldt = B; g.aux = m->G1; g.lda = d.Hp;
+    if ((rc = plan_add(m, 0, 0, {m->Xb, B, d.Dk, m->W1b, d.Hp, d.Dk, d.Dk, B, d.Hp, 1, bnh, nth, 1}, g))) return rc;
+    // layer 2
+    g = cfg0(E_GELU);
+    g.bias = m->b2p; g.out = m->A2; g.ldo = d.Hp; g.outT = m->A2T; g.ldt = B; g.aux = m->G2; g.lda = d.Hp;
+    if ((rc = plan_add(m, 1, 0, {m->A1, B, d.Hp, m->W2b, d.Hp, d.Hp, d.Hp, B, d.Hp, 1, bnh, nth, 1}, g))) return rc;
+    // layer 3 + softmax cross-entropy: dZ3 = (softmax - onehot) / B
+    g = cfg0(E_SOFTMAX);
+    g.bias = m->b3p; g.out = m->dZ3; g.ldo = d.Gk; g.outT = m->dZ3T; g.ldt = B; g.colsum = m->cs3; g.ldc = d.G;
+    g.y = m->yb; g.scale = 1.0f / (float)B; g.loss = m->st->loss;
+    if ((rc = plan_add(m, 2, 0, {m->A2, B, d.Hp, m->W3b, d.G, d.Hp, d.Hp, B, d.G, m->nch3, m->bn3, 1, 1}, g)))
+        return rc;
+    // dZ2 = (dZ3 W3) * GELU'(z2)
+    g = cfg0(E_MUL);
+    g.aux = m->G2; g.lda = d.Hp; g.out = m->dZ2; g.ldo = d.Hp; g.outT = m->dZ2T; g.ldt = B; g.colsum = m->cs2;
+    g.ldc = d.Hp;
+    if ((rc = plan_add(m, 3, 0, {m->dZ3, B, d.Gk, m->W3T, d.Hp, d.Gk, d.Gk, B, d.Hp, 1, bnh, nth, 1}, g))) return rc;
+    // dZ1 = (dZ2 W2) * GELU'(z1)
+    g = cfg0(E_MUL);
+    g.aux = m->G1; g.lda = d.Hp; g.outT = m->dZ1T; g.ldt = B; g.colsum = m->cs1; g.ldc = d.Hp;
+    if ((rc = plan_add(m, 4, 0, {m->dZ2, B, d.Hp, m->W2T, d.Hp, d.Hp, d.Hp, B, d.Hp, 1, bnh, nth, 1}, g))) return rc;
+    // weight gradients, contracted over the batch: dW3 = dZ3^T A2, dW2 = dZ2^T A1, dW1 = dZ1^T X
+    g = cfg0(E_F32);
+    g.part = m->pW3; g.ldp = d.Hp; g.part_split = (int64_t)d.G * d.Hp;
+    if ((rc = plan_add(m, 5, 0, {m->dZ3T, d.G, B, m->A2T, d.Hp, B, B, d.G, d.Hp, 1, d.Hp, 1, m->s3}, g))) return rc;
+    g = cfg0(E_F32);
+    g.part = m->pW2; g.ldp = d.Hp; g.part_split = (int64_t)d.Hp * d.Hp;
+    if ((rc = plan_add(m, 5, 1, {m->dZ2T, d.Hp, B, m->A1T, d.Hp, B, B, d.Hp, d.Hp, 1, d.Hp, 1, m->s2}, g))) return rc;
+    g = cfg0(E_F32);
+    g.part = m->pW1; g.ldp = d.Dn; g.part_split = (int64_t)d.Hp * d.Dn;
+    return plan_add(m, 5, 2, {m->dZ1T, d.Hp, B, m->XbT, d.Dn, B, B, d.Hp, d.Dn, 1, d.Dn, 1, m->s1}, g);
+}
+
 int alloc_batch(kmeans_mlp *m, int B) {
     if (m->B == B) return KM_OK;
     for (void *p : m->batch_allocs) cudaFreeAsync(p, m->stream);
@@ -954,17 +1183,13 @@ int alloc_batch(kmeans_mlp *m, int B) {
     m->B = 0;
     const MlpDims &d = m->d;
     auto &L = m->batch_allocs;
-    // split-K of the weight gradients: at least 4 slices of 64 per CTA, about
-    // one wave of CTAs
-    auto splits_for = [&](int mrows) {
-        const int tiles = (mrows + kMM - 1) / kMM;
-        int s = 1;
-        while (s * 2 * tiles <= m->num_sms && (B / 64) % (s * 2) == 0 && B / 64 / (s * 2) >= 4) s *= 2;
-        return s;
-    };
-    m->s1 = splits_for(d.Hp);
-    m->s2 = splits_for(d.Hp);
-    m->s3 = splits_for(d.G);
+    // split-K of the weight gradients: at least 4 slices of 64 per CTA, at most
+    // one wave of CTAs for the three products together (fewer partial sums to
+    // write and read back than with a wave for each)
+    const int tiles = 2 * ((d.Hp + kMM - 1) / kMM) + (d.G + kMM - 1) / kMM;
+    int sk = 1;
+    while (sk * 2 * tiles <= m->num_sms && (B / 64) % (sk * 2) == 0 && B / 64 / (sk * 2) >= 4) sk *= 2;
+    m->s1 = m->s2 = m->s3 = sk;
     MLP_CUDA(m, mlp_alloc(m, &m->Xb, (size_t)B * d.Dk, L));
     MLP_CUDA(m, mlp_alloc(m, &m->XbT, (size_t)d.Dn * B, L));
     MLP_CUDA(m, mlp_alloc(m, &m->A1, (size_t)B * d.Hp, L));
@@ -985,6 +1210,8 @@ int alloc_batch(kmeans_mlp *m, int B) {
     MLP_CUDA(m, mlp_alloc(m, &m->cs2, (size_t)(B / 32) * d.Hp, L));
     MLP_CUDA(m, mlp_alloc(m, &m->cs3, (size_t)(B / 32) * d.G, L));
     MLP_CUDA(m, mlp_alloc(m, &m->yb, (size_t)B, L));
+    const int rc = plan_batch(m, B);
+    if (rc) return rc;
     m->B = B;
     return KM_OK;
 }
@@ -992,43 +1219,8 @@ int alloc_batch(kmeans_mlp *m, int B) {
 // forward + backward of one batch already gathered into Xb / XbT / yb;
 // leaves the split-K partials and the column sums for k_mlp_apply
 int enqueue_fwd_bwd(kmeans_mlp *m, cudaStream_t s) {
-    const MlpDims &d = m->d;
-    const int B = m->B;
-    int rc, bnh, nth;
-    hidden_tiles(m, B, bnh, nth);
-    // layer 1: A1 = GELU(Xb W1^T + b1), with A1^T and GELU'(z1)
-    GemmCfg g = cfg0(E_GELU);
-    g.bias = m->b1p; g.out = m->A1; g.ldo = d.Hp; g.outT = m->A1T; g.ldt = B; g.aux = m->G1; g.lda = d.Hp;
-    if ((rc = launch_gemm(m, {m->Xb, B, d.Dk, m->W1b, d.Hp, d.Dk, d.Dk, B, d.Hp, 1, bnh, nth, 1}, g, s))) return rc;
-    // layer 2
-    g = cfg0(E_GELU);
-    g.bias = m->b2p; g.out = m->A2; g.ldo = d.Hp; g.outT = m->A2T; g.ldt = B; g.aux = m->G2; g.lda = d.Hp;
-    if ((rc = launch_gemm(m, {m->A1, B, d.Hp, m->W2b, d.Hp, d.Hp, d.Hp, B, d.Hp, 1, bnh, nth, 1}, g, s))) return rc;
-    // layer 3 + softmax cross-entropy: dZ3 = (softmax - onehot) / B
-    g = cfg0(E_SOFTMAX);
-    g.bias = m->b3p; g.out = m->dZ3; g.ldo = d.Gk; g.outT = m->dZ3T; g.ldt = B; g.colsum = m->cs3; g.ldc = d.G;
-    g.y = m->yb; g.scale = 1.0f / (float)B; g.loss = m->st->loss;
-    if ((rc = launch_gemm(m, {m->A2, B, d.Hp, m->W3b, d.G, d.Hp, d.Hp, B, d.G, m->nch3, m->bn3, 1, 1}, g, s)))
-        return rc;
-    // dZ2 = (dZ3 W3) * GELU'(z2)
-    g = cfg0(E_MUL);
-    g.aux = m->G2; g.lda = d.Hp; g.out = m->dZ2; g.ldo = d.Hp; g.outT = m->dZ2T; g.ldt = B; g.colsum = m->cs2;
-    g.ldc = d.Hp;
-    if ((rc = launch_gemm(m, {m->dZ3, B, d.Gk, m->W3T, d.Hp, d.Gk, d.Gk, B, d.Hp, 1, bnh, nth, 1}, g, s))) return rc;
-    // dZ1 = (dZ2 W2) * GELU'(z1)
-    g = cfg0(E_MUL);
-    g.aux = m->G1; g.lda = d.Hp; g.outT = m->dZ1T; g.ldt = B; g.colsum = m->cs1; g.ldc = d.Hp;
-    if ((rc = launch_gemm(m, {m->dZ2, B, d.Hp, m->W2T, d.Hp, d.Hp, d.Hp, B, d.Hp, 1, bnh, nth, 1}, g, s))) return rc;
-    // weight gradients, contracted over the batch: dW3 = dZ3^T A2, dW2 = dZ2^T A1, dW1 = dZ1^T X
-    g = cfg0(E_F32);
-    g.part = m->pW3; g.ldp = d.Hp; g.part_split = (int64_t)d.G * d.Hp;
-    if ((rc = launch_gemm(m, {m->dZ3T, d.G, B, m->A2T, d.Hp, B, B, d.G, d.Hp, 1, d.Hp, 1, m->s3}, g, s))) return rc;
-    g = cfg0(E_F32);
-    g.part = m->pW2; g.ldp = d.Hp; g.part_split = (int64_t)d.Hp * d.Hp;
-    if ((rc = launch_gemm(m, {m->dZ2T, d.Hp, B, m->A1T, d.Hp, B, B, d.Hp, d.Hp, 1, d.Hp, 1, m->s2}, g, s))) return rc;
-    g = cfg0(E_F32);
-    g.part = m->pW1; g.ldp = d.Dn; g.part_split = (int64_t)d.Hp * d.Dn;
-    if ((rc = launch_gemm(m, {m->dZ1T, d.Hp, B, m->XbT, d.Dn, B, B, d.Hp, d.Dn, 1, d.Dn, 1, m->s1}, g, s))) return rc;
+    for (int k = 0; k < kmeans_mlp::kPlans; ++k)
+        if (int rc = launch_plan(m, k, s)) return rc;
     return KM_OK;
 }
 
@@ -1050,21 +1242,42 @@ ApplyArgs apply_args(kmeans_mlp *m, int mode) {
     return a;
 }
 
-int launch_apply(kmeans_mlp *m, const ApplyArgs &a, cudaStream_t s) {
-    const int64_t blocks = std::min<int64_t>((m->d.P + 255) / 256, (int64_t)m->num_sms * 8);
-    count_launch();
-    k_mlp_apply<<<(unsigned)blocks, 256, 0, s>>>(m->d, a);
-    cudaError_t e = cudaGetLastError();
+int launch_apply(kmeans_mlp *m, ApplyArgs a, cudaStream_t s) {
+    const MlpDims &d = m->d;
+    const int64_t nw = (int64_t)d.H * d.D + (int64_t)d.H * d.H + (int64_t)d.G * d.H;
+    a.wblocks = (int)std::min<int64_t>((nw + kApplyThreads - 1) / kApplyThreads, (int64_t)m->num_sms * 8);
+    const int bblocks = (2 * d.H + d.G + 31) / 32;
+    const cudaError_t e = launch_pdl(k_mlp_apply, (unsigned)(a.wblocks + bblocks), kApplyThreads, 0, s, d, a);
     if (e != cudaSuccess) return mlp_fail(m, KM_ECUDA, "k_mlp_apply launch: %s", cudaGetErrorString(e));
     return KM_OK;
 }
 
-int check_err(kmeans_mlp *m) {
-    int h = 0;
-    MLP_CUDA(m, cudaMemcpyAsync(&h, m->err, 4, cudaMemcpyDeviceToHost, m->stream));
-    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
-    if (h) return mlp_fail(m, KM_ETIMEOUT, "a bounded wait in a tensor-core product gave up");
+// the batch's rows (of N) and classes into Xb / XbT / yb
+int launch_gather(kmeans_mlp *m, const float *X, int64_t N, const int32_t *labels, int K, uint64_t seed,
+                  cudaStream_t s) {
+    const MlpDims &d = m->d;
+    count_launch();
+    k_mlp_gather<<<(unsigned)((m->B + kGatherRows - 1) / kGatherRows), kGatherThreads, 0, s>>>(
+        X, N, d.D, labels, K, d.G, m->B, d.Dk, d.Dn, seed, m->st, m->Xb, m->XbT, m->yb);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return mlp_fail(m, KM_ECUDA, "k_mlp_gather launch: %s", cudaGetErrorString(e));
     return KM_OK;
+}
+
+// waits for the stream and reads the state (error flag, loss) back
+int read_state(kmeans_mlp *m, MlpState &h) {
+    MLP_CUDA(m, cudaMemcpyAsync(&h, m->st, sizeof(h), cudaMemcpyDeviceToHost, m->stream));
+    MLP_CUDA(m, cudaStreamSynchronize(m->stream));
+    if (h.err) return mlp_fail(m, KM_ETIMEOUT, "a bounded wait in a tensor-core product gave up");
+    return KM_OK;
+}
+int check_err(kmeans_mlp *m) {
+    MlpState h;
+    return read_state(m, h);
+}
+// the error flag and the loss sums to zero (not the step counter)
+cudaError_t clear_state(kmeans_mlp *m) {
+    return cudaMemsetAsync(&m->st->err, 0, sizeof(MlpState) - offsetof(MlpState, err), m->stream);
 }
 
 struct DevGuard {
@@ -1196,7 +1409,8 @@ KM_API int kmeans_mlp_create(kmeans_mlp **out, int32_t D, int32_t hidden, int32_
     MC(mlp_alloc(m, &m->b2p, (size_t)d.Hp, m->allocs));
     MC(mlp_alloc(m, &m->b3p, (size_t)classes, m->allocs));
     MC(mlp_alloc(m, &m->st, 1, m->allocs));
-    MC(mlp_alloc(m, &m->err, 1, m->allocs));
+    m->err = &m->st->err;
+    MC(cudaFuncSetAttribute(k_mlp_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem_optin));
     count_launch();
     k_mlp_init<<<(unsigned)std::min<int64_t>((d.P + 255) / 256, (int64_t)m->num_sms * 8), 256, 0, m->stream>>>(
         d, m->master, seed);
@@ -1254,21 +1468,15 @@ KM_API int kmeans_mlp_gradient(kmeans_mlp *m, const float *X, const int32_t *y, 
     int rc;
     if ((rc = alloc_batch(m, B))) return rc;
     cudaStream_t s = m->stream;
-    MLP_CUDA(m, cudaMemsetAsync(m->err, 0, 4, s));
-    MLP_CUDA(m, cudaMemsetAsync(m->st->loss, 0, sizeof(double) * 3, s));
-    count_launch();
-    k_mlp_gather<<<B, 64, 0, s>>>(X, B, m->d.D, y, 0, m->d.G, B, m->d.Dk, m->d.Dn, ~0ull, m->st, m->Xb, m->XbT, m->yb);
-    MLP_CUDA(m, cudaGetLastError());
+    MLP_CUDA(m, clear_state(m));
+    if ((rc = launch_gather(m, X, B, y, 0, ~0ull, s))) return rc;
     if ((rc = enqueue_fwd_bwd(m, s))) return rc;
     ApplyArgs a = apply_args(m, 0);
     a.grad = grad;
     if ((rc = launch_apply(m, a, s))) return rc;
-    if ((rc = check_err(m))) return rc;
-    if (loss) {
-        double h[3];
-        MLP_CUDA(m, cudaMemcpy(h, m->st->loss, sizeof(h), cudaMemcpyDeviceToHost));
-        *loss = h[2] > 0 ? h[0] / h[2] : 0.0;
-    }
+    MlpState h;
+    if ((rc = read_state(m, h))) return rc;
+    if (loss) *loss = h.loss[2] > 0 ? h.loss[0] / h.loss[2] : 0.0;
     return KM_OK;
 }
 
@@ -1286,8 +1494,7 @@ KM_API int kmeans_mlp_train(kmeans_mlp *m, const float *X, int64_t N, const int3
     int rc;
     if ((rc = alloc_batch(m, batch))) return rc;
     cudaStream_t s = m->stream;
-    MLP_CUDA(m, cudaMemsetAsync(m->err, 0, 4, s));
-    MLP_CUDA(m, cudaMemsetAsync(m->st->loss, 0, sizeof(double) * 3, s));
+    MLP_CUDA(m, clear_state(m));
     // one step recorded once as a CUDA graph, replayed `steps` times (the
     // step counter on the device drives the row draw and Adam's bias correction)
     cudaStream_t cap = nullptr;
@@ -1297,10 +1504,8 @@ KM_API int kmeans_mlp_train(kmeans_mlp *m, const float *X, int64_t N, const int3
         ~CapGuard() { cudaStreamDestroy(s); }
     } cg{cap};
     MLP_CUDA(m, cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-    count_launch();
-    k_mlp_gather<<<batch, 64, 0, cap>>>(X, N, m->d.D, labels, K, m->d.G, batch, m->d.Dk, m->d.Dn, seed, m->st, m->Xb,
-                                        m->XbT, m->yb);
-    rc = cudaGetLastError() == cudaSuccess ? enqueue_fwd_bwd(m, cap) : mlp_fail(m, KM_ECUDA, "gather launch failed");
+    rc = launch_gather(m, X, N, labels, K, seed, cap);
+    if (!rc) rc = enqueue_fwd_bwd(m, cap);
     if (!rc) {
         ApplyArgs a = apply_args(m, 1);
         a.lr = lr;
@@ -1326,11 +1531,10 @@ KM_API int kmeans_mlp_train(kmeans_mlp *m, const float *X, int64_t N, const int3
         ~ExecGuard() { cudaGraphExecDestroy(x); }
     } eg{ex};
     for (int64_t i = 0; i < steps; ++i) MLP_CUDA(m, cudaGraphLaunch(ex, s));
-    if ((rc = check_err(m))) return rc;
-    double h[3];
-    MLP_CUDA(m, cudaMemcpy(h, m->st->loss, sizeof(h), cudaMemcpyDeviceToHost));
-    if (mean_loss) *mean_loss = h[2] > 0 ? h[0] / h[2] : 0.0;
-    if (accuracy) *accuracy = h[2] > 0 ? h[1] / h[2] : 0.0;
+    MlpState h;
+    if ((rc = read_state(m, h))) return rc;
+    if (mean_loss) *mean_loss = h.loss[2] > 0 ? h.loss[0] / h.loss[2] : 0.0;
+    if (accuracy) *accuracy = h.loss[2] > 0 ? h.loss[1] / h.loss[2] : 0.0;
     return KM_OK;
 }
 

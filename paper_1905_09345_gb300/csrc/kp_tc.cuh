@@ -81,6 +81,16 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16]) {
                  : "memory");
 }
 
+// 16 columns back to TMEM, complete on return
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n\t"
+        "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+
 // byte offset of the 16-byte chunk holding bfloat16 elements [8q, 8q+8) of
 // `row` in a 128-byte-swizzled K-major tile (64 elements per 128-byte row)
 __device__ __forceinline__ uint32_t swz_chunk(int row, int q, int atom_bytes) {

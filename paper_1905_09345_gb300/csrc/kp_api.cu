@@ -389,7 +389,7 @@ cudaError_t enqueue_assign(kmeans_ctx *c, const Params &p, cudaStream_t s, bool 
 }
 
 cudaError_t enqueue_update(kmeans_ctx *c, const Params &p, cudaStream_t s, int final_only, int respect_done) {
-    return timed(c, s, KM_KERNEL_UPDATE, [&] { return launch_update(p, s, final_only, respect_done); });
+    return timed(c, s, KM_KERNEL_UPDATE, [&] { return launch_update(p, s, final_only, respect_done, c->num_sms); });
 }
 
 // Iteration 0 seeded by the learned proposal: predictions, the centroid

@@ -388,7 +388,7 @@ cudaError_t launch_filter(const Params &p, cudaStream_t s, int respect_done, int
 cudaError_t launch_survivor(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem_limit);
 bool survivor_tp_eligible(const Params &p);
 cudaError_t launch_survivor_tp(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem_limit);
-cudaError_t launch_update(const Params &p, cudaStream_t s, int final_only, int respect_done);
+cudaError_t launch_update(const Params &p, cudaStream_t s, int final_only, int respect_done, int num_sms);
 cudaError_t launch_arm(const Params &p, cudaStream_t s, int max_iter, double tol);
 cudaError_t launch_set_cond(const Params &p, cudaStream_t s);
 cudaError_t launch_rebase(const Params &p, cudaStream_t s, int num_sms);

@@ -6,9 +6,7 @@
 // not removed, and at t = 0 nothing is removed yet), and for every iteration
 // of plain Lloyd, the comparison baseline.
 //
-// One thread per point: x lives in registers, centroid tiles are staged in
-// shared memory and read by all threads at the same address (broadcast).  The
-// distance is the direct difference sum (x_i - c_i)^2 in FP32; its rounding
+// The distance is the direct difference sum (x_i - c_i)^2 in FP32; its rounding
 // error is bounded (Params::eps_hi/eps_lo), and when the two nearest FP32
 // values cannot be ordered by that bound the point is settled in FP64 with the
 // summation order of the FP64 definition, so labels are exact.
@@ -17,40 +15,27 @@
 namespace kp {
 
 constexpr int kDenseThreads = 128;
+constexpr int kDenseWarps = kDenseThreads / 32;
 constexpr int kDenseTileBytes = 64 * 1024;
+constexpr int kDenseLbBytes = 48 * 1024;
 
-template <int DP>
-struct XRow {
-    float v[DP];
-};
+using f32x2 = unsigned long long;  // two FP32 values in one 64-bit register pair
 
-// squared distance of x (registers) to centroid row c (shared, DP floats)
-template <int DP>
-__device__ __forceinline__ float sqdist_reg(const XRow<DP> &x, const float *__restrict__ c) {
-    float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-    for (int i = 0; i < DP; i += 8) {
-        float4 c0 = *reinterpret_cast<const float4 *>(c + i);
-        float t0 = x.v[i + 0] - c0.x, t1 = x.v[i + 1] - c0.y;
-        float t2 = x.v[i + 2] - c0.z, t3 = x.v[i + 3] - c0.w;
-        a0 = fmaf(t0, t0, a0);
-        a0 = fmaf(t1, t1, a0);
-        a0 = fmaf(t2, t2, a0);
-        a0 = fmaf(t3, t3, a0);
-        if (i + 4 < DP) {
-            float4 c1 = *reinterpret_cast<const float4 *>(c + i + 4);
-            float u0 = x.v[i + 4] - c1.x, u1 = x.v[i + 5] - c1.y;
-            float u2 = x.v[i + 6] - c1.z, u3 = x.v[i + 7] - c1.w;
-            a1 = fmaf(u0, u0, a1);
-            a1 = fmaf(u1, u1, a1);
-            a1 = fmaf(u2, u2, a1);
-            a1 = fmaf(u3, u3, a1);
-        }
-    }
-    return a0 + a1;
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void fma2_sq(f32x2 &acc, f32x2 d) {
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc) : "l"(d));
+}
+__device__ __forceinline__ float sum2(f32x2 a) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    return lo + hi;
 }
 
-// generic D: x and c in global memory (c with stride Dp)
+// any D: x and c in global memory (c with stride Dp)
 __device__ __forceinline__ float sqdist_gen(const float *__restrict__ x, const float *__restrict__ c, int D) {
     float a0 = 0.f, a1 = 0.f;
     int i = 0;
@@ -66,237 +51,382 @@ __device__ __forceinline__ float sqdist_gen(const float *__restrict__ x, const f
     return a0 + a1;
 }
 
-template <int DP>
-__device__ __forceinline__ void load_x(XRow<DP> &x, const Params &p, int64_t n) {
-    const float *row = p.X + n * p.D;
-    if (p.x_vec4 && DP == p.D) {
-#pragma unroll
-        for (int i = 0; i < DP; i += 4) {
-            float4 t = __ldg(reinterpret_cast<const float4 *>(row + i));
-            x.v[i] = t.x;
-            x.v[i + 1] = t.y;
-            x.v[i + 2] = t.z;
-            x.v[i + 3] = t.w;
+// What the scan over the centroids leaves of a point.
+struct Nearest {
+    float s1, s2;    // smallest and second smallest value
+    int best;        // centroid of s1
+    float bg_m2;     // smallest value in the best's group without the best
+    float gm1, gm2;  // the same two of the group being scanned
+    int ga;          // its best centroid
+
+    __device__ __forceinline__ void init() {
+        s1 = s2 = bg_m2 = gm1 = gm2 = INFINITY;
+        best = ga = 0;
+    }
+    // (a NaN is never below anything and leaves both minima alone)
+    __device__ __forceinline__ void visit(int c, float s) {
+        const bool q = s < gm1;
+        gm2 = fminf(gm2, q ? gm1 : s);
+        gm1 = fminf(gm1, s);
+        ga = q ? c : ga;
+    }
+    // end of a group: its smallest value, for the caller's bound
+    __device__ __forceinline__ float close() {
+        const float m = gm1;
+        if (gm1 < s1) {
+            s2 = fminf(s1, gm2);
+            s1 = gm1;
+            best = ga;
+            bg_m2 = gm2;
+        } else {
+            s2 = fminf(s2, gm1);
         }
-    } else {
+        gm1 = gm2 = INFINITY;
+        return m;
+    }
+};
+
+__device__ __forceinline__ float bound_dn(float s, const Params &p) { return s == INFINITY ? INFINITY : dist_dn(s, p); }
+
+// Finish a warp's points (lane: point n if active, its scan's result; row: its
+// group bounds, in shared or global memory).  Near-ties are settled by the
+// whole warp, one point at a time: the lanes share the centroids out, those
+// that the FP32 bound cannot separate from the best are compared in FP64.
+// Returns the lane's number of settled points; `changed` counts its moves.
+__device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool active, int64_t n, Nearest &t,
+                                             float *row, bool bounds, int first, int v, int &changed) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool near = active && t.s2 != INFINITY && unresolved(t.s1, t.s2, p);
+    unsigned todo = __ballot_sync(full, near);
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int64_t m = __shfl_sync(full, n, src);
+        const float ref = __shfl_sync(full, t.s1, src);
+        const int was = __shfl_sync(full, t.best, src);
+        const float *xr = p.X + m * p.D;
+        double bd = INFINITY;
+        int bi = was;
+        float bs = ref;
+        for (int c = lane; c < p.K; c += 32) {
+            const float s = sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D);
+            if (!unresolved(ref, s, p)) continue;
+            const double d = dist2_f64(xr, p.C + (size_t)c * p.Dp, p.D);
+            if (d < bd || (d == bd && tie_key(p, c) < tie_key(p, bi))) { bd = d; bi = c; bs = s; }
+        }
 #pragma unroll
-        for (int i = 0; i < DP; ++i) x.v[i] = i < p.D ? __ldg(row + i) : 0.f;
+        for (int o = 16; o > 0; o >>= 1) {
+            const double od = __shfl_xor_sync(full, bd, o);
+            const int oi = __shfl_xor_sync(full, bi, o);
+            const float os = __shfl_xor_sync(full, bs, o);
+            if (od < bd || (od == bd && tie_key(p, oi) < tie_key(p, bi))) { bd = od; bi = oi; bs = os; }
+        }
+        if (bi != was) {
+            if (bounds) {  // group bounds must now exclude the new best
+                float *r = reinterpret_cast<float *>(__shfl_sync(full, reinterpret_cast<unsigned long long>(row), src));
+                for (int g = lane; g < p.G; g += 32) {
+                    float mn = INFINITY;
+                    for (int c = p.gstart[g]; c < p.gstart[g + 1]; ++c)
+                        if (c != bi) mn = fminf(mn, sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D));
+                    r[g] = bound_dn(mn, p);
+                }
+                __syncwarp();
+            }
+            if (lane == src) {
+                t.best = bi;
+                t.s1 = bs;
+                t.bg_m2 = -1.f;  // already written
+            }
+        }
+    }
+    int old = t.best;
+    if (active) {
+        if (bounds) {
+            if (t.bg_m2 >= 0.f) row[p.grp[t.best]] = bound_dn(t.bg_m2, p);
+            p.u[n] = dist_up(t.s1, p);
+            p.stamp[n] = make_stamp(v, v);
+        }
+        old = first ? -1 : p.label[n];
+        p.label[n] = t.best;
+    }
+    const bool moved = old != t.best;
+    changed += moved;
+    if (!first) {
+        const unsigned mv = __ballot_sync(full, moved);
+        if (mv) {
+            int slot = 0;
+            if (lane == __ffs(mv) - 1) slot = atomicAdd(&ctrl->moved_count, __popc(mv));
+            slot = __shfl_sync(full, slot, __ffs(mv) - 1) + __popc(mv & ((1u << lane) - 1u));
+            if (moved) {
+                p.moved[slot] = (int)n;
+                p.moved_old[slot] = old;
+            }
+        }
+    }
+    return near;
+}
+
+// counters: one atomic per warp
+__device__ __forceinline__ void add_counters(Ctrl *ctrl, int changed, int settled, int64_t dist) {
+    changed = __reduce_add_sync(0xffffffffu, changed);
+    settled = __reduce_add_sync(0xffffffffu, settled);
+    if ((threadIdx.x & 31) == 0) {
+        if (changed) atomicAdd(&ctrl->n_changed, (unsigned long long)changed);
+        if (settled) atomicAdd(&ctrl->n_recheck, (unsigned long long)settled);
+        if (dist) atomicAdd(&ctrl->n_dist, (unsigned long long)dist);
     }
 }
 
-// The FP32 value of the distance from point n to centroid c, computed exactly
-// as in the main loop (global-memory operands; same arithmetic, same order).
-template <int DP>
-__device__ __forceinline__ float sqdist_again(const Params &p, const XRow<(DP > 0 ? DP : 1)> &x, int64_t n, int c) {
-    if constexpr (DP > 0) {
-        return sqdist_reg<DP>(x, p.C + (size_t)c * p.Dp);
-    } else {
-        return sqdist_gen(p.X + n * p.D, p.C + (size_t)c * p.Dp, p.D);
-    }
-}
-
-// Dense assignment.  first: iteration 0 of this context (all points count as
-// moved and are added to the sums by the caller).  Writes labels; for the
-// filtered method also u, lbg, lb and stamps (exact at the current version).
-template <int DP>
-__global__ void __launch_bounds__(kDenseThreads) k_dense_assign(Params p, int first, int respect_done, int if_dense) {
+// Dense assignment, D <= 128.  first: iteration 0 of this context (all points
+// count as moved and are added to the sums by the caller).  Writes labels; for
+// the filtered method also u, lbg, lb and stamps (exact at the current
+// version).
+//
+// Bound by the FP32 pipe: a subtraction and a multiply-add per point, centroid
+// and coordinate.  Both go through the packed instructions (f32x2), which halve
+// the issue slots, and every value read from shared memory serves P points per
+// lane, held in registers, of Q centroids at a time, so that 4 P packed
+// instructions follow a 16-byte broadcast read and 2 P Q sums are in flight.
+// Rows of more than 64 coordinates are cut over L lanes (32 / L lanes apart),
+// whose partial sums meet in a transposing shuffle that leaves each lane the
+// P / L points it owns.
+//
+// Measured, K = 256 (before: one point per lane, scalar, two centroids): 262,144
+// x 64: 599 -> 333 us, the FP32 pipe busy in 75% of the cycles; 600,000 x 8:
+// 286 -> 124; x 16: 377 -> 212; x 32: 673 -> 399; x 50: 1177 -> 667; x 128: 3358
+// -> 1699.
+template <int DPL, int L, int P, int Q, int MB>
+__global__ void __launch_bounds__(kDenseThreads, MB) k_dense_assign(Params p, int first, int respect_done,
+                                                                   int if_dense) {
     extern __shared__ __align__(128) float smem[];
+    constexpr int OWN = P / L;                   // points a lane owns
+    constexpr int PW = 32 * OWN;                 // points of a warp
+    constexpr int PB = PW * kDenseWarps;         // points of a block
+    constexpr int SEG = L > 1 ? DPL + 4 : DPL;   // a lane's part of a staged row (skewed: no bank conflicts)
+    constexpr int RS = L * SEG;                  // staged row stride
+    static_assert(DPL % 4 == 0 && P % L == 0 && (L == 1 || L == 2 || L == 4), "shape");
     Ctrl *ctrl = p.ctrl;
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;
     if (if_dense && !*(volatile int *)&ctrl->dense_mode) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->path = KM_PATH_DENSE_FP32;
     const int v = ctrl->v;
-    const int K = p.K;
-    const int G = p.G;
+    const int K = p.K, D = p.D;
     const bool bounds = p.algo == KM_ALGO_FILTERED;
-    constexpr int DPs = DP > 0 ? DP : 4;  // shared row stride (unused for DP = 0)
-    const int KT = DP > 0 ? min(K, kDenseTileBytes / (DPs * 4)) : 0;
+    const int KT = min(K, kDenseTileBytes / (RS * 4));
+    const bool resident = KT == K;
     float *cs = smem;
-    const int lbs_stride = p.Gp + 1;
-    const bool stage_lb = bounds && (size_t)lbs_stride * kDenseThreads * 4 <= 48 * 1024;
-    float *lbs = smem + (size_t)KT * DPs;
-    const bool c_resident = DP > 0 && KT == K;
+    const int ls = p.Gp + 1;
+    const bool stage_lb = bounds && (size_t)ls * PB * 4 <= kDenseLbBytes;
+    float *lbs = smem + (size_t)KT * RS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int part = lane / (32 / L);      // which coordinates
+    const int lidx = lane % (32 / L);      // which points
 
-    if (c_resident) {  // whole centroid set fits: stage once for all point tiles
-        for (int idx = threadIdx.x; idx < K * (DPs / 4); idx += blockDim.x) {
-            int r = idx / (DPs / 4), q = idx % (DPs / 4);
-            reinterpret_cast<float4 *>(cs)[idx] = *reinterpret_cast<const float4 *>(p.C + (size_t)r * p.Dp + q * 4);
+    auto stage = [&](int c0, int kt) {
+        for (int i = threadIdx.x; i < kt * (L * DPL / 4); i += kDenseThreads) {
+            const int r = i / (L * DPL / 4), q = (i % (L * DPL / 4)) * 4;
+            const float *c = p.C + (size_t)(c0 + r) * p.Dp;
+            float4 w;
+            if (q + 4 <= p.Dp) {  // the padding up to Dp is zero
+                w = *reinterpret_cast<const float4 *>(c + q);
+            } else {
+                w.x = w.y = w.z = w.w = 0.f;
+            }
+            *reinterpret_cast<float4 *>(cs + r * RS + (q / DPL) * SEG + q % DPL) = w;
         }
+    };
+    if (resident) {
+        stage(0, K);
         __syncthreads();
     }
 
-    unsigned long long my_changed = 0, my_recheck = 0;
+    int changed = 0, settled = 0;
+    int64_t dist = 0;
+    for (int64_t base = (int64_t)blockIdx.x * PB; base < p.N; base += (int64_t)gridDim.x * PB) {
+        const int64_t w0 = base + warp * PW;  // the warp's points, 32 / L apart per lane
+        f32x2 x[P][DPL / 2];
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+            const int64_t n = w0 + j * (32 / L) + lidx;
+            const float *row = p.X + min(n, p.N - 1) * D;
+            if (p.x_vec4) {
+#pragma unroll
+                for (int i = 0; i < DPL; i += 4) {
+                    ulonglong2 w = make_ulonglong2(0ull, 0ull);
+                    if (part * DPL + i < D) w = __ldg(reinterpret_cast<const ulonglong2 *>(row + part * DPL + i));
+                    x[j][i / 2] = w.x;
+                    x[j][i / 2 + 1] = w.y;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < DPL; i += 2) {
+                    const int q = part * DPL + i;
+                    const float a = q < D ? __ldg(row + q) : 0.f, b = q + 1 < D ? __ldg(row + q + 1) : 0.f;
+                    asm("mov.b64 %0, {%1, %2};" : "=l"(x[j][i / 2]) : "f"(a), "f"(b));
+                }
+            }
+        }
+        // the point in slot o of this lane
+        auto own = [&](int o) { return w0 + (part * OWN + o) * (32 / L) + lidx; };
+        auto lb_row = [&](int o) {
+            const int64_t n = min(own(o), p.N - 1);
+            return stage_lb ? lbs + (int)(own(o) - base) * ls : p.lb + n * p.Gp;
+        };
+        Nearest t[OWN];
+#pragma unroll
+        for (int o = 0; o < OWN; ++o) t[o].init();
+        int g = 0, gend = bounds ? p.gstart[1] : K;
+        auto close_group = [&]() {
+#pragma unroll
+            for (int o = 0; o < OWN; ++o) {
+                const float m = t[o].close();
+                if (bounds && (stage_lb || own(o) < p.N)) lb_row(o)[g] = bound_dn(m, p);
+            }
+        };
+        // centroid c's sums of this lane's part of its P points, to the owners
+        auto visit = [&](int c, const f32x2 *acc) {
+            while (c == gend) {  // same for all threads
+                close_group();
+                gend = p.gstart[++g + 1];
+            }
+            float s[P];
+#pragma unroll
+            for (int j = 0; j < P; ++j) s[j] = sum2(acc[j]);
+#pragma unroll
+            for (int h = L / 2; h > 0; h >>= 1) {  // h: the bit of `part` that this step settles
+                const bool up = part & h;
+                const int half = OWN * h;
+#pragma unroll
+                for (int j = 0; j < half; ++j) {
+                    const float mine = up ? s[j + half] : s[j], give = up ? s[j] : s[j + half];
+                    s[j] = mine + __shfl_xor_sync(0xffffffffu, give, h * (32 / L));
+                }
+            }
+#pragma unroll
+            for (int o = 0; o < OWN; ++o) t[o].visit(c, s[o]);
+        };
+        for (int c0 = 0; c0 < K; c0 += KT) {
+            const int kt = min(KT, K - c0);
+            if (!resident) {
+                __syncthreads();
+                stage(c0, kt);
+                __syncthreads();
+            }
+            const float *cp = cs + part * SEG;
+            for (int k = 0; k < kt; k += Q) {
+                f32x2 acc[Q][P];
+                const float *c[Q];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    c[q] = cp + min(k + q, kt - 1) * RS;
+#pragma unroll
+                    for (int j = 0; j < P; ++j) acc[q][j] = 0ull;
+                }
+#pragma unroll
+                for (int i = 0; i < DPL / 2; i += 2) {
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(c[q] + 2 * i);
+#pragma unroll
+                        for (int j = 0; j < P; ++j) {
+                            fma2_sq(acc[q][j], sub2(x[j][i], u.x));
+                            fma2_sq(acc[q][j], sub2(x[j][i + 1], u.y));
+                        }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (k + q < kt) visit(c0 + k + q, acc[q]);
+            }
+        }
+        while (true) {  // the last group, and empty ones behind it
+            close_group();
+            if (!bounds || ++g >= p.G) break;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = 0; o < OWN; ++o) {
+            const int64_t n = own(o);
+            settled += finish_points(p, ctrl, n < p.N, n, t[o], lb_row(o), bounds, first, v, changed);
+        }
+        dist += max((int64_t)0, min((int64_t)PW, p.N - w0)) * K;
+        if (bounds) {
+            __syncwarp();
+            // lbg = min over the row, then a coalesced copy of the warp's rows
+#pragma unroll
+            for (int o = 0; o < OWN; ++o) {
+                if (own(o) < p.N) {
+                    const float *r = lb_row(o);
+                    float m = INFINITY;
+                    for (int q = 0; q < p.G; ++q) m = fminf(m, r[q]);
+                    p.lbg[own(o)] = m;
+                }
+            }
+            if (stage_lb && w0 < p.N) {
+                const int count = (int)min((int64_t)PW, p.N - w0) * p.Gp;
+                const float *src = lbs + warp * PW * ls;
+                float *dst = p.lb + w0 * p.Gp;
+                for (int i = lane; i < count; i += 32) {
+                    const int r = i / p.Gp, q = i - r * p.Gp;
+                    dst[i] = q < p.G ? src[r * ls + q] : 0.f;
+                }
+            }
+            __syncwarp();
+        }
+    }
+    add_counters(ctrl, changed, settled, lane == 0 ? dist : 0);
+}
+
+// Dense assignment, any D: one point per lane, operands in global memory.
+__global__ void __launch_bounds__(kDenseThreads) k_dense_assign_any(Params p, int first, int respect_done,
+                                                                    int if_dense) {
+    Ctrl *ctrl = p.ctrl;
+    count_kernel(ctrl);
+    if (respect_done && *(volatile int *)&ctrl->done) return;
+    if (if_dense && !*(volatile int *)&ctrl->dense_mode) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->path = KM_PATH_DENSE_FP32;
+    const int v = ctrl->v;
+    const bool bounds = p.algo == KM_ALGO_FILTERED;
+    int changed = 0, settled = 0;
+    int64_t dist = 0;
     for (int64_t base = (int64_t)blockIdx.x * kDenseThreads; base < p.N; base += (int64_t)gridDim.x * kDenseThreads) {
         const int64_t n = base + threadIdx.x;
         const bool active = n < p.N;
-        XRow<(DP > 0 ? DP : 1)> x;
-        if constexpr (DP > 0) {
-            if (active) load_x<DP>(x, p, n);
-            else {
-#pragma unroll
-                for (int i = 0; i < DP; ++i) x.v[i] = 0.f;
-            }
-        }
-        int best = 0;
-        float s1 = INFINITY, s2 = INFINITY;   // best / second-best over all centroids
-        int cur_g = 0;
-        float gm1 = INFINITY, gm2 = INFINITY;  // two smallest in the current group
-        float bg_m2 = INFINITY;                // second smallest of the best's group
-        bool best_in_cur = false;
-
-        auto close_group = [&](int g) {
-            if (bounds && active) {
-                float d = gm1 == INFINITY ? INFINITY : dist_dn(gm1, p);
-                if (stage_lb) lbs[threadIdx.x * lbs_stride + g] = d;
-                else p.lb[n * p.Gp + g] = d;
-            }
-            if (best_in_cur) bg_m2 = gm2;
-            best_in_cur = false;
-            gm1 = gm2 = INFINITY;
-        };
-        auto visit = [&](int c, float s) {
-            int g = p.grp[c];
-            if (g != cur_g) {
-                close_group(cur_g);
-                cur_g = g;
-            }
-            if (s < gm1) { gm2 = gm1; gm1 = s; }
-            else if (s < gm2) gm2 = s;
-            if (s < s1) {
-                s2 = s1;
-                s1 = s;
-                best = c;
-                best_in_cur = true;
-            } else if (s < s2) {
-                s2 = s;
-            }
-        };
-
-        if constexpr (DP > 0) {
-            for (int c0 = 0; c0 < K; c0 += KT) {
-                const int kt = min(KT, K - c0);
-                if (!c_resident) {
-                    __syncthreads();
-                    for (int idx = threadIdx.x; idx < kt * (DP / 4); idx += blockDim.x) {
-                        int r = idx / (DP / 4), q = idx % (DP / 4);
-                        reinterpret_cast<float4 *>(cs)[idx] =
-                            *reinterpret_cast<const float4 *>(p.C + (size_t)(c0 + r) * p.Dp + q * 4);
-                    }
-                    __syncthreads();
-                }
-                int j = 0;
-                for (; j + 1 < kt; j += 2) {
-                    float sa = sqdist_reg<DP>(x, cs + (size_t)j * DP);
-                    float sb = sqdist_reg<DP>(x, cs + (size_t)(j + 1) * DP);
-                    visit(c0 + j, sa);
-                    visit(c0 + j + 1, sb);
-                }
-                if (j < kt) visit(c0 + j, sqdist_reg<DP>(x, cs + (size_t)j * DP));
-            }
-        } else {
-            if (active) {
-                const float *xr = p.X + n * p.D;
-                for (int c = 0; c < K; ++c) visit(c, sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D));
-            }
-        }
-        close_group(cur_g);
-
+        const int64_t row = min(n, p.N - 1);
+        float *lb = p.lb + row * p.Gp;
+        Nearest t;
+        t.init();
         if (active) {
-            // near-tie: settle in FP64 among every centroid the FP32 error
-            // bound cannot separate from the FP32 best
-            if (s2 != INFINITY && unresolved(s1, s2, p)) {
-                const float s1_ref = s1;
-                double bd = INFINITY;
-                int bi = best;
-                float bs = s1;
-                for (int c = 0; c < K; ++c) {
-                    float s = sqdist_again<DP>(p, x, n, c);
-                    if (!unresolved(s1_ref, s, p)) continue;
-                    double d64 = dist2_f64(p.X + n * p.D, p.C + (size_t)c * p.Dp, p.D);
-                    if (d64 < bd || (d64 == bd && tie_key(p, c) < tie_key(p, bi))) { bd = d64; bi = c; bs = s; }
+            const float *x = p.X + row * p.D;
+            int g = 0, gend = bounds ? p.gstart[1] : p.K;
+            for (int c = 0; c <= p.K; ++c) {
+                while (c == gend) {
+                    const float m = t.close();
+                    if (!bounds) break;
+                    lb[g] = bound_dn(m, p);
+                    if (++g == p.G) break;
+                    gend = p.gstart[g + 1];
                 }
-                my_recheck += 1;
-                if (bi != best) {
-                    best = bi;
-                    s1 = bs;
-                    if (bounds) {  // group bounds must now exclude the new best
-                        for (int g = 0; g < G; ++g) {
-                            float m = INFINITY;
-                            for (int c = p.gstart[g]; c < p.gstart[g + 1]; ++c)
-                                if (c != best) m = fminf(m, sqdist_again<DP>(p, x, n, c));
-                            float d = m == INFINITY ? INFINITY : dist_dn(m, p);
-                            if (stage_lb) lbs[threadIdx.x * lbs_stride + g] = d;
-                            else p.lb[n * p.Gp + g] = d;
-                        }
-                        bg_m2 = -1.f;  // already written
-                    }
-                }
-            }
-            if (bounds && bg_m2 >= 0.f) {
-                int g = p.grp[best];
-                float d = bg_m2 == INFINITY ? INFINITY : dist_dn(bg_m2, p);
-                if (stage_lb) lbs[threadIdx.x * lbs_stride + g] = d;
-                else p.lb[n * p.Gp + g] = d;
-            }
-            const int old = first ? -1 : p.label[n];
-            p.label[n] = best;
-            if (bounds) {
-                p.u[n] = dist_up(s1, p);
-                p.stamp[n] = make_stamp(v, v);
-            }
-            if (old != best) {
-                my_changed += 1;
-                if (!first) {
-                    int slot = atomicAdd(&ctrl->moved_count, 1);
-                    p.moved[slot] = (int)n;
-                    p.moved_old[slot] = old;
-                }
+                if (c < p.K) t.visit(c, sqdist_gen(x, p.C + (size_t)c * p.Dp, p.D));
             }
         }
+        settled += finish_points(p, ctrl, active, n, t, lb, bounds, first, v, changed);
+        dist += active ? p.K : 0;
         if (bounds) {
-            if (stage_lb) {
-                __syncthreads();
-                // lbg = min over the row, then a coalesced copy of the rows
-                if (active) {
-                    float m = INFINITY;
-                    for (int g = 0; g < G; ++g) m = fminf(m, lbs[threadIdx.x * lbs_stride + g]);
-                    p.lbg[n] = m;
-                }
-                const int64_t rows = min((int64_t)kDenseThreads, p.N - base);
-                for (int64_t idx = threadIdx.x; idx < rows * p.Gp; idx += blockDim.x) {
-                    int64_t r = idx / p.Gp;
-                    int g = (int)(idx % p.Gp);
-                    p.lb[(base + r) * p.Gp + g] = g < G ? lbs[r * lbs_stride + g] : 0.f;
-                }
-                __syncthreads();
-            } else if (active) {
+            __syncwarp();
+            if (active) {
                 float m = INFINITY;
-                for (int g = 0; g < G; ++g) m = fminf(m, p.lb[n * p.Gp + g]);
+                for (int g = 0; g < p.G; ++g) m = fminf(m, lb[g]);
                 p.lbg[n] = m;
+                for (int g = p.G; g < p.Gp; ++g) lb[g] = 0.f;
             }
         }
     }
-    // counters: one atomic per warp
-    unsigned long long ch = my_changed, rc = my_recheck;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ch += __shfl_xor_sync(0xffffffffu, ch, o);
-        rc += __shfl_xor_sync(0xffffffffu, rc, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (ch) atomicAdd(&ctrl->n_changed, ch);
-        if (rc) atomicAdd(&ctrl->n_recheck, rc);
-        int64_t lo = (int64_t)blockIdx.x * kDenseThreads + (threadIdx.x & ~31);
-        (void)lo;
-    }
-    if (threadIdx.x == 0) {
-        // points this block assigned, times K distances each
-        int64_t pts = 0;
-        for (int64_t base = (int64_t)blockIdx.x * kDenseThreads; base < p.N; base += (int64_t)gridDim.x * kDenseThreads)
-            pts += min((int64_t)kDenseThreads, p.N - base);
-        atomicAdd(&ctrl->n_dist, (unsigned long long)(pts * K));
-    }
+    for (int o = 16; o > 0; o >>= 1) dist += __shfl_xor_sync(0xffffffffu, dist, o);
+    add_counters(ctrl, changed, settled, (threadIdx.x & 31) == 0 ? dist : 0);
 }
 
 // Cluster statistics for moved points: S[new] += x, S[old] -= x (FP64),
@@ -372,37 +502,71 @@ int dense_dp(int D) {
     return 0;
 }
 
-template <int DP>
+template <int DPL, int L, int P, int Q, int MB>
 static cudaError_t launch_dense_t(const Params &p, cudaStream_t s, int first, int respect_done, int num_sms,
                                   int if_dense) {
-    constexpr int DPs = DP > 0 ? DP : 4;
-    const int KT = DP > 0 ? std::min(p.K, kDenseTileBytes / (DPs * 4)) : 0;
-    size_t smem = (size_t)KT * DPs * 4;
-    const bool bounds = p.algo == KM_ALGO_FILTERED;
-    if (bounds && (size_t)(p.Gp + 1) * kDenseThreads * 4 <= 48 * 1024) smem += (size_t)(p.Gp + 1) * kDenseThreads * 4;
-    cudaError_t e = cudaFuncSetAttribute(k_dense_assign<DP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int PB = P / L * kDenseThreads;
+    constexpr int RS = L * (L > 1 ? DPL + 4 : DPL);
+    size_t smem = (size_t)std::min(p.K, kDenseTileBytes / (RS * 4)) * RS * 4;
+    const size_t lb = (size_t)(p.Gp + 1) * PB * 4;
+    if (p.algo == KM_ALGO_FILTERED && lb <= (size_t)kDenseLbBytes) smem += lb;
+    auto kernel = k_dense_assign<DPL, L, P, Q, MB>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dense_assign<DP>, kDenseThreads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kDenseThreads, smem);
     if (e != cudaSuccess) return e;
-    int64_t tiles = (p.N + kDenseThreads - 1) / kDenseThreads;
-    int64_t grid = std::min<int64_t>(tiles, (int64_t)num_sms * std::max(per_sm, 1));
+    const int64_t tiles = (p.N + PB - 1) / PB;
+    const int64_t grid = std::min<int64_t>(tiles, (int64_t)num_sms * std::max(per_sm, 1));
     count_launch();
-    k_dense_assign<DP><<<(unsigned)grid, kDenseThreads, smem, s>>>(p, first, respect_done, if_dense);
+    kernel<<<(unsigned)grid, kDenseThreads, smem, s>>>(p, first, respect_done, if_dense);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dense_assign(const Params &p, cudaStream_t s, int first, int respect_done, int num_sms,
                                 int if_dense) {
-    switch (dense_dp(p.D)) {
-    case 4: return launch_dense_t<4>(p, s, first, respect_done, num_sms, if_dense);
-    case 8: return launch_dense_t<8>(p, s, first, respect_done, num_sms, if_dense);
-    case 16: return launch_dense_t<16>(p, s, first, respect_done, num_sms, if_dense);
-    case 32: return launch_dense_t<32>(p, s, first, respect_done, num_sms, if_dense);
-    case 64: return launch_dense_t<64>(p, s, first, respect_done, num_sms, if_dense);
-    case 128: return launch_dense_t<128>(p, s, first, respect_done, num_sms, if_dense);
-    default: return launch_dense_t<0>(p, s, first, respect_done, num_sms, if_dense);
-    }
+    // few points: one per lane, so that they spread over more warps
+    // (200 centroids in 17 dimensions: 60,000 points 33 us against 35, 120,000
+    // the same, 250,000 101 against 92)
+    // Otherwise P and Q by width, as measured (600,000 points, K = 256): up to 8
+    // coordinates 4 points and 2 centroids (123 us against 136 with 2 and 4),
+    // beyond 2 and 4 (D = 16: 212 against 224; 32: 400 against 387, but 65 against
+    // 71 for K = 32); D = 128: a row on two lanes 1699, on one 1689, on four 1805
+    const bool few = p.N < (int64_t)num_sms * kDenseThreads * 4;
+#define DENSE(DPL, L, P, Q, MB) return launch_dense_t<DPL, L, P, Q, MB>(p, s, first, respect_done, num_sms, if_dense)
+#define DENSE_F(DPL, P, Q, MB)            \
+    do {                                  \
+        if (few) DENSE(DPL, 1, 1, 4, MB); \
+        else DENSE(DPL, 1, P, Q, MB);     \
+    } while (0)
+    if (p.D <= 32) switch ((p.D + 3) / 4) {
+        case 1: DENSE_F(4, 4, 2, 4);
+        case 2: DENSE_F(8, 4, 2, 4);
+        case 3: DENSE_F(12, 2, 4, 4);
+        case 4: DENSE_F(16, 2, 4, 4);
+        case 5: DENSE_F(20, 2, 4, 4);
+        case 6: DENSE_F(24, 2, 4, 4);
+        case 7: DENSE_F(28, 2, 4, 4);
+        default: DENSE_F(32, 2, 4, 3);
+        }
+    if (p.D <= 64) switch ((p.D + 7) / 8) {
+        case 5: DENSE_F(40, 2, 4, 2);
+        case 6: DENSE_F(48, 2, 4, 2);
+        case 7: DENSE_F(56, 2, 4, 2);
+        default: DENSE_F(64, 2, 4, 2);
+        }
+    if (p.D <= 128) switch ((p.D + 15) / 16) {
+        case 5: DENSE(40, 2, 2, 4, 2);
+        case 6: DENSE(48, 2, 2, 4, 2);
+        case 7: DENSE(56, 2, 2, 4, 2);
+        default: DENSE(64, 2, 2, 4, 2);
+        }
+#undef DENSE_F
+#undef DENSE
+    const int64_t grid = std::min<int64_t>((p.N + kDenseThreads - 1) / kDenseThreads, (int64_t)num_sms * 8);
+    count_launch();
+    k_dense_assign_any<<<(unsigned)grid, kDenseThreads, 0, s>>>(p, first, respect_done, if_dense);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_apply_moves(const Params &p, cudaStream_t s, int all_points, int respect_done, int num_sms,

@@ -198,6 +198,62 @@ __device__ __forceinline__ double dist2_f64(const float *x, const float *c, int 
     return s;
 }
 
+// s + e == a + b exactly (Knuth's TwoSum; barring overflow)
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// Which of two centroids a point is nearer to, in the order of the FP64
+// definition, without FP64 arithmetic: 0: ca, 1: cb, -1: not decided here
+// (the caller computes the FP64 distances).  Called by whole warps; the lanes
+// share the coordinates.  A lone FP64 distance is a chain of D dependent
+// additions on a pipe that takes 16 cycles for a warp's instruction, and the
+// kernel whose last warp meets one waits for it: over 20 us a pass at D = 64.
+//
+// The distances are summed as FP32 pairs h + l: x - c exactly (TwoSum), its
+// square but for 2^-45 of it, TwoSum into h, everything else into l.  With n
+// coordinates per lane, l meets n + 10 additions of magnitudes below
+// (n + 9) 2^-24 of the sum, so that the pair is within (n^2 + 16 n + 100) 2^-48
+// of it; the FP64 sum is within (D + 2) 2^-53.  The order is decided when the
+// pairs differ by more than twice both errors of both sums (and what
+// underflow can hide); NaN and infinity decide nothing.
+__device__ __forceinline__ int pair_order(const float *x, const float *ca, const float *cb, int D) {
+    float ha = 0.f, la = 0.f, hb = 0.f, lb = 0.f;
+    auto acc = [](float &h, float &l, float xv, float c) {
+        float dh, dl, e;
+        two_sum(xv, -c, dh, dl);
+        const float sq = __fmul_rn(dh, dh);
+        const float sqe = __fmaf_rn(dh, dh, -sq);
+        const float cross = __fmaf_rn(__fmul_rn(2.f, dh), dl, __fmul_rn(dl, dl));
+        two_sum(h, sq, h, e);
+        l = __fadd_rn(l, __fadd_rn(e, __fadd_rn(sqe, cross)));
+    };
+    for (int i = threadIdx.x & 31; i < D; i += 32) {
+        const float xv = __ldg(x + i);
+        acc(ha, la, xv, ca[i]);
+        acc(hb, lb, xv, cb[i]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        float e;
+        const float h1 = __shfl_xor_sync(0xffffffffu, ha, o), l1 = __shfl_xor_sync(0xffffffffu, la, o);
+        const float h2 = __shfl_xor_sync(0xffffffffu, hb, o), l2 = __shfl_xor_sync(0xffffffffu, lb, o);
+        two_sum(ha, h1, ha, e);
+        la = __fadd_rn(__fadd_rn(la, l1), e);
+        two_sum(hb, h2, hb, e);
+        lb = __fadd_rn(__fadd_rn(lb, l2), e);
+    }
+    float s, e;
+    two_sum(ha, -hb, s, e);
+    const float diff = __fadd_rn(s, __fadd_rn(e, __fsub_rn(la, lb)));
+    const float n = (float)((D + 31) / 32);
+    const float rel = (n * n + 16.f * n + 100.f) * 0x1p-47f + (float)(D + 2) * 0x1p-52f;
+    const float margin = __fmaf_ru(rel, __fadd_ru(ha, hb), (float)(D + 4) * 0x1p-140f);
+    return diff < -margin ? 0 : (diff > margin ? 1 : -1);
+}
+
 // ---------------------------------------------------------------------------
 // warp reductions
 // ---------------------------------------------------------------------------

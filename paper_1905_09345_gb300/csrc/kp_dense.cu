@@ -454,11 +454,6 @@ __global__ void __launch_bounds__(256) k_apply_moves(Params p, int all_points, i
         // squares, compensated sums): FP64 arithmetic is slow on these SMs;
         // only the atomics are FP64
         float qh = 0.f, ql = 0.f, oh = 0.f, ol = 0.f;
-        auto two_sum = [](float a, float b, float &s, float &e) {  // s + e == a + b exactly
-            s = __fadd_rn(a, b);
-            const float bb = __fsub_rn(s, a);
-            e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-        };
         // (x - r)^2 into the pair (h, l): x - r as the exact pair dh + dl, its
         // square as sq + sqe (exact) plus 2 dh dl + dl^2 (below 2^-47 of it)
         auto acc = [&](float &h, float &l, float xv, float r) {

@@ -134,11 +134,6 @@ constexpr int kSumBatch = 8;            // points whose loads are in flight toge
 struct Sum3 {
     float h, l, m;
     __device__ __forceinline__ void clear() { h = l = m = 0.f; }
-    static __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {  // s + e == a + b
-        s = __fadd_rn(a, b);
-        const float bb = __fsub_rn(s, a);
-        e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    }
     __device__ __forceinline__ void add(float x) {
         float e, f;
         two_sum(h, x, h, e);
@@ -235,12 +230,12 @@ __global__ void __launch_bounds__(kSumThreads) k_noalloc_sums(Params p, int segs
                     // (x - r)^2 exactly but for 2^-47 of it: x - r = dh + dl, its
                     // square sq + sqe, and 2 dh dl + dl^2
                     float dh, dl, e;
-                    Sum3::two_sum(xv[b], -ref, dh, dl);
+                    two_sum(xv[b], -ref, dh, dl);
                     const float sq = __fmul_rn(dh, dh);
                     const float sqe = __fmaf_rn(dh, dh, -sq);
                     q.add(sq);
                     const float cross = __fmaf_rn(__fmul_rn(2.f, dh), dl, __fmul_rn(dl, dl));
-                    Sum3::two_sum(q.l, __fadd_rn(sqe, cross), q.l, e);
+                    two_sum(q.l, __fadd_rn(sqe, cross), q.l, e);
                     q.m = __fadd_rn(q.m, e);
                 }
             }
@@ -259,7 +254,7 @@ __global__ void __launch_bounds__(kSumThreads) k_noalloc_sums(Params p, int segs
                 const float m = __shfl_xor_sync(0xffffffffu, q.m, o);
                 float e;
                 q.m = __fadd_rn(q.m, m);
-                Sum3::two_sum(q.l, l, q.l, e);
+                two_sum(q.l, l, q.l, e);
                 q.m = __fadd_rn(q.m, e);
                 q.add(h);
             }

@@ -12,22 +12,11 @@
 namespace kp {
 namespace {
 
-// ---------------------------------------------------------------------------
-// k_settle: the exact decision for the rows the tensor-core epilogue queued
-// (runner-up inside the error window).  A sub-warp of D / 8 lanes per
-// request, eight coordinates per lane, candidates one after another so that
-// the sub-warp never diverges: FP32 direct-difference distances reduced
-// across the sub-warp, the smallest with the lowest index; where FP32 cannot
-// separate it from the runner-up, every candidate again in FP64 with the
-// summation order of the FP64 definition (lanes over candidates).  The candidates are the centroids
-// of the groups whose tensor-core minimum lies in the window (a group mask,
-// or -- for the streamed-centroid pass -- the groups whose written bound is
-// within the window's edge).  Writes the label, corrects u / lb / lbg when
-// the winner is not i1, and appends label changes to the moved-point list
-// 32 at a time.
-// ---------------------------------------------------------------------------
 constexpr int kSettleThreads = 256;
 constexpr int kSettleWarps = kSettleThreads / 32;
+constexpr int kSub = 8;              // lanes per request
+constexpr int kPer = 32 / kSub;      // requests a warp works on at a time
+constexpr int kGrabMax = 4 * kPer;   // requests a warp claims at a time, at most
 
 // The bitmap's set bits, compacted into the settle queue: a warp takes 32
 // words, scans their populations and reserves its slots with one atomic.
@@ -72,26 +61,101 @@ __device__ __forceinline__ double settle_fp64(const float *x, const float *c, in
     return s;
 }
 
+// FP32 squared distance by one lane (D a multiple of 4)
+__device__ __forceinline__ float settle_fp32(const float *x, const float *c, int D) {
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < D; i += 4) {
+        const float4 xv = __ldg(reinterpret_cast<const float4 *>(x + i)), cv = *reinterpret_cast<const float4 *>(c + i);
+        const float d0 = xv.x - cv.x, d1 = xv.y - cv.y, d2 = xv.z - cv.z, d3 = xv.w - cv.w;
+        a0 = fmaf(d0, d0, a0);
+        a1 = fmaf(d1, d1, a1);
+        a0 = fmaf(d2, d2, a0);
+        a1 = fmaf(d3, d3, a1);
+    }
+    return a0 + a1;
+}
+
+// The three smallest FP32 distances met so far, the first two with their
+// centroids.
+struct Top3 {
+    float s1, s2, s3;
+    int i1, i2;
+    __device__ __forceinline__ void add(float s, int c) {  // (a NaN is never below anything)
+        const bool f = s < s1, g = s < s2;
+        s3 = g ? s2 : fminf(s3, s);
+        s2 = f ? s1 : (g ? s : s2);
+        i2 = f ? i1 : (g ? c : i2);
+        s1 = f ? s : s1;
+        i1 = f ? c : i1;
+    }
+    // with the list of the lane `o` away; both lanes get the same result
+    __device__ __forceinline__ void merge(int o) {
+        const unsigned full = 0xffffffffu;
+        const float b1 = __shfl_xor_sync(full, s1, o), b2 = __shfl_xor_sync(full, s2, o);
+        const float b3 = __shfl_xor_sync(full, s3, o);
+        const int j1 = __shfl_xor_sync(full, i1, o), j2 = __shfl_xor_sync(full, i2, o);
+        const bool f = b1 < s1 || (b1 == s1 && j1 < i1);
+        const float x1 = f ? s1 : b1, x2 = f ? s2 : b2;                       // the list that lost
+        const float y2 = f ? b2 : s2, y3 = f ? b3 : s3;                       // what is left of the other
+        const int k1 = f ? i1 : j1, k2 = f ? j2 : i2;
+        s1 = f ? b1 : s1;
+        i1 = f ? j1 : i1;
+        const bool g = x1 < y2 || (x1 == y2 && k1 < k2);
+        s2 = g ? x1 : y2;
+        i2 = g ? k1 : k2;
+        s3 = g ? fminf(x2, y2) : fminf(x1, y3);
+    }
+};
+
+// ---------------------------------------------------------------------------
+// k_settle: the exact decision for the rows the tensor-core epilogue queued
+// (runner-up inside the error window).  The candidates are the centroids of
+// the groups whose tensor-core minimum lies in the window (a group mask, or --
+// for the streamed-centroid pass -- the groups whose written bound is within
+// the window's edge).  The smallest FP32 distance decides; where FP32 cannot separate it from the
+// runner-up alone the two are ordered by pair_order, and what is left (three
+// that FP32 cannot separate, exact ties) by the FP64 distances of every
+// candidate, lanes over centroids, ties to the lowest index.  Writes the
+// label, corrects u / lb / lbg when the winner is not i1, and appends label
+// changes to the moved-point list 32 at a time.
+//
+// Bound by the latency of the chain count -> request -> row -> candidates and,
+// with many requests, by the shared-memory reads of the candidates' rows.
+// Eight lanes per request: lane l reads the 16-byte pieces l, l + 8, ... of a
+// candidate's row, so that the eight read 128 consecutive bytes and the four
+// requests of a warp never conflict, whatever rows they are at.  (A thread
+// per request read rows of its own: up to 32 rows a read, twelve times the
+// wavefronts, and as many trips as the longest of 32 lists.)  Four candidates
+// go together: their partial sums are handed over in a transposing shuffle
+// that leaves each pair of lanes one of the four.
+//
+// Measured, a pass: 31,000 of 300,007 x 64 rows, K = 200: 64 -> 25 us (20 us of it
+// FP64 near-ties, a dozen of them); 115,000 of 1,048,576 x 64, K = 256: 85 -> 65;
+// 500,000 of 4,194,304 x 128, K = 1024 (centroids in L2): 1270 -> 560.
+// ---------------------------------------------------------------------------
 template <int D>
-__global__ void __launch_bounds__(kSettleThreads, 1) k_settle(Params p, int first, int respect_done, int staged) {
-    // a request per SUB lanes, 8 coordinates per lane
-    constexpr int PL = 8, SUB = D / PL, PER = 32 / SUB;
-    extern __shared__ __align__(16) float sm_settle[];  // C (K x D) | group starts
+__global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int first, int respect_done, int staged) {
+    constexpr int NC = D / 32;  // 16-byte pieces of a row per lane
+    extern __shared__ __align__(128) float sm_settle[];  // C (K x D) | group starts
     __shared__ int32_t mv_n[kSettleWarps][32], mv_old[kSettleWarps][32];  // moves not yet appended
     Ctrl *ctrl = p.ctrl;
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;
     // the requests of this iteration's dense pass, if it ran on the tensor cores
     if (*(volatile int *)&ctrl->path != KM_PATH_DENSE_TC) return;
-    int64_t total = *(volatile int *)&ctrl->settle_count;
+    int total = *(volatile int *)&ctrl->settle_count;
     if (total < 0 || total > p.N) {  // cannot happen: at most one request per row
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ctrl->err, kErrQueue);
         total = 0;
     }
+    const unsigned full = 0xffffffffu;
     const int warp_in = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int sub = lane / SUB, sl = lane - sub * SUB;  // sub-warp and lane in it
-    const unsigned smask = (SUB == 32 ? 0xffffffffu : ((1u << SUB) - 1u)) << (sub * SUB);
-    if ((int64_t)blockIdx.x * kSettleWarps * PER >= total) return;  // uniform per block
+    const int sub = lane / kSub, sl = lane % kSub;
+    // requests per claim: enough claims for every warp of the grid
+    const int64_t nwarps = (int64_t)gridDim.x * kSettleWarps;
+    const int grab = (int)min((int64_t)kGrabMax, max((int64_t)kPer, total / (2 * nwarps) / kPer * kPer));
+    if ((int64_t)blockIdx.x * grab >= total) return;  // uniform per block
     const int K = p.K, G = p.G;
     // C in shared memory (row stride D) when it fits, else read from L2
     const int cst = staged ? D : p.Dp;
@@ -106,14 +170,14 @@ __global__ void __launch_bounds__(kSettleThreads, 1) k_settle(Params p, int firs
     for (int i = threadIdx.x; i <= G; i += kSettleThreads) gs_s[i] = p.gstart[i];
     __syncthreads();
     const bool bounds = p.algo == KM_ALGO_FILTERED;
-    unsigned long long c_changed = 0, c_recheck = 0;
+    int c_changed = 0, c_recheck = 0;
     int mcount = 0;  // warp-uniform
     // append the buffered moves (one slot reservation per warp)
     auto flush_moves = [&]() {
         if (mcount) {
             int base = 0;
             if (lane == 0) base = atomicAdd(&ctrl->moved_count, mcount);
-            base = __shfl_sync(0xffffffffu, base, 0);
+            base = __shfl_sync(full, base, 0);
             if (lane < mcount) {
                 p.moved[base + lane] = mv_n[warp_in][lane];
                 p.moved_old[base + lane] = mv_old[warp_in][lane];
@@ -122,435 +186,218 @@ __global__ void __launch_bounds__(kSettleThreads, 1) k_settle(Params p, int firs
             mcount = 0;
         }
     };
-    // dynamic schedule: each warp takes the next kGrab requests from a counter
-    // (the requests differ in work; a fixed split leaves SMs idle at the end)
-    // and gives them to its sub-warps, PER at a time (warp-uniform trips)
-    constexpr int kGrab = 4 * PER;
-    int r0 = 0, j = kGrab;  // the warp's current grab and its next unused slot
+    // the candidates of a request: the centroids of the masked groups; all K
+    // when the mask holds every group
+    auto all_of = [&](unsigned long long gmask) { return gmask == ~0ull || (gmask == 0ull && !p.lb); };
+    // dynamic schedule: a warp claims `grab` requests (they differ in work),
+    // its lanes read them, and its sub-warps take them kPer at a time
     for (;;) {
-        if (j == kGrab) {
-            if (lane == 0) r0 = atomicAdd(&ctrl->settle_next, kGrab);
-            r0 = __shfl_sync(0xffffffffu, r0, 0);
-            j = 0;
+        int r0 = 0;
+        if (lane == 0) r0 = atomicAdd(&ctrl->settle_next, grab);
+        r0 = __shfl_sync(full, r0, 0);
+        if (r0 >= total || r0 < 0) break;
+        const int cnt = min(grab, total - r0);
+        SettleReq mine;
+        mine.n = -1;
+        mine.old = -1;
+        mine.i1 = 0;
+        mine.lb_alt = mine.lim = 0.f;
+        mine.gmask = 0ull;
+        if (lane < cnt) {
+            const int n = p.squeue[r0 + lane];
+            if (n >= 0 && n < p.N) mine = p.sreq[n];
+            if (n < 0 || n >= p.N || mine.n != n || (unsigned)mine.i1 >= (unsigned)K) {
+                atomicExch(&ctrl->err, kErrQueue);
+                mine.n = -1;
+            }
         }
-        if (r0 >= total) break;
-        const int64_t r = (int64_t)r0 + j + sub;
-        j += PER;
-        bool moved = false;
-        int64_t n = -1;
-        int old = -1;
-        if (r < total) {
-            n = p.squeue[r];
-            const SettleReq q = p.sreq[n >= 0 && n < p.N ? n : 0];
-            if (n < 0 || n >= p.N || q.n != n || (unsigned)q.i1 >= (unsigned)K) {  // sub-warp-uniform
-                if (sl == 0) atomicExch(&ctrl->err, kErrQueue);
-            } else {
-                old = q.old;
-                const float *xg = p.X + n * D;
-                float xv[PL];
+        for (int j = 0; j < cnt; j += kPer) {  // warp-uniform
+            const int from = j + sub;  // < 32
+            const int n = __shfl_sync(full, mine.n, from), old = __shfl_sync(full, mine.old, from);
+            const int w1 = __shfl_sync(full, mine.i1, from);
+            const float lim = __shfl_sync(full, mine.lim, from), lb_alt = __shfl_sync(full, mine.lb_alt, from);
+            const unsigned long long gmask = __shfl_sync(full, mine.gmask, from);
+            const bool act = n >= 0;
+            const int64_t row = act ? n : 0;
+            ulonglong2 xv[NC];
 #pragma unroll
-                for (int k4 = 0; k4 < PL / 4; ++k4) {
-                    const float4 a = __ldg(reinterpret_cast<const float4 *>(xg + sl * PL) + k4);
-                    xv[4 * k4] = a.x;
-                    xv[4 * k4 + 1] = a.y;
-                    xv[4 * k4 + 2] = a.z;
-                    xv[4 * k4 + 3] = a.w;
+            for (int k = 0; k < NC; ++k)
+                xv[k] = __ldg(reinterpret_cast<const ulonglong2 *>(p.X + row * D) + sl + kSub * k);
+            Top3 t;
+            t.s1 = t.s2 = t.s3 = INFINITY;
+            t.i1 = t.i2 = w1;
+            // the walk: centroids [col, cend) of the current group, then the next
+            // group of the mask m (group ids base + bit).  For the bounds' window
+            // m is refilled with 32 groups at a time, four per lane.
+            const bool window = gmask == 0ull && p.lb;
+            int col = 0, cend = act && all_of(gmask) ? K : 0;
+            unsigned long long m = act && !all_of(gmask) && !window ? gmask : 0ull;
+            int seg = act && window ? 0 : G;  // next group of the row's bounds to test
+            const float *lbr = p.lb + row * p.Gp;
+            const float4 none = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+            auto bounds4 = [&](int g) {
+                return g < p.Gp ? *reinterpret_cast<const float4 *>(lbr + g) : none;
+            };
+            float4 ahead = seg < G ? bounds4(4 * sl) : none;
+            int base = 0;
+            for (;;) {  // warp-uniform trips
+                if (col >= cend && m) {
+                    const int b = __ffsll((long long)m) - 1;
+                    m &= m - 1;
+                    // (a window's mask has bit 8 t + l for group base + 4 l + t)
+                    const int g = window ? base + 4 * (b & 7) + (b >> 3) : b;
+                    if (g < G) {
+                        col = gs_s[g];
+                        cend = gs_s[g + 1];
+                    }
                 }
-                // FP32 distance to centroid col, reduced across the sub-warp
-                auto part = [&](int col) __attribute__((always_inline)) {
-                    const float4 *cp = reinterpret_cast<const float4 *>(Cb + (size_t)col * cst + sl * PL);
-                    float a0 = 0.f, a1 = 0.f;
+                const bool dry = col >= cend && !m;
+                if (__any_sync(full, dry && seg < G)) {
+                    const bool take = dry && seg < G;
+                    const float4 v = ahead;
+                    unsigned mk = 0;
 #pragma unroll
-                    for (int k4 = 0; k4 < PL / 4; ++k4) {
-                        const float4 c = cp[k4];
-                        const float d0 = xv[4 * k4] - c.x, d1 = xv[4 * k4 + 1] - c.y;
-                        const float d2 = xv[4 * k4 + 2] - c.z, d3 = xv[4 * k4 + 3] - c.w;
-                        a0 = fmaf(d0, d0, a0);
-                        a1 = fmaf(d1, d1, a1);
-                        a0 = fmaf(d2, d2, a0);
-                        a1 = fmaf(d3, d3, a1);
+                    for (int k = 0; k < 4; ++k) {
+                        const float b = k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
+                        const unsigned in = __ballot_sync(full, b <= lim && seg + 4 * sl + k < G);
+                        mk |= ((in >> (sub * kSub)) & 0xffu) << (8 * k);
                     }
-                    return a0 + a1;
-                };
-                // the candidates in ascending index (a sub-warp-uniform walk)
-                auto for_groups = [&](auto &&fn) __attribute__((always_inline)) {
-                    if (q.gmask == ~0ull || (q.gmask == 0ull && !p.lb)) {
-                        fn(0, K);
-                        return;
+                    if (take) {
+                        m = mk;
+                        base = seg;
+                        seg += 32;
+                        if (seg < G) ahead = bounds4(seg + 4 * sl);
                     }
-                    if (q.gmask == 0ull) {  // the groups whose bound is within the window's edge
-                        const float *lbr = p.lb + n * p.Gp;
-                        for (int g0 = 0; g0 < G; g0 += SUB) {
-                            const bool in = g0 + sl < G && lbr[g0 + sl] <= q.lim;
-                            unsigned m = (__ballot_sync(smask, in) >> (sub * SUB)) &
-                                         (SUB == 32 ? 0xffffffffu : ((1u << SUB) - 1u));
-                            while (m) {
-                                const int g = g0 + __ffs(m) - 1;
-                                m &= m - 1;
-                                fn(gs_s[g], gs_s[g + 1]);
-                            }
-                        }
-                        return;
-                    }
-                    unsigned long long m = q.gmask;
-                    while (m) {
-                        const int g = __ffsll((long long)m) - 1;
-                        m &= m - 1;
-                        if (g >= G) break;
-                        fn(gs_s[g], gs_s[g + 1]);
-                    }
-                };
-                float s1 = INFINITY, s2 = INFINITY;
-                int bi = q.i1;
-                for_groups([&](int c0, int c1) __attribute__((always_inline)) {
-                    for (int col = c0; col < c1; col += 2) {  // two at a time: independent chains
-                        const bool two = col + 1 < c1;
-                        float pa = part(col), pb = part(two ? col + 1 : col);
+                    continue;
+                }
+                if (!__any_sync(full, col < cend || m)) break;
+                if (!__any_sync(full, col < cend)) continue;  // (an empty group)
+                const int last = max(cend - 1, 0);
+                float s[4];
 #pragma unroll
-                        for (int o = SUB / 2; o > 0; o >>= 1) {
-                            pa += __shfl_xor_sync(smask, pa, o, SUB);
-                            pb += __shfl_xor_sync(smask, pb, o, SUB);
-                        }
-                        if (pa < s1) {
-                            s2 = s1;
-                            s1 = pa;
-                            bi = col;
-                        } else {
-                            s2 = fminf(s2, pa);
-                        }
-                        if (two) {
-                            if (pb < s1) {
-                                s2 = s1;
-                                s1 = pb;
-                                bi = col + 1;
-                            } else {
-                                s2 = fminf(s2, pb);
-                            }
-                        }
+                for (int k = 0; k < 4; ++k) {
+                    const ulonglong2 *c = reinterpret_cast<const ulonglong2 *>(Cb + (size_t)min(col + k, last) * cst) + sl;
+                    unsigned long long a0 = 0ull, a1 = 0ull;
+#pragma unroll
+                    for (int q = 0; q < NC; ++q) {
+                        const ulonglong2 c2 = c[kSub * q];
+                        unsigned long long d0, d1;
+                        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d0) : "l"(xv[q].x), "l"(c2.x));
+                        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d1) : "l"(xv[q].y), "l"(c2.y));
+                        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a0) : "l"(d0));
+                        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a1) : "l"(d1));
                     }
-                });
-                float bs = s1;
-                if (s2 != INFINITY && unresolved(s1, s2, p)) {
-                    // FP64 over every candidate, lanes over candidates
+                    float l0, h0, l1, h1;
+                    asm("mov.b64 {%0, %1}, %2;" : "=f"(l0), "=f"(h0) : "l"(a0));
+                    asm("mov.b64 {%0, %1}, %2;" : "=f"(l1), "=f"(h1) : "l"(a1));
+                    s[k] = (l0 + h0) + (l1 + h1);
+                }
+                // lanes 4 apart: two candidates each; 2 apart: one each; then the pair's sum
+                const bool u4 = sl & 4, u2 = sl & 2;
+                const float r0v = (u4 ? s[2] : s[0]) + __shfl_xor_sync(full, u4 ? s[0] : s[2], 4);
+                const float r1v = (u4 ? s[3] : s[1]) + __shfl_xor_sync(full, u4 ? s[1] : s[3], 4);
+                float sx = (u2 ? r1v : r0v) + __shfl_xor_sync(full, u2 ? r0v : r1v, 2);
+                sx += __shfl_xor_sync(full, sx, 1);
+                const int cc = col + (u4 ? 2 : 0) + (u2 ? 1 : 0);
+                if (cc < cend) t.add(sx, cc);
+                col += 4;
+            }
+            t.merge(2);
+            t.merge(4);
+            // near-ties, one request after another, by the whole warp
+            int bi = t.i1;
+            float bs = t.s1;
+            unsigned rm = __ballot_sync(full, sl == 0 && act && t.s2 != INFINITY && unresolved(t.s1, t.s2, p));
+            while (rm) {
+                const int src = __ffs(rm) - 1;
+                rm &= rm - 1;
+                const int64_t nr = __shfl_sync(full, n, src);
+                const int a1 = __shfl_sync(full, t.i1, src), a2 = __shfl_sync(full, t.i2, src);
+                const float v1 = __shfl_sync(full, t.s1, src), v2 = __shfl_sync(full, t.s2, src);
+                const float v3 = __shfl_sync(full, t.s3, src);
+                const float *xg = p.X + nr * D;
+                int bj = a1;
+                float bsr = v1;
+                int o = -1;
+                if (v3 == INFINITY || !unresolved(v1, v3, p))
+                    o = pair_order(xg, Cb + (size_t)a1 * cst, Cb + (size_t)a2 * cst, D);
+                if (o == 1) {
+                    bj = a2;
+                    bsr = v2;
+                } else if (o < 0) {
+                    const unsigned long long gm = __shfl_sync(full, gmask, src);
+                    const float lm = __shfl_sync(full, lim, src);
+                    const float *lbn = p.lb + nr * p.Gp;
                     double bd = INFINITY;
-                    int bj = 0x7fffffff;
-                    for_groups([&](int c0, int c1) __attribute__((always_inline)) {
-                        for (int col = c0 + sl; col < c1; col += SUB) {
-                            const double d64 = settle_fp64(xg, Cb + (size_t)col * cst, D);
-                            if (d64 < bd || (d64 == bd && tie_key(p, col) < tie_key(p, bj))) {
-                                bd = d64;
-                                bj = col;
-                            }
+                    bj = 0x7fffffff;
+                    for (int c = lane; c < K; c += 32) {
+                        bool cand = all_of(gm);
+                        if (!cand) {
+                            const int g = p.grp[c];
+                            cand = gm == 0ull ? lbn[g] <= lm : (g < 64 && ((gm >> g) & 1ull));
                         }
-                    });
+                        if (!cand || !unresolved(v1, settle_fp32(xg, Cb + (size_t)c * cst, D), p)) continue;
+                        const double d64 = settle_fp64(xg, Cb + (size_t)c * cst, D);
+                        if (d64 < bd || (d64 == bd && tie_key(p, c) < tie_key(p, bj))) {
+                            bd = d64;
+                            bj = c;
+                        }
+                    }
 #pragma unroll
-                    for (int o = SUB / 2; o > 0; o >>= 1) {
-                        const double ov = __shfl_xor_sync(smask, bd, o, SUB);
-                        const int oi = __shfl_xor_sync(smask, bj, o, SUB);
+                    for (int w = 16; w > 0; w >>= 1) {
+                        const double ov = __shfl_xor_sync(full, bd, w);
+                        const int oi = __shfl_xor_sync(full, bj, w);
                         if (ov < bd || (ov == bd && tie_key(p, oi) < tie_key(p, bj))) {
                             bd = ov;
                             bj = oi;
                         }
                     }
-                    if (bj != bi) {  // its FP32 distance, for u
-                        float pc = part(bj);
-#pragma unroll
-                        for (int o = SUB / 2; o > 0; o >>= 1) pc += __shfl_xor_sync(smask, pc, o, SUB);
-                        bs = pc;
-                    }
-                    bi = bj;
-                    c_recheck += sl == 0 ? 1 : 0;
+                    if (bj == 0x7fffffff) bj = a1;
+                    // for u: its FP32 distance, or the smallest (it is no farther than a1)
+                    bsr = bj == a2 ? v2 : v1;
                 }
-                if (sl == 0) {
-                    p.label[n] = bi;
-                    if (bounds) {
-                        p.u[n] = dist_up(bs, p);
-                        if (bi != q.i1) {
-                            p.lb[n * p.Gp + p.grp[q.i1]] = q.lb_alt;
-                            p.lb[n * p.Gp + p.grp[bi]] = q.lb_alt;
-                            p.lbg[n] = q.lb_alt;
-                        }
+                if (lane / kSub == src / kSub) {
+                    bi = bj;
+                    bs = bsr;
+                }
+                c_recheck += lane == 0;
+            }
+            bool moved = false;
+            if (act && sl == 0) {
+                p.label[n] = bi;
+                if (bounds) {
+                    p.u[n] = dist_up(bs, p);
+                    if (bi != w1) {
+                        p.lb[row * p.Gp + p.grp[w1]] = lb_alt;
+                        p.lb[row * p.Gp + p.grp[bi]] = lb_alt;
+                        p.lbg[n] = lb_alt;
                     }
                 }
                 moved = bi != old;
-                c_changed += (moved && sl == 0) ? 1 : 0;
+                c_changed += moved;
             }
-        }
-        // label changes: the sub-warp leaders' moves, appended 32 at a time
-        __syncwarp();
-        if (!first) {
-            const unsigned mm = __ballot_sync(0xffffffffu, moved && sl == 0);
-            if (mm) {
-                const int k = mcount + __popc(mm & ((1u << lane) - 1u));
-                if (moved && sl == 0) {
-                    mv_n[warp_in][k] = (int32_t)n;
-                    mv_old[warp_in][k] = old;
+            // label changes: the sub-warp leaders' moves, appended 32 at a time
+            if (!first) {
+                const unsigned mm = __ballot_sync(full, moved);
+                if (mm) {
+                    const int k = mcount + __popc(mm & ((1u << lane) - 1u));
+                    if (moved) {
+                        mv_n[warp_in][k] = n;
+                        mv_old[warp_in][k] = old;
+                    }
+                    mcount += __popc(mm);
+                    __syncwarp();
+                    if (mcount > 32 - kPer) flush_moves();
                 }
-                mcount += __popc(mm);
             }
-            __syncwarp();
-            if (mcount > 32 - PER) flush_moves();
         }
     }
     if (!first) flush_moves();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c_changed += __shfl_xor_sync(0xffffffffu, c_changed, o);
-        c_recheck += __shfl_xor_sync(0xffffffffu, c_recheck, o);
-    }
+    c_changed = __reduce_add_sync(full, c_changed);
+    c_recheck = __reduce_add_sync(full, c_recheck);
     if (lane == 0) {
-        if (c_changed) atomicAdd(&ctrl->n_changed, c_changed);
-        if (c_recheck) atomicAdd(&ctrl->n_recheck, c_recheck);
-    }
-}
-
-// The staged variant for short rows (D <= 64, C in shared memory): one
-// thread per request with the row in registers.  Its candidate walks diverge
-// across the warp, but with C in shared memory that costs less than the
-// sub-warp reductions above (measured: about 100 against 135 us per pass on
-// the 1M x 64, K = 256 workload).  The rare near-ties that need FP64 are
-// settled afterwards by the whole warp, one request at a time.
-// FP32 squared distance of the row (packed pairs in registers) to a centroid
-// row in shared memory: packed FP32x2 subtract / fused multiply-add (each
-// half an ordinary round-to-nearest FP32 operation; four partial sums)
-template <int D>
-__device__ __forceinline__ float settle_fp32(const ulonglong2 (&xr)[D / 4], const float *c) {
-    const ulonglong2 *c2p = reinterpret_cast<const ulonglong2 *>(c);
-    unsigned long long a0 = 0ull, a1 = 0ull;
-#pragma unroll
-    for (int i = 0; i < D / 4; ++i) {
-        const ulonglong2 c2 = c2p[i];
-        unsigned long long d0, d1;
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d0) : "l"(xr[i].x), "l"(c2.x));
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d1) : "l"(xr[i].y), "l"(c2.y));
-        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a0) : "l"(d0));
-        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a1) : "l"(d1));
-    }
-    float l0, h0, l1, h1;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(l0), "=f"(h0) : "l"(a0));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(l1), "=f"(h1) : "l"(a1));
-    return (l0 + h0) + (l1 + h1);
-}
-// The same FP32 distance with the row read from memory (16-byte aligned, D a
-// multiple of 4): the packing and every rounding step of settle_fp32
-template <int D>
-__device__ __forceinline__ float settle_fp32_mem(const float *x, const float *c) {
-    const ulonglong2 *x2p = reinterpret_cast<const ulonglong2 *>(x);
-    const ulonglong2 *c2p = reinterpret_cast<const ulonglong2 *>(c);
-    unsigned long long a0 = 0ull, a1 = 0ull;
-#pragma unroll 4
-    for (int i = 0; i < D / 4; ++i) {
-        const ulonglong2 x2 = __ldg(x2p + i);
-        const ulonglong2 c2 = c2p[i];
-        unsigned long long d0, d1;
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d0) : "l"(x2.x), "l"(c2.x));
-        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d1) : "l"(x2.y), "l"(c2.y));
-        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a0) : "l"(d0));
-        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a1) : "l"(d1));
-    }
-    float l0, h0, l1, h1;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(l0), "=f"(h0) : "l"(a0));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(l1), "=f"(h1) : "l"(a1));
-    return (l0 + h0) + (l1 + h1);
-}
-
-template <int D>
-__global__ void __launch_bounds__(kSettleThreads, 2) k_settle_t(Params p, int first, int respect_done, int staged) {
-    static_assert(D <= 64 && D % 4 == 0, "the row lives in registers");
-    extern __shared__ __align__(16) float sm_settle[];  // C (K rows, stride SD) | group starts
-    Ctrl *ctrl = p.ctrl;
-    count_kernel(ctrl);
-    if (respect_done && *(volatile int *)&ctrl->done) return;
-    // the requests of this iteration's dense pass, if it ran on the tensor cores
-    if (*(volatile int *)&ctrl->path != KM_PATH_DENSE_TC) return;
-    int64_t total = *(volatile int *)&ctrl->settle_count;
-    if (total < 0 || total > p.N) {  // cannot happen: at most one request per row
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&ctrl->err, kErrQueue);
-        total = 0;
-    }
-    const int lane = threadIdx.x & 31;
-    if ((int64_t)blockIdx.x * kSettleThreads >= total) return;  // uniform per block
-    const int K = p.K, G = p.G;
-    // C staged with a row stride of D + 4 floats (16-byte reads of different
-    // rows by the threads of a warp spread over the banks), or read from
-    // global memory when it does not fit
-    const int SD = staged ? D + 4 : p.Dp;
-    const float *Cs = staged ? sm_settle : p.C;
-    int32_t *gs_s = reinterpret_cast<int32_t *>(sm_settle + (staged ? (size_t)K * SD : 0));
-    if (staged)
-        for (int i = threadIdx.x; i < K * (D / 4); i += kSettleThreads) {
-            const int row = i / (D / 4), q4 = i - row * (D / 4);
-            reinterpret_cast<float4 *>(sm_settle + (size_t)row * SD)[q4] =
-                __ldg(reinterpret_cast<const float4 *>(p.C + (size_t)row * p.Dp) + q4);
-        }
-    for (int i = threadIdx.x; i <= G; i += kSettleThreads) gs_s[i] = p.gstart[i];
-    __syncthreads();
-    const bool bounds = p.algo == KM_ALGO_FILTERED;
-    unsigned long long c_changed = 0, c_recheck = 0;
-    // the candidates of a request: the centroids of the masked groups; all K
-    // when the mask holds every group
-    auto all_of = [&](const SettleReq &q) { return q.gmask == ~0ull || (q.gmask == 0ull && !p.lb); };
-    // dynamic schedule: each warp takes the next 32 requests (one per lane)
-    // from a counter; the requests differ in work, and a fixed split left
-    // many SMs idle while a few finished their share
-    for (;;) {
-        int r0 = 0;
-        if (lane == 0) r0 = atomicAdd(&ctrl->settle_next, 32);
-        r0 = __shfl_sync(0xffffffffu, r0, 0);
-        if (r0 >= total) break;
-        const int64_t r = (int64_t)r0 + lane;
-        bool act = r < total;
-        int64_t n = 0;
-        SettleReq q;
-        q.n = -1;
-        q.old = -1;
-        q.i1 = 0;
-        q.lb_alt = 0.f;
-        q.gmask = 0ull;
-        q.lim = 0.f;
-        if (act) {
-            n = p.squeue[r];
-            if (n < 0 || n >= p.N) {
-                atomicExch(&ctrl->err, kErrQueue);
-                act = false;
-            }
-        }
-        if (act) {
-            q = p.sreq[n];
-            if (q.n != n || (unsigned)q.i1 >= (unsigned)K) {
-                atomicExch(&ctrl->err, kErrQueue);
-                act = false;
-            }
-        }
-        float s1 = INFINITY, s2 = INFINITY;
-        int bi = q.i1;
-        if (act) {
-            // the row in registers
-            ulonglong2 xr[D / 4];
-            {
-                const ulonglong2 *xp = reinterpret_cast<const ulonglong2 *>(p.X + n * D);
-#pragma unroll
-                for (int i = 0; i < D / 4; ++i) xr[i] = __ldg(xp + i);
-            }
-            // smallest (first in ascending order on ties) and runner-up over the
-            // candidates in ascending index
-            auto visit = [&](int col) {
-                const float sx = settle_fp32<D>(xr, Cs + (size_t)col * SD);
-                if (sx < s1) {
-                    s2 = s1;
-                    s1 = sx;
-                    bi = col;
-                } else {
-                    s2 = fminf(s2, sx);
-                }
-            };
-            if (all_of(q)) {
-                for (int col = 0; col < K; ++col) visit(col);
-            } else if (q.gmask == 0ull) {  // the groups whose bound is within the window's edge
-                const float *lbr = p.lb + n * p.Gp;
-                for (int g = 0; g < G; ++g)
-                    if (lbr[g] <= q.lim)
-                        for (int col = gs_s[g]; col < gs_s[g + 1]; ++col) visit(col);
-            } else {
-                unsigned long long m = q.gmask;
-                while (m) {
-                    const int g = __ffsll((long long)m) - 1;
-                    m &= m - 1;
-                    if (g >= G) break;
-                    for (int col = gs_s[g]; col < gs_s[g + 1]; ++col) visit(col);
-                }
-            }
-        }
-        float bs = s1;
-        // near-ties (FP32 cannot order the two smallest): the smallest FP64
-        // distance among the candidates that FP32 cannot separate from s1,
-        // lowest index on equal distances; settled one request at a time by the
-        // whole warp, lanes over the centroids, so that one lane's FP64 work
-        // does not hold up the warp's other requests
-        const bool rc = act && s2 != INFINITY && unresolved(s1, s2, p);
-        unsigned rm = __ballot_sync(0xffffffffu, rc);
-        while (rm) {
-            const int src = __ffs(rm) - 1;
-            rm &= rm - 1;
-            const int64_t nr = __shfl_sync(0xffffffffu, n, src);
-            const float s1r = __shfl_sync(0xffffffffu, s1, src);
-            const int bir = __shfl_sync(0xffffffffu, bi, src);
-            SettleReq qr;
-            qr.gmask = __shfl_sync(0xffffffffu, q.gmask, src);
-            qr.lim = __shfl_sync(0xffffffffu, q.lim, src);
-            const bool all = all_of(qr);
-            const float *xg = p.X + nr * D;
-            const float *lbr = p.lb + nr * p.Gp;
-            double bd = INFINITY;
-            int bj = 0x7fffffff;
-            for (int c = lane; c < K; c += 32) {  // ascending: the first of equal distances stays
-                bool cand = all;
-                if (!cand) {
-                    const int g = p.grp[c];
-                    cand = qr.gmask == 0ull ? lbr[g] <= qr.lim : (g < 64 && ((qr.gmask >> g) & 1ull));
-                }
-                if (!cand || !unresolved(s1r, settle_fp32_mem<D>(xg, Cs + (size_t)c * SD), p)) continue;
-                const double d64 = settle_fp64(xg, Cs + (size_t)c * SD, D);
-                if (d64 < bd || (d64 == bd && tie_key(p, c) < tie_key(p, bj))) {
-                    bd = d64;
-                    bj = c;
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ov = __shfl_xor_sync(0xffffffffu, bd, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bj, o);
-                if (ov < bd || (ov == bd && tie_key(p, oi) < tie_key(p, bj))) {
-                    bd = ov;
-                    bj = oi;
-                }
-            }
-            // bir is among them (its own FP32 distance is s1r)
-            if (bj == 0x7fffffff) bj = bir;
-            const float bsr = bj != bir ? settle_fp32_mem<D>(xg, Cs + (size_t)bj * SD) : s1r;
-            if (lane == src) {
-                bi = bj;
-                bs = bsr;
-                c_recheck += 1;
-            }
-        }
-        bool moved = false;
-        if (act) {
-            p.label[n] = bi;
-            if (bounds) {
-                p.u[n] = dist_up(bs, p);
-                if (bi != q.i1) {
-                    p.lb[n * p.Gp + p.grp[q.i1]] = q.lb_alt;
-                    p.lb[n * p.Gp + p.grp[bi]] = q.lb_alt;
-                    p.lbg[n] = q.lb_alt;
-                }
-            }
-            moved = bi != q.old;
-            c_changed += moved ? 1 : 0;
-        }
-        // label changes: one slot reservation per warp
-        if (!first) {
-            const unsigned mm = __ballot_sync(0xffffffffu, moved);
-            if (mm) {
-                int base = 0;
-                if (lane == 0) base = atomicAdd(&ctrl->moved_count, __popc(mm));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (moved) {
-                    const int slot = base + __popc(mm & ((1u << lane) - 1u));
-                    p.moved[slot] = (int32_t)n;
-                    p.moved_old[slot] = q.old;
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c_changed += __shfl_xor_sync(0xffffffffu, c_changed, o);
-        c_recheck += __shfl_xor_sync(0xffffffffu, c_recheck, o);
-    }
-    if (lane == 0) {
-        if (c_changed) atomicAdd(&ctrl->n_changed, c_changed);
-        if (c_recheck) atomicAdd(&ctrl->n_recheck, c_recheck);
+        if (c_changed) atomicAdd(&ctrl->n_changed, (unsigned long long)c_changed);
+        if (c_recheck) atomicAdd(&ctrl->n_recheck, (unsigned long long)c_recheck);
     }
 }
 
@@ -558,22 +405,17 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle_t(Params p, int fi
 
 cudaError_t launch_settle(const Params &p, cudaStream_t s, int first, int respect_done, int num_sms) {
     if (p.D != 32 && p.D != 64 && p.D != 128) return cudaErrorInvalidValue;
-    // compact the request bitmap (one warp per 32 words), then one thread per request
+    // compact the request bitmap (one warp per 32 words), then the requests
     const int64_t words = (p.N + 31) / 32;
     const int64_t gblocks = std::max<int64_t>(1, std::min<int64_t>((words + 255) / 256, (int64_t)num_sms * 8));
     count_launch();
     k_settle_gather<<<(unsigned)gblocks, 256, 0, s>>>(p, respect_done);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // C in shared memory when it fits (up to 160 KB), else read from L2; short
-    // rows with C in shared memory: thread per request (C rows padded by 4
-    // floats), else sub-warps (C rows unpadded)
-    const int staged = (size_t)p.K * (p.D + 4) * 4 <= ((size_t)160 << 10);
-    const bool per_thread = staged && p.D <= 64;
-    const size_t cbytes = staged ? (size_t)p.K * (p.D + (per_thread ? 4 : 0)) * 4 : 0;
-    const size_t smem = cbytes + (size_t)(p.G + 1) * 4;
-    auto kern = per_thread ? (p.D == 32 ? k_settle_t<32> : k_settle_t<64>)
-                           : (p.D == 32 ? k_settle<32> : (p.D == 64 ? k_settle<64> : k_settle<128>));
+    // C in shared memory when it fits (up to 160 KB), else read from L2
+    const int staged = (size_t)p.K * p.D * 4 <= ((size_t)160 << 10);
+    const size_t smem = (staged ? (size_t)p.K * p.D * 4 : 0) + (size_t)(p.G + 1) * 4;
+    auto kern = p.D == 32 ? k_settle<32> : (p.D == 64 ? k_settle<64> : k_settle<128>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;

@@ -197,13 +197,6 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_scatter(Params p, int r
     }
 }
 
-// Error-free transformation of a sum (Knuth's TwoSum): s + e == a + b exactly.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // Each warp sums a run of consecutive sorted entries, lanes over the
 // coordinates, eight entries' loads in flight at a time, and adds its partial
 // sums to S and Q (and, in incremental mode, the count change to cnt) whenever

@@ -90,8 +90,9 @@ __device__ __forceinline__ float bound_dn(float s, const Params &p) { return s =
 
 // Finish a warp's points (lane: point n if active, its scan's result; row: its
 // group bounds, in shared or global memory).  Near-ties are settled by the
-// whole warp, one point at a time: the lanes share the centroids out, those
-// that the FP32 bound cannot separate from the best are compared in FP64.
+// whole warp, one point at a time: the lanes share the centroids out; a single
+// one that the FP32 bound cannot separate from the best is ordered by
+// pair_order, several (or what that leaves open) in FP64.
 // Returns the lane's number of settled points; `changed` counts its moves.
 __device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool active, int64_t n, Nearest &t,
                                              float *row, bool bounds, int first, int v, int &changed) {
@@ -106,21 +107,41 @@ __device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool a
         const float ref = __shfl_sync(full, t.s1, src);
         const int was = __shfl_sync(full, t.best, src);
         const float *xr = p.X + m * p.D;
-        double bd = INFINITY;
+        // the centroids that FP32 cannot separate from the best
+        int many = 0, other = was;
+        float so = ref;
+        for (int c0 = 0; c0 < p.K; c0 += 32) {
+            const int c = c0 + lane;
+            const float s = c < p.K ? sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D) : INFINITY;
+            const unsigned in = __ballot_sync(full, c < p.K && c != was && unresolved(ref, s, p));
+            many += __popc(in);
+            if (in) {
+                other = c0 + __ffs(in) - 1;
+                so = __shfl_sync(full, s, __ffs(in) - 1);
+            }
+        }
         int bi = was;
         float bs = ref;
-        for (int c = lane; c < p.K; c += 32) {
-            const float s = sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D);
-            if (!unresolved(ref, s, p)) continue;
-            const double d = dist2_f64(xr, p.C + (size_t)c * p.Dp, p.D);
-            if (d < bd || (d == bd && tie_key(p, c) < tie_key(p, bi))) { bd = d; bi = c; bs = s; }
-        }
+        const int o =
+            many == 1 ? pair_order(xr, p.C + (size_t)was * p.Dp, p.C + (size_t)other * p.Dp, p.D) : (many ? -1 : 0);
+        if (o == 1) {
+            bi = other;
+            bs = so;
+        } else if (o < 0) {
+            double bd = INFINITY;
+            for (int c = lane; c < p.K; c += 32) {
+                const float s = sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D);
+                if (c != was && !unresolved(ref, s, p)) continue;
+                const double d = dist2_f64(xr, p.C + (size_t)c * p.Dp, p.D);
+                if (d < bd || (d == bd && tie_key(p, c) < tie_key(p, bi))) { bd = d; bi = c; bs = s; }
+            }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double od = __shfl_xor_sync(full, bd, o);
-            const int oi = __shfl_xor_sync(full, bi, o);
-            const float os = __shfl_xor_sync(full, bs, o);
-            if (od < bd || (od == bd && tie_key(p, oi) < tie_key(p, bi))) { bd = od; bi = oi; bs = os; }
+            for (int w = 16; w > 0; w >>= 1) {
+                const double od = __shfl_xor_sync(full, bd, w);
+                const int oi = __shfl_xor_sync(full, bi, w);
+                const float os = __shfl_xor_sync(full, bs, w);
+                if (od < bd || (od == bd && tie_key(p, oi) < tie_key(p, bi))) { bd = od; bi = oi; bs = os; }
+            }
         }
         if (bi != was) {
             if (bounds) {  // group bounds must now exclude the new best
@@ -193,7 +214,7 @@ __device__ __forceinline__ void add_counters(Ctrl *ctrl, int changed, int settle
 // P / L points it owns.
 //
 // Measured, K = 256 (before: one point per lane, scalar, two centroids): 262,144
-// x 64: 599 -> 333 us, the FP32 pipe busy in 75% of the cycles; 600,000 x 8:
+// x 64: 599 -> 310 us, the FP32 pipe busy in 75% of the cycles; 600,000 x 8:
 // 286 -> 124; x 16: 377 -> 212; x 32: 673 -> 399; x 50: 1177 -> 667; x 128: 3358
 // -> 1699.
 template <int DPL, int L, int P, int Q, int MB>

@@ -22,10 +22,14 @@
 //     group that holds the running best keeps both the value that excludes
 //     the best and the value that includes it, in case the best moves on;
 //   * a point whose FP32 best and runner-up cannot be separated by the FP32
-//     error bound is settled over all K centroids, in FP64 where needed, and
-//     its bounds are rebuilt from that full scan -- by the whole warp, after
-//     the batch's points are done, so that one lane does not hold up the
-//     other 31 (and the SM) for the length of a K-centroid scan;
+//     error bound is settled by the whole warp, after the batch's points are
+//     done: the two are ordered by compensated FP32 sums (pair_order), and
+//     only where that decides nothing, or a third is as near, by a scan over
+//     all K centroids with FP64 distances, from which the bounds are rebuilt
+//     (that scan for every near-tie, some 300 of a million survivors, was a
+//     quarter of the kernel's time with many centroids: 4,194,304 x 128,
+//     K = 1024: 1060 -> 774 us an iteration; 1,048,576 x 32, K = 4096: 767 ->
+//     607);
 //   * label changes go to the moved-point list; the cluster sums are updated
 //     by the moves kernel afterwards.
 #include "kp_common.cuh"
@@ -153,7 +157,7 @@ __device__ __forceinline__ double dist2_f64_mem(const Params &p, const float *xg
 // is its FP32 squared distance.  (One lane alone took about 125 us for this
 // at K = 256, D = 64, against about 28 us for a whole batch of 32 points.)
 template <int DP>
-__device__ __forceinline__ int settle_warp(const Params &p, const float *Cs, const int32_t *gs, int64_t n, float s1,
+__device__ __noinline__ int settle_warp(const Params &p, const float *Cs, const int32_t *gs, int64_t n, float s1,
                                         int i1, float *s_win, float *lbg_out) {
     const int K = p.K, G = p.G, D = p.D;
     const int lane = threadIdx.x & 31;
@@ -218,7 +222,8 @@ struct TpLayout {
 // two blocks per SM up to 64 coordinates; at 128 the point's registers (64
 // for x alone) leave room for one
 template <int DP, bool STAGE>
-__global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Params p, int respect_done) {
+__global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2)
+    k_survivor_tp(const __grid_constant__ Params p, int respect_done) {
     extern __shared__ __align__(128) float smem[];
     __shared__ __align__(8) uint64_t bar;
     Ctrl *ctrl = p.ctrl;
@@ -271,8 +276,8 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Par
         int a = 0;
         // a point deferred to the warp's settle: its FP32 best, index and global bound
         bool rc = false;
-        float rc_s = 0.f, rc_lbg = 0.f;
-        int rc_best = 0;
+        float rc_s = 0.f, rc_lbg = 0.f, rc_s2 = 0.f;
+        int rc_best = 0, rc_sec = -1;  // the runner-up, -1: not the only one FP32 cannot separate
         const unsigned long long c_dist0 = c_dist;  // this lane's count before its point
         if (active) {
             n = p.queue[it];
@@ -309,8 +314,8 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Par
                 const float *dcw = p.Dc + (size_t)wl * K;
                 const float *dgw = p.Dg + (size_t)wl * Gp;
 
-                float s_best = sa, s_sec = INFINITY, bd_up = ut;
-                int best = a;
+                float s_best = sa, s_sec = INFINITY, s_third = INFINITY, bd_up = ut;
+                int best = a, sec = a;
                 int bg = -1;                      // group holding the running best, once visited
                 float bg_val = INFINITY, bg_m1 = INFINITY;  // its bound without / with the best
                 float lmin = INFINITY;            // minimum over the other groups' new bounds
@@ -368,13 +373,19 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Par
                                 const float s = sqdist_xr<DP>(xr, Cs + (size_t)c * p.Dp);
                                 c_dist += 1;
                                 if (s < s_best || (s == s_best && c < best)) {
-                                    s_sec = fminf(s_sec, s_best);
+                                    s_third = s_sec;
+                                    s_sec = s_best;
+                                    sec = best;
                                     s_best = s;
                                     best = c;
                                     best_moved = true;
                                     bd_up = fminf(bd_up, dist_up(s, p));
+                                } else if (s < s_sec) {
+                                    s_third = s_sec;
+                                    s_sec = s;
+                                    sec = c;
                                 } else {
-                                    s_sec = fminf(s_sec, s);
+                                    s_third = fminf(s_third, s);
                                 }
                                 if (s < sm1) {
                                     sm2 = sm1;
@@ -437,6 +448,8 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Par
                     rc_s = s_best;
                     rc_best = best;
                     rc_lbg = lbg_new;
+                    rc_s2 = s_sec;
+                    rc_sec = s_third == INFINITY || !unresolved(s_best, s_third, p) ? sec : -1;
                 } else {
                     p.lbg[n] = lbg_new;
                     p.u[n] = dist_up(s_best, p);
@@ -456,12 +469,29 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Par
             const int64_t nr = __shfl_sync(0xffffffffu, n, src);
             const float s1 = __shfl_sync(0xffffffffu, rc_s, src);
             const int i1 = __shfl_sync(0xffffffffu, rc_best, src);
-            float sw = s1, lg = __shfl_sync(0xffffffffu, rc_lbg, src);
-            const int w = settle_warp<DP>(p, Cs, gs, nr, s1, i1, &sw, &lg);
-            if (lane == src) {
-                rc_best = w;
-                rc_s = sw;
-                rc_lbg = lg;
+            const int i2 = __shfl_sync(0xffffffffu, rc_sec, src);
+            const int o = i2 < 0 ? -1
+                                 : pair_order(p.X + nr * p.D, Cs + (size_t)i1 * p.Dp, Cs + (size_t)i2 * p.Dp, p.D);
+            if (o == 1) {
+                // the runner-up it is: every bound holds (its group's still counts
+                // it), but for those that left out i1
+                if (lane == src) {
+                    float *lb1 = p.lb + n * Gp + sgrp[i1];
+                    const float d1 = dist_dn(s1, p);
+                    *lb1 = fminf(*lb1, d1);
+                    rc_lbg = fminf(rc_lbg, d1);
+                    rc_best = i2;
+                    rc_s = rc_s2;
+                }
+            } else if (o < 0) {
+                float sw = s1, lg = __shfl_sync(0xffffffffu, rc_lbg, src);
+                const int w = settle_warp<DP>(p, Cs, gs, nr, s1, i1, &sw, &lg);
+                if (lane == src) {
+                    rc_best = w;
+                    rc_s = sw;
+                    rc_lbg = lg;
+                    c_dist = c_dist0 + (unsigned long long)K;  // evaluated against all K: K, not scan + K
+                }
             }
         }
         if (rc) {
@@ -470,7 +500,6 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2) k_survivor_tp(Par
             p.label[n] = rc_best;
             p.stamp[n] = make_stamp(v, v);
             moved = rc_best != a;
-            c_dist = c_dist0 + (unsigned long long)K;  // evaluated against all K: K, not scan + K
             c_recheck += 1;
         }
         // moved points: one atomic per warp for the list slots
@@ -531,21 +560,30 @@ cudaError_t launch_tp(const Params &p, cudaStream_t s, int respect_done, int num
 }  // namespace
 
 bool survivor_tp_eligible(const Params &p) {
-    const int dp = dense_dp(p.D);
-    return dp > 0 && dp <= 128 && p.K < 0x7fffffff;
+    return p.D <= 128 && p.K < 0x7fffffff;
 }
 
 cudaError_t launch_survivor_tp(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem_limit) {
     smem_limit -= 64;  // static shared (mbarrier)
-    switch (dense_dp(p.D)) {
-    case 4: return launch_tp<4>(p, s, respect_done, num_sms, smem_limit);
-    case 8: return launch_tp<8>(p, s, respect_done, num_sms, smem_limit);
-    case 16: return launch_tp<16>(p, s, respect_done, num_sms, smem_limit);
-    case 32: return launch_tp<32>(p, s, respect_done, num_sms, smem_limit);
-    case 64: return launch_tp<64>(p, s, respect_done, num_sms, smem_limit);
-    case 128: return launch_tp<128>(p, s, respect_done, num_sms, smem_limit);
-    default: return cudaErrorInvalidValue;
-    }
+    // the row's registers in steps of 4 coordinates up to 32, then 16 and 32 (a
+    // centroid's staged row is padded at least that far): 200,003 x 17, K = 100:
+    // 33 us an iteration on 32 coordinates, 31 on 20
+#define TP(DP) \
+    if (p.D <= DP) return launch_tp<DP>(p, s, respect_done, num_sms, smem_limit)
+    TP(4);
+    TP(8);
+    TP(12);
+    TP(16);
+    TP(20);
+    TP(24);
+    TP(28);
+    TP(32);
+    TP(48);
+    TP(64);
+    TP(96);
+    TP(128);
+#undef TP
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace kp

@@ -74,8 +74,8 @@ struct SettleReq {
     int32_t old;     // label before this pass (-1: none)
     int32_t i1;      // tensor-core winner (the bounds were written for it)
     float lb_alt;    // group bound that holds for every column (from the smallest estimate)
-    unsigned long long gmask;  // groups that can hold the winner (all ones: every group;
-                               // zero: the groups g with lb[n][g] <= lim)
+    unsigned long long gmask[2];  // their union: groups that can hold the winner (all ones: every
+                                  // group; zero: the groups g with lb[n][g] <= lim)
     float lim;       // bound of the window's edge (used when gmask is zero)
 };
 

@@ -21,7 +21,16 @@
 // each scanning half of the columns) read the accumulators back with
 // tcgen05.ld, one TMEM lane (= point) per thread, and turn
 // t_k = ||c_k||^2 - 2 x.c_k into the winner, the runner-up and the per-group
-// minima.  Lower bounds are t-based with the error E(x) subtracted, the upper
+// minima, four columns at a time (Scan4 in kp_tc.cuh).
+//
+// Bound by the scan: of 200 us for 1,048,576 x 64, K = 256, G = 26, loads,
+// products and TMEM reads alone take 76, the scan 80 (the minima and maxima of
+// four columns are 13 instructions on the half-rate pipe), the rows' bounds and
+// labels 45.  Measured: that pass 226 -> 200 us, 300,007 x 64, K = 200, plain
+// Lloyd, 55 -> 47 (column-by-column scan, rows finished by one of the two
+// halves, a lane per centroid's norm before).
+//
+  Lower bounds are t-based with the error E(x) subtracted, the upper
 // bound adds it; when the runner-up lies within 2E of the winner the point is
 // settled exactly by kp_settle.cu (FP32 direct differences, then FP64 if the
 // FP32 error bound cannot decide), so labels are exact.
@@ -88,10 +97,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     uint8_t *sBl = sm + NA * b_atom;
     uint8_t *sA = sm + cfg.off_A;  // stage s: [NA atoms of x_h][NA atoms of x_l]
     float *cn = reinterpret_cast<float *>(sm + cfg.off_cn);  // [Kp] ||c||^2 (+inf: padding)
-    float *pen = cn + Kp;  // [Kp] +inf where a group opens, else 0
+    int32_t *gtab = reinterpret_cast<int32_t *>(cn + Kp);  // [Kp] group of each column (padding: the last)
     uint32_t *bm = reinterpret_cast<uint32_t *>(sm + cfg.off_gs);  // [Kp / 32] group-start masks
     float *stage = reinterpret_cast<float *>(sm + cfg.off_stage);  // [2 groups x 128 rows][Gp + 1]
-    float4 *mrg = reinterpret_cast<float4 *>(stage + (size_t)kGroups * kTM * (p.Gp + 1));  // [2 x 128]
+    float4 *t4 = reinterpret_cast<float4 *>(stage + (size_t)kGroups * kTM * (p.Gp + 1));  // one per scanning lane
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + cfg.off_bar);
     const int S = cfg.stages;
     uint64_t *full_a = bars;
@@ -102,10 +111,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * S + 2 * kGroups + 1);
     float *c2max_s = reinterpret_cast<float *>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the broadcast tells the compiler that the warp index is warp-uniform)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int v = ctrl->v;
     const int K = p.K, G = p.G;
 
+    // a tile of points to stage s
+    auto load_tile = [&](int tile, int s) {
+        uint8_t *st = sA + (size_t)s * 2 * NA * kAtomBytes;
+        mbar_arrive_expect_tx(&full_a[s], (uint32_t)(2 * NA * kAtomBytes));
+        for (int a = 0; a < NA; ++a) {
+            tma_2d(st + a * kAtomBytes, &tmh, 64 * a, tile * kTM, &full_a[s]);
+            tma_2d(st + (NA + a) * kAtomBytes, &tml, 64 * a, tile * kTM, &full_a[s]);
+        }
+    };
     if (threadIdx.x == 0) {
         for (int i = 0; i < S; ++i) {
             bar_init(&full_a[i], 1);
@@ -118,6 +137,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         bar_init(mma_done, 1);
         *c2max_s = 0.f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // the first tiles of points, on their way while the centroids are split
+        int s = 0;
+        for (int tile = blockIdx.x; tile < cfg.num_tiles && s < S; tile += gridDim.x, ++s) load_tile(tile, s);
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -126,58 +148,62 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int c = threadIdx.x; c < Kp / 32; c += blockDim.x) bm[c] = 0u;
-    // the centroid block, split into x_h / x_l bfloat16 tiles (128-byte swizzle),
-    // and the exact FP32 norms (padding rows: zero tiles, norm +inf)
-    for (int idx = threadIdx.x; idx < Kp * (D / 8); idx += blockDim.x) {
-        const int row = idx / (D / 8), q = idx - row * (D / 8);
-        float vals[8];
-        if (row < K && q * 8 < p.D) {  // coordinates beyond D: zero padding
-            const float4 a = *reinterpret_cast<const float4 *>(p.C + (size_t)row * p.Dp + q * 8);
-            const float4 b = *reinterpret_cast<const float4 *>(p.C + (size_t)row * p.Dp + q * 8 + 4);
-            vals[0] = a.x; vals[1] = a.y; vals[2] = a.z; vals[3] = a.w;
-            vals[4] = b.x; vals[5] = b.y; vals[6] = b.z; vals[7] = b.w;
-            if (p.mu)  // c - mu (mu's padding columns are zero)
+    // The centroid block, split into x_h / x_l bfloat16 tiles (128-byte swizzle),
+    // and the FP32 norms of the values split (padding rows: zero tiles, norm
+    // +inf).  Eight coordinates per thread, a row on D / 8 neighbouring lanes;
+    // the loads of four rounds go out together, so that every launch pays their
+    // latency once or twice.
+    float cm = 0.f;
+    constexpr int kRounds = 4;
+    for (int i0 = threadIdx.x; i0 < Kp * (D / 8); i0 += kRounds * kTcThreads) {  // (whole warps: Kp D / 8 is a multiple of 32)
+        const int q = i0 % (D / 8);  // the same in every round: kTcThreads is a multiple of D / 8
+        float4 w[kRounds][2], m[2];
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool in = q * 8 < p.D;  // coordinates beyond D: zero padding
 #pragma unroll
-                for (int i = 0; i < 8; ++i) vals[i] = __fsub_rn(vals[i], p.mu[q * 8 + i]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) vals[i] = 0.f;
+        for (int s = 0; s < kRounds; ++s) {
+            const int row = (i0 + s * kTcThreads) / (D / 8);
+            const float4 *c = reinterpret_cast<const float4 *>(p.C + (size_t)min(row, K - 1) * p.Dp + q * 8);
+            w[s][0] = in ? c[0] : zero;
+            w[s][1] = in ? c[1] : zero;
         }
-        uint4 h, l;
-        split8(vals, h, l);
-        *reinterpret_cast<uint4 *>(sBh + swz_chunk(row, q, b_atom)) = h;
-        *reinterpret_cast<uint4 *>(sBl + swz_chunk(row, q, b_atom)) = l;
+        const float4 *mu = reinterpret_cast<const float4 *>(p.mu + q * 8);  // (mu's padding columns are zero)
+        m[0] = in && p.mu ? mu[0] : zero;
+        m[1] = in && p.mu ? mu[1] : zero;
+#pragma unroll
+        for (int s = 0; s < kRounds; ++s) {
+            const int row = (i0 + s * kTcThreads) / (D / 8);
+            if (row >= Kp) break;  // warp-uniform
+            const bool real = row < K;
+            float vals[8] = {__fsub_rn(w[s][0].x, m[0].x), __fsub_rn(w[s][0].y, m[0].y), __fsub_rn(w[s][0].z, m[0].z),
+                             __fsub_rn(w[s][0].w, m[0].w), __fsub_rn(w[s][1].x, m[1].x), __fsub_rn(w[s][1].y, m[1].y),
+                             __fsub_rn(w[s][1].z, m[1].z), __fsub_rn(w[s][1].w, m[1].w)};
+            float ss = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                vals[k] = real ? vals[k] : 0.f;
+                ss = fmaf(vals[k], vals[k], ss);
+            }
+            uint4 h, l;
+            split8(vals, h, l);
+            *reinterpret_cast<uint4 *>(sBh + swz_chunk(row, q, b_atom)) = h;
+            *reinterpret_cast<uint4 *>(sBl + swz_chunk(row, q, b_atom)) = l;
+#pragma unroll
+            for (int o = D / 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            if (q == 0) {
+                cn[row] = real ? ss : INFINITY;
+                gtab[row] = real ? p.grp[row] : G - 1;
+            }
+            if (real) cm = fmaxf(cm, ss);
+        }
     }
-    {
-        float cm = 0.f;
-        for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
-            float s2 = INFINITY;
-            if (k < K) {
-                const float *c = p.C + (size_t)k * p.Dp;
-                float a0 = 0.f, a1 = 0.f;
-                for (int d = 0; d + 1 < p.D; d += 2) {  // ||c - mu||^2, the values split above
-                    const float v0 = p.mu ? __fsub_rn(c[d], p.mu[d]) : c[d];
-                    const float v1 = p.mu ? __fsub_rn(c[d + 1], p.mu[d + 1]) : c[d + 1];
-                    a0 = fmaf(v0, v0, a0);
-                    a1 = fmaf(v1, v1, a1);
-                }
-                s2 = a0 + a1;
-                cm = fmaxf(cm, s2);
-            }
-            cn[k] = s2;
-            pen[k] = 0.f;
-        }
-        cm = warp_max(cm);
-        __syncthreads();  // c2max_s and the masks initialised
-        if (lane == 0 && cm > 0.f) atomicMax(reinterpret_cast<int *>(c2max_s), __float_as_int(cm));
-        // group g >= 1 starts at column gstart[g] (< K <= Kp)
-        for (int g = 1 + threadIdx.x; g < G; g += blockDim.x) {
-            const int col = p.gstart[g];
-            if ((unsigned)col < (unsigned)Kp) {
-                atomicOr(&bm[col >> 5], 1u << (col & 31));
-                pen[col] = INFINITY;
-            }
-        }
+    cm = warp_max(cm);
+    __syncthreads();  // c2max_s and the masks initialised
+    if (lane == 0 && cm > 0.f) atomicMax(reinterpret_cast<int *>(c2max_s), __float_as_int(cm));
+    // group g >= 1 starts at column gstart[g] (< K <= Kp)
+    for (int g = 1 + threadIdx.x; g < G; g += blockDim.x) {
+        const int col = p.gstart[g];
+        if ((unsigned)col < (unsigned)Kp) atomicOr(&bm[col >> 5], 1u << (col & 31));
     }
     // generic-proxy writes of the B tiles must be visible to the tensor cores
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -189,20 +215,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (warp == 0) {
         // ------------------------------------------------------------ TMA
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmh) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tml) : "memory");
             int i = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < cfg.num_tiles && ok; tile += gridDim.x, ++i) {
                 const int s = i % S, f = i / S;
-                if (f > 0) ok = bar_wait(&empty_a[s], (f - 1) & 1, ctrl);
+                if (f == 0) continue;  // (issued above)
+                ok = bar_wait(&empty_a[s], (f - 1) & 1, ctrl);
                 if (!ok) break;
-                uint8_t *st = sA + (size_t)s * 2 * NA * kAtomBytes;
-                mbar_arrive_expect_tx(&full_a[s], (uint32_t)(2 * NA * kAtomBytes));
-                for (int a = 0; a < NA; ++a) {
-                    tma_2d(st + a * kAtomBytes, &tmh, 64 * a, tile * kTM, &full_a[s]);
-                    tma_2d(st + (NA + a) * kAtomBytes, &tml, 64 * a, tile * kTM, &full_a[s]);
-                }
+                load_tile(tile, s);
             }
             // drain: every issued copy has landed before the block can exit
             const int issued = i;
@@ -257,273 +277,214 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
     } else {
         // ------------------------------------------------------- epilogue
-        // Two warps per TMEM lane quadrant and group: half 0 scans the first
-        // half of the accumulator columns and finishes the rows, half 1 scans
-        // the second half; the pair meets at a 64-thread named barrier (1..8).
+        // Two warps per TMEM lane quadrant and group, one lane per row in both:
+        // half 0 scans the first half of the accumulator columns, half 1 the
+        // second.  They meet three times a tile (64-thread named barriers 1..8):
+        // at its start, when half 1's result is in shared memory, and when half
+        // 0's merged result is.  Everything else is each half's own: the group
+        // minima it has scanned (half 0's slots are the group numbers, half 1's
+        // the group numbers plus one), their bounds, and its share of the row.
         const int e = warp - 2;
         const int grp_id = e / kEpiWarps;
         const int half = (e % kEpiWarps) / 4;
-        const int pid = 1 + grp_id * 4 + ((e % kEpiWarps) & 3);
+        const int pid = 1 + grp_id * 4 + (e & 3);
         const int q = warp & 3;  // TMEM lane quadrant of this warp
         const int r = q * 32 + lane;
         const bool bounds = p.algo == KM_ALGO_FILTERED;
         const float c2max = __fmul_ru(*c2max_s, 1.0f + 1.0f / 1024);
         const float cmax = sqrt_hi(c2max);
         const float ec2 = __fmul_ru(cfg.e_c2, c2max);
-        float *row = stage + (size_t)(grp_id * kTM + r) * (p.Gp + 1);  // shared by the pair
-        float4 *mrow = mrg + grp_id * kTM + r;                       // half 1's result for half 0
-        // column chunks of 32: half 0 takes [0, ha), half 1 [ha, nch); half 1's
-        // first store lands in the slot of the group open at its first column's
-        // left neighbour, which half 0 merges with its own last minimum
-        const int nch = Kp >> 5, ha = (nch + 1) >> 1;
-        const int k0 = half ? ha : 0, k1 = half ? nch : ha;
-        const int gsplit = nch > 1 ? group_of(bm, 32 * ha - 1) : 0;
-        unsigned long long c_changed = 0, c_recheck = 0, c_dist = 0;
-        auto write_req = [&](int64_t n, int old, int i1, float xlo, float b1, float E, unsigned long long gmask) {
-            SettleReq rq;
-            rq.n = (int32_t)n;
-            rq.old = old;
-            rq.i1 = i1;
-            // every column is at least b1: when i1 loses, this bounds both i1's
-            // group (which now keeps i1) and the winner's group
-            rq.lb_alt = sqrt_lo(__fsub_rd(__fadd_rd(xlo, b1), E));
-            rq.gmask = gmask;
-            rq.lim = 0.f;
-            p.sreq[n] = rq;
+        const uint32_t row = smem_u32(stage + (size_t)(grp_id * kTM + r) * (p.Gp + 1));  // shared by the pair
+        // halves in steps of 16 columns; the group open across their border has
+        // a part in both
+        const int csplit = ((Kp >> 4) + 1) / 2 * 16;
+        const int c0 = half ? csplit : 0, c1 = half ? Kp : csplit;
+        const int gsplit = __shfl_sync(0xffffffffu, gtab[csplit - 1], 0);
+        // the groups whose bounds this half writes, and the slot of group 0
+        const int glo = half ? gsplit + 1 : 0, ghi = half || gsplit == G - 1 ? G : gsplit + 1;
+        const uint32_t slot0 = row + 4u * half;
+        const uint32_t mine = smem_u32(t4 + e * 32 + lane), other = smem_u32(t4 + (e ^ 4) * 32 + lane);
+        Scan4 sc;
+        sc.row = row;
+        sc.t4 = mine;
+        int c_changed = 0;
+        int64_t c_dist = 0;
+        auto put4 = [](uint32_t at, float x, float y, int z, float w) {
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(x), "f"(y), "f"(__int_as_float(z)), "f"(w)
+                         : "memory");
         };
-        // the lb-row store: this lane's first float4 of a 16-row block and the
-        // step of 32 float4s, as (row, column) pairs
-        const int st_q4 = p.Gp >> 2;
-        const int st_r0 = lane / st_q4, st_g0 = lane - st_r0 * st_q4;
-        const int st_dr = 32 / st_q4, st_dg = 32 - st_dr * st_q4;
+        auto get4 = [](uint32_t at) {
+            float4 v;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
+            return v;
+        };
         int i = grp_id;
         for (int tile = blockIdx.x + grp_id * gridDim.x; tile < cfg.num_tiles;
              tile += kGroups * gridDim.x, i += kGroups) {
             const int u = i / kGroups;
+            const int64_t n = (int64_t)tile * kTM + r;
+            const bool valid = n < p.N;
+            // read now, so that their latency hides behind the wait and the scan
+            const int old = half == 0 && valid && !first ? p.label[n] : -1;
+            const float xn = valid ? p.xnorm[n] : 0.f;
             // waits are warp-uniform (the TMEM loads below are warp-collective)
             // and pair-uniform (the named barriers need both warps)
             const bool ok = __all_sync(0xffffffffu, bar_wait(&acc_full[grp_id], u & 1, ctrl));
             if (!pair_and(ok, pid)) break;
             tc_fence_after();
-            const int64_t n = (int64_t)tile * kTM + r;
-            const bool valid = n < p.N;
-            int old = -1;
-            float xlo = 0.f, xup = 0.f, E = 0.f, xn = 0.f;
-            bool need_row = false;  // half 0: this row's settle request, written after the conversion
-            int best_row = 0;
-            float b1_row = 0.f;
-            if (half == 0) {
-                // the previous label and the row norm, read now so that their
-                // latency hides behind the scan (the error window that needs the
-                // norm is formed after it)
-                old = valid ? (first ? -1 : p.label[n]) : -1;
-                xn = valid ? p.xnorm[n] : 0.f;
-            }
             const uint32_t tb = tmem + (uint32_t)(grp_id * cfg.buf_cols) + ((uint32_t)(q * 32) << 16);
 
-            // pass 1: group minima (staged), winner (lowest index on ties), runner-up
-            // over this half's columns; the next 32 columns are read from TMEM
-            // while the current ones are scanned
-            RowScan A;
-            A.init(half ? row + gsplit : row);
-            if (k0 < k1) {  // 16 columns at a time, the next 16 in flight
-                const int c0 = 32 * k0, c1 = 32 * k1;
+            // group minima, winner (lowest index on ties) and runner-up over this
+            // half's columns, 16 at a time, the next 16 in flight
+            sc.b1 = sc.b2 = sc.gm = INFINITY;
+            sc.c4 = c0;
+            sc.pend = half ? gsplit + 1 : 0;
+            auto sixteen = [&](const uint32_t(&acc)[16], int c) {
+                // (a broadcast, so that the compiler knows the mask to be warp-uniform)
+                const uint32_t m16 = __shfl_sync(0xffffffffu, bm[c >> 5], 0) >> (c & 31);
+                const float4 *cn4 = reinterpret_cast<const float4 *>(cn + c);
+#pragma unroll
+                for (int j = 0; j < 16; j += 4) sc.four(&acc[j], cn4[j >> 2], (m16 >> j) & 15u, c + j);
+            };
+            {
                 uint32_t ra[16], rb[16];
                 tmem_ld16_async(tb + c0, ra);
-                for (int c = c0; c < c1; c += 32) {  // warp-uniform; c1 - c0 is a multiple of 32
+#pragma unroll 1
+                for (int c = c0; c < c1; c += 32) {
                     tmem_wait16(ra);
-                    tmem_ld16_async(tb + c + 16, rb);
-                    scan_one<16>(A, ra, c, cn, pen);
-                    tmem_wait16(rb);
-                    if (c + 32 < c1) tmem_ld16_async(tb + c + 32, ra);
-                    scan_one<16>(A, rb, c + 16, cn, pen);
+                    if (c + 16 < c1) tmem_ld16_async(tb + c + 16, rb);
+                    sixteen(ra, c);
+                    if (c + 16 < c1) {
+                        tmem_wait16(rb);
+                        if (c + 32 < c1) tmem_ld16_async(tb + c + 32, ra);
+                        sixteen(rb, c + 16);
+                    }
                 }
             }
             // accumulators no longer needed
             tc_fence_before();
             __syncwarp();
             if (lane == 0) bar_arrive(&acc_empty[grp_id]);
-            if (half) {
-                if (nch > 1) A.close();
-                float c1, c2;
-                int ci;
-                A.result(c1, ci, c2);
-                *mrow = make_float4(c1, c2, __int_as_float(ci), 0.f);
-            }
-            pair_sync(pid);  // half 1's minima and result are in shared memory
+            // the open group's minimum, and this half's result
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + 4u * (uint32_t)sc.pend), "f"(sc.gm) : "memory");
+            float b1 = sc.b1, b2 = sc.b2;
+            int i1 = sc.winner();
+            if (half) put4(mine, b1, b2, i1, lds_f(slot0 + 4u * (uint32_t)gsplit));
+            pair_sync(pid);
             if (half == 0) {
-                float b1, b2;
-                int i1;
-                {
-                    if (nch > 1) {
-                        const float gmA = A.gm;
-                        row[gsplit] = fminf(row[gsplit], gmA);
-                    } else {
-                        A.close();
-                    }
-                    float a1, a2;
-                    int ai;
-                    A.result(a1, ai, a2);
-                    const float4 m = *mrow;
-                    const float c1 = m.x, c2 = m.y;
-                    const int ci = __float_as_int(m.z);
-                    // half 0 holds the lower indices: it wins ties
-                    const bool bw = c1 < a1;
-                    b1 = bw ? c1 : a1;
-                    i1 = bw ? ci : ai;
-                    b2 = fminf(fminf(a2, c2), fmaxf(a1, c1));
-                }
-                xlo = __fmul_rd(xn, cfg.xn_lo);
-                xup = __fmul_ru(xn, cfg.xn_hi);
-                E = __fmaf_ru(cfg.e_lin, __fmul_ru(sqrt_hi(xup), cmax), ec2);
-                const float R = __fadd_ru(sqrt_hi(xup), cmax);  // bounds ||x - mu|| + ||c - mu||
-                E = __fmaf_ru(p.e_cen, __fmul_ru(R, R), E);
-                const float twoE = __fmul_ru(2.f, E);
-                const float thr = __fadd_ru(b1, twoE);
-
-                // Rows whose runner-up is inside the error window go to the settle
-                // queue: k_settle decides them exactly afterwards from FP32 (and
-                // FP64) distances to the centroids of the groups whose minimum lies
-                // in the window (every other centroid is strictly farther than the
-                // tensor-core winner i1, which is among them).  The epilogue writes
-                // such a row's bounds as if the tensor-core winner i1 won; k_settle
-                // corrects them when it does not.
-                const bool need = valid && b2 <= thr;
-                need_row = bounds && need;
-                best_row = i1;
-                b1_row = b1;
-                {
-                    const unsigned nm = __ballot_sync(0xffffffffu, need);
-                    // The groups that can hold a window column: group minimum
-                    // within the window (at most 64 groups; more: all of them).
-                    // With bounds, the pair tests its halves of the groups while
-                    // converting them, and half 0 writes the request afterwards.
-                    if (nm && !bounds) {
-                        unsigned long long gmask = ~0ull;
-                        if (G <= 64) {
-                            gmask = 0ull;
-                            for (int g = 0; g < G; ++g) gmask |= (row[g] <= thr) ? (1ull << g) : 0ull;
-                        }
-                        if (need) write_req(n, old, i1, xlo, b1, E, gmask);
-                    }
-                    // the warp's 32 rows in the request bitmap (every word is written
-                    // by every dense pass, so the bitmap needs no clearing)
-                    if (lane == 0) p.sbits[(int64_t)tile * (kTM / 32) + q] = nm;
-                }
-
-                const int best = i1;
-                if (valid) {
-                    c_dist += (unsigned long long)K;
-                    if (!need) p.label[n] = best;
-                    if (bounds) {
-                        // the winner's group must exclude the winner: every other
-                        // column is at least the runner-up b2 (at least b1 when the
-                        // exact winner is not the tensor-core winner); staged in t
-                        // and converted with the other groups below
-                        const float tw = best == i1 ? b2 : b1;
-                        const float lw = tw == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xlo, tw), E));
-                        row[group_of(bm, best)] = tw;
-                        // the bound is monotone in t, so the smallest group bound is
-                        // the bound of the smallest column other than the winner
-                        p.lbg[n] = lw;
-                        p.u[n] = sqrt_hi(__fadd_ru(__fadd_ru(xup, b1), E));
-                        p.stamp[n] = make_stamp(v, v);
-                    }
-                }
-                *mrow = make_float4(xlo, E, thr, 0.f);  // for half 1's share of the conversion
-                {
-                    // label changes: one slot reservation per warp
-                    const bool moved = valid && !need && old != best;
-                    const unsigned mm = __ballot_sync(0xffffffffu, moved);
-                    c_changed += moved ? 1 : 0;
-                    if (mm && !first) {
-                        int base = 0;
-                        if (lane == 0) base = atomicAdd(&ctrl->moved_count, __popc(mm));
-                        base = __shfl_sync(0xffffffffu, base, 0);
-                        if (moved) {
-                            const int slot = base + __popc(mm & ((1u << lane) - 1u));
-                            p.moved[slot] = (int)n;
-                            p.moved_old[slot] = old;
-                        }
-                    }
-                }
+                const float4 m = get4(other);
+                const bool bw = m.x < b1;  // half 0 holds the lower indices: it wins ties
+                b2 = fminf(fminf(b2, m.y), fmaxf(b1, m.x));
+                i1 = bw ? __float_as_int(m.z) : i1;
+                b1 = fminf(b1, m.x);
+                put4(mine, b1, b2, i1, 0.f);
+                const uint32_t at = row + 4u * (uint32_t)gsplit;
+                const float gm = fminf(lds_f(at), m.w);
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(at), "f"(gm) : "memory");
             }
-            pair_sync(pid);  // half 0's winner fixes and (x_lo, E) are in shared memory
+            pair_sync(pid);
+            if (half) {
+                const float4 m = get4(other);
+                b1 = m.x;
+                b2 = m.y;
+                i1 = __float_as_int(m.z);
+            }
+            const float xlo = __fmul_rd(xn, cfg.xn_lo), xup = __fmul_ru(xn, cfg.xn_hi);
+            const float R = __fadd_ru(sqrt_hi(xup), cmax);  // bounds ||x - mu|| + ||c - mu||
+            const float E = __fmaf_ru(p.e_cen, __fmul_ru(R, R), __fmaf_ru(cfg.e_lin, __fmul_ru(sqrt_hi(xup), cmax), ec2));
+            const float thr = __fadd_ru(b1, __fmul_ru(2.f, E));
+            auto bound_of = [&](float t) { return t == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xlo, t), E)); };
+
+            // Rows whose runner-up is inside the error window go to the settle
+            // queue: k_settle decides them exactly afterwards from FP32 (and
+            // FP64) distances to the centroids of the groups whose minimum lies
+            // in the window (every other centroid is strictly farther than the
+            // tensor-core winner i1, which is among them).  The epilogue writes
+            // such a row's bounds as if i1 won; k_settle corrects them when it
+            // does not.
+            const bool need = valid && b2 <= thr;
+            const unsigned nm = __ballot_sync(0xffffffffu, need);
+            const bool moved = half == 0 && valid && !need && old != i1;
+            int mbase = 0;
+            const unsigned mm = __ballot_sync(0xffffffffu, moved);
+            if (half == 0) {
+                // label changes: one slot reservation per warp, used at the end
+                if (mm && !first && lane == 0) mbase = atomicAdd(&ctrl->moved_count, __popc(mm));
+                c_changed += moved;
+                c_dist += valid ? K : 0;
+                // the warp's 32 rows in the request bitmap (every word is written
+                // by every dense pass, so the bitmap needs no clearing)
+                if (lane == 0) p.sbits[(int64_t)tile * (kTM / 32) + q] = nm;
+                if (valid && !need) p.label[n] = i1;
+            }
+            // this half's groups that can hold a window column (at most 64
+            // groups; more: all of them), before the winner's own is replaced
+            unsigned long long gmask = G <= 64 ? 0ull : ~0ull;
+            if (nm && G <= 64)
+                for (int g = glo; g < ghi; ++g)
+                    gmask |= lds_f(slot0 + 4u * (uint32_t)g) <= thr ? 1ull << g : 0ull;
             if (bounds) {
-                // s_c >= xn_lo + t_c - E for every column c: the pair converts the
-                // row's group minima, half 0 the first half of the groups
-                // and each half marks its groups whose minimum is within the
-                // window (bit g - g0; the winner's group holds tw = b2 <= thr)
-                const int gh = (G + 1) >> 1;
-                uint32_t gbits = 0u;
-                if (valid) {
-                    const float4 xe = *mrow;
-                    const int g0 = half ? gh : 0, g1 = half ? G : gh;
-                    if (G <= 64) {  // gh <= 32: one 32-bit word per half
-#pragma unroll 4
-                        for (int g = g0; g < g1; ++g) {
-                            const float tg = row[g];
-                            gbits |= (tg <= xe.z ? 1u : 0u) << (g - g0);
-                            row[g] = tg == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xe.x, tg), xe.y));
-                        }
-                    } else {
-#pragma unroll 4
-                        for (int g = g0; g < g1; ++g) {
-                            const float tg = row[g];
-                            row[g] = tg == INFINITY ? INFINITY : sqrt_lo(__fsub_rd(__fadd_rd(xe.x, tg), xe.y));
-                        }
+                // the winner's group must exclude the winner: every other column
+                // is at least the runner-up b2.  The bound is monotone in t, so the
+                // smallest group bound is the bound of the runner-up.
+                const int gb = gtab[i1];
+                if (gb >= glo && gb < ghi)
+                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(slot0 + 4u * (uint32_t)gb), "f"(b2) : "memory");
+                if (half && valid) {
+                    p.lbg[n] = bound_of(b2);
+                    p.u[n] = sqrt_hi(__fadd_ru(__fadd_ru(xup, b1), E));
+                    p.stamp[n] = make_stamp(v, v);
+                }
+                // s_c >= xn_lo + t_c - E for every column c: the bounds of the
+                // groups, four at a time to the row (the four that both halves
+                // have a part of one by one; the padding with the last group)
+                float *lbrow = p.lb + n * p.Gp;
+                for (int g = glo & ~3; g < ghi; g += 4) {
+                    float o[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int gk = min(max(g + k, glo), ghi - 1);
+                        o[k] = g + k < G ? bound_of(lds_f(slot0 + 4u * (uint32_t)gk)) : 0.f;
                     }
-                    if (half) row[p.Gp] = __uint_as_float(gbits);  // the slot past the groups
-                }
-                pair_sync(pid);  // the rows' bounds and half 1's group bits are complete
-                if (half == 0 && need_row) {
-                    const unsigned long long gmask =
-                        G <= 64 ? ((unsigned long long)gbits | ((unsigned long long)__float_as_uint(row[p.Gp]) << gh))
-                                : ~0ull;
-                    write_req(n, old, best_row, xlo, b1_row, E, gmask);
-                }
-                // the quadrant's 32 rows (consecutive points) as one contiguous
-                // block, half 0 the first 16 rows, half 1 the rest
-                const int64_t n0 = (int64_t)tile * kTM + q * 32;
-                const int rows = (int)min((int64_t)32, p.N - n0);
-                const int r0 = half * 16, r1 = min(rows, r0 + 16);
-                if (r1 > r0) {
-                    // rows x Gp floats, contiguous in lb: 16-byte stores (Gp is a
-                    // multiple of 4, so no vector crosses a row); lane-strided
-                    // element e = rw * q4 + gq, (rw, gq) stepped without division
-                    const int Gp = p.Gp;
-                    const float *st0 = stage + (size_t)(grp_id * kTM + q * 32) * (Gp + 1);
-                    float4 *dst = reinterpret_cast<float4 *>(p.lb + n0 * Gp);
-                    for (int rw = r0 + st_r0, gq = st_g0; rw < r1;) {
-                        const int g = gq * 4;
-                        const float *src = st0 + rw * (Gp + 1) + g;
-                        float4 v4;
-                        v4.x = g < G ? src[0] : 0.f;
-                        v4.y = g + 1 < G ? src[1] : 0.f;
-                        v4.z = g + 2 < G ? src[2] : 0.f;
-                        v4.w = g + 3 < G ? src[3] : 0.f;
-                        dst[rw * st_q4 + gq] = v4;
-                        rw += st_dr;
-                        gq += st_dg;
-                        if (gq >= st_q4) {
-                            gq -= st_q4;
-                            ++rw;
+                    if (valid) {
+                        if (g >= glo && (g + 4 <= ghi || ghi == G)) {  // warp-uniform
+                            *reinterpret_cast<float4 *>(lbrow + g) = make_float4(o[0], o[1], o[2], o[3]);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                if (g + k >= glo && (g + k < ghi || ghi == G)) lbrow[g + k] = o[k];
                         }
                     }
                 }
             }
-            pair_sync(pid);  // the row slots are free for the pair's next tile
+            if (need) {
+                SettleReq *rq = p.sreq + n;
+                rq->gmask[half] = gmask;
+                if (half == 0) {
+                    rq->n = (int32_t)n;
+                    rq->old = old;
+                    rq->i1 = i1;
+                    // every column is at least b1: when i1 loses, this bounds both i1's
+                    // group (which now keeps i1) and the winner's group
+                    rq->lb_alt = bound_of(b1);
+                    rq->lim = 0.f;
+                }
+            }
+            if (mm && !first) {
+                mbase = __shfl_sync(0xffffffffu, mbase, 0);
+                if (moved) {
+                    const int slot = mbase + __popc(mm & ((1u << lane) - 1u));
+                    p.moved[slot] = (int)n;
+                    p.moved_old[slot] = old;
+                }
+            }
         }
+        c_changed = __reduce_add_sync(0xffffffffu, c_changed);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            c_changed += __shfl_xor_sync(0xffffffffu, c_changed, o);
-            c_recheck += __shfl_xor_sync(0xffffffffu, c_recheck, o);
-            c_dist += __shfl_xor_sync(0xffffffffu, c_dist, o);
-        }
+        for (int o = 16; o > 0; o >>= 1) c_dist += __shfl_xor_sync(0xffffffffu, c_dist, o);
         if (lane == 0) {
-            if (c_changed) atomicAdd(&ctrl->n_changed, c_changed);
-            if (c_recheck) atomicAdd(&ctrl->n_recheck, c_recheck);
-            if (c_dist) atomicAdd(&ctrl->n_dist, c_dist);
+            if (c_changed) atomicAdd(&ctrl->n_changed, (unsigned long long)c_changed);
+            if (c_dist) atomicAdd(&ctrl->n_dist, (unsigned long long)c_dist);
         }
     }
     tc_fence_before();
@@ -595,11 +556,14 @@ bool plan(const Params &p, size_t smem_limit, TcCfg &cfg, size_t &smem) {
     const size_t NA = Dt / 64;
     const size_t b_bytes = 2 * NA * (size_t)cfg.Kp * 128;
     const size_t a_stage = 2 * NA * (size_t)kAtomBytes;
-    const size_t cn_bytes = (size_t)cfg.Kp * 8;  // norms and group-opening penalties
+    const size_t cn_bytes = (size_t)cfg.Kp * 8;  // norms and groups of the columns
     const size_t gs_bytes = (((size_t)cfg.Kp / 32) * 4 + 15) & ~size_t(15);  // group-start masks
-    const size_t stage_bytes = (size_t)kGroups * kTM * (p.Gp + 1) * 4 + (size_t)kGroups * kTM * 16;
+    // the rows' minima, and 16 bytes per scanning lane.  A shape is taken when two
+    // stages of points fit beside half of those; at the border one stage is left.
+    const size_t rows_bytes = (size_t)kGroups * kTM * (p.Gp + 1) * 4, lane_bytes = (size_t)kGroups * kEpiWarps * 32 * 16;
+    const size_t stage_bytes = rows_bytes + lane_bytes;
     const size_t fixed = 1024 + b_bytes + cn_bytes + gs_bytes + stage_bytes + 64 * 8 + 64;
-    if (fixed + 2 * a_stage > smem_limit) return false;
+    if (fixed - lane_bytes / 2 + 2 * a_stage > smem_limit) return false;
     cfg.stages = (int)std::min<size_t>(6, (smem_limit - fixed) / a_stage);
     size_t off = b_bytes;
     cfg.off_A = (uint32_t)off;

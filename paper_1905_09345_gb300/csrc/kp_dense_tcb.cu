@@ -54,100 +54,6 @@ struct TcbCfg {
     float e_lin, e_c2, xn_lo, xn_hi;
 };
 
-__device__ __forceinline__ unsigned long long pack_f2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-
-__device__ __forceinline__ float min3(float a, float b, float c) {
-    float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
-// Running scan of one row over an ascending run of accumulator columns, four
-// at a time: the smallest value and the runner-up from the sorted pairs of the
-// four, the winner as the index of its group of four (whose values the lane
-// keeps in shared memory, from which the column is read off at the end), and
-// the open group's minimum.  A group boundary among the four columns (the
-// same for every row) closes the minimum into the row's next staging slot.
-// The stores carry no memory clobber, so that the scan's loads may move
-// across them; what they wrote is read back by volatile accesses only.
-struct Scan4 {
-    float b1, b2, gm;
-    int c4;        // first column of the four that hold b1
-    uint32_t row;  // staging slots of the row
-    uint32_t t4;   // the lane's four values
-    int pend;      // closed minima staged (warp-uniform)
-
-    __device__ __forceinline__ void four(const uint32_t *acc, const float4 &cn, uint32_t nib, int c) {
-        unsigned long long t01, t23;
-        const unsigned long long m2 = 0xc0000000c0000000ull;  // (-2, -2)
-        asm("fma.rn.f32x2 %0, %1, %2, %3;"
-            : "=l"(t01)
-            : "l"(pack_f2(__uint_as_float(acc[0]), __uint_as_float(acc[1]))), "l"(m2), "l"(pack_f2(cn.x, cn.y)));
-        asm("fma.rn.f32x2 %0, %1, %2, %3;"
-            : "=l"(t23)
-            : "l"(pack_f2(__uint_as_float(acc[2]), __uint_as_float(acc[3]))), "l"(m2), "l"(pack_f2(cn.z, cn.w)));
-        float t[4];
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[0]), "=f"(t[1]) : "l"(t01));
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[2]), "=f"(t[3]) : "l"(t23));
-        const float l0 = fminf(t[0], t[1]), h0 = fmaxf(t[0], t[1]);
-        const float l1 = fminf(t[2], t[3]), h1 = fmaxf(t[2], t[3]);
-        const float m = fminf(l0, l1);
-        const float s = min3(fmaxf(l0, l1), h0, h1);  // the second smallest of the four
-        b2 = min3(b2, s, fmaxf(b1, m));
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %6, %7;\n\t@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t"
-            "selp.s32 %0, %8, %0, p;\n\t}"
-            : "+r"(c4)
-            : "r"(t4), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(m), "f"(b1), "r"(c));
-        b1 = fminf(b1, m);
-        if (nib == 0) {
-            gm = fminf(gm, m);
-        } else {  // (branches on nib are warp-uniform)
-            auto close = [&](float v) {
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + 4u * (uint32_t)pend), "f"(v));
-                ++pend;
-            };
-            if (nib & 1u) {
-                close(gm);
-                gm = INFINITY;
-            }
-            if (nib & 2u) {
-                close(fminf(gm, t[0]));
-                gm = t[1];
-            } else {
-                gm = fminf(gm, l0);
-            }
-            if (nib & 4u) {
-                close(gm);
-                gm = INFINITY;
-            }
-            if (nib & 8u) {
-                close(fminf(gm, t[2]));
-                gm = t[3];
-            } else {
-                gm = fminf(gm, l1);
-            }
-        }
-    }
-    // the winner's column (lowest among equal values)
-    __device__ __forceinline__ int winner() const {
-        float t0, t1, t2, t3;
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t0), "=f"(t1), "=f"(t2), "=f"(t3) : "r"(t4));
-        if (b1 == INFINITY) return c4;
-        return c4 + (t0 == b1 ? 0 : (t1 == b1 ? 1 : (t2 == b1 ? 2 : 3)));
-    }
-};
-
-__device__ __forceinline__ float lds_f(uint32_t a) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
-    return v;
-}
-
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
     k_dense_tcb(const __grid_constant__ CUtensorMap tmh, const __grid_constant__ CUtensorMap tml,
@@ -532,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 rq.old = old;
                 rq.i1 = i1;
                 rq.lb_alt = sqrt_lo(__fsub_rd(__fadd_rd(xlo, b1), E));
-                rq.gmask = 0ull;
+                rq.gmask[0] = rq.gmask[1] = 0ull;
                 rq.lim = sqrt_hi(__fsub_ru(__fadd_ru(xup, thr), E));
                 p.sreq[n] = rq;
             }

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int firs
         mine.old = -1;
         mine.i1 = 0;
         mine.lb_alt = mine.lim = 0.f;
-        mine.gmask = 0ull;
+        mine.gmask[0] = mine.gmask[1] = 0ull;
         if (lane < cnt) {
             const int n = p.squeue[r0 + lane];
             if (n >= 0 && n < p.N) mine = p.sreq[n];
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int firs
             const int n = __shfl_sync(full, mine.n, from), old = __shfl_sync(full, mine.old, from);
             const int w1 = __shfl_sync(full, mine.i1, from);
             const float lim = __shfl_sync(full, mine.lim, from), lb_alt = __shfl_sync(full, mine.lb_alt, from);
-            const unsigned long long gmask = __shfl_sync(full, mine.gmask, from);
+            const unsigned long long gmask = __shfl_sync(full, mine.gmask[0] | mine.gmask[1], from);
             const bool act = n >= 0;
             const int64_t row = act ? n : 0;
             ulonglong2 xv[NC];

@@ -1,7 +1,7 @@
 // kp_tc.cuh -- pieces shared by the tensor-core dense kernels: mbarrier and
 // TMA helpers, tcgen05 descriptors and TMEM loads, the bfloat16 split, the
-// 128-byte-swizzled tile layout, and the branch-free row scan of the
-// epilogue (group minima, winner, runner-up).
+// 128-byte-swizzled tile layout, and the row scan of the epilogue (group
+// minima, winner, runner-up).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -110,76 +110,98 @@ __device__ __forceinline__ void split8(const float *v, uint4 &h, uint4 &l) {
     h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
     l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
-// Running scan of one row over a run of accumulator columns: the per-group
-// minima (stored into the row's shared-memory slots as each group closes),
-// and the smallest value with its index and the runner-up, in two independent
-// chains (even and odd columns).  Branch-free: pen[c] is +inf where column c
-// opens a group (0 elsewhere), so that gm + pen restarts the running minimum,
-// and the closing minimum is stored by a predicated shared store.  A row is
-// scanned as two such runs (the two halves of its columns) interleaved column
-// by column, for instruction-level parallelism; merge() joins them.
-struct RowScan {
-    float b1[2], b2[2];
-    int i1[2];
-    float gm;     // minimum of the open group
-    uint32_t rp;  // shared-memory address of the open group's slot
+__device__ __forceinline__ unsigned long long pack_f2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
 
-    __device__ __forceinline__ void init(const float *slot) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            b1[c] = INFINITY;
-            b2[c] = INFINITY;
-            i1[c] = 0;  // kept when no column is below +inf (then column 0)
-        }
-        gm = INFINITY;
-        rp = smem_u32(slot);
-    }
-    __device__ __forceinline__ void col(float acc, float cnv, float pen, int c, int jpar) {
-        const float t = fmaf(-2.f, acc, cnv);
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Running scan of one row over an ascending run of accumulator columns, four
+// at a time: the smallest value and the runner-up from the sorted pairs of the
+// four, the winner as the index of its group of four (whose values the lane
+// keeps in shared memory, from which the column is read off at the end), and
+// the open group's minimum.  A group boundary among the four columns (the
+// same for every row) closes the minimum into the row's next slot.
+// The stores carry no memory clobber, so that the scan's loads may move
+// across them; what they wrote is read back by volatile accesses only.
+struct Scan4 {
+    float b1, b2, gm;
+    int c4;        // first column of the four that hold b1
+    uint32_t row;  // slots of the row's group minima
+    uint32_t t4;   // the lane's four values
+    int pend;      // the open group's slot (warp-uniform)
+
+    __device__ __forceinline__ void four(const uint32_t *acc, const float4 &cn, uint32_t nib, int c) {
+        unsigned long long t01, t23;
+        const unsigned long long m2 = 0xc0000000c0000000ull;  // (-2, -2)
+        asm("fma.rn.f32x2 %0, %1, %2, %3;"
+            : "=l"(t01)
+            : "l"(pack_f2(__uint_as_float(acc[0]), __uint_as_float(acc[1]))), "l"(m2), "l"(pack_f2(cn.x, cn.y)));
+        asm("fma.rn.f32x2 %0, %1, %2, %3;"
+            : "=l"(t23)
+            : "l"(pack_f2(__uint_as_float(acc[2]), __uint_as_float(acc[3]))), "l"(m2), "l"(pack_f2(cn.z, cn.w)));
+        float t[4];
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[0]), "=f"(t[1]) : "l"(t01));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[2]), "=f"(t[3]) : "l"(t23));
+        const float l0 = fminf(t[0], t[1]), h0 = fmaxf(t[0], t[1]);
+        const float l1 = fminf(t[2], t[3]), h1 = fmaxf(t[2], t[3]);
+        const float m = fminf(l0, l1);
+        const float s = min3(fmaxf(l0, l1), h0, h1);  // the second smallest of the four
+        b2 = min3(b2, s, fmaxf(b1, m));
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.f32 p, %2, 0f00000000;\n\t@p st.shared.f32 [%0], %1;\n\t"
-            "@p add.u32 %0, %0, 4;\n\t}"
-            : "+r"(rp)
-            : "f"(gm), "f"(pen)
-            : "memory");
-        gm = fminf(__fadd_rn(gm, pen), t);
-        b2[jpar] = fminf(b2[jpar], fmaxf(b1[jpar], t));
-        const bool lt = t < b1[jpar];
-        b1[jpar] = lt ? t : b1[jpar];
-        i1[jpar] = lt ? c : i1[jpar];
+            "{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %6, %7;\n\t@p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t"
+            "selp.s32 %0, %8, %0, p;\n\t}"
+            : "+r"(c4)
+            : "r"(t4), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(m), "f"(b1), "r"(c));
+        b1 = fminf(b1, m);
+        if (nib == 0) {
+            gm = fminf(gm, m);
+        } else {  // (branches on nib are warp-uniform)
+            auto close = [&](float v) {
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(row + 4u * (uint32_t)pend), "f"(v));
+                ++pend;
+            };
+            if (nib & 1u) {
+                close(gm);
+                gm = INFINITY;
+            }
+            if (nib & 2u) {
+                close(fminf(gm, t[0]));
+                gm = t[1];
+            } else {
+                gm = fminf(gm, l0);
+            }
+            if (nib & 4u) {
+                close(gm);
+                gm = INFINITY;
+            }
+            if (nib & 8u) {
+                close(fminf(gm, t[2]));
+                gm = t[3];
+            } else {
+                gm = fminf(gm, l1);
+            }
+        }
     }
-    // store the open group's minimum
-    __device__ __forceinline__ void close() const {
-        asm volatile("st.shared.f32 [%0], %1;" ::"r"(rp), "f"(gm) : "memory");
-    }
-    // winner (lowest index among equal values) and runner-up of both chains
-    __device__ __forceinline__ void result(float &w1, int &wi, float &w2) const {
-        const bool odd = b1[1] < b1[0] || (b1[1] == b1[0] && i1[1] < i1[0]);
-        w1 = odd ? b1[1] : b1[0];
-        wi = odd ? i1[1] : i1[0];
-        w2 = fminf(fminf(b2[0], b2[1]), fmaxf(b1[0], b1[1]));
+    // the winner's column (lowest among equal values)
+    __device__ __forceinline__ int winner() const {
+        float t0, t1, t2, t3;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t0), "=f"(t1), "=f"(t2), "=f"(t3) : "r"(t4));
+        if (b1 == INFINITY) return c4;
+        return c4 + (t0 == b1 ? 0 : (t1 == b1 ? 1 : (t2 == b1 ? 2 : 3)));
     }
 };
 
-template <int W>
-__device__ __forceinline__ void scan_one(RowScan &A, const uint32_t (&ra)[W], int ca, const float *cn,
-                                         const float *pen) {
-#pragma unroll
-    for (int j = 0; j < W; j += 4) {
-        const float4 na = *reinterpret_cast<const float4 *>(cn + ca + j);
-        const float4 pa = *reinterpret_cast<const float4 *>(pen + ca + j);
-        const float nav[4] = {na.x, na.y, na.z, na.w}, pav[4] = {pa.x, pa.y, pa.z, pa.w};
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) A.col(__uint_as_float(ra[j + jj]), nav[jj], pav[jj], ca + j + jj, jj & 1);
-    }
-}
-
-// group of column `col` from the boundary masks (contiguous groups)
-__device__ __forceinline__ int group_of(const uint32_t *bm, int col) {
-    const int c = col >> 5;
-    int g = __popc(bm[c] & ((2u << (col & 31)) - 1u));
-    for (int i = 0; i < c; ++i) g += __popc(bm[i]);
-    return g;
+__device__ __forceinline__ float lds_f(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {

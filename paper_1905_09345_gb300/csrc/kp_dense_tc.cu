@@ -21,7 +21,11 @@
 // each scanning half of the columns) read the accumulators back with
 // tcgen05.ld, one TMEM lane (= point) per thread, and turn
 // t_k = ||c_k||^2 - 2 x.c_k into the winner, the runner-up and the per-group
-// minima, four columns at a time (Scan4 in kp_tc.cuh).
+// minima, four columns at a time (Scan4 in kp_tc.cuh).  Lower bounds are
+// t-based with the error E(x) subtracted, the upper
+// bound adds it; when the runner-up lies within 2E of the winner the point is
+// settled exactly by kp_settle.cu (FP32 direct differences, then FP64 if the
+// FP32 error bound cannot decide), so labels are exact.
 //
 // Bound by the scan: of 200 us for 1,048,576 x 64, K = 256, G = 26, loads,
 // products and TMEM reads alone take 76, the scan 80 (the minima and maxima of
@@ -29,11 +33,6 @@
 // labels 45.  Measured: that pass 226 -> 200 us, 300,007 x 64, K = 200, plain
 // Lloyd, 55 -> 47 (column-by-column scan, rows finished by one of the two
 // halves, a lane per centroid's norm before).
-//
-  Lower bounds are t-based with the error E(x) subtracted, the upper
-// bound adds it; when the runner-up lies within 2E of the winner the point is
-// settled exactly by kp_settle.cu (FP32 direct differences, then FP64 if the
-// FP32 error bound cannot decide), so labels are exact.
 //
 // Error model of t_k (per point; c_max = max ||c_k||, c2_max = max ||c_k||^2):
 //   the split leaves |v - v_h - v_l| <= 2^-16 |v| (bfloat16 unit roundoff

@@ -31,7 +31,9 @@ __device__ __forceinline__ float round_up_f(double x) { return __double2float_ru
 // reduction, each on half of the lanes; and a cluster whose reference point is
 // its centroid (right after the sums were rebuilt) has no terms to add.
 // Measured: K = 16, D = 16: 11.5 -> 9.1 us; K = 100, D = 17: 11.7 -> 9.6; K = 256,
-// D = 64: 14.3 -> 11.9 (eight centroids to a block and three reductions before).
+// D = 64: 14.3 -> 11.9 (eight centroids to a block and three reductions before);
+// 8.1, 8.8 and 9.7 with the last block's inputs read ahead and the drift's root
+// taken in FP32.
 __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_only, int respect_done, int wpb) {
     __shared__ double red_d[kUpdWarps * 32];
     __shared__ float red_f[kUpdWarps];
@@ -43,6 +45,14 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x * wpb + warp;
     const int D = p.D;
+    // what the last block needs of the control block and the groups, read now
+    Ctrl cs;
+    if (threadIdx.x == 0) cs = *ctrl;
+    int gs0 = 0, gs1 = 0;
+    if (threadIdx.x < p.G) {
+        gs0 = p.gstart[threadIdx.x];
+        gs1 = p.gstart[threadIdx.x + 1];
+    }
     if (warp < wpb && k < p.K) {
         const unsigned long long nk = p.cnt[k];
         const double nkd = (double)nk;
@@ -71,10 +81,13 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
         for (int o = 8; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
         if (lane == 0) p.Jk[k] = p.Q[k] + r;
         if (lane == 16 && !final_only) {
-            // sqrt of an FP64 sum of D squares: relative error below
-            // (D + 4) 2^-53; inflate by that, then round up to FP32
-            const double dk = sqrt(r) * (1.0 + (double)(D + 4) * 1.1102230246251565e-16);
-            const float dlt = round_up_f(dk);
+            // an FP64 sum of D squares: relative error below (D + 4) 2^-53;
+            // inflate by twice that, then the smallest FP32 value whose square
+            // (exact in FP64) reaches it: the root rounded up, or the value below
+            const double dk = r * (1.0 + (double)(D + 4) * 2.220446049250313e-16);
+            float dlt = __fsqrt_ru(round_up_f(dk));
+            const float below = __int_as_float(max(__float_as_int(dlt) - 1, 0));
+            if ((double)below * (double)below >= dk) dlt = below;
             p.delta[k] = dlt;
             p.Dc[(size_t)(v + 1) * p.K + k] = __fadd_ru(p.Dc[(size_t)v * p.K + k], dlt);
         }
@@ -98,7 +111,9 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
     if (!final_only) {
         for (int g = threadIdx.x; g < p.G; g += blockDim.x) {
             float m = 0.f;
-            for (int kk = p.gstart[g]; kk < p.gstart[g + 1]; ++kk) m = fmaxf(m, p.delta[kk]);
+            const bool have = g == (int)threadIdx.x;
+            const int k0 = have ? gs0 : p.gstart[g], k1 = have ? gs1 : p.gstart[g + 1];
+            for (int kk = k0; kk < k1; ++kk) m = fmaxf(m, p.delta[kk]);
             p.Dg[(size_t)(v + 1) * p.Gp + g] = __fadd_ru(p.Dg[(size_t)v * p.Gp + g], m);
             dmax = fmaxf(dmax, m);
         }
@@ -116,17 +131,17 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
     if (threadIdx.x == 0) {
         const double J = jp;
         const float dm = dmax;
-        const int t = ctrl->t;
+        const int t = cs.t;
         kmeans_iter_stats st;
         memset(&st, 0, sizeof(st));
         st.iter = t;
-        st.n_changed = (int64_t)ctrl->n_changed;
-        st.n_survivors = (int64_t)ctrl->n_survivors;
-        st.n_scanned = (int64_t)ctrl->n_scanned;
-        st.n_dist = (int64_t)ctrl->n_dist;
-        st.n_recheck = (int64_t)ctrl->n_recheck;
-        st.path = ctrl->path;
-        st.n_settle = ctrl->settle_count;
+        st.n_changed = (int64_t)cs.n_changed;
+        st.n_survivors = (int64_t)cs.n_survivors;
+        st.n_scanned = (int64_t)cs.n_scanned;
+        st.n_dist = (int64_t)cs.n_dist;
+        st.n_recheck = (int64_t)cs.n_recheck;
+        st.path = cs.path;
+        st.n_settle = cs.settle_count;
         st.objective = J;
         if (final_only) {
             ctrl->jfinal = J;
@@ -135,16 +150,16 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
         } else {
             p.Dm[v + 1] = __fadd_ru(p.Dm[v], dm);
             st.max_drift = (double)dm;
-            ctrl->iters_left -= 1;
-            int stop = ctrl->iters_left <= 0 || st.n_changed == 0 ||
-                       (ctrl->have_jprev && (ctrl->jprev - J) < ctrl->tol * ctrl->jprev);
+            ctrl->iters_left = cs.iters_left - 1;
+            int stop = cs.iters_left <= 1 || st.n_changed == 0 ||
+                       (cs.have_jprev && (cs.jprev - J) < cs.tol * cs.jprev);
             st.done = stop;
             ctrl->done = stop;
             ctrl->jprev = J;
             ctrl->have_jprev = 1;
             ctrl->v = v + 1;
             ctrl->t = t + 1;
-            ctrl->fit_n_iter += 1;
+            ctrl->fit_n_iter = cs.fit_n_iter + 1;
             p.stats[t % kStatsCap] = st;
             if (p.cond) cudaGraphSetConditional((cudaGraphConditionalHandle)p.cond, stop ? 0u : 1u);
         }

@@ -53,7 +53,7 @@ struct Ctrl {
     unsigned long long kernels;  // kernels of this context run on the device
     int32_t settle_count;  // rows queued for the exact settle by the tensor-core pass
     int32_t surv_next;     // next queue entry to hand out in the survivor kernel
-    int32_t stats_full;    // the cluster sums of this iteration are recomputed in full
+    int32_t stats_full;    // how this iteration's cluster sums are made (kp_stats.cu: 1 = from all points)
     uint32_t stats_ticket; // last-block-done counter of k_stats_hist
     int32_t settle_next;   // next settle request to hand out
 };
@@ -390,6 +390,52 @@ __device__ __forceinline__ int checked_label(const Params &p, int64_t n) {
         return -1;
     }
     return k;
+}
+
+// Cluster statistics of one point, by a whole warp, lanes over the coordinates:
+// from cluster `old` (-1: none) to its label.  ||x - R_k||^2 of both clusters is
+// summed as FP32 pairs (exact squares, compensated sums): FP64 arithmetic is
+// slow on these SMs; only the atomics are FP64.
+__device__ __forceinline__ void move_point(const Params &p, int64_t n, int old) {
+    const int lane = threadIdx.x & 31;
+    const int nw = checked_label(p, n);
+    if (nw < 0) return;  // warp-uniform: one point per warp
+    if (old >= p.K) {
+        atomicExch(&p.ctrl->err, kErrLabel);
+        return;
+    }
+    const float *x = p.X + n * p.D;
+    float qh = 0.f, ql = 0.f, oh = 0.f, ol = 0.f;
+    // (x - r)^2 into the pair (h, l): x - r as the exact pair dh + dl, its
+    // square as sq + sqe (exact) plus 2 dh dl + dl^2 (below 2^-47 of it)
+    auto acc = [](float &h, float &l, float xv, float r) {
+        float dh, dl, s, e;
+        two_sum(xv, -r, dh, dl);
+        const float sq = __fmul_rn(dh, dh);
+        const float sqe = __fmaf_rn(dh, dh, -sq);
+        const float cross = __fmaf_rn(__fmul_rn(2.f, dh), dl, __fmul_rn(dl, dl));
+        two_sum(h, sq, s, e);
+        h = s;
+        l = __fadd_rn(l, __fadd_rn(e, __fadd_rn(sqe, cross)));
+    };
+    for (int i = lane; i < p.D; i += 32) {
+        const float xf = __ldg(x + i);
+        acc(qh, ql, xf, p.R[(size_t)nw * p.Dp + i]);
+        if (old >= 0) acc(oh, ol, xf, p.R[(size_t)old * p.Dp + i]);
+        const double xi = (double)xf;
+        atomicAdd(&p.S[(size_t)nw * p.D + i], xi);
+        if (old >= 0) atomicAdd(&p.S[(size_t)old * p.D + i], -xi);
+    }
+    const double q = warp_sum_d((double)qh + (double)ql);
+    const double qo = warp_sum_d((double)oh + (double)ol);
+    if (lane == 0) {
+        atomicAdd(&p.Q[nw], q);
+        atomicAdd(&p.cnt[nw], 1ull);
+        if (old >= 0) {
+            atomicAdd(&p.Q[old], -qo);
+            atomicAdd(&p.cnt[old], ~0ull);  // -1
+        }
+    }
 }
 
 // drift of centroid k between versions w and v (upper bound)

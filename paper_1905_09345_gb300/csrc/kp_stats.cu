@@ -14,6 +14,8 @@
 //     +x under its new label and -x under its old one (the sign in bit 31 of
 //     the entry's id), added to the sums as they stand; the counts change by
 //     the entries' signs.
+// When only a handful of labels changed, k_stats_hist moves those points
+// itself, one atomic per coordinate, and the other two have nothing to do.
 #include "kp_common.cuh"
 
 namespace kp {
@@ -29,6 +31,21 @@ constexpr int kSumMaxPer = 8;                  // coordinates per lane (D <= 256
 __device__ __forceinline__ bool stats_full_rule(const Params &p, int all_points) {
     return all_points || (int64_t)p.ctrl->moved_count * 2 > p.N;
 }
+
+// Few moved points: at most so many, per cluster and in coordinates.  An FP64
+// atomic per coordinate costs less than the sort's three chains of dependent
+// loads as long as the L2 takes them (60 a nanosecond in all, one address about
+// every 40 ns) in the time of one such chain; the bounds keep the worst case,
+// every move between the same two clusters, near 40 us.  Measured, the three
+// kernels of an iteration: 16,384 x 16, K = 16, 25 moved points: 14.6 us sorted,
+// 9.6 moved one by one, but 3,300 moved points 15 sorted and 64 one by one;
+// 200,003 x 17, K = 100, 500 to 800 moved points: 20 sorted, 9 one by one.  Whole
+// fits with 2, 4, 8, 16, 32 points per cluster (48 problems): 15.3, 15.1, 15.0,
+// 15.0, 15.0 ms, sorted always 15.7.
+constexpr int64_t kDirectCoords = 1 << 17;
+constexpr int64_t kDirectPer = 8;
+constexpr int64_t kDirectMax = 1024;
+constexpr int kStatsSorted = 0, kStatsFull = 1, kStatsDirect = 2;  // Ctrl::stats_full
 
 constexpr uint32_t kNegEntry = 0x80000000u;  // entry id bit: subtract the point
 
@@ -59,7 +76,7 @@ __device__ __forceinline__ int64_t stats_entries(const Params &p, bool full) {
     return full ? p.N : 2 * (int64_t)p.ctrl->moved_count;
 }
 
-// Decide the mode; in full mode zero S and Q; count the entries per cluster
+// Decide the mode; move the points if they are few; in full mode zero S and Q; count the entries per cluster
 // (shared-memory histogram when K fits), and let the last block turn the
 // counts into segment offsets (hcur) and, in full mode, the new cluster sizes
 // (cnt).
@@ -71,10 +88,18 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_hist(Params p, int all_
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;
     const bool full = stats_full_rule(p, all_points);
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->stats_full = full ? 1 : 0;
     const int K = p.K, D = p.D;
     const bool local = K <= p.hist_smem_k;
     const int64_t m = full ? 0 : (int64_t)ctrl->moved_count;
+    const bool direct = !full && m <= kDirectMax && m <= kDirectPer * K && m * D <= kDirectCoords;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        ctrl->stats_full = full ? kStatsFull : (direct ? kStatsDirect : kStatsSorted);
+    if (direct) {
+        for (int64_t it = ((int64_t)blockIdx.x * kStatsThreads + threadIdx.x) >> 5; it < m;
+             it += ((int64_t)gridDim.x * kStatsThreads) >> 5)
+            move_point(p, p.moved[it], p.moved_old[it]);
+        return;
+    }
     const int64_t ne = stats_entries(p, full);
     // blocks taking part: one per tile of entries (the others leave at once;
     // few moved points need few blocks)
@@ -145,7 +170,9 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_scatter(Params p, int r
     Ctrl *ctrl = p.ctrl;
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;
-    const bool full = *(volatile int *)&ctrl->stats_full;
+    const int mode = *(volatile int *)&ctrl->stats_full;
+    if (mode == kStatsDirect) return;
+    const bool full = mode == kStatsFull;
     const int64_t m = full ? 0 : (int64_t)ctrl->moved_count;
     const int64_t ne = stats_entries(p, full);
     const int K = p.K;
@@ -213,7 +240,9 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_sum(Params p, int respe
     Ctrl *ctrl = p.ctrl;
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;
-    const bool full = *(volatile int *)&ctrl->stats_full;
+    const int mode = *(volatile int *)&ctrl->stats_full;
+    if (mode == kStatsDirect) return;
+    const bool full = mode == kStatsFull;
     const int64_t ne = stats_entries(p, full);
     const int D = p.D;
     const int lane = threadIdx.x & 31;

@@ -246,6 +246,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 const uint8_t *st = sA + (size_t)s * 2 * NA * kAtomBytes;
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
+                    if (D == 64 && 16 * ks >= p.D) break;  // 32 coordinates: the padding to 64 adds nothing
                     const int a = ks >> 2, j = ks & 3;
                     const uint64_t dah = desc_sw128(smem_u32(st + a * kAtomBytes + j * 32));
                     const uint64_t dal = desc_sw128(smem_u32(st + (NA + a) * kAtomBytes + j * 32));

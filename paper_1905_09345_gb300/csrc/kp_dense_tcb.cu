@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             auto product = [&](uint32_t d_tmem, const uint8_t *sa, const uint8_t *sb, bool fresh) {
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
+                    if (D == 64 && 16 * ks >= p.D) break;  // 32 coordinates: the padding to 64 adds nothing
                     const int a = ks >> 2, jj = ks & 3;
                     const uint64_t da = desc_sw128(smem_u32(sa + a * kAtomBytes + jj * 32));
                     const uint64_t db = desc_sw128(smem_u32(sb + a * kBAtom + jj * 32));

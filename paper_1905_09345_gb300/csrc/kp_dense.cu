@@ -19,13 +19,6 @@ constexpr int kDenseWarps = kDenseThreads / 32;
 constexpr int kDenseTileBytes = 64 * 1024;
 constexpr int kDenseLbBytes = 48 * 1024;
 
-using f32x2 = unsigned long long;  // two FP32 values in one 64-bit register pair
-
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ void fma2_sq(f32x2 &acc, f32x2 d) {
     asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc) : "l"(d));
 }

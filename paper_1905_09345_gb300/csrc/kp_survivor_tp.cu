@@ -41,14 +41,6 @@ constexpr int kTpThreads = 256;
 
 // x is kept as packed pairs of FP32 values: xr[q] holds coordinates
 // 4q .. 4q+3 as two 64-bit registers (low half = lower coordinate)
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(unsigned long long v, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
 __device__ __forceinline__ float hsum2(unsigned long long v) {
     float lo, hi;
     unpack2(v, lo, hi);

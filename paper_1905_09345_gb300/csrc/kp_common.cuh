@@ -538,7 +538,7 @@ cudaError_t launch_bounds_out(const Params &p, cudaStream_t s, float *u, float *
 // and state (kmeanspp_state_bytes()) are scratch; *err_out (host) is set
 // nonzero if a drawn index fell out of range
 cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const double *u, float *C, long long *idx,
-                            double *dmin, unsigned long long *Q, float *ub, unsigned long long *sums, void *state,
+                            double *dmin, unsigned long long *Q, float2 *ub, unsigned long long *sums, void *state,
                             cudaStream_t s, int num_sms, long long *err_out);
 size_t kmeanspp_state_bytes();
 int kmeanspp_chunk_log2(int64_t N);

@@ -22,7 +22,14 @@
 // the new centre is not nearer.  The others are collected per block (FP64
 // costs a warp the same for one lane as for 32) and get their FP64 distance;
 // the conversions of x to FP64, which share that pipe, are made on the integer
-// one.  What is left is one read of X per centre.
+// one.
+//
+// Nor does every point need its FP32 distance: with the nearest centre a(x)
+// kept beside D(x)^2, ||c - a(x)||^2 >= 4 D(x)^2 shows by the triangle
+// inequality that the new centre c is not nearer, from eight bytes of the point
+// and a table of the distances between c and the other centres, which every
+// block makes for itself.  What is left of X to read per centre are the rows
+// near c and those that no centre is near to yet.
 //
 // The weights need no FP64 either: Q(x) = floor(D(x)^2 2^(64 - e0)), 64 bits
 // with 2^e0 > max D^2 at the time e0 was set, is made from the bits of D^2
@@ -38,9 +45,10 @@
 // holding T, then the point in it, copied to the output centroids.  Every
 // block owns a run of chunks.
 // Measured on GB300 (1,048,576 x 32, K = 128): 337 us per centre and 43.9 ms in
-// all with FP64 distances to every point; now 46 us once half a dozen centres
-// stand (21 the read of X, at 6.4 TB/s; 8 the FP64 distances; 8 the draw; 5
-// the launch) and 7.0 ms in all.  3,878 x 100: 45 -> 22 us per centre.
+// all with FP64 distances to every point; 50 us and 6.9 ms with the FP32 filter
+// alone (21 the read of X, 8 the FP64 distances, 8 the draw, 5 the launch);
+// 38 us and 5.4 ms with the bound's filter before it.  3,878 x 100: 45 -> 22 us per
+// centre with the FP32 filter.
 #include <cmath>
 
 #include "kp_common.cuh"
@@ -56,6 +64,7 @@ constexpr int kPPWarps = kPPThreads / 32;
 constexpr int kPPBlocks = 3, kPPU = 8;
 constexpr int kPPSegment = 2048;   // points filtered between two looks at the list
 constexpr int kPPList = 2 * kPPSegment;
+constexpr int kPPTable = 1024;     // centres whose distances to the new one the first filter uses
 constexpr int kPPMaxChunks = 4096; // chunk size: the power of two >= 32 that gives at most so many
 constexpr int kPPBins = 65;        // leading zeros of Q (64: zero)
 constexpr unsigned long long kPPNaN = ~0ull;  // Q of a point whose D^2 is NaN: weight 0
@@ -190,7 +199,8 @@ struct PPArgs {
     int D;
     double *dmin;                 // N: D(x)^2
     unsigned long long *Q;        // N
-    float *ub;                    // N: D(x)^2 rounded up to FP32 (the filter's bound)
+    float2 *ub;                   // N: D(x)^2 rounded up to FP32 (the filters' bound); the nearest
+                                  // centre so far (an int in the second half)
     unsigned long long *sums[2];  // chunk sums of the weights
     int csh;                      // log2 of the chunk size
     long long nb;                 // chunks
@@ -417,7 +427,7 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_quant(PPArgs a) {
             const double d = a.dmin[n];
             const unsigned long long q = quant(d, e0);
             a.Q[n] = q;
-            a.ub[n] = d == d ? __double2float_ru(d) : INFINITY;
+            a.ub[n] = make_float2(d == d ? __double2float_ru(d) : INFINITY, __int_as_float(0));
             s0 += weight(q, k);
             s1 += weight(q, k + 1);
             if (q != kPPNaN) atomicAdd(&hist[bin_of(q)], 1);
@@ -442,15 +452,19 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_quant(PPArgs a) {
 // next.
 template <bool VEC>
 __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int j, int lprl, float eps_lo, float tiny) {
-    extern __shared__ double sd[];  // the centre: FP64 (D), then FP32 padded to a multiple of LPR vectors with zeros
+    // the centre: FP64 (D), then FP32 padded to a multiple of LPR vectors with
+    // zeros; the first filter's table (kPPTable) and list (kPPSegment)
+    extern __shared__ double sd[];
     __shared__ unsigned list[kPPList];
     __shared__ int hist[kPPBins];
-    __shared__ int nlist;
+    __shared__ int nlist, nkept;
     const int D = a.D, LPR = 1 << lprl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *sc = reinterpret_cast<float *>(sd + ((D + 1) & ~1));
     constexpr int W = VEC ? 4 : 1;
     const int nv = D / W;                      // vectors of a row
     const int steps = (nv + LPR - 1) >> lprl;  // vectors per lane
+    float *far = sc + steps * LPR * W;         // what D(x)^2 has to exceed for the new centre to matter
+    unsigned short *kept = reinterpret_cast<unsigned short *>(far + kPPTable);
     {
         const float *c = a.X + a.st->pick * D;
         for (int i = threadIdx.x; i < steps * LPR * W; i += kPPThreads) {
@@ -460,7 +474,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
         }
     }
     if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) nlist = 0;
+    if (threadIdx.x == 0) nlist = nkept = 0;
     const int e0 = a.st->e0, k = a.st->k;
     unsigned long long *sums0 = a.sums[a.st->cur], *sums1 = a.sums[a.st->cur ^ 1];
     const long long c0 = chunk0(a, blockIdx.x), c1 = chunk0(a, blockIdx.x + 1);
@@ -476,22 +490,73 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
     __syncthreads();
 
     const int sub = lane >> lprl, l = lane & (LPR - 1), rows = 32 >> lprl;
+    // a quarter of the squared distances between the new centre and the others,
+    // rounded down with room for the FP64 sums' own error: a point whose D^2 is
+    // no larger is, by the triangle inequality, no nearer to the new centre
+    const int ntab = min(j - 1, kPPTable);
+    for (int g0 = warp * rows; g0 < ntab; g0 += kPPWarps * rows) {  // warp-uniform
+        const int g = g0 + sub;
+        float s = 0.f;
+        for (int t = 0; t < steps; ++t) {
+            const int q = l + (t << lprl);
+            if (g < ntab && q < nv) {
+                if constexpr (VEC) {
+                    const float4 x = *(reinterpret_cast<const float4 *>(a.C + (long long)g * D) + q);
+                    const float4 cc = *reinterpret_cast<const float4 *>(sc + 4 * q);
+                    const float d0 = x.x - cc.x, d1 = x.y - cc.y, d2 = x.z - cc.z, d3 = x.w - cc.w;
+                    s = fmaf(d3, d3, fmaf(d2, d2, fmaf(d1, d1, fmaf(d0, d0, s))));
+                } else {
+                    const float d = a.C[(long long)g * D + q] - sc[q];
+                    s = fmaf(d, d, s);
+                }
+            }
+        }
+        for (int o = LPR >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (l == 0 && g < ntab)
+            far[g] = s < INFINITY ? __fmul_rd(__fsub_rd(__fmul_rd(s, eps_lo), tiny), 0.249997f) : -1.f;
+    }
+    __syncthreads();
     constexpr int U = kPPU;  // row groups in flight
     for (long long q0 = p0; q0 < p1; q0 += kPPSegment) {
         // the filter, on a segment of this block's points
         const int cnt = (int)min((long long)kPPSegment, p1 - q0);
         // (odd centres: the segments and their rows from the end)
         const long long s0 = (j & 1) ? p1 - (q0 - p0) - cnt : q0;
-        for (int g0 = warp * U * rows; g0 < cnt; g0 += kPPWarps * U * rows) {
+        // first by the bound alone, a thread per point
+        {
+            constexpr int kPer = kPPSegment / kPPThreads;
+            float2 b[kPer];
+#pragma unroll
+            for (int v = 0; v < kPer; ++v) {
+                const int i = v * kPPThreads + threadIdx.x;
+                b[v] = i < cnt ? a.ub[s0 + i] : make_float2(-1.f, 0.f);
+            }
+#pragma unroll
+            for (int v = 0; v < kPer; ++v) {
+                const int i = v * kPPThreads + threadIdx.x, c = __float_as_int(b[v].y);
+                const bool keep = i < cnt && !(c < ntab && b[v].x <= far[c]);
+                const unsigned m = __ballot_sync(0xffffffffu, keep);
+                if (m) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&nkept, __popc(m));
+                    at = __shfl_sync(0xffffffffu, at, 0);
+                    if (keep) kept[at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)i;
+                }
+            }
+        }
+        __syncthreads();
+        const int nk = nkept;
+        // then by the FP32 distance
+        for (int g0 = warp * U * rows; g0 < nk; g0 += kPPWarps * U * rows) {
             float s[U], ub[U];
             int r[U];
 #pragma unroll
             for (int v = 0; v < U; ++v) {
                 s[v] = 0.f;
                 r[v] = g0 + v * rows + sub;
-                if (j & 1) r[v] = cnt - 1 - r[v];  // below zero past the end
-                if (r[v] >= cnt) r[v] = -1;
-                ub[v] = l == 0 && r[v] >= 0 ? a.ub[s0 + r[v]] : 0.f;
+                if (j & 1) r[v] = nk - 1 - r[v];  // below zero past the end
+                r[v] = r[v] >= 0 && r[v] < nk ? kept[r[v]] : -1;
+                ub[v] = l == 0 && r[v] >= 0 ? a.ub[s0 + r[v]].x : 0.f;
             }
             for (int t = 0; t < steps; ++t) {
                 const int q = l + (t << lprl);
@@ -541,9 +606,11 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
             }
         }
         __syncthreads();
+        if (threadIdx.x == 0) nkept = 0;
         // the FP64 distances of the points it kept, when they fill the block or
         // the points end
         const int n = nlist;
+        __syncthreads();
         if (n < kPPSegment / 2 && q0 + kPPSegment < p1) continue;  // (room for a whole segment is left)
         for (int i = threadIdx.x; i < n; i += kPPThreads) {
             const long long pt = p0 + list[i];
@@ -552,7 +619,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
             if (m < d || (d != d && m == m)) {
                 const unsigned long long qo = a.Q[pt], qn = quant(m, e0);
                 a.dmin[pt] = m;
-                a.ub[pt] = __double2float_ru(m);
+                a.ub[pt] = make_float2(__double2float_ru(m), __int_as_float(j - 1));
                 a.Q[pt] = qn;
                 const long long b = pt >> a.csh;
                 atomicAdd(&sums0[b], weight(qn, k) - weight(qo, k));  // modulo 2^64
@@ -572,7 +639,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
 }  // namespace
 
 cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const double *u, float *C, long long *idx,
-                            double *dmin, unsigned long long *Q, float *ub, unsigned long long *sums, void *state,
+                            double *dmin, unsigned long long *Q, float2 *ub, unsigned long long *sums, void *state,
                             cudaStream_t s, int num_sms, long long *err_out) {
     PPArgs a;
     a.X = X;
@@ -598,7 +665,8 @@ cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const doubl
     int lprl = 0;
     while ((1 << lprl) < nv && lprl < 5) ++lprl;
     const int steps = (nv + (1 << lprl) - 1) >> lprl;
-    const size_t smem = (size_t)((D + 1) & ~1) * 8 + (size_t)steps * (4u << lprl) * (vec ? 4 : 1);
+    const size_t smem = (size_t)((D + 1) & ~1) * 8 + (size_t)steps * (4u << lprl) * (vec ? 4 : 1) + kPPTable * 4 +
+                        kPPSegment * 2;
     auto step = vec ? k_pp_step<true> : k_pp_step<false>;
     if ((e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
@@ -664,7 +732,7 @@ KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K,
         return fail(KM_ECUDA, "device query failed");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t nb = ((N - 1) >> kmeanspp_chunk_log2(N)) + 1;
-    float *ub = nullptr;
+    float2 *ub = nullptr;
     double *dmin = nullptr, *ud = nullptr;
     unsigned long long *bsum = nullptr, *Q = nullptr;
     void *st = nullptr;
@@ -673,7 +741,7 @@ KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K,
     long long err = 0;
     cudaError_t e = pool_alloc(dev, reinterpret_cast<void **>(&dmin), (size_t)N * 8, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&Q), (size_t)N * 8, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ub), (size_t)N * 4, s);
+    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ub), (size_t)N * 8, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&bsum), (size_t)nb * 16, s);
     if (e == cudaSuccess) e = pool_alloc(dev, &st, kmeanspp_state_bytes(), s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ud), (size_t)K * 8, s);

@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_scatter(Params p, int r
 // 512 bytes) and summed before the next is asked for.  The run's ids are in
 // registers before its first batch, so that a batch waits for its rows only, and
 // two coordinates of a lane go through the arithmetic together (f32x2).
-// Measured, all points: 1,048,576 x 64: 139 -> 115 us; 300,007 x 64: 54 -> 40;
+// Measured, all points: 1,048,576 x 64: 139 -> 105 us; 300,007 x 64: 54 -> 37;
 // 4,194,304 x 128: 900 -> 670.  A ring of rows in shared memory, seven ahead, with
 // a rolled loop over the points measured 157, 54 and 900.
 // The same operations on one value and on two (kp_common.cuh)

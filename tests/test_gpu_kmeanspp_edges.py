@@ -69,3 +69,19 @@ def test_far_from_origin_and_subnormal(kp):
     Y[::3, 0] = 0.0
     check(kp, Y, 50, seed=3)
     check(kp, np.zeros((500, 3), np.float32), 20, seed=4)  # every weight zero
+
+
+@pytest.mark.parametrize("N,D,K", [(6000, 3, 1100), (5000, 20, 400), (70000, 32, 64)])
+@pytest.mark.parametrize("kind", ["blobs", "line", "copies"])
+def test_bound_alone(kp, N, D, K, kind):
+    """The filter by the bound alone where it skips nearly everything, more
+    centres than its table holds, points and centres on a line (the triangle
+    inequality holds with equality there) and many copies of few points."""
+    rng = np.random.default_rng(N + D)
+    if kind == "blobs":
+        X = rng.normal(size=(50, D))[rng.integers(0, 50, size=N)] * 100.0 + rng.normal(size=(N, D))
+    elif kind == "line":
+        X = rng.integers(0, 4096, size=(N, 1)) * np.ones((1, D))
+    else:
+        X = rng.integers(-2, 3, size=(max(K // 2, 2), D))[rng.integers(0, max(K // 2, 2), size=N)]
+    check(kp, X.astype(np.float32), K, seed=K)

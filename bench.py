@@ -623,7 +623,7 @@ def run_ours(args):
     near = {"n_recheck_total": int(sum(s_["n_recheck"] for s_ in stats) + fstats["n_recheck"]),
             "n_settle_total": int(sum(s_["n_settle"] for s_ in stats) + fstats["n_settle"]),
             "per_iteration_n_recheck": [s_["n_recheck"] for s_ in stats],
-            "what": "n_recheck: points whose label was settled in FP64 (the FP32 error bound could not "
+            "what": "n_recheck: points whose label was settled beyond FP32 (the FP32 error bound could not "
                     "order their two nearest centroids); n_settle: rows the tensor-core pass sent to the "
                     "exact settle.  Labels are exact for all of them."}
     e2e = {"value": e2e_value, "unit": UNIT,

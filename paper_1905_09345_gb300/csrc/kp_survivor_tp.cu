@@ -482,7 +482,6 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2)
                     rc_best = w;
                     rc_s = sw;
                     rc_lbg = lg;
-                    c_dist = c_dist0 + (unsigned long long)K;  // evaluated against all K: K, not scan + K
                 }
             }
         }
@@ -492,6 +491,7 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2)
             p.label[n] = rc_best;
             p.stamp[n] = make_stamp(v, v);
             moved = rc_best != a;
+            c_dist = c_dist0 + (unsigned long long)K;  // counted as K, not scan + K, however it was settled
             c_recheck += 1;
         }
         // moved points: one atomic per warp for the list slots

@@ -186,7 +186,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                             // the block's norms.  Their slot was last read for this half's
                             // block four uses ago; the slot of c_h just waited for (at most
                             // two blocks back) was multiplied after the scan of this half's
-                            // block three uses ago had released its accumulators.
+                            // block three uses ago had released its accumulators, and a warp
+                            // that releases one block has read the one before (a second
+                            // tile without a successor: see `late` below).
                             uint64_t *cb = &cn_full[h * kCnSlots + (uh[h] & (kCnSlots - 1))];
                             mbar_arrive_expect_tx(cb, kNB * 4);
                             tma_bulk_g2s(cnr + (h * kCnSlots + (uh[h] & (kCnSlots - 1))) * kNB, p.cnorm + j * kNB,
@@ -252,8 +254,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tc_fence_after();
                         const uint8_t *sb = sB + (size_t)bs * NA * kBAtom;
                         if (part == 0 && uses > 0) {
-                            // the (tile, half) buffers are scanned; at a pair's start also a
-                            // missing second tile's, whose last scan may still read the norms
+                            // the (tile, half) buffers are read; at a pair's start also a
+                            // missing second tile's, whose last release follows its last
+                            // read of the norms
                             for (int g = 0; g < (k < 2 ? 2 : ng) && ok; ++g)
                                 ok = bar_wait(&acc_empty[g * 2 + h], (uses - 1) & 1, ctrl);
                             if (!ok) break;
@@ -373,6 +376,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                 };
+                // A second tile's warps are not waited for again when the CTA's last pair
+                // lacks it: their last release before that pair says that the block's
+                // norms are read too, so that their slot may be filled again.
+                const bool late = g == 1 && b == nblk - 1 && i + 2 >= ntile;
+                auto release = [&]() {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(&acc_empty[g * 2 + h]);
+                };
                 uint32_t ra[16], rb[16];
                 tmem_ld16_async(tb, ra);
 #pragma unroll 1
@@ -383,13 +395,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem_wait16(rb);
                     if (c0 + 32 < kNB) {
                         tmem_ld16_async(tb + c0 + 32, ra);
-                    } else {  // the accumulators are read: release them
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) bar_arrive(&acc_empty[g * 2 + h]);
+                    } else if (!late) {  // the accumulators are read: release them
+                        release();
                     }
                     sixteen(rb, c0 + 16);
                 }
+                if (late) release();
             }
             if (!ok) break;  // a wait timed out (error recorded)
             // the open group's minimum

@@ -44,3 +44,17 @@ def test_clustered_singletons(kp):  # noqa: F811
         st = lockstep(kp, X, C0, G, 3, algo=algo, check_bounds=algo == kp.KM_ALGO_FILTERED,
                       grouping=kp.KM_GROUP_CLUSTERED)
         assert st[0]["path"] == kp.KM_PATH_DENSE_TC
+
+
+@pytest.mark.parametrize("D,K", [(32, 900), (32, 1025), (128, 900)])
+def test_last_pair_lacks_second_tile(kp, D, K):  # noqa: F811
+    """Three tiles per CTA and four or more centroid blocks per half: the last
+    pair has one tile, and the norms' slots are filled again while nobody waits
+    for the second tile's warps block by block."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    N = 3 * 128 * sms - 77
+    rng = np.random.default_rng(K + D)
+    X, _ = synth.gaussian_mixture(rng, N, D, 64, centre_range=10.0, scale="blob_uniform", scale_args=(0.5, 2.0))
+    C0 = synth.sample_init(rng, X, K)
+    st = lockstep(kp, X, C0, K // 10, 2, algo=kp.KM_ALGO_LLOYD, check_bounds=False)
+    assert all(s["path"] == kp.KM_PATH_DENSE_TC for s in st)

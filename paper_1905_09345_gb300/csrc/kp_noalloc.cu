@@ -258,7 +258,15 @@ __global__ void __launch_bounds__(kSumThreads) k_noalloc_sums(Params p, int segs
                 q.m = __fadd_rn(q.m, e);
                 q.add(h);
             }
-            if (lane == 0) {
+            if (__any_sync(0xffffffffu, !isfinite(q.h))) {  // (as for S; the points' own squares may fit FP32)
+                double t = 0.0;
+                for (int a = from; a < end; ++a) {
+                    const double d = on ? (double)__ldg(p.X + (base + (order[a] & (kSumTile - 1))) * D + i) - (double)ref : 0.0;
+                    t += d * d;
+                }
+                t = warp_sum_d(t);
+                if (lane == 0) atomicAdd(&p.Q[k], t);
+            } else if (lane == 0) {
                 const int at = atomicAdd(&nparts, 1);
                 part[at] = q.h;
                 part[most + at] = q.l;

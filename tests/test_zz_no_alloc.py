@@ -86,3 +86,54 @@ def test_noalloc_step_rejects_oversize_and_host_memory(kp):
     with pytest.raises(kp.KMeansError) as e:  # host memory is refused, not staged
         kp.kmeans_lloyd_step_noalloc(X, 3000, 8, C0, 16, lab, torch.empty(16, 8, device="cuda"), J)
     assert e.value.status == kp.KM_EINVAL
+
+
+def _step_vs_oracle(kp, oracle, X, C0):
+    N, D = X.shape
+    K = C0.shape[0]
+    labels = torch.full((N,), -1, dtype=torch.int32, device="cuda")
+    C_new = torch.empty(K, D, dtype=torch.float32, device="cuda")
+    J = torch.zeros(1, dtype=torch.float64, device="cuda")
+    kp.kmeans_lloyd_step_noalloc(torch.from_numpy(X).cuda(), N, D, torch.from_numpy(C0).cuda(), K, labels, C_new, J)
+    torch.cuda.synchronize()
+    Cin = C0.astype(np.float64)
+    o_lab, _, _, _ = oracle.lloyd_assign(X, Cin)
+    o_C, counts, o_J = oracle.lloyd_update(X, o_lab, Cin)
+    assert np.array_equal(labels.cpu().numpy(), o_lab)
+    a = C_new.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(a - o_C).max(0) <= CENTROID_RTOL * np.maximum(1.0, np.abs(o_C).max(0)))
+    assert abs(J.item() - o_J) <= OBJECTIVE_RTOL * o_J, (J.item(), o_J)
+    return counts
+
+
+# one point; one segment and a second slice; the most clusters and coordinates;
+# several tiles of a segment in four slices and in one
+SUM_SHAPES = [(1, 1, 1), (1500, 33, 7), (5000, 128, 1024), (400003, 100, 50), (1400000, 3, 5)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,D,K", SUM_SHAPES, ids=[f"N{s[0]}_D{s[1]}_K{s[2]}" for s in SUM_SHAPES])
+def test_noalloc_sums(kp, oracle_lib, N, D, K):
+    """Two clusters are empty where there are more than two."""
+    X, C0 = _data(N=N, D=D, K=K, seed=N + D)
+    C0 = C0 + np.float32(0.25)
+    if K > 2:
+        C0[[1, K - 1]] = 1e4
+    counts = _step_vs_oracle(kp, oracle_lib, X, C0)
+    assert K <= 2 or (counts[1] == 0 and counts[K - 1] == 0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["squares17", "squares18", "coordinate"])
+def test_noalloc_sums_beyond_fp32(kp, oracle_lib, kind):
+    """A cluster's sum of squares, or of one coordinate, leaves FP32 while the
+    points and their distances do not: every result is exact all the same."""
+    rng = np.random.default_rng(4)
+    N, D, K = 6000, 64, 4
+    X = rng.normal(size=(N, D))
+    if kind == "coordinate":
+        X[:, 5] = 2e36  # the same for all points: no difference
+    else:
+        X *= 10.0 ** int(kind[-2:])
+    X = X.astype(np.float32)
+    _step_vs_oracle(kp, oracle_lib, X, X[:K].copy())

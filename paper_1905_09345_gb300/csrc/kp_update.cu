@@ -83,11 +83,17 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
         if (lane == 16 && !final_only) {
             // an FP64 sum of D squares: relative error below (D + 4) 2^-53;
             // inflate by twice that, then the smallest FP32 value whose square
-            // (exact in FP64) reaches it: the root rounded up, or the value below
+            // (exact in FP64) reaches it: the root rounded up, or the value
+            // below.  Squares outside FP32's normal range: the FP64 root.
             const double dk = r * (1.0 + (double)(D + 4) * 2.220446049250313e-16);
-            float dlt = __fsqrt_ru(round_up_f(dk));
-            const float below = __int_as_float(max(__float_as_int(dlt) - 1, 0));
-            if ((double)below * (double)below >= dk) dlt = below;
+            float dlt;
+            if (dk == 0.0 || (dk >= 0x1p-126 && dk <= 0x1p127)) {
+                dlt = __fsqrt_ru(round_up_f(dk));
+                const float below = __int_as_float(max(__float_as_int(dlt) - 1, 0));
+                if ((double)below * (double)below >= dk) dlt = below;
+            } else {
+                dlt = round_up_f(__dsqrt_ru(dk));
+            }
             p.delta[k] = dlt;
             p.Dc[(size_t)(v + 1) * p.K + k] = __fadd_ru(p.Dc[(size_t)v * p.K + k], dlt);
         }

@@ -172,8 +172,9 @@ __device__ __forceinline__ bool epi_all(bool v) {
 }
 
 // Programmatic dependent launch: the next kernel of the chain may start its
-// set-up on idle SMs (trigger); it touches nothing that earlier kernels write
-// or read before they have finished (wait).
+// set-up on idle SMs once a thread of every CTA has said so (trigger); it
+// touches nothing that earlier kernels write or read before they have finished
+// (wait).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -209,8 +210,10 @@ __global__ void __launch_bounds__(kMThreads, 1) k_mlp_gemm(const __grid_constant
                      "r"(gb.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        // Only now may the next product's CTAs come: they take TMEM columns and hold
+        // them until this kernel has ended, which it could not if it still needed them.
+        pdl_trigger();
     }
-    pdl_trigger();
     pdl_wait();
     if (g.bias)  // this CTA's columns, zero past the output
         for (int i = threadIdx.x; i < g.nch * g.bn; i += kMThreads) sbias[i] = nb + i < g.N ? g.bias[nb + i] : 0.f;
@@ -1085,7 +1088,6 @@ int plan_add(kmeans_mlp *m, int k, int idx, const GemmSpec &sp, GemmCfg g) {
     int stages = 4;
     while (stages > 2 && fixed + stages * (size_t)b.st_bytes > m->smem_optin) --stages;
     b.stages = stages;
-    // (the 576 threads' registers let one CTA reside on an SM, so the TMEM columns always suffice)
     m->smem[k] = fixed + stages * (size_t)b.st_bytes;
     if (m->smem[k] > m->smem_optin) return mlp_fail(m, KM_EINVAL, "product tile does not fit in shared memory");
     return KM_OK;

@@ -1336,7 +1336,6 @@ int mlp_predict_enqueue(kmeans_mlp *m, const float *X, int64_t N, int32_t *pred,
     if ((rc = make_map(m, &t1, m->W1b, d.Hp, d.Dk, d.Dk, d.Hp))) return rc;
     if ((rc = make_map(m, &t2, m->W2b, d.Hp, d.Hp, d.Hp, d.Hp))) return rc;
     if ((rc = make_map(m, &t3, m->W3b, d.G, d.Hp, d.Hp, m->bn3))) return rc;
-    MLP_CUDA(m, cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     count_launch();
     k_mlp_infer<<<(unsigned)std::min<int64_t>(c.tiles, m->num_sms), kInThreads, smem, s>>>(t1, t2, t3, c);
     MLP_CUDA(m, cudaGetLastError());
@@ -1412,7 +1411,9 @@ KM_API int kmeans_mlp_create(kmeans_mlp **out, int32_t D, int32_t hidden, int32_
     MC(mlp_alloc(m, &m->b3p, (size_t)classes, m->allocs));
     MC(mlp_alloc(m, &m->st, 1, m->allocs));
     m->err = &m->st->err;
+    // (one value for every network: it is the process's, and another thread's network may be launching)
     MC(cudaFuncSetAttribute(k_mlp_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem_optin));
+    MC(cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->smem_optin));
     count_launch();
     k_mlp_init<<<(unsigned)std::min<int64_t>((d.P + 255) / 256, (int64_t)m->num_sms * 8), 256, 0, m->stream>>>(
         d, m->master, seed);

@@ -1,0 +1,47 @@
+"""Calls from several host threads at a time: contexts, networks and seedings are
+independent of one another, whatever sizes the others have (a kernel's
+shared-memory limit is one value per process)."""
+import threading
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from test_gpu_parity import kp  # noqa: E402,F401
+
+pytestmark = pytest.mark.gpu
+
+
+def together(*loops):
+    """Every loop in a thread of its own; their first error is raised."""
+    errors = []
+
+    def guard(f):
+        try:
+            f()
+        except BaseException as e:  # noqa: BLE001
+            errors.append(e)
+    ts = [threading.Thread(target=guard, args=(f,)) for f in loops]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def test_networks_of_two_sizes(kp):  # noqa: F811
+    def loop(D, H, C, N):
+        net = kp.MLP(D, H, C, seed=3)
+        X = torch.randn(N, D, device="cuda")
+        want = torch.empty(N, dtype=torch.int32, device="cuda")
+        got = torch.empty_like(want)
+
+        def run():
+            with torch.cuda.device(0):
+                net.predict(X, want)
+                for _ in range(2000):
+                    net.predict(X, got)
+                assert torch.equal(got, want)
+        return run
+    together(loop(256, 256, 512, 300), loop(8, 16, 2, 300), loop(64, 64, 40, 300))

@@ -65,6 +65,7 @@ constexpr int kPPBlocks = 3, kPPU = 8;
 constexpr int kPPSegment = 2048;   // points filtered between two looks at the list
 constexpr int kPPList = 2 * kPPSegment;
 constexpr int kPPTable = 1024;     // centres whose distances to the new one the first filter uses
+constexpr int kPPMaxD = 4096;      // coordinates of a point (the centre is in shared memory)
 constexpr int kPPMaxChunks = 4096; // chunk size: the power of two >= 32 that gives at most so many
 constexpr int kPPBins = 65;        // leading zeros of Q (64: zero)
 constexpr unsigned long long kPPNaN = ~0ull;  // Q of a point whose D^2 is NaN: weight 0
@@ -668,8 +669,9 @@ cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const doubl
     const size_t smem = (size_t)((D + 1) & ~1) * 8 + (size_t)steps * (4u << lprl) * (vec ? 4 : 1) + kPPTable * 4 +
                         kPPSegment * 2;
     auto step = vec ? k_pp_step<true> : k_pp_step<false>;
-    if ((e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
+    // (one value for every call: it is the process's, and another thread may be launching)
+    constexpr int most = kPPMaxD * 12 + kPPTable * 4 + kPPSegment * 2;
+    if ((e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
     // FP32 error of a D-term sum of squared differences (any order), with room
     // for the FP64 sum's own (2^-53 relative): true >= computed (1 - eps) - tiny
     const double eps = (D + 8) * std::ldexp(1.0, -24) * (1.0 + 1.0 / 1024);
@@ -718,7 +720,7 @@ KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K,
         return code;
     };
     if (!X || !u || !centroids) return fail(KM_EINVAL, "a pointer argument is NULL");
-    if (N < 1 || N >= ((int64_t)1 << 40) || D < 1 || D > 4096 || K < 1 || (int64_t)K > N)
+    if (N < 1 || N >= ((int64_t)1 << 40) || D < 1 || D > kPPMaxD || K < 1 || (int64_t)K > N)
         return fail(KM_EINVAL, "need 1 <= K <= N < 2^40 and 1 <= D <= 4096");
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, X) != cudaSuccess ||

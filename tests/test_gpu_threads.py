@@ -3,6 +3,7 @@ independent of one another, whatever sizes the others have (a kernel's
 shared-memory limit is one value per process)."""
 import threading
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -45,3 +46,22 @@ def test_networks_of_two_sizes(kp):  # noqa: F811
                 assert torch.equal(got, want)
         return run
     together(loop(256, 256, 512, 300), loop(8, 16, 2, 300), loop(64, 64, 40, 300))
+
+
+def test_seedings_of_two_widths(kp):  # noqa: F811
+    def loop(N, D, K, reps):
+        rng = np.random.default_rng(D)
+        X = torch.from_numpy(rng.normal(size=(N, D)).astype(np.float32)).cuda()
+        u = rng.uniform(size=K)
+        C = torch.empty(K, D, device="cuda")
+        want = torch.empty(K, dtype=torch.int64, device="cuda")
+        got = torch.empty_like(want)
+
+        def run():
+            with torch.cuda.device(0):
+                kp.kmeans_init_kmeanspp(X, N, D, K, u, C, want)
+                for _ in range(reps):
+                    kp.kmeans_init_kmeanspp(X, N, D, K, u, C, got)
+                    assert torch.equal(got, want)
+        return run
+    together(loop(200, 4096, 4, 1500), loop(200, 4, 4, 1500), loop(200, 900, 4, 1500))

@@ -484,7 +484,9 @@ static cudaError_t launch_dense_t(const Params &p, cudaStream_t s, int first, in
     const size_t lb = (size_t)(p.Gp + 1) * PB * 4;
     if (p.algo == KM_ALGO_FILTERED && lb <= (size_t)kDenseLbBytes) smem += lb;
     auto kernel = k_dense_assign<DPL, L, P, Q, MB>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one value for every context: it is the process's, and another thread's context may be launching)
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kDenseTileBytes + kDenseLbBytes);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kDenseThreads, smem);

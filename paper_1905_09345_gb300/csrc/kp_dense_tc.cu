@@ -612,7 +612,8 @@ cudaError_t launch_t(const Params &p, cudaStream_t s, int first, int respect_don
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_dense_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one value for every context: it is the process's, and another thread's context may be launching)
+    cudaError_t e = cudaFuncSetAttribute(k_dense_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
     if (e != cudaSuccess) return e;
     const int grid = std::min(cfg.num_tiles, num_sms);
     count_launch();

@@ -623,7 +623,8 @@ cudaError_t launch_b(const Params &p, cudaStream_t s, int first, int respect_don
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaFuncSetAttribute(k_dense_tcb<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one value for every context: it is the process's, and another thread's context may be launching)
+    cudaError_t e = cudaFuncSetAttribute(k_dense_tcb<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
     if (e != cudaSuccess) return e;
     const int grid = std::min(cfg.num_tiles, num_sms);
     count_launch();

@@ -548,12 +548,10 @@ cudaError_t launch_filter(const Params &p, cudaStream_t s, int respect_done, int
     int64_t warps = (p.N + 127) / 128;
     int64_t grid = std::min<int64_t>((warps + 7) / 8, (int64_t)num_sms * 2);
     grid = std::max<int64_t>(grid, 1);
-    const size_t smem1 = (size_t)p.nbucket * 4, smem2 = 2 * smem1;
-    cudaError_t e = cudaFuncSetAttribute(k_filter_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-    if (e != cudaSuccess) return e;
+    const size_t smem1 = (size_t)p.nbucket * 4, smem2 = 2 * smem1;  // at most 32 KB
     count_launch();
     k_filter<<<(unsigned)grid, kFilterThreads, smem1, s>>>(p, respect_done);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     count_launch();
     k_filter_scatter<<<(unsigned)grid, kFilterThreads, smem2, s>>>(p, respect_done);
@@ -570,7 +568,9 @@ static cudaError_t launch_surv_t(const Params &p, cudaStream_t s, int respect_do
     while (wpb > 1 && cbytes + per_warp * wpb > smem_limit) wpb >>= 1;
     size_t smem = cbytes + per_warp * wpb;
     if (smem > smem_limit) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaFuncSetAttribute(k_survivor<DP, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one value for every context: it is the process's, and another thread's context may be launching)
+    cudaError_t e =
+        cudaFuncSetAttribute(k_survivor<DP, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_survivor<DP, STAGE>, wpb * 32, smem);
@@ -595,7 +595,7 @@ static cudaError_t launch_surv_dp(const Params &p, cudaStream_t s, int respect_d
 
 cudaError_t launch_survivor(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem_limit) {
     if (survivor_tp_eligible(p)) return launch_survivor_tp(p, s, respect_done, num_sms, smem_limit);
-    smem_limit -= 64;  // static shared (mbarrier)
+    smem_limit -= 128;  // static shared (mbarrier, in an aligned block of its own)
     switch (dense_dp(p.D)) {
     case 4: return launch_surv_dp<4>(p, s, respect_done, num_sms, smem_limit);
     case 8: return launch_surv_dp<8>(p, s, respect_done, num_sms, smem_limit);

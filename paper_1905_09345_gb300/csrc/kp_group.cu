@@ -15,6 +15,7 @@ namespace kp {
 namespace {
 
 constexpr int GRP_THREADS = 256;
+constexpr int kGrpMaxD = 4096;  // coordinates of a context's points at most
 
 // grp[k] = argmin_g ||c_k - cen_g||^2 (lowest g on ties).  Warp per
 // centroid, lanes over the groups; the centres sit in shared memory with a
@@ -117,11 +118,9 @@ cudaError_t launch_clustered_groups(const float *C, int K, int D, int G, int ite
     const size_t smem_a = sm_ck + (cen_smem ? sm_cen : 0);
     const size_t smem_u = (size_t)D * 4 + (size_t)GRP_THREADS * 4 + 32 * 4;
     if (smem_a > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_grp_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a);
-        if (e != cudaSuccess) return e;
-    }
-    if (smem_u > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_grp_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_u);
+        // (one value for every context: it is the process's, and another thread's context may be launching)
+        cudaError_t e =
+            cudaFuncSetAttribute(k_grp_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, nw * kGrpMaxD * 4);
         if (e != cudaSuccess) return e;
     }
     const unsigned ga = (unsigned)std::max(1, std::min((K + nw - 1) / nw, num_sms));

@@ -17,6 +17,7 @@ constexpr int kSettleWarps = kSettleThreads / 32;
 constexpr int kSub = 8;              // lanes per request
 constexpr int kPer = 32 / kSub;      // requests a warp works on at a time
 constexpr int kGrabMax = 4 * kPer;   // requests a warp claims at a time, at most
+constexpr int kSettleStaged = 160 << 10;  // bytes of centroids kept in shared memory, at most
 
 // The bitmap's set bits, compacted into the settle queue: a warp takes 32
 // words, scans their populations and reserves its slots with one atomic.
@@ -413,10 +414,12 @@ cudaError_t launch_settle(const Params &p, cudaStream_t s, int first, int respec
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // C in shared memory when it fits (up to 160 KB), else read from L2
-    const int staged = (size_t)p.K * p.D * 4 <= ((size_t)160 << 10);
+    const int staged = (size_t)p.K * p.D * 4 <= (size_t)kSettleStaged;
     const size_t smem = (staged ? (size_t)p.K * p.D * 4 : 0) + (size_t)(p.G + 1) * 4;
     auto kern = p.D == 32 ? k_settle<32> : (p.D == 64 ? k_settle<64> : k_settle<128>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one value for every context: it is the process's, and another thread's
+    // context may be launching; K of a tensor-core pass is at most 4096)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSettleStaged + 4 * (4096 + 1));
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSettleThreads, smem);

@@ -380,7 +380,9 @@ cudaError_t launch_stats_full(const Params &p, cudaStream_t s, int all_points, i
     {
         const size_t h1 = p.K <= p.hist_smem_k ? (size_t)p.K * 4 : 0;
         const size_t h2 = 2 * h1;
-        cudaError_t e = cudaFuncSetAttribute(k_stats_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h2);
+        // (one value for every context: it is the process's, and another thread's context may be launching)
+        cudaError_t e =
+            cudaFuncSetAttribute(k_stats_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, p.hist_smem_k * 8);
         if (e != cudaSuccess) return e;
         const int64_t blocks = (p.N + kStatsTile - 1) / kStatsTile;
         // two blocks per SM: each block adds its counts to the K global ones

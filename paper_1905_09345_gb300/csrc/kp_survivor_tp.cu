@@ -524,9 +524,10 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2)
 }
 
 template <int DP, bool STAGE>
-cudaError_t launch_tp2(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem) {
+cudaError_t launch_tp2(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem, size_t smem_limit) {
     auto kern = k_survivor_tp<DP, STAGE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one value for every context: it is the process's, and another thread's context may be launching)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTpThreads, smem);
@@ -545,8 +546,8 @@ cudaError_t launch_tp(const Params &p, cudaStream_t s, int respect_done, int num
     const bool stage = TpLayout(p, true).total * 4 <= smem_limit && cbytes < (1u << 31);
     const size_t smem = TpLayout(p, stage).total * 4;
     if (smem > smem_limit) return cudaErrorInvalidConfiguration;
-    return stage ? launch_tp2<DP, true>(p, s, respect_done, num_sms, smem)
-                 : launch_tp2<DP, false>(p, s, respect_done, num_sms, smem);
+    return stage ? launch_tp2<DP, true>(p, s, respect_done, num_sms, smem, smem_limit)
+                 : launch_tp2<DP, false>(p, s, respect_done, num_sms, smem, smem_limit);
 }
 
 }  // namespace
@@ -556,7 +557,7 @@ bool survivor_tp_eligible(const Params &p) {
 }
 
 cudaError_t launch_survivor_tp(const Params &p, cudaStream_t s, int respect_done, int num_sms, size_t smem_limit) {
-    smem_limit -= 64;  // static shared (mbarrier)
+    smem_limit -= 128;  // static shared (mbarrier, in an aligned block of its own)
     // the row's registers in steps of 4 coordinates up to 32, then 16 and 32 (a
     // centroid's staged row is padded at least that far): 200,003 x 17, K = 100:
     // 33 us an iteration on 32 coordinates, 31 on 20

@@ -65,3 +65,29 @@ def test_seedings_of_two_widths(kp):  # noqa: F811
                     assert torch.equal(got, want)
         return run
     together(loop(200, 4096, 4, 1500), loop(200, 4, 4, 1500), loop(200, 900, 4, 1500))
+
+
+def test_contexts_of_many_sizes(kp):  # noqa: F811
+    """Contexts made, fitted and closed side by side: every dense engine, the
+    settle, both survivor kernels, clustered groups."""
+    def loop(N, D, K, G, grouping, reps):
+        rng = np.random.default_rng(D + K)
+        centres = rng.normal(size=(K, D)) * 4.0
+        X = (centres[rng.integers(0, K, size=N)] + rng.normal(size=(N, D))).astype(np.float32)
+        X, C0 = torch.from_numpy(X).cuda(), torch.from_numpy(X[:K].copy()).cuda()
+        got = torch.empty(N, dtype=torch.int32, device="cuda")
+
+        def run():
+            with torch.cuda.device(0):
+                want = None
+                for _ in range(reps):
+                    km = kp.KMeans(X, C0, G, grouping=grouping)
+                    r = km.fit(4, 0.0, got)
+                    km.close()
+                    want = got.clone() if want is None else want
+                    assert torch.equal(got, want) and r.n_iter <= 4
+        return run
+    sizes = [(1500, 32, 256, 25, 0), (1500, 32, 1500, 150, 1), (1500, 64, 200, 20, 0), (1500, 128, 32, 3, 0),
+             (1500, 128, 900, 90, 0), (1500, 17, 100, 10, 1), (1500, 17, 1400, 10, 0), (700, 400, 64, 6, 1),
+             (700, 300, 500, 50, 0)]
+    together(*[loop(*s, 60) for s in sizes])

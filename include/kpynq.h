@@ -343,8 +343,8 @@ KM_API int kmeans_shard_update(kmeans_ctx *ctx, int32_t final_pass, const double
  * give the same centres on any implementation.  X: N x D float32, device
  * memory; u: K doubles; centroids: K x D float32 out; indices: K int64 out
  * (nullable); u and the outputs may be host or device memory.  Work on
- * `stream` with stream-ordered scratch (24 N bytes and a little); returns after
- * it finished.  Errors: KM_EINVAL, KM_ENOMEM, KM_ECUDA; message in
+ * `stream` with stream-ordered scratch (16 N bytes and a little, or 8 N, more
+ * slowly, where that does not fit); returns after it finished.  Errors: KM_EINVAL, KM_ENOMEM, KM_ECUDA; message in
  * kmeans_last_error(NULL).
  */
 KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K, const double *u,

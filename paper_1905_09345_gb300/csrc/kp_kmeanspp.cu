@@ -31,14 +31,17 @@
 // block makes for itself.  What is left of X to read per centre are the rows
 // near c and those that no centre is near to yet.
 //
-// The weights need no FP64 either: Q(x) = floor(D(x)^2 2^(64 - e0)), 64 bits
-// with 2^e0 > max D^2 at the time e0 was set, is made from the bits of D^2
-// when that changes, and for max D^2 in [2^(e-1), 2^e), e = e0 - k <= e0,
-// q(x) = Q(x) >> (32 - k) exactly (a floor of a floor).  k, the leading zeros
-// of max Q, is the first occupied bin of a histogram of leading zeros.  The
-// histogram and the chunk sums of q change only with the points that change;
-// a second set of sums is kept for k + 1, so that the usual step of k costs a
-// re-summation during the next sweep only.
+// The weights need no FP64 either: for max D^2 in [2^(e-1), 2^e), q(x) is a
+// shift of the significand of D(x)^2.  e = e0 - k, with 2^e0 > max D^2 when e0
+// was set and k the first occupied bin of a histogram of the points by the
+// binary orders that D(x)^2 lies below 2^e0.  The histogram and the chunk sums
+// of q change only with the points that change; a second set of sums is kept
+// for k + 1, so that the usual step of k costs a re-summation during the next
+// sweep only.
+//
+// Scratch: D(x)^2, and beside it what the bound's filter reads (a(x) and D(x)^2
+// in FP32).  Where memory for the second half is short the sweeps do without
+// that filter.
 //
 // One launch per centre (k_pp_step): the distances to the centre drawn last,
 // the sums, and -- in the last block to finish -- the next draw: the chunk
@@ -67,19 +70,18 @@ constexpr int kPPList = 2 * kPPSegment;
 constexpr int kPPTable = 1024;     // centres whose distances to the new one the first filter uses
 constexpr int kPPMaxD = 4096;      // coordinates of a point (the centre is in shared memory)
 constexpr int kPPMaxChunks = 4096; // chunk size: the power of two >= 32 that gives at most so many
-constexpr int kPPBins = 65;        // leading zeros of Q (64: zero)
-constexpr unsigned long long kPPNaN = ~0ull;  // Q of a point whose D^2 is NaN: weight 0
+constexpr int kPPBins = 65;        // binary orders of D^2 below 2^e0 (64: more, or zero)
 
 struct PPState {
     unsigned long long wmax;  // after the first centre: bit pattern of max D^2 (doubles >= 0 order as their bits)
     long long pick;           // the centre chosen last
     long long err;            // nonzero: an index out of range was produced
-    int e0;                   // scale of Q
-    int k;                    // leading zeros of max Q when the last draw was made
+    int e0;                   // scale of the histogram
+    int k;                    // its first occupied bin when the last draw was made
     int cur;                  // sums[cur]: of the weights at k; sums[cur ^ 1]: at k + 1
     int resum;                // sums[cur ^ 1] must be made anew
     unsigned ticket;          // blocks done
-    int hist[kPPBins];        // points by leading zeros of Q
+    int hist[kPPBins];        // points by the binary order of D^2 (NaN: in none)
 };
 
 __device__ __forceinline__ long long uniform_index(double u, long long N) {
@@ -91,21 +93,24 @@ __device__ __forceinline__ long long uniform_index(double u, long long N) {
 // FP32 points is at least 2^-298)
 __device__ __forceinline__ int exponent_of(unsigned long long bits) { return (int)((bits >> 52) & 0x7ff) - 1022; }
 
-// floor(d 2^(64 - e0)) for 0 <= d < 2^e0, from the bits of d
-__device__ __forceinline__ unsigned long long quant(double d, int e0) {
+// the weights floor(d 2^(32 - e)) for 0 <= d < 2^e, from the bits of d (NaN: 0),
+// at e and at e - 1
+struct Weights {
+    unsigned long long at, next;
+};
+__device__ __forceinline__ Weights weights(double d, int e) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
-    const int ex = (int)(bits >> 52);
-    if (ex >= 0x7ff && d != d) return kPPNaN;
-    if (ex == 0) return 0ull;  // zero (or below every weight)
-    const unsigned long long m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
-    const int sh = ex - 1011 - e0;  // d = m 2^(ex - 1075)
-    return sh >= 0 ? m << min(sh, 11) : (sh > -64 ? m >> -sh : 0ull);
+    const int ex = (int)(bits >> 52);  // d = m 2^(ex - 1075)
+    const unsigned long long m = ex == 0 || d != d ? 0ull : (bits & 0xfffffffffffffull) | 0x10000000000000ull;
+    const unsigned long long next = m >> (min(max(1043 + e - ex, 1), 64) - 1);
+    return {next >> 1, next};
 }
-// the weight at e = e0 - k; k > 32 only when every Q is zero
-__device__ __forceinline__ unsigned long long weight(unsigned long long q, int k) {
-    return q == kPPNaN ? 0ull : q >> (32 - min(k, 32));
+
+// the bin of d (not NaN)
+__device__ __forceinline__ int bin_of(double d, int e0) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+    return (bits >> 52) ? min(max(e0 - exponent_of(bits), 0), 64) : 64;
 }
-__device__ __forceinline__ int bin_of(unsigned long long q) { return q ? __clzll((long long)q) : 64; }
 
 // float to double on the integer pipe, exact for zero and normal numbers;
 // others set `odd` (no branch, so that several conversions and products are in
@@ -199,9 +204,8 @@ struct PPArgs {
     long long N;
     int D;
     double *dmin;                 // N: D(x)^2
-    unsigned long long *Q;        // N
     float2 *ub;                   // N: D(x)^2 rounded up to FP32 (the filters' bound); the nearest
-                                  // centre so far (an int in the second half)
+                                  // centre so far (an int in the second half); may be missing
     unsigned long long *sums[2];  // chunk sums of the weights
     int csh;                      // log2 of the chunk size
     long long nb;                 // chunks
@@ -258,16 +262,15 @@ __device__ void draw(const PPArgs &a, int j) {
         s_pick = a.N;
     }
     __syncthreads();
-    int kt = s_k, resum = 0;
-    if (kt == kg + 1 && kt <= 32) {
+    int kt = s_k, resum = 0, e0 = st->e0;
+    if (kt == kg + 1 && kt < 64) {
         cur ^= 1;
         resum = 1;
     } else if (kt != kg) {
         // the maximum fell by more than a factor of two: both sums are made anew
-        // (with a new Q when max Q has lost its leading bits)
-        int e0 = st->e0;
-        const bool requant = kt > 32;
-        if (requant) {
+        // (and the histogram, when it fell out of that)
+        const bool rebase = kt == 64;
+        if (rebase) {
             unsigned long long m = 0;
             for (long long n = tid; n < a.N; n += kPPThreads) {
                 const double d = __ldcg(a.dmin + n);
@@ -287,16 +290,11 @@ __device__ void draw(const PPArgs &a, int j) {
             unsigned long long s0 = 0, s1 = 0;
             const long long n1 = min(a.N, (b + 1) << a.csh);
             for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
-                unsigned long long q;
-                if (requant) {
-                    q = quant(__ldcg(a.dmin + n), e0);
-                    a.Q[n] = q;
-                    if (q != kPPNaN) atomicAdd(&st->hist[bin_of(q)], 1);
-                } else {
-                    q = __ldcg(a.Q + n);
-                }
-                s0 += weight(q, kt);
-                s1 += weight(q, kt + 1);
+                const double d = __ldcg(a.dmin + n);
+                if (rebase && d == d) atomicAdd(&st->hist[bin_of(d, e0)], 1);
+                const Weights w = weights(d, e0 - kt);
+                s0 += w.at;
+                s1 += w.next;
             }
             s0 = warp_sum_u(s0);
             s1 = warp_sum_u(s1);
@@ -309,6 +307,7 @@ __device__ void draw(const PPArgs &a, int j) {
         __threadfence();
         __syncthreads();
     }
+    const int e = e0 - kt;
     if (kt != kg) load_sums(a.sums[cur]);
     // per-thread run of consecutive chunk sums, scanned across the block
 #pragma unroll
@@ -352,7 +351,7 @@ __device__ void draw(const PPArgs &a, int j) {
             const long long n1 = min(a.N, (b + 1) << a.csh);
             for (long long n0 = b << a.csh; n0 < n1; n0 += kPPThreads) {
                 const long long n = n0 + tid;
-                const unsigned long long q = n < n1 ? weight(__ldcg(a.Q + n), kt) : 0ull;
+                const unsigned long long q = n < n1 ? weights(__ldcg(a.dmin + n), e).at : 0ull;
                 unsigned long long tot;
                 const unsigned long long in = before + block_scan_incl(q, sh, &tot);
                 if (in > T && in - q <= T) s_pick = n;  // the first run above T
@@ -387,8 +386,8 @@ __device__ __forceinline__ bool last_block(PPState *st) {
     return last;
 }
 
-// Centre 0, drawn uniformly: every point's FP64 distance, and the scale of Q
-// (k_pp_quant then makes Q).
+// Centre 0, drawn uniformly: every point's FP64 distance, and the scale of the
+// weights.
 template <bool VEC>
 __global__ void __launch_bounds__(kPPThreads) k_pp_first(PPArgs a) {
     extern __shared__ double sd[];  // the centre (D)
@@ -413,9 +412,9 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_first(PPArgs a) {
     }
 }
 
-// Q and the filter's bound of every point, the chunk sums and the histogram,
-// the draw of centre 1
-__global__ void __launch_bounds__(kPPThreads) k_pp_quant(PPArgs a) {
+// The filter's bound of every point, the chunk sums and the histogram, the draw
+// of centre 1
+__global__ void __launch_bounds__(kPPThreads) k_pp_weigh(PPArgs a) {
     __shared__ int hist[kPPBins];
     if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
     __syncthreads();
@@ -426,12 +425,11 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_quant(PPArgs a) {
         const long long n1 = min(a.N, (b + 1) << a.csh);
         for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
             const double d = a.dmin[n];
-            const unsigned long long q = quant(d, e0);
-            a.Q[n] = q;
-            a.ub[n] = make_float2(d == d ? __double2float_ru(d) : INFINITY, __int_as_float(0));
-            s0 += weight(q, k);
-            s1 += weight(q, k + 1);
-            if (q != kPPNaN) atomicAdd(&hist[bin_of(q)], 1);
+            if (a.ub) a.ub[n] = make_float2(d == d ? __double2float_ru(d) : INFINITY, __int_as_float(0));
+            const Weights w = weights(d, e0 - k);
+            s0 += w.at;
+            s1 += w.next;
+            if (d == d) atomicAdd(&hist[bin_of(d, e0)], 1);
         }
         s0 = warp_sum_u(s0);
         s1 = warp_sum_u(s1);
@@ -450,8 +448,8 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_quant(PPArgs a) {
 // multiple of 4 and 16-byte aligned rows) or one coordinate each, so that a
 // warp's loads are contiguous; successive centres sweep a block's points in
 // opposite directions, so that the end of one sweep is found in L2 by the
-// next.
-template <bool VEC>
+// next.  BOUND: the bound's filter comes first.
+template <bool VEC, bool BOUND>
 __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int j, int lprl, float eps_lo, float tiny) {
     // the centre: FP64 (D), then FP32 padded to a multiple of LPR vectors with
     // zeros; the first filter's table (kPPTable) and list (kPPSegment)
@@ -484,7 +482,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
         for (long long b = c0 + warp; b < c1; b += kPPWarps) {
             unsigned long long s = 0;
             const long long n1 = min(a.N, (b + 1) << a.csh);
-            for (long long n = (b << a.csh) + lane; n < n1; n += 32) s += weight(a.Q[n], k + 1);
+            for (long long n = (b << a.csh) + lane; n < n1; n += 32) s += weights(a.dmin[n], e0 - k).next;
             s = warp_sum_u(s);
             if (lane == 0) sums1[b] = s;
         }
@@ -494,7 +492,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
     // a quarter of the squared distances between the new centre and the others,
     // rounded down with room for the FP64 sums' own error: a point whose D^2 is
     // no larger is, by the triangle inequality, no nearer to the new centre
-    const int ntab = min(j - 1, kPPTable);
+    const int ntab = BOUND ? min(j - 1, kPPTable) : 0;
     for (int g0 = warp * rows; g0 < ntab; g0 += kPPWarps * rows) {  // warp-uniform
         const int g = g0 + sub;
         float s = 0.f;
@@ -517,6 +515,11 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
             far[g] = s < INFINITY ? __fmul_rd(__fsub_rd(__fmul_rd(s, eps_lo), tiny), 0.249997f) : -1.f;
     }
     __syncthreads();
+    auto bound = [&](long long n) {
+        if constexpr (BOUND) return a.ub[n].x;
+        const double d = a.dmin[n];
+        return d == d ? __double2float_ru(d) : INFINITY;
+    };
     constexpr int U = kPPU;  // row groups in flight
     for (long long q0 = p0; q0 < p1; q0 += kPPSegment) {
         // the filter, on a segment of this block's points
@@ -530,12 +533,12 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
 #pragma unroll
             for (int v = 0; v < kPer; ++v) {
                 const int i = v * kPPThreads + threadIdx.x;
-                b[v] = i < cnt ? a.ub[s0 + i] : make_float2(-1.f, 0.f);
+                b[v] = BOUND && i < cnt ? a.ub[s0 + i] : make_float2(-1.f, 0.f);
             }
 #pragma unroll
             for (int v = 0; v < kPer; ++v) {
                 const int i = v * kPPThreads + threadIdx.x, c = __float_as_int(b[v].y);
-                const bool keep = i < cnt && !(c < ntab && b[v].x <= far[c]);
+                const bool keep = i < cnt && !(BOUND && c < ntab && b[v].x <= far[c]);
                 const unsigned m = __ballot_sync(0xffffffffu, keep);
                 if (m) {
                     int at = 0;
@@ -557,7 +560,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
                 r[v] = g0 + v * rows + sub;
                 if (j & 1) r[v] = nk - 1 - r[v];  // below zero past the end
                 r[v] = r[v] >= 0 && r[v] < nk ? kept[r[v]] : -1;
-                ub[v] = l == 0 && r[v] >= 0 ? a.ub[s0 + r[v]].x : 0.f;
+                ub[v] = l == 0 && r[v] >= 0 ? bound(s0 + r[v]) : 0.f;
             }
             for (int t = 0; t < steps; ++t) {
                 const int q = l + (t << lprl);
@@ -618,15 +621,14 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
             const double s = dist2<VEC>(a.X + pt * D, sd, D);
             const double d = a.dmin[pt], m = fmin(d, s);
             if (m < d || (d != d && m == m)) {
-                const unsigned long long qo = a.Q[pt], qn = quant(m, e0);
                 a.dmin[pt] = m;
-                a.ub[pt] = make_float2(__double2float_ru(m), __int_as_float(j - 1));
-                a.Q[pt] = qn;
+                if constexpr (BOUND) a.ub[pt] = make_float2(__double2float_ru(m), __int_as_float(j - 1));
                 const long long b = pt >> a.csh;
-                atomicAdd(&sums0[b], weight(qn, k) - weight(qo, k));  // modulo 2^64
-                atomicAdd(&sums1[b], weight(qn, k + 1) - weight(qo, k + 1));
-                if (qo != kPPNaN) atomicAdd(&hist[bin_of(qo)], -1);
-                atomicAdd(&hist[bin_of(qn)], 1);
+                const Weights wm = weights(m, e0 - k), wd = weights(d, e0 - k);
+                atomicAdd(&sums0[b], wm.at - wd.at);  // modulo 2^64
+                atomicAdd(&sums1[b], wm.next - wd.next);
+                if (d == d) atomicAdd(&hist[bin_of(d, e0)], -1);
+                atomicAdd(&hist[bin_of(m, e0)], 1);
             }
         }
         __syncthreads();
@@ -640,14 +642,13 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
 }  // namespace
 
 cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const double *u, float *C, long long *idx,
-                            double *dmin, unsigned long long *Q, float2 *ub, unsigned long long *sums, void *state,
-                            cudaStream_t s, int num_sms, long long *err_out) {
+                            double *dmin, float2 *ub, unsigned long long *sums, void *state, cudaStream_t s,
+                            int num_sms, long long *err_out) {
     PPArgs a;
     a.X = X;
     a.N = N;
     a.D = D;
     a.dmin = dmin;
-    a.Q = Q;
     a.ub = ub;
     a.csh = kmeanspp_chunk_log2(N);
     a.nb = (N + ((int64_t)1 << a.csh) - 1) >> a.csh;
@@ -668,7 +669,8 @@ cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const doubl
     const int steps = (nv + (1 << lprl) - 1) >> lprl;
     const size_t smem = (size_t)((D + 1) & ~1) * 8 + (size_t)steps * (4u << lprl) * (vec ? 4 : 1) + kPPTable * 4 +
                         kPPSegment * 2;
-    auto step = vec ? k_pp_step<true> : k_pp_step<false>;
+    auto step = ub ? (vec ? k_pp_step<true, true> : k_pp_step<false, true>)
+                   : (vec ? k_pp_step<true, false> : k_pp_step<false, false>);
     // (one value for every call: it is the process's, and another thread may be launching)
     constexpr int most = kPPMaxD * 12 + kPPTable * 4 + kPPSegment * 2;
     if ((e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
@@ -687,7 +689,7 @@ cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const doubl
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (K > 1) {
         count_launch();
-        k_pp_quant<<<grid, kPPThreads, 0, s>>>(a);
+        k_pp_weigh<<<grid, kPPThreads, 0, s>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     for (int j = 2; j < K; ++j) {
@@ -736,24 +738,30 @@ KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K,
     const int64_t nb = ((N - 1) >> kmeanspp_chunk_log2(N)) + 1;
     float2 *ub = nullptr;
     double *dmin = nullptr, *ud = nullptr;
-    unsigned long long *bsum = nullptr, *Q = nullptr;
+    unsigned long long *bsum = nullptr;
     void *st = nullptr;
     float *Cd = nullptr;
     long long *idx = nullptr;
     long long err = 0;
     cudaError_t e = pool_alloc(dev, reinterpret_cast<void **>(&dmin), (size_t)N * 8, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&Q), (size_t)N * 8, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ub), (size_t)N * 8, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&bsum), (size_t)nb * 16, s);
     if (e == cudaSuccess) e = pool_alloc(dev, &st, kmeanspp_state_bytes(), s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ud), (size_t)K * 8, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&Cd), (size_t)K * D * 4, s);
     if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&idx), (size_t)K * 8, s);
+    if (e == cudaSuccess && K > 2) {  // (the sweeps' only; they can do without)
+        e = pool_alloc(dev, reinterpret_cast<void **>(&ub), (size_t)N * 8, s);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            ub = nullptr;
+            e = cudaSuccess;
+        }
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(ud, u, (size_t)K * 8, cudaMemcpyDefault, s);
-    if (e == cudaSuccess) e = launch_kmeanspp(X, N, D, K, ud, Cd, idx, dmin, Q, ub, bsum, st, s, sms, &err);
+    if (e == cudaSuccess) e = launch_kmeanspp(X, N, D, K, ud, Cd, idx, dmin, ub, bsum, st, s, sms, &err);
     if (e == cudaSuccess) e = cudaMemcpyAsync(centroids, Cd, (size_t)K * D * 4, cudaMemcpyDefault, s);
     if (e == cudaSuccess && indices) e = cudaMemcpyAsync(indices, idx, (size_t)K * 8, cudaMemcpyDefault, s);
-    for (void *p : {(void *)dmin, (void *)Q, (void *)ub, (void *)bsum, st, (void *)ud, (void *)Cd, (void *)idx})
+    for (void *p : {(void *)dmin, (void *)ub, (void *)bsum, st, (void *)ud, (void *)Cd, (void *)idx})
         if (p) cudaFreeAsync(p, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {

@@ -269,7 +269,7 @@ __device__ void draw(const PPArgs &a, int j) {
     } else if (kt != kg) {
         // the maximum fell by more than a factor of two: both sums are made anew
         // (and the histogram, when it fell out of that)
-        const bool rebase = kt == 64;
+        const bool rebase = kt == 64 || kg == 64;  // (no distance before: no scale either)
         if (rebase) {
             unsigned long long m = 0;
             for (long long n = tid; n < a.N; n += kPPThreads) {

@@ -85,3 +85,63 @@ def test_bound_alone(kp, N, D, K, kind):
     else:
         X = rng.integers(-2, 3, size=(max(K // 2, 2), D))[rng.integers(0, max(K // 2, 2), size=N)]
     check(kp, X.astype(np.float32), K, seed=K)
+
+
+def weights_reference(X, K, u):
+    """The draw of the header with Python integers.  A NaN distance never becomes
+    the smallest and weighs nothing; an infinite one weighs 2^64 - 1, sums modulo
+    2^64."""
+    N = len(X)
+    X = X.astype(np.float64)
+    d = np.full(N, np.nan)
+    idx = []
+    for j in range(K):
+        pick = min(int(np.floor(u[j] * N)), N - 1)
+        w = d[~np.isnan(d)].max(initial=0.0)
+        if w > 0:
+            e = 1025 if np.isinf(w) else np.frexp(w)[1]
+            q = [0 if np.isnan(v) else (2 ** 64 - 1 if np.isinf(v) else int(np.floor(np.ldexp(v, 32 - e)))) for v in d]
+            W = sum(q) % 2 ** 64
+            if W:
+                T = min(int(np.floor(u[j] * float(W))), W - 1)
+                run = 0
+                for pick in range(N):
+                    run = (run + q[pick]) % 2 ** 64
+                    if run > T:
+                        break
+        idx.append(pick)
+        s = np.zeros(N)
+        with np.errstate(invalid="ignore", over="ignore"):
+            for i in range(X.shape[1]):
+                t = X[:, i] - X[pick, i]
+                s = s + t * t
+        d = np.fmin(d, s)
+    return np.array(idx)
+
+
+def check_weights(kp, X, K, seed, u0):
+    N, D = X.shape
+    u = np.random.default_rng(seed).uniform(size=K) * 0.99
+    u[0] = u0
+    C = torch.empty(K, D, dtype=torch.float32, device="cuda")
+    idx = torch.empty(K, dtype=torch.int64, device="cuda")
+    kp.kmeans_init_kmeanspp(torch.from_numpy(X).cuda(), N, D, K, u, C, idx)
+    got, ref = idx.cpu().numpy(), weights_reference(X, K, u)
+    assert np.array_equal(got, ref), (got, ref)
+
+
+@pytest.mark.parametrize("where", ["first", "later"])
+@pytest.mark.parametrize("scale", [1e-6, 1.0, 1e6])
+def test_nan_rows(kp, where, scale):
+    """Rows with a NaN: as the first centre one leaves no distance to scale by,
+    and the next draw is uniform."""
+    rng = np.random.default_rng(3)
+    X = (rng.normal(size=(700, 6)) * np.exp2(rng.uniform(-6, 6, size=(700, 1))) * scale).astype(np.float32)
+    X[10:700:97, 2] = np.nan
+    check_weights(kp, X, 12, 6, (10 if where == "first" else 11) / 700 + 1e-9)
+    X[10:20] = np.nan  # (two such centres in a row)
+    u = np.concatenate([[10.5 / 700, 12.5 / 700], np.random.default_rng(5).uniform(size=8)])
+    C = torch.empty(10, 6, device="cuda")
+    idx = torch.empty(10, dtype=torch.int64, device="cuda")
+    kp.kmeans_init_kmeanspp(torch.from_numpy(X).cuda(), 700, 6, 10, u, C, idx)
+    assert np.array_equal(idx.cpu().numpy(), weights_reference(X, 10, u))

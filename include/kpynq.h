@@ -340,7 +340,9 @@ KM_API int kmeans_shard_update(kmeans_ctx *ctx, int32_t final_pass, const double
  * power of two that puts the largest in [2^31, 2^32), T = floor(u[j] * W)
  * for their sum W, and the centre is the first point whose running weight
  * sum exceeds T (uniform floor(u[j] * N) when W = 0) -- so the same uniforms
- * give the same centres on any implementation.  X: N x D float32, device
+ * give the same centres on any implementation.  (Not meant for, but taken: a
+ * row with a NaN weighs nothing, an infinite distance 2^64 - 1, sums modulo
+ * 2^64.)  X: N x D float32, device
  * memory; u: K doubles; centroids: K x D float32 out; indices: K int64 out
  * (nullable); u and the outputs may be host or device memory.  Work on
  * `stream` with stream-ordered scratch (16 N bytes and a little, or 8 N, more

@@ -93,8 +93,8 @@ __device__ __forceinline__ long long uniform_index(double u, long long N) {
 // FP32 points is at least 2^-298)
 __device__ __forceinline__ int exponent_of(unsigned long long bits) { return (int)((bits >> 52) & 0x7ff) - 1022; }
 
-// the weights floor(d 2^(32 - e)) for 0 <= d < 2^e, from the bits of d (NaN: 0),
-// at e and at e - 1
+// the weights floor(d 2^(32 - e)) for 0 <= d < 2^e, from the bits of d (NaN: 0;
+// infinity: the largest integer), at e and at e - 1
 struct Weights {
     unsigned long long at, next;
 };
@@ -103,6 +103,7 @@ __device__ __forceinline__ Weights weights(double d, int e) {
     const int ex = (int)(bits >> 52);  // d = m 2^(ex - 1075)
     const unsigned long long m = ex == 0 || d != d ? 0ull : (bits & 0xfffffffffffffull) | 0x10000000000000ull;
     const unsigned long long next = m >> (min(max(1043 + e - ex, 1), 64) - 1);
+    if (ex == 0x7ff && m != 0ull) return {~0ull, ~0ull};
     return {next >> 1, next};
 }
 

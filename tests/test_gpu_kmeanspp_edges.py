@@ -145,3 +145,15 @@ def test_nan_rows(kp, where, scale):
     idx = torch.empty(10, dtype=torch.int64, device="cuda")
     kp.kmeans_init_kmeanspp(torch.from_numpy(X).cuda(), 700, 6, 10, u, C, idx)
     assert np.array_equal(idx.cpu().numpy(), weights_reference(X, 10, u))
+
+
+@pytest.mark.parametrize("first", [0, 300])
+def test_infinite_coordinates(kp, first):
+    """Infinite distances outweigh all others together, the first of them every
+    time; as the first centre such a row leaves the rest infinitely far."""
+    rng = np.random.default_rng(first)
+    X = rng.normal(size=(900, 5)).astype(np.float32)
+    X[300, 1] = np.inf
+    X[450, 3] = -np.inf
+    X[700, 1] = np.inf
+    check_weights(kp, X, 9, 2, (first + 0.5) / 900)

@@ -81,7 +81,7 @@ struct PPState {
     int cur;                  // sums[cur]: of the weights at k; sums[cur ^ 1]: at k + 1
     int resum;                // sums[cur ^ 1] must be made anew
     unsigned ticket;          // blocks done
-    int hist[kPPBins];        // points by the binary order of D^2 (NaN: in none)
+    unsigned long long hist[kPPBins];  // points by the binary order of D^2 (NaN: in none)
 };
 
 __device__ __forceinline__ long long uniform_index(double u, long long N) {
@@ -254,7 +254,7 @@ __device__ void draw(const PPArgs &a, int j) {
     };
     load_sums(a.sums[cur]);
     if (warp == 0) {  // the first occupied bin
-        const int h0 = __ldcg(&st->hist[lane]), h1 = __ldcg(&st->hist[32 + lane]);
+        const unsigned long long h0 = __ldcg(&st->hist[lane]), h1 = __ldcg(&st->hist[32 + lane]);
         const unsigned b0 = __ballot_sync(0xffffffffu, h0 != 0), b1 = __ballot_sync(0xffffffffu, h1 != 0);
         if (lane == 0) s_k = b0 ? __ffs(b0) - 1 : (b1 ? 31 + __ffs(b1) : 64);
     }
@@ -279,7 +279,7 @@ __device__ void draw(const PPArgs &a, int j) {
             }
             m = warp_max_u(m);
             if (lane == 0) sh[warp] = m;
-            if (tid < kPPBins) st->hist[tid] = 0;
+            if (tid < kPPBins) st->hist[tid] = 0ull;
             __syncthreads();
             m = 0;
             for (int w = 0; w < kPPWarps; ++w) m = max(m, sh[w]);
@@ -292,7 +292,7 @@ __device__ void draw(const PPArgs &a, int j) {
             const long long n1 = min(a.N, (b + 1) << a.csh);
             for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
                 const double d = __ldcg(a.dmin + n);
-                if (rebase && d == d) atomicAdd(&st->hist[bin_of(d, e0)], 1);
+                if (rebase && d == d) atomicAdd(&st->hist[bin_of(d, e0)], 1ull);
                 const Weights w = weights(d, e0 - kt);
                 s0 += w.at;
                 s1 += w.next;
@@ -440,7 +440,8 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_weigh(PPArgs a) {
         }
     }
     __syncthreads();
-    if (threadIdx.x < kPPBins && hist[threadIdx.x]) atomicAdd(&a.st->hist[threadIdx.x], hist[threadIdx.x]);
+    if (threadIdx.x < kPPBins && hist[threadIdx.x])  // (a block's points fit 31 bits, all together need not)
+        atomicAdd(&a.st->hist[threadIdx.x], (unsigned long long)(long long)hist[threadIdx.x]);
     if (last_block(a.st)) draw(a, 1);
 }
 
@@ -636,7 +637,8 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
         if (threadIdx.x == 0) nlist = 0;
         __syncthreads();
     }
-    if (threadIdx.x < kPPBins && hist[threadIdx.x]) atomicAdd(&a.st->hist[threadIdx.x], hist[threadIdx.x]);
+    if (threadIdx.x < kPPBins && hist[threadIdx.x])  // (a block's points fit 31 bits, all together need not)
+        atomicAdd(&a.st->hist[threadIdx.x], (unsigned long long)(long long)hist[threadIdx.x]);
     if (last_block(a.st)) draw(a, j);
 }
 

@@ -46,3 +46,27 @@ def test_eight_bytes_a_point(N, D, K, tmp_path):
     assert r.returncode == 0, r.stderr[-1500:]
     ref, _ = oracle.kmeanspp(X.astype(np.float64), K, u)
     assert np.array_equal(np.load(tmp_path / "idx.npy"), ref)
+
+
+@pytest.mark.gpu
+def test_more_points_than_32_bits_count(kp_lib):
+    """2^32 points at the largest distance: with a 32-bit count of them, zero, the
+    weights would be scaled by the one point that is nearer."""
+    N, K = 2 ** 32 + 2, 2
+    if torch.cuda.mem_get_info()[0] < 16 * N:
+        pytest.skip("needs 64 GB of device memory")
+    X = torch.ones(N, 1, device="cuda")
+    X[0], X[1] = 0.0, 0.5
+    C = torch.empty(K, 1, device="cuda")
+    idx = torch.empty(K, dtype=torch.int64, device="cuda")
+    kp_lib.kmeans_init_kmeanspp(X, N, 1, K, np.array([0.0, 0.25]), C, idx)
+    assert idx.tolist() == [0, 1 + 2 ** 30]
+    assert C.flatten().tolist() == [0.0, 1.0]
+
+
+@pytest.fixture
+def kp_lib():
+    from paper_1905_09345_gb300 import build, kpynq
+    build.build()
+    yield kpynq
+    torch.cuda.empty_cache()

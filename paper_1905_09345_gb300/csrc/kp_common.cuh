@@ -533,15 +533,6 @@ cudaError_t launch_arm(const Params &p, cudaStream_t s, int max_iter, double tol
 cudaError_t launch_set_cond(const Params &p, cudaStream_t s);
 cudaError_t launch_rebase(const Params &p, cudaStream_t s, int num_sms);
 cudaError_t launch_bounds_out(const Params &p, cudaStream_t s, float *u, float *lbg, float *lb, int num_sms);
-// k-means++ seeding (kp_kmeanspp.cu): K centres of X into C / idx; dmin (N
-// doubles), ub (N, or NULL: slower), sums (2 per chunk of
-// 2^kmeanspp_chunk_log2(N) points) and state (kmeanspp_state_bytes()) are
-// scratch; *err_out (host) is set nonzero if a drawn index fell out of range
-cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const double *u, float *C, long long *idx,
-                            double *dmin, float2 *ub, unsigned long long *sums, void *state, cudaStream_t s,
-                            int num_sms, long long *err_out);
-size_t kmeanspp_state_bytes();
-int kmeanspp_chunk_log2(int64_t N);
 // stream-ordered allocation from the library's own pool on `dev` (it keeps
 // freed memory mapped across synchronisations, unlike the default pool with
 // its zero release threshold); free with cudaFreeAsync

@@ -37,21 +37,27 @@
 // binary orders that D(x)^2 lies below 2^e0.  The histogram and the chunk sums
 // of q change only with the points that change; a second set of sums is kept
 // for k + 1, so that the usual step of k costs a re-summation during the next
-// sweep only.
+// sweep only.  When the maximum falls further (the first centres do that, and
+// outliers) the sums are made anew by all blocks: the next launch does that
+// instead of a sweep, and the host makes up for the launches spent so (one to
+// spare is always launched).
+// (16,777,216 x 2, K = 4, one such fall: 35 ms with the last block making the
+// sums, 1.4 now, 1.9 with FP64 distances to every point.)
 //
 // Scratch: D(x)^2, and beside it what the bound's filter reads (a(x) and D(x)^2
 // in FP32).  Where memory for the second half is short the sweeps do without
 // that filter.
 //
-// One launch per centre (k_pp_step): the distances to the centre drawn last,
-// the sums, and -- in the last block to finish -- the next draw: the chunk
+// One launch per centre as a rule (k_pp_step): the distances to the centre drawn
+// last, the sums, and -- in the last block to finish -- the next draw: the chunk
 // holding T, then the point in it, copied to the output centroids.  Every
 // block owns a run of chunks.
 // Measured on GB300 (1,048,576 x 32, K = 128): 337 us per centre and 43.9 ms in
 // all with FP64 distances to every point; 50 us and 6.9 ms with the FP32 filter
 // alone (21 the read of X, 8 the FP64 distances, 8 the draw, 5 the launch);
-// 38 us and 5.4 ms with the bound's filter before it.  3,878 x 100: 45 -> 22 us per
-// centre with the FP32 filter.
+// 38 us and 5.4 ms with the bound's filter before it; 4.9 ms without a copy of the
+// arguments in local memory.  3,878 x 100: 45 -> 22 us per centre with the FP32
+// filter.
 #include <cmath>
 
 #include "kp_common.cuh"
@@ -72,14 +78,24 @@ constexpr int kPPMaxD = 4096;      // coordinates of a point (the centre is in s
 constexpr int kPPMaxChunks = 4096; // chunk size: the power of two >= 32 that gives at most so many
 constexpr int kPPBins = 65;        // binary orders of D^2 below 2^e0 (64: more, or zero)
 
+// what the next launch does
+enum PPTodo : int {
+    kPPSweep,  // the distances to the last centre
+    kPPSums,   // the chunk sums anew
+    kPPMax,    // the largest distance
+    kPPHist    // the histogram and the chunk sums anew
+};
+
 struct PPState {
-    unsigned long long wmax;  // after the first centre: bit pattern of max D^2 (doubles >= 0 order as their bits)
+    int chosen;               // centres chosen so far
+    int err;                  // nonzero: an index out of range was produced
     long long pick;           // the centre chosen last
-    long long err;            // nonzero: an index out of range was produced
+    unsigned long long wmax;  // bit pattern of max D^2 (doubles >= 0 order as their bits)
+    int todo;                 // PPTodo
     int e0;                   // scale of the histogram
     int k;                    // its first occupied bin when the last draw was made
-    int cur;                  // sums[cur]: of the weights at k; sums[cur ^ 1]: at k + 1
-    int resum;                // sums[cur ^ 1] must be made anew
+    int cur;                  // the set of sums of the weights at k; the other: at k + 1
+    int resum;                // the other set must be made anew
     unsigned ticket;          // blocks done
     unsigned long long hist[kPPBins];  // points by the binary order of D^2 (NaN: in none)
 };
@@ -203,11 +219,11 @@ __device__ __forceinline__ unsigned long long warp_max_u(unsigned long long v) {
 struct PPArgs {
     const float *X;
     long long N;
-    int D;
+    int D, K;
     double *dmin;                 // N: D(x)^2
     float2 *ub;                   // N: D(x)^2 rounded up to FP32 (the filters' bound); the nearest
                                   // centre so far (an int in the second half); may be missing
-    unsigned long long *sums[2];  // chunk sums of the weights
+    unsigned long long *sums0, *sums1;  // chunk sums of the weights (two sets)
     int csh;                      // log2 of the chunk size
     long long nb;                 // chunks
     const double *u;
@@ -215,6 +231,21 @@ struct PPArgs {
     float *C;
     long long *idx;
 };
+
+// (an index into the kernel's arguments would copy them to local memory)
+__device__ __forceinline__ unsigned long long *sums_of(const PPArgs &a, int set) { return set ? a.sums1 : a.sums0; }
+
+// a load that stays where it is written
+__device__ __forceinline__ int ld_now(const int *p) {
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ long long ld_now(const long long *p) {
+    long long v;
+    asm volatile("ld.global.s64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
+}
 
 // the chunks of this block: [first, last)
 __device__ __forceinline__ long long chunk0(const PPArgs &a, unsigned blk) {
@@ -230,9 +261,64 @@ __device__ __forceinline__ void take_centre(const PPArgs &a, int j, long long pi
     }
 }
 
-// The last block to finish (whole block): the draw of centre j from the chunk
-// sums.  Every other block's results are visible (fence and ticket).
-__device__ void draw(const PPArgs &a, int j) {
+// d = D(x_n)^2 of the points n of chunk b, lanes over the points, four loads in
+// flight
+template <class F>
+__device__ __forceinline__ void each_distance(const PPArgs &a, long long b, F f) {
+    const long long n1 = min(a.N, (b + 1) << a.csh);
+    for (long long n0 = (b << a.csh) + (threadIdx.x & 31); n0 < n1; n0 += 128) {
+        double d[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) d[v] = n0 + 32 * v < n1 ? __ldcg(a.dmin + n0 + 32 * v) : 0.0;
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            if (n0 + 32 * v < n1) f(n0 + 32 * v, d[v]);
+    }
+}
+
+// A block's part of what a fall of the maximum asks for (PPTodo); with `ub` also
+// the filter's bound of every point, nearest centre 0.
+__device__ __forceinline__ void remake(const PPArgs &a, int todo, float2 *ub) {
+    __shared__ int hist[kPPBins];
+    if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
+    __syncthreads();
+    const PPState *st = a.st;
+    const int e0 = st->e0, e = e0 - st->k, cur = st->cur, lane = threadIdx.x & 31;
+    const long long c1 = chunk0(a, blockIdx.x + 1);
+    unsigned long long m = 0;
+    for (long long b = chunk0(a, blockIdx.x) + (threadIdx.x >> 5); b < c1; b += kPPWarps) {
+        if (todo == kPPMax) {
+            each_distance(a, b, [&](long long, double d) {
+                if (d == d) m = max(m, (unsigned long long)__double_as_longlong(d));
+            });
+            continue;
+        }
+        unsigned long long s0 = 0, s1 = 0;
+        each_distance(a, b, [&](long long n, double d) {
+            if (ub) ub[n] = make_float2(d == d ? __double2float_ru(d) : INFINITY, __int_as_float(0));
+            const Weights w = weights(d, e);
+            s0 += w.at;
+            s1 += w.next;
+            if (todo == kPPHist && d == d) atomicAdd(&hist[bin_of(d, e0)], 1);
+        });
+        s0 = warp_sum_u(s0);
+        s1 = warp_sum_u(s1);
+        if (lane == 0) {
+            sums_of(a, cur)[b] = s0;
+            sums_of(a, cur ^ 1)[b] = s1;
+        }
+    }
+    m = warp_max_u(m);
+    if (lane == 0 && m) atomicMax(&a.st->wmax, m);
+    __syncthreads();
+    if (threadIdx.x < kPPBins && hist[threadIdx.x])  // (a block's points fit 31 bits, all together need not)
+        atomicAdd(&a.st->hist[threadIdx.x], (unsigned long long)hist[threadIdx.x]);
+}
+
+// The last block to finish (whole block): the draw of the next centre from the
+// chunk sums, or the order to remake them first.  Every other block's results are
+// visible (fence and ticket).
+__device__ __forceinline__ void draw(const PPArgs &a) {
     __shared__ unsigned long long sh[kPPWarps];
     __shared__ unsigned long long s_before;
     __shared__ long long s_block, s_pick;
@@ -241,8 +327,8 @@ __device__ void draw(const PPArgs &a, int j) {
     constexpr int kPer = kPPMaxChunks / kPPThreads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     PPState *st = a.st;
-    int cur = st->cur;
-    const int kg = st->k;
+    int cur = ld_now(&st->cur);
+    const int kg = ld_now(&st->k), j = ld_now(&st->chosen), e0 = ld_now(&st->e0), todo = ld_now(&st->todo);
     // the sums at k, read before k is known to stand
     unsigned long long v[kPer];
     auto load_sums = [&](const unsigned long long *bs) {
@@ -252,7 +338,8 @@ __device__ void draw(const PPArgs &a, int j) {
             v[i] = b < a.nb ? __ldcg(bs + b) : 0ull;
         }
     };
-    load_sums(a.sums[cur]);
+    load_sums(sums_of(a, cur));
+    const double u = *const_cast<const volatile double *>(a.u + min(j, a.K - 1));  // (now: nothing else depends on it yet)
     if (warp == 0) {  // the first occupied bin
         const unsigned long long h0 = __ldcg(&st->hist[lane]), h1 = __ldcg(&st->hist[32 + lane]);
         const unsigned b0 = __ballot_sync(0xffffffffu, h0 != 0), b1 = __ballot_sync(0xffffffffu, h1 != 0);
@@ -263,53 +350,37 @@ __device__ void draw(const PPArgs &a, int j) {
         s_pick = a.N;
     }
     __syncthreads();
-    int kt = s_k, resum = 0, e0 = st->e0;
-    if (kt == kg + 1 && kt < 64) {
+    if (todo == kPPMax) {  // the scale; then the histogram
+        if (tid < kPPBins) st->hist[tid] = 0ull;
+        if (tid == 0) {
+            const unsigned long long w = __ldcg(&st->wmax);
+            if (w) st->e0 = exponent_of(w);
+            st->k = w ? 0 : 64;  // all zero: it stays so
+            st->todo = kPPHist;
+            st->ticket = 0u;
+        }
+        return;
+    }
+    const int kt = s_k, resum = kt == kg + 1 && kt < 64;
+    if (resum) {
         cur ^= 1;
-        resum = 1;
-    } else if (kt != kg) {
-        // the maximum fell by more than a factor of two: both sums are made anew
-        // (and the histogram, when it fell out of that)
-        const bool rebase = kt == 64 || kg == 64;  // (no distance before: no scale either)
-        if (rebase) {
-            unsigned long long m = 0;
-            for (long long n = tid; n < a.N; n += kPPThreads) {
-                const double d = __ldcg(a.dmin + n);
-                if (d == d) m = max(m, (unsigned long long)__double_as_longlong(d));
+    } else if (kt != kg) {  // (not after kPPSums and kPPHist)
+        // the maximum fell by more than a factor of two, or (64) there was or is
+        // none in the histogram's reach
+        if (tid == 0) {
+            if (kt == 64 || kg == 64) {
+                st->todo = kPPMax;
+                st->wmax = 0ull;
+            } else {
+                st->todo = kPPSums;
+                st->k = kt;
             }
-            m = warp_max_u(m);
-            if (lane == 0) sh[warp] = m;
-            if (tid < kPPBins) st->hist[tid] = 0ull;
-            __syncthreads();
-            m = 0;
-            for (int w = 0; w < kPPWarps; ++w) m = max(m, sh[w]);
-            kt = m ? 0 : 64;  // all zero: it stays so
-            e0 = m ? exponent_of(m) : e0;
-            __syncthreads();
+            st->ticket = 0u;
         }
-        for (long long b = warp; b < a.nb; b += kPPWarps) {
-            unsigned long long s0 = 0, s1 = 0;
-            const long long n1 = min(a.N, (b + 1) << a.csh);
-            for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
-                const double d = __ldcg(a.dmin + n);
-                if (rebase && d == d) atomicAdd(&st->hist[bin_of(d, e0)], 1ull);
-                const Weights w = weights(d, e0 - kt);
-                s0 += w.at;
-                s1 += w.next;
-            }
-            s0 = warp_sum_u(s0);
-            s1 = warp_sum_u(s1);
-            if (lane == 0) {
-                a.sums[cur][b] = s0;
-                a.sums[cur ^ 1][b] = s1;
-            }
-        }
-        if (tid == 0) st->e0 = e0;
-        __threadfence();
-        __syncthreads();
+        return;
     }
     const int e = e0 - kt;
-    if (kt != kg) load_sums(a.sums[cur]);
+    if (resum) load_sums(sums_of(a, cur));
     // per-thread run of consecutive chunk sums, scanned across the block
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
@@ -329,9 +400,9 @@ __device__ void draw(const PPArgs &a, int j) {
     unsigned long long W = 0;
     const unsigned long long incl = block_scan_incl(run, sh, &W);
     if (W == 0) {  // every weight is zero: a uniform draw
-        if (tid == 0) s_pick = uniform_index(a.u[j], a.N);
+        if (tid == 0) s_pick = uniform_index(u, a.N);
     } else {
-        unsigned long long T = (unsigned long long)floor(__dmul_rn(a.u[j], (double)W));
+        unsigned long long T = (unsigned long long)floor(__dmul_rn(u, (double)W));
         if (T >= W) T = W - 1;
         unsigned long long acc = incl - run;
         if (acc <= T && T < incl) {  // exactly one thread: its run holds T
@@ -372,6 +443,8 @@ __device__ void draw(const PPArgs &a, int j) {
         st->k = kt;
         st->cur = cur;
         st->resum = resum;
+        st->chosen = j + 1;
+        st->todo = kPPSweep;
         st->ticket = 0u;
     }
 }
@@ -409,6 +482,7 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_first(PPArgs a) {
         const unsigned long long w = __ldcg(&a.st->wmax);
         a.st->e0 = w ? exponent_of(w) : 0;
         a.st->k = w ? 0 : 64;
+        a.st->chosen = 1;
         a.st->ticket = 0u;
     }
 }
@@ -416,49 +490,26 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_first(PPArgs a) {
 // The filter's bound of every point, the chunk sums and the histogram, the draw
 // of centre 1
 __global__ void __launch_bounds__(kPPThreads) k_pp_weigh(PPArgs a) {
-    __shared__ int hist[kPPBins];
-    if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
-    __syncthreads();
-    const int e0 = a.st->e0, k = a.st->k, lane = threadIdx.x & 31;
-    const long long c1 = chunk0(a, blockIdx.x + 1);
-    for (long long b = chunk0(a, blockIdx.x) + (threadIdx.x >> 5); b < c1; b += kPPWarps) {
-        unsigned long long s0 = 0, s1 = 0;
-        const long long n1 = min(a.N, (b + 1) << a.csh);
-        for (long long n = (b << a.csh) + lane; n < n1; n += 32) {
-            const double d = a.dmin[n];
-            if (a.ub) a.ub[n] = make_float2(d == d ? __double2float_ru(d) : INFINITY, __int_as_float(0));
-            const Weights w = weights(d, e0 - k);
-            s0 += w.at;
-            s1 += w.next;
-            if (d == d) atomicAdd(&hist[bin_of(d, e0)], 1);
-        }
-        s0 = warp_sum_u(s0);
-        s1 = warp_sum_u(s1);
-        if (lane == 0) {
-            a.sums[0][b] = s0;
-            a.sums[1][b] = s1;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < kPPBins && hist[threadIdx.x])  // (a block's points fit 31 bits, all together need not)
-        atomicAdd(&a.st->hist[threadIdx.x], (unsigned long long)(long long)hist[threadIdx.x]);
-    if (last_block(a.st)) draw(a, 1);
+    remake(a, kPPHist, a.ub);
+    if (last_block(a.st)) draw(a);
 }
 
-// Centre j - 1 (drawn last): the distances it shortens, the sums, the draw of
-// centre j.  A row is read by LPR = 2^lprl lanes, 16 bytes each (VEC: D a
-// multiple of 4 and 16-byte aligned rows) or one coordinate each, so that a
-// warp's loads are contiguous; successive centres sweep a block's points in
-// opposite directions, so that the end of one sweep is found in L2 by the
-// next.  BOUND: the bound's filter comes first.
+// The centre drawn last: the distances it shortens, and the sums.  A row is read
+// by LPR = 2^lprl lanes, 16 bytes each (VEC: D a multiple of 4 and 16-byte
+// aligned rows) or one coordinate each, so that a warp's loads are contiguous;
+// successive centres sweep a block's points in opposite directions (`odd`), so
+// that the end of one sweep is found in L2 by the next.  BOUND: the bound's
+// filter comes first.
 template <bool VEC, bool BOUND>
-__global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int j, int lprl, float eps_lo, float tiny) {
+__device__ __forceinline__ void sweep(const PPArgs &a, int chosen, long long pick, int e0, int k, int cur, int resum,
+                                      int odd, int lprl, float eps_lo, float tiny) {
     // the centre: FP64 (D), then FP32 padded to a multiple of LPR vectors with
     // zeros; the first filter's table (kPPTable) and list (kPPSegment)
     extern __shared__ double sd[];
     __shared__ unsigned list[kPPList];
     __shared__ int hist[kPPBins];
     __shared__ int nlist, nkept;
+    __shared__ int newest, s_e0, s_k, s_cur;  // the centre drawn last; of the state (registers are short)
     const int D = a.D, LPR = 1 << lprl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *sc = reinterpret_cast<float *>(sd + ((D + 1) & ~1));
     constexpr int W = VEC ? 4 : 1;
@@ -467,7 +518,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
     float *far = sc + steps * LPR * W;         // what D(x)^2 has to exceed for the new centre to matter
     unsigned short *kept = reinterpret_cast<unsigned short *>(far + kPPTable);
     {
-        const float *c = a.X + a.st->pick * D;
+        const float *c = a.X + pick * D;
         for (int i = threadIdx.x; i < steps * LPR * W; i += kPPThreads) {
             const float v = i < D ? c[i] : 0.f;
             sc[i] = v;
@@ -475,18 +526,22 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
         }
     }
     if (threadIdx.x < kPPBins) hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) nlist = nkept = 0;
-    const int e0 = a.st->e0, k = a.st->k;
-    unsigned long long *sums0 = a.sums[a.st->cur], *sums1 = a.sums[a.st->cur ^ 1];
+    if (threadIdx.x == 0) {
+        nlist = nkept = 0;
+        newest = chosen - 1;
+        s_e0 = e0;
+        s_k = k;
+        s_cur = cur;
+    }
     const long long c0 = chunk0(a, blockIdx.x), c1 = chunk0(a, blockIdx.x + 1);
     const long long p0 = c0 << a.csh, p1 = min(a.N, c1 << a.csh);  // this block's points
-    if (a.st->resum)
+    if (resum)
         for (long long b = c0 + warp; b < c1; b += kPPWarps) {
             unsigned long long s = 0;
             const long long n1 = min(a.N, (b + 1) << a.csh);
             for (long long n = (b << a.csh) + lane; n < n1; n += 32) s += weights(a.dmin[n], e0 - k).next;
             s = warp_sum_u(s);
-            if (lane == 0) sums1[b] = s;
+            if (lane == 0) sums_of(a, cur ^ 1)[b] = s;
         }
     __syncthreads();
 
@@ -494,7 +549,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
     // a quarter of the squared distances between the new centre and the others,
     // rounded down with room for the FP64 sums' own error: a point whose D^2 is
     // no larger is, by the triangle inequality, no nearer to the new centre
-    const int ntab = BOUND ? min(j - 1, kPPTable) : 0;
+    const int ntab = BOUND ? min(chosen - 1, kPPTable) : 0;
     for (int g0 = warp * rows; g0 < ntab; g0 += kPPWarps * rows) {  // warp-uniform
         const int g = g0 + sub;
         float s = 0.f;
@@ -526,8 +581,8 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
     for (long long q0 = p0; q0 < p1; q0 += kPPSegment) {
         // the filter, on a segment of this block's points
         const int cnt = (int)min((long long)kPPSegment, p1 - q0);
-        // (odd centres: the segments and their rows from the end)
-        const long long s0 = (j & 1) ? p1 - (q0 - p0) - cnt : q0;
+        // (odd: the segments and their rows from the end)
+        const long long s0 = odd ? p1 - (q0 - p0) - cnt : q0;
         // first by the bound alone, a thread per point
         {
             constexpr int kPer = kPPSegment / kPPThreads;
@@ -560,7 +615,7 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
             for (int v = 0; v < U; ++v) {
                 s[v] = 0.f;
                 r[v] = g0 + v * rows + sub;
-                if (j & 1) r[v] = nk - 1 - r[v];  // below zero past the end
+                if (odd) r[v] = nk - 1 - r[v];  // below zero past the end
                 r[v] = r[v] >= 0 && r[v] < nk ? kept[r[v]] : -1;
                 ub[v] = l == 0 && r[v] >= 0 ? bound(s0 + r[v]) : 0.f;
             }
@@ -624,13 +679,14 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
             const double d = a.dmin[pt], m = fmin(d, s);
             if (m < d || (d != d && m == m)) {
                 a.dmin[pt] = m;
-                if constexpr (BOUND) a.ub[pt] = make_float2(__double2float_ru(m), __int_as_float(j - 1));
+                if constexpr (BOUND) a.ub[pt] = make_float2(__double2float_ru(m), __int_as_float(newest));
                 const long long b = pt >> a.csh;
-                const Weights wm = weights(m, e0 - k), wd = weights(d, e0 - k);
-                atomicAdd(&sums0[b], wm.at - wd.at);  // modulo 2^64
-                atomicAdd(&sums1[b], wm.next - wd.next);
-                if (d == d) atomicAdd(&hist[bin_of(d, e0)], -1);
-                atomicAdd(&hist[bin_of(m, e0)], 1);
+                const int e = s_e0 - s_k;
+                const Weights wm = weights(m, e), wd = weights(d, e);
+                atomicAdd(&sums_of(a, s_cur)[b], wm.at - wd.at);  // modulo 2^64
+                atomicAdd(&sums_of(a, s_cur ^ 1)[b], wm.next - wd.next);
+                if (d == d) atomicAdd(&hist[bin_of(d, s_e0)], -1);
+                atomicAdd(&hist[bin_of(m, s_e0)], 1);
             }
         }
         __syncthreads();
@@ -639,30 +695,60 @@ __global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int
     }
     if (threadIdx.x < kPPBins && hist[threadIdx.x])  // (a block's points fit 31 bits, all together need not)
         atomicAdd(&a.st->hist[threadIdx.x], (unsigned long long)(long long)hist[threadIdx.x]);
-    if (last_block(a.st)) draw(a, j);
 }
 
-}  // namespace
+// A sweep and the draw of the next centre, or what has to be done before that
+// draw.
+template <bool VEC, bool BOUND>
+__global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int odd, int lprl, float eps_lo, float tiny) {
+    // the state's fields in one go, before the first of them is looked at
+    const int chosen = ld_now(&a.st->chosen), todo = ld_now(&a.st->todo);
+    const int e0 = ld_now(&a.st->e0), k = ld_now(&a.st->k), cur = ld_now(&a.st->cur), resum = ld_now(&a.st->resum);
+    const long long pick = ld_now(&a.st->pick);
+    if (chosen >= a.K) return;
+    if (todo == kPPSweep) sweep<VEC, BOUND>(a, chosen, pick, e0, k, cur, resum, odd, lprl, eps_lo, tiny);
+    else remake(a, todo, nullptr);
+    if (last_block(a.st)) draw(a);
+}
 
-cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const double *u, float *C, long long *idx,
-                            double *dmin, float2 *ub, unsigned long long *sums, void *state, cudaStream_t s,
-                            int num_sms, long long *err_out) {
+int kmeanspp_chunk_log2(int64_t N) {
+    int c = 5;
+    while (((N - 1) >> c) >= kPPMaxChunks) ++c;
+    return c;
+}
+
+// device memory of a call
+struct PPScratch {
+    double *dmin;              // N
+    float2 *ub;                // N, or NULL: the sweeps do without the bound's filter
+    unsigned long long *sums;  // 2 per chunk
+    PPState *st;
+    double *u;                 // K
+    float *C;                  // K x D
+    long long *idx;            // K
+};
+
+// The launches that choose centres `chosen` .. K - 1, if the maximum falls
+// slowly; a launch spent on remaking the sums leaves one centre more to the
+// next call.
+cudaError_t launch_kmeanspp(const PPScratch &w, const float *X, int64_t N, int D, int K, int chosen, cudaStream_t s,
+                            int num_sms) {
     PPArgs a;
     a.X = X;
     a.N = N;
     a.D = D;
-    a.dmin = dmin;
-    a.ub = ub;
+    a.K = K;
+    a.dmin = w.dmin;
+    a.ub = w.ub;
     a.csh = kmeanspp_chunk_log2(N);
     a.nb = (N + ((int64_t)1 << a.csh) - 1) >> a.csh;
-    a.sums[0] = sums;
-    a.sums[1] = sums + a.nb;
-    a.u = u;
-    a.st = static_cast<PPState *>(state);
-    a.C = C;
-    a.idx = idx;
+    a.sums0 = w.sums;
+    a.sums1 = w.sums + a.nb;
+    a.u = w.u;
+    a.st = w.st;
+    a.C = w.C;
+    a.idx = w.idx;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(state, 0, sizeof(PPState), s)) != cudaSuccess) return e;
     // 16-byte loads where the rows allow; lanes per row: its vectors rounded up
     // to a power of two, at most a warp
     const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
@@ -672,8 +758,8 @@ cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const doubl
     const int steps = (nv + (1 << lprl) - 1) >> lprl;
     const size_t smem = (size_t)((D + 1) & ~1) * 8 + (size_t)steps * (4u << lprl) * (vec ? 4 : 1) + kPPTable * 4 +
                         kPPSegment * 2;
-    auto step = ub ? (vec ? k_pp_step<true, true> : k_pp_step<false, true>)
-                   : (vec ? k_pp_step<true, false> : k_pp_step<false, false>);
+    auto step = a.ub ? (vec ? k_pp_step<true, true> : k_pp_step<false, true>)
+                     : (vec ? k_pp_step<true, false> : k_pp_step<false, false>);
     // (one value for every call: it is the process's, and another thread may be launching)
     constexpr int most = kPPMaxD * 12 + kPPTable * 4 + kPPSegment * 2;
     if ((e = cudaFuncSetAttribute(step, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
@@ -686,32 +772,29 @@ cudaError_t launch_kmeanspp(const float *X, int64_t N, int D, int K, const doubl
     // one wave of blocks that own whole chunks
     const unsigned grid = (unsigned)std::min<int64_t>(a.nb, (int64_t)num_sms * kPPBlocks);
     const unsigned fg = (unsigned)std::min<int64_t>((N + kPPThreads - 1) / kPPThreads, (int64_t)num_sms * 8);
-    count_launch();
-    if (vec) k_pp_first<true><<<fg, kPPThreads, (size_t)D * 8, s>>>(a);
-    else k_pp_first<false><<<fg, kPPThreads, (size_t)D * 8, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (K > 1) {
+    if (chosen == 0) {
+        if ((e = cudaMemsetAsync(w.st, 0, sizeof(PPState), s)) != cudaSuccess) return e;
         count_launch();
-        k_pp_weigh<<<grid, kPPThreads, 0, s>>>(a);
+        if (vec) k_pp_first<true><<<fg, kPPThreads, (size_t)D * 8, s>>>(a);
+        else k_pp_first<false><<<fg, kPPThreads, (size_t)D * 8, s>>>(a);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (K > 1) {
+            count_launch();
+            k_pp_weigh<<<grid, kPPThreads, 0, s>>>(a);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        chosen = 2;
+    }
+    // (one launch to spare, K - chosen + 1 in all: 2 us against the 25 us of another look)
+    for (int j = chosen; j < K + (K > 2); ++j) {
+        count_launch();
+        step<<<grid, kPPThreads, smem, s>>>(a, j & 1, lprl, eps_lo, tiny);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    for (int j = 2; j < K; ++j) {
-        count_launch();
-        step<<<grid, kPPThreads, smem, s>>>(a, j, lprl, eps_lo, tiny);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (err_out) return cudaMemcpyAsync(err_out, &a.st->err, 8, cudaMemcpyDeviceToHost, s);
     return cudaSuccess;
 }
 
-int kmeanspp_chunk_log2(int64_t N) {
-    int c = 5;
-    while (((N - 1) >> c) >= kPPMaxChunks) ++c;
-    return c;
-}
-
-size_t kmeanspp_state_bytes() { return sizeof(PPState); }
-
+}  // namespace
 }  // namespace kp
 
 using namespace kp;
@@ -739,39 +822,53 @@ KM_API int kmeans_init_kmeanspp(const float *X, int64_t N, int32_t D, int32_t K,
         return fail(KM_ECUDA, "device query failed");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t nb = ((N - 1) >> kmeanspp_chunk_log2(N)) + 1;
-    float2 *ub = nullptr;
-    double *dmin = nullptr, *ud = nullptr;
-    unsigned long long *bsum = nullptr;
-    void *st = nullptr;
-    float *Cd = nullptr;
-    long long *idx = nullptr;
-    long long err = 0;
-    cudaError_t e = pool_alloc(dev, reinterpret_cast<void **>(&dmin), (size_t)N * 8, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&bsum), (size_t)nb * 16, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, &st, kmeanspp_state_bytes(), s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&ud), (size_t)K * 8, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&Cd), (size_t)K * D * 4, s);
-    if (e == cudaSuccess) e = pool_alloc(dev, reinterpret_cast<void **>(&idx), (size_t)K * 8, s);
+    // one piece of memory, 256-byte aligned parts
+    size_t bytes = 0;
+    auto part = [&](size_t n) {
+        const size_t at = bytes;
+        bytes = (bytes + n + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t o_dmin = part((size_t)N * 8), o_sums = part((size_t)nb * 16), o_st = part(sizeof(PPState)),
+                 o_u = part((size_t)K * 8), o_C = part((size_t)K * D * 4), o_idx = part((size_t)K * 8);
+    char *base = nullptr;
+    PPScratch w = {};
+    cudaError_t e = pool_alloc(dev, reinterpret_cast<void **>(&base), bytes, s);
+    if (e == cudaSuccess) {
+        w.dmin = reinterpret_cast<double *>(base + o_dmin);
+        w.sums = reinterpret_cast<unsigned long long *>(base + o_sums);
+        w.st = reinterpret_cast<PPState *>(base + o_st);
+        w.u = reinterpret_cast<double *>(base + o_u);
+        w.C = reinterpret_cast<float *>(base + o_C);
+        w.idx = reinterpret_cast<long long *>(base + o_idx);
+        e = cudaMemcpyAsync(w.u, u, (size_t)K * 8, cudaMemcpyDefault, s);
+    }
     if (e == cudaSuccess && K > 2) {  // (the sweeps' only; they can do without)
-        e = pool_alloc(dev, reinterpret_cast<void **>(&ub), (size_t)N * 8, s);
+        e = pool_alloc(dev, reinterpret_cast<void **>(&w.ub), (size_t)N * 8, s);
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
-            ub = nullptr;
+            w.ub = nullptr;
             e = cudaSuccess;
         }
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ud, u, (size_t)K * 8, cudaMemcpyDefault, s);
-    if (e == cudaSuccess) e = launch_kmeanspp(X, N, D, K, ud, Cd, idx, dmin, ub, bsum, st, s, sms, &err);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(centroids, Cd, (size_t)K * D * 4, cudaMemcpyDefault, s);
-    if (e == cudaSuccess && indices) e = cudaMemcpyAsync(indices, idx, (size_t)K * 8, cudaMemcpyDefault, s);
-    for (void *p : {(void *)dmin, (void *)ub, (void *)bsum, st, (void *)ud, (void *)Cd, (void *)idx})
+    struct {
+        int chosen, err;  // as in PPState
+    } h = {0, 0};
+    // every launch chooses a centre or gets nearer to it, at most three to a centre
+    for (int64_t round = 0; e == cudaSuccess && h.chosen < K && !h.err && round <= 3 * (int64_t)K; ++round) {
+        e = launch_kmeanspp(w, X, N, D, K, h.chosen, s, sms);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&h, w.st, sizeof(h), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(centroids, w.C, (size_t)K * D * 4, cudaMemcpyDefault, s);
+        if (e == cudaSuccess && indices) e = cudaMemcpyAsync(indices, w.idx, (size_t)K * 8, cudaMemcpyDefault, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
+    for (void *p : {(void *)base, (void *)w.ub})
         if (p) cudaFreeAsync(p, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(e == cudaErrorMemoryAllocation ? KM_ENOMEM : KM_ECUDA, cudaGetErrorString(e));
     }
-    if (err) return fail(KM_ECUDA, "the draw produced an index out of range");
+    if (h.err || h.chosen < K) return fail(KM_ECUDA, "the draw produced an index out of range");
     return KM_OK;
 }
 

@@ -29,7 +29,8 @@
 // inequality that the new centre c is not nearer, from eight bytes of the point
 // and a table of the distances between c and the other centres, which every
 // block makes for itself.  What is left of X to read per centre are the rows
-// near c and those that no centre is near to yet.
+// near c and those that no centre is near to yet.  (For few points a block there
+// is no table: making it would cost more than reading them.)
 //
 // The weights need no FP64 either: for max D^2 in [2^(e-1), 2^e), q(x) is a
 // shift of the significand of D(x)^2.  e = e0 - k, with 2^e0 > max D^2 when e0
@@ -502,7 +503,7 @@ __global__ void __launch_bounds__(kPPThreads) k_pp_weigh(PPArgs a) {
 // filter comes first.
 template <bool VEC, bool BOUND>
 __device__ __forceinline__ void sweep(const PPArgs &a, int chosen, long long pick, int e0, int k, int cur, int resum,
-                                      int odd, int lprl, float eps_lo, float tiny) {
+                                      int odd, int table, int lprl, float eps_lo, float tiny) {
     // the centre: FP64 (D), then FP32 padded to a multiple of LPR vectors with
     // zeros; the first filter's table (kPPTable) and list (kPPSegment)
     extern __shared__ double sd[];
@@ -549,7 +550,7 @@ __device__ __forceinline__ void sweep(const PPArgs &a, int chosen, long long pic
     // a quarter of the squared distances between the new centre and the others,
     // rounded down with room for the FP64 sums' own error: a point whose D^2 is
     // no larger is, by the triangle inequality, no nearer to the new centre
-    const int ntab = BOUND ? min(chosen - 1, kPPTable) : 0;
+    const int ntab = BOUND ? min(chosen - 1, table) : 0;
     for (int g0 = warp * rows; g0 < ntab; g0 += kPPWarps * rows) {  // warp-uniform
         const int g = g0 + sub;
         float s = 0.f;
@@ -700,13 +701,14 @@ __device__ __forceinline__ void sweep(const PPArgs &a, int chosen, long long pic
 // A sweep and the draw of the next centre, or what has to be done before that
 // draw.
 template <bool VEC, bool BOUND>
-__global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int odd, int lprl, float eps_lo, float tiny) {
+__global__ void __launch_bounds__(kPPThreads, kPPBlocks) k_pp_step(PPArgs a, int odd, int table, int lprl,
+                                                                       float eps_lo, float tiny) {
     // the state's fields in one go, before the first of them is looked at
     const int chosen = ld_now(&a.st->chosen), todo = ld_now(&a.st->todo);
     const int e0 = ld_now(&a.st->e0), k = ld_now(&a.st->k), cur = ld_now(&a.st->cur), resum = ld_now(&a.st->resum);
     const long long pick = ld_now(&a.st->pick);
     if (chosen >= a.K) return;
-    if (todo == kPPSweep) sweep<VEC, BOUND>(a, chosen, pick, e0, k, cur, resum, odd, lprl, eps_lo, tiny);
+    if (todo == kPPSweep) sweep<VEC, BOUND>(a, chosen, pick, e0, k, cur, resum, odd, table, lprl, eps_lo, tiny);
     else remake(a, todo, nullptr);
     if (last_block(a.st)) draw(a);
 }
@@ -771,6 +773,14 @@ cudaError_t launch_kmeanspp(const PPScratch &w, const float *X, int64_t N, int D
     const float tiny = std::ldexp((float)(D + 8), -149);
     // one wave of blocks that own whole chunks
     const unsigned grid = (unsigned)std::min<int64_t>(a.nb, (int64_t)num_sms * kPPBlocks);
+    // Every block makes the table for itself: as many distances as half of its
+    // points, and none for few points.  K = 300, all centres in the table / half the
+    // points / none: 2,000 x 100: 9.8 / 7.4 / 7.1 ms (32 points a block), 40,000 x 32:
+    // 5.8 / 5.4 / 5.0 (88), 60,000 x 784: 44 / 44 / 51 (132), 335,544 x 100: 13.2 / 13.2
+    // / 21.5 (736), points in clusters; without clusters the table gains nothing and
+    // costs 26 / 26 / 21.5 in the last case, 9.9 / 9.0 / 7.4 at 100,000 x 17 (219).
+    const int64_t points = N / grid;
+    const int table = points < 128 ? 0 : (int)std::min<int64_t>(kPPTable, points / 2);
     const unsigned fg = (unsigned)std::min<int64_t>((N + kPPThreads - 1) / kPPThreads, (int64_t)num_sms * 8);
     if (chosen == 0) {
         if ((e = cudaMemsetAsync(w.st, 0, sizeof(PPState), s)) != cudaSuccess) return e;
@@ -788,7 +798,7 @@ cudaError_t launch_kmeanspp(const PPScratch &w, const float *X, int64_t N, int D
     // (one launch to spare, K - chosen + 1 in all: 2 us against the 25 us of another look)
     for (int j = chosen; j < K + (K > 2); ++j) {
         count_launch();
-        step<<<grid, kPPThreads, smem, s>>>(a, j & 1, lprl, eps_lo, tiny);
+        step<<<grid, kPPThreads, smem, s>>>(a, j & 1, table, lprl, eps_lo, tiny);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -157,3 +157,12 @@ def test_infinite_coordinates(kp, first):
     X[450, 3] = -np.inf
     X[700, 1] = np.inf
     check_weights(kp, X, 9, 2, (first + 0.5) / 900)
+
+
+@pytest.mark.parametrize("N,D,K", [(120000, 3, 400), (60000, 8, 90), (940000, 2, 1060)])
+def test_more_centres_than_the_table(kp, N, D, K):
+    """The table of the bound's filter holds half as many centres as a block has
+    points (none below 128 points), and 1024 at most."""
+    rng = np.random.default_rng(N)
+    X = rng.normal(size=(K, D))[rng.integers(0, K, size=N)] * 50.0 + rng.normal(size=(N, D)) * 0.1
+    check(kp, X.astype(np.float32), K, seed=K)

@@ -74,10 +74,12 @@ struct SettleReq {
     int32_t old;     // label before this pass (-1: none)
     int32_t i1;      // tensor-core winner (the bounds were written for it)
     float lb_alt;    // group bound that holds for every column (from the smallest estimate)
-    unsigned long long gmask[2];  // their union: groups that can hold the winner (all ones: every
-                                  // group; zero: the groups g with lb[n][g] <= lim)
-    float lim;       // bound of the window's edge (used when gmask is zero)
+    // K <= 256: the union of the two is the set of groups that can hold the winner
+    // (all ones: every group).  K > 256: the low half of the second is the bound of
+    // the window's edge, lim, and the groups are those with lb[n][g] <= lim.
+    unsigned long long gmask[2];
 };
+static_assert(sizeof(SettleReq) == 32, "a request per point: context memory");
 
 // Everything a kernel needs, passed by value.
 struct Params {

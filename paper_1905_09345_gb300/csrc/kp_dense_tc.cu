@@ -467,7 +467,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     // every column is at least b1: when i1 loses, this bounds both i1's
                     // group (which now keeps i1) and the winner's group
                     rq->lb_alt = bound_of(b1);
-                    rq->lim = 0.f;
                 }
             }
             if (mm && !first) {

@@ -450,8 +450,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 rq.old = old;
                 rq.i1 = i1;
                 rq.lb_alt = sqrt_lo(__fsub_rd(__fadd_rd(xlo, b1), E));
-                rq.gmask[0] = rq.gmask[1] = 0ull;
-                rq.lim = sqrt_hi(__fsub_ru(__fadd_ru(xup, thr), E));
+                rq.gmask[0] = 0ull;
+                rq.gmask[1] = __float_as_uint(sqrt_hi(__fsub_ru(__fadd_ru(xup, thr), E)));
                 p.sreq[n] = rq;
             }
             if (lane == 0) p.sbits[(int64_t)tile * (kTM / 32) + q] = nm;

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int firs
         mine.n = -1;
         mine.old = -1;
         mine.i1 = 0;
-        mine.lb_alt = mine.lim = 0.f;
+        mine.lb_alt = 0.f;
         mine.gmask[0] = mine.gmask[1] = 0ull;
         if (lane < cnt) {
             const int n = p.squeue[r0 + lane];
@@ -212,12 +212,18 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int firs
                 mine.n = -1;
             }
         }
+        float mine_lim = 0.f;
+        unsigned long long mine_mask = mine.gmask[0] | mine.gmask[1];
+        if (K > 256) {  // requests of the streamed-centroid pass
+            mine_lim = __uint_as_float((uint32_t)mine.gmask[1]);
+            mine_mask = 0ull;
+        }
         for (int j = 0; j < cnt; j += kPer) {  // warp-uniform
             const int from = j + sub;  // < 32
             const int n = __shfl_sync(full, mine.n, from), old = __shfl_sync(full, mine.old, from);
             const int w1 = __shfl_sync(full, mine.i1, from);
-            const float lim = __shfl_sync(full, mine.lim, from), lb_alt = __shfl_sync(full, mine.lb_alt, from);
-            const unsigned long long gmask = __shfl_sync(full, mine.gmask[0] | mine.gmask[1], from);
+            const float lim = __shfl_sync(full, mine_lim, from), lb_alt = __shfl_sync(full, mine.lb_alt, from);
+            const unsigned long long gmask = __shfl_sync(full, mine_mask, from);
             const bool act = n >= 0;
             const int64_t row = act ? n : 0;
             ulonglong2 xv[NC];

@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(kUpdWarps * 32) k_update(Params p, int final_o
             // below.  Squares outside FP32's normal range: the FP64 root.
             const double dk = r * (1.0 + (double)(D + 4) * 2.220446049250313e-16);
             float dlt;
-            if (dk == 0.0 || (dk >= 0x1p-126 && dk <= 0x1p127)) {
+            const unsigned hi = (unsigned)__double2hiint(dk);  // (FP64 comparisons share the slow pipe)
+            if (hi - 0x38100000u < 0x0fd00000u || (hi | (unsigned)__double2loint(dk)) == 0u) {  // [2^-126, 2^127), 0
                 dlt = __fsqrt_ru(round_up_f(dk));
                 const float below = __int_as_float(max(__float_as_int(dlt) - 1, 0));
                 if ((double)below * (double)below >= dk) dlt = below;

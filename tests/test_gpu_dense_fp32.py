@@ -38,3 +38,17 @@ def test_dense_fp32_ties(kp, D):  # noqa: F811
     C0 = np.concatenate([X[:20], X[:12]]).astype(np.float32)
     for grouping in (kp.KM_GROUP_CONTIGUOUS, kp.KM_GROUP_CLUSTERED):
         lockstep(kp, X, C0, 5, 2, dense=kp.KM_DENSE_FP32, check_bounds=True, grouping=grouping)
+
+
+@pytest.mark.parametrize("N,D,K,G", [(2000, 130, 33, 4), (1537, 200, 64, 6), (900, 401, 21, 21), (5000, 256, 130, 13),
+                                     (700, 1000, 9, 2)])
+def test_dense_fp32_wide(kp, N, D, K, G):  # noqa: F811
+    """Rows of more than 128 coordinates, and exact ties among them."""
+    rng = np.random.default_rng(N + D)
+    X, _ = synth.gaussian_mixture(rng, N, D, min(K, 32), centre_range=4.0, scale="blob_uniform",
+                                  scale_args=(0.5, 2.0))
+    Y = rng.integers(0, 2, size=(400, D)).astype(np.float32)
+    Y[:, 20:] = 0.0
+    for algo in (kp.KM_ALGO_FILTERED, kp.KM_ALGO_LLOYD):
+        lockstep(kp, X, synth.sample_init(rng, X, K), G, 3, algo=algo, check_bounds=N * K < 150_000)
+        lockstep(kp, Y, Y[:K].copy(), G, 2, algo=algo, check_bounds=True)

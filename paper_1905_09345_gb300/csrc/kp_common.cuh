@@ -218,6 +218,11 @@ __device__ __forceinline__ f32x2 pack2(float lo, float hi) {
 __device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
+__device__ __forceinline__ float sum2(f32x2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return lo + hi;
+}
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     f32x2 r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -255,7 +260,7 @@ __device__ __forceinline__ void two_sum2(f32x2 a, f32x2 b, f32x2 &s, f32x2 &e) {
 // The distances are summed as FP32 pairs h + l: x - c exactly (TwoSum), its
 // square but for 2^-45 of it, TwoSum into h, everything else into l.  With n
 // coordinates per lane, l meets n + 10 additions of magnitudes below
-// (n + 9) 2^-24 of the sum, so that the pair is within (n^2 + 16 n + 100) 2^-48
+// (n + 9) 2^-24 of the sum, so that the pair is within (n^2 + 20 n + 100) 2^-48
 // of it; the FP64 sum is within (D + 2) 2^-53.  The order is decided when the
 // pairs differ by more than twice both errors of both sums (and what
 // underflow can hide); NaN and infinity decide nothing.
@@ -289,7 +294,7 @@ __device__ __forceinline__ int pair_order(const float *x, const float *ca, const
     two_sum(ha, -hb, s, e);
     const float diff = __fadd_rn(s, __fadd_rn(e, __fsub_rn(la, lb)));
     const float n = (float)((D + 31) / 32);
-    const float rel = (n * n + 16.f * n + 100.f) * 0x1p-47f + (float)(D + 2) * 0x1p-52f;
+    const float rel = (n * n + 20.f * n + 100.f) * 0x1p-47f + (float)(D + 2) * 0x1p-52f;
     const float margin = __fmaf_ru(rel, __fadd_ru(ha, hb), (float)(D + 4) * 0x1p-140f);
     return diff < -margin ? 0 : (diff > margin ? 1 : -1);
 }

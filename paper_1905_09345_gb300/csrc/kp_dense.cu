@@ -8,8 +8,9 @@
 //
 // The distance is the direct difference sum (x_i - c_i)^2 in FP32; its rounding
 // error is bounded (Params::eps_hi/eps_lo), and when the two nearest FP32
-// values cannot be ordered by that bound the point is settled in FP64 with the
-// summation order of the FP64 definition, so labels are exact.
+// values cannot be ordered by that bound the two are ordered by compensated FP32
+// sums (pair_order), or, where those decide nothing or a third is as near, in FP64
+// with the summation order of the FP64 definition, so labels are exact.
 #include "kp_common.cuh"
 
 namespace kp {
@@ -19,15 +20,10 @@ constexpr int kDenseWarps = kDenseThreads / 32;
 constexpr int kDenseTileBytes = 64 * 1024;
 constexpr int kDenseLbBytes = 48 * 1024;
 
+// acc += d d (in place: fma2 in its stead takes up to 8 registers more here)
 __device__ __forceinline__ void fma2_sq(f32x2 &acc, f32x2 d) {
     asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc) : "l"(d));
 }
-__device__ __forceinline__ float sum2(f32x2 a) {
-    float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
-    return lo + hi;
-}
-
 // any D: x and c in global memory (c with stride Dp)
 __device__ __forceinline__ float sqdist_gen(const float *__restrict__ x, const float *__restrict__ c, int D) {
     float a0 = 0.f, a1 = 0.f;
@@ -219,7 +215,7 @@ __global__ void __launch_bounds__(kDenseThreads, MB) k_dense_assign(Params p, in
     constexpr int PB = PW * kDenseWarps;         // points of a block
     constexpr int SEG = L > 1 ? DPL + 4 : DPL;   // a lane's part of a staged row (skewed: no bank conflicts)
     constexpr int RS = L * SEG;                  // staged row stride
-    static_assert(DPL % 4 == 0 && P % L == 0 && (L == 1 || L == 2 || L == 4), "shape");
+    static_assert(DPL % 4 == 0 && P % L == 0 && (L == 1 || L == 2), "shape");
     Ctrl *ctrl = p.ctrl;
     count_kernel(ctrl);
     if (respect_done && *(volatile int *)&ctrl->done) return;

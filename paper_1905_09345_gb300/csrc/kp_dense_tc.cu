@@ -24,8 +24,8 @@
 // minima, four columns at a time (Scan4 in kp_tc.cuh).  Lower bounds are
 // t-based with the error E(x) subtracted, the upper
 // bound adds it; when the runner-up lies within 2E of the winner the point is
-// settled exactly by kp_settle.cu (FP32 direct differences, then FP64 if the
-// FP32 error bound cannot decide), so labels are exact.
+// settled exactly by kp_settle.cu (FP32 direct differences, then compensated FP32
+// sums, then FP64, each where the one before cannot decide), so labels are exact.
 //
 // Bound by the scan: of 200 us for 1,048,576 x 64, K = 256, G = 26, loads,
 // products and TMEM reads alone take 76, the scan 80 (the minima and maxima of

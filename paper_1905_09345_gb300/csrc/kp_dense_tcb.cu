@@ -538,9 +538,12 @@ bool plan_b(const Params &p, size_t smem_limit, TcbCfg &cfg, size_t &smem) {
     if (cfg.Kp > kMaxKp) return false;
     cfg.nb = cfg.Kp / kNB;
     cfg.hb = (cfg.nb + 1) / 2;
-    // groups that 64 columns (the span between two flushes of the staged
-    // minima) can close under the contiguous grouping j -> j G / K, plus the
-    // one still open
+    // The shapes that this engine takes are those of an earlier layout, which kept
+    // every norm and the minima of 64 columns' groups (under the contiguous grouping
+    // j -> j G / K, whatever the context's) in shared memory.  The present layout
+    // needs less, and at most 229,208 bytes: 128 coordinates with K = 4096, with K =
+    // 1024 and more than 368 groups, or with K = 257 and more than 106 would fit too
+    // and still go to the FP32 engine.
     int most = 0;
     for (int j = 0; j < cfg.Kp / 64; ++j) {
         const int64_t c0 = (int64_t)j * 64, c1 = std::min<int64_t>((int64_t)(j + 1) * 64, p.K) - 1;
@@ -552,8 +555,6 @@ bool plan_b(const Params &p, size_t smem_limit, TcbCfg &cfg, size_t &smem) {
     const size_t NA = Dt / 64;
     const size_t a_bytes = 2 * 2 * NA * (size_t)kAtomBytes;
     const size_t half = NA * (size_t)kBAtom;
-    // the shapes this engine takes: a bound on Kp and on the groups that 64
-    // columns hold (beyond it the FP32 engine runs)
     if (1024 + a_bytes + 2 * half + (size_t)cfg.Kp * 8 + (size_t)cfg.Kp / 32 * 4 + 256 * (size_t)srow * 4 + 184 >
         smem_limit)
         return false;

@@ -69,8 +69,6 @@ struct GemmCfg {
     int mt, nt;        // CTAs along M and N (the rest of a product's CTAs split K)
     int k_steps;       // K slices of 64 per CTA (split-K: the CTA's split selects the slice range)
     int nch, bn;       // N chunks per CTA and columns per chunk (multiple of 16, <= 256)
-    int tmem_cols;     // power of two >= nch * bn
-    int stages;
     int mode;          // Epi
     const float *bias; // N (GELU, SOFTMAX)
     uint16_t *out;     // row-major bfloat16 M x ldo (nullable)

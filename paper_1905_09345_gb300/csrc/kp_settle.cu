@@ -3,10 +3,10 @@
 // The tensor-core passes (kp_dense_tc.cu, kp_dense_tcb.cu) estimate every
 // distance with a bounded error; a row whose runner-up lies inside the error
 // window of its winner is queued (a per-row request and one bit in a bitmap),
-// and the kernels here decide it exactly from FP32 direct differences, with
-// FP64 where the FP32 error bound cannot order the two smallest, so that the
-// labels are those of the exact argmin (KPynq Sec. I: the distance
-// calculator's result).
+// and the kernels here decide it exactly from FP32 direct differences, from
+// compensated FP32 sums where their error bound cannot order the two smallest, and
+// in FP64 where those cannot either or a third is as near, so that the labels are
+// those of the exact argmin (KPynq Sec. I: the distance calculator's result).
 #include "kp_common.cuh"
 
 namespace kp {
@@ -114,8 +114,8 @@ struct Top3 {
 // (runner-up inside the error window).  The candidates are the centroids of
 // the groups whose tensor-core minimum lies in the window (a group mask, or --
 // for the streamed-centroid pass -- the groups whose written bound is within
-// the window's edge).  The smallest FP32 distance decides; where FP32 cannot separate it from the
-// runner-up alone the two are ordered by pair_order, and what is left (three
+// the window's edge).  The smallest FP32 distance decides; where FP32 cannot
+// separate it from the runner-up alone the two are ordered by pair_order, and what is left (three
 // that FP32 cannot separate, exact ties) by the FP64 distances of every
 // candidate, lanes over centroids, ties to the lowest index.  Writes the
 // label, corrects u / lb / lbg when the winner is not i1, and appends label
@@ -284,20 +284,15 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int firs
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const ulonglong2 *c = reinterpret_cast<const ulonglong2 *>(Cb + (size_t)min(col + k, last) * cst) + sl;
-                    unsigned long long a0 = 0ull, a1 = 0ull;
+                    f32x2 a0 = 0ull, a1 = 0ull;
 #pragma unroll
                     for (int q = 0; q < NC; ++q) {
                         const ulonglong2 c2 = c[kSub * q];
-                        unsigned long long d0, d1;
-                        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d0) : "l"(xv[q].x), "l"(c2.x));
-                        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d1) : "l"(xv[q].y), "l"(c2.y));
-                        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a0) : "l"(d0));
-                        asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a1) : "l"(d1));
+                        const f32x2 d0 = sub2(xv[q].x, c2.x), d1 = sub2(xv[q].y, c2.y);
+                        a0 = fma2(d0, d0, a0);
+                        a1 = fma2(d1, d1, a1);
                     }
-                    float l0, h0, l1, h1;
-                    asm("mov.b64 {%0, %1}, %2;" : "=f"(l0), "=f"(h0) : "l"(a0));
-                    asm("mov.b64 {%0, %1}, %2;" : "=f"(l1), "=f"(h1) : "l"(a1));
-                    s[k] = (l0 + h0) + (l1 + h1);
+                    s[k] = sum2(a0) + sum2(a1);
                 }
                 // lanes 4 apart: two candidates each; 2 apart: one each; then the pair's sum
                 const bool u4 = sl & 4, u2 = sl & 2;

@@ -78,10 +78,10 @@ __device__ __forceinline__ int64_t stats_entries(const Params &p, bool full) {
     return full ? p.N : 2 * (int64_t)p.ctrl->moved_count;
 }
 
-// Decide the mode; move the points if they are few; in full mode zero S and Q; count the entries per cluster
-// (shared-memory histogram when K fits), and let the last block turn the
-// counts into segment offsets (hcur) and, in full mode, the new cluster sizes
-// (cnt).
+// Decide the mode; move the points if they are few; in full mode zero S and Q;
+// count the entries per cluster (shared-memory histogram when K fits), and let
+// the last block turn the counts into segment offsets (hcur) and, in full mode,
+// the new cluster sizes (cnt).
 __global__ void __launch_bounds__(kStatsThreads) k_stats_hist(Params p, int all_points, int respect_done) {
     extern __shared__ int hist[];
     __shared__ int last;
@@ -226,6 +226,18 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_scatter(Params p, int r
     }
 }
 
+// The same operations on one value and on two (kp_common.cuh)
+__device__ __forceinline__ float add2(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float mul2(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma2(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ void two_sum2(float a, float b, float &s, float &e) { two_sum(a, b, s, e); }
+__device__ __forceinline__ float flip2(float a, bool neg) { return neg ? -a : a; }
+__device__ __forceinline__ f32x2 flip2(f32x2 a, bool neg) { return a ^ (neg ? kNeg2 : 0ull); }
+__device__ __forceinline__ void put2(float &v, float lo, float) { v = lo; }
+__device__ __forceinline__ void put2(f32x2 &v, float lo, float hi) { v = pack2(lo, hi); }
+__device__ __forceinline__ void get2(float v, float &lo, float &hi) { lo = v, hi = 0.f; }
+__device__ __forceinline__ void get2(f32x2 v, float &lo, float &hi) { unpack2(v, lo, hi); }
+
 // Each warp sums a run of consecutive sorted entries, lanes over the
 // coordinates, eight entries' loads in flight at a time, and adds its partial
 // sums to S and Q (and, in incremental mode, the count change to cnt) whenever
@@ -245,18 +257,6 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats_scatter(Params p, int r
 // Measured, all points: 1,048,576 x 64: 139 -> 105 us; 300,007 x 64: 54 -> 37;
 // 4,194,304 x 128: 900 -> 670.  A ring of rows in shared memory, seven ahead, with
 // a rolled loop over the points measured 157, 54 and 900.
-// The same operations on one value and on two (kp_common.cuh)
-__device__ __forceinline__ float add2(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float mul2(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float fma2(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ void two_sum2(float a, float b, float &s, float &e) { two_sum(a, b, s, e); }
-__device__ __forceinline__ float flip2(float a, bool neg) { return neg ? -a : a; }
-__device__ __forceinline__ f32x2 flip2(f32x2 a, bool neg) { return a ^ (neg ? kNeg2 : 0ull); }
-__device__ __forceinline__ void put2(float &v, float lo, float) { v = lo; }
-__device__ __forceinline__ void put2(f32x2 &v, float lo, float hi) { v = pack2(lo, hi); }
-__device__ __forceinline__ void get2(float v, float &lo, float &hi) { lo = v, hi = 0.f; }
-__device__ __forceinline__ void get2(f32x2 v, float &lo, float &hi) { unpack2(v, lo, hi); }
-
 template <int NPER>  // coordinates per lane: ceil(D / 32), in pairs beyond one
 __global__ void __launch_bounds__(kStatsThreads, NPER <= 2 ? 3 : (NPER == 4 ? 2 : 1)) k_stats_sum(Params p, int respect_done) {
     Ctrl *ctrl = p.ctrl;

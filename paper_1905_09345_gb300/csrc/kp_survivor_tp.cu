@@ -41,12 +41,7 @@ constexpr int kTpThreads = 256;
 
 // x is kept as packed pairs of FP32 values: xr[q] holds coordinates
 // 4q .. 4q+3 as two 64-bit registers (low half = lower coordinate)
-__device__ __forceinline__ float hsum2(unsigned long long v) {
-    float lo, hi;
-    unpack2(v, lo, hi);
-    return lo + hi;
-}
-
+//
 // Direct-difference squared distance sum_i (x_i - c_i)^2 with packed FP32x2
 // subtract and fused multiply-add (each lane of a pair is an ordinary
 // round-to-nearest FP32 operation): four partial sums of D/4 terms each, so
@@ -64,7 +59,7 @@ __device__ __forceinline__ float sqdist_xr(const ulonglong2 (&xr)[DP / 4], const
         asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a0) : "l"(d0));
         asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a1) : "l"(d1));
     }
-    return hsum2(a0) + hsum2(a1);
+    return sum2(a0) + sum2(a1);
 }
 
 template <int DP>
@@ -116,7 +111,7 @@ __device__ __forceinline__ float sqdist_mem(const Params &p, const float *xg, co
         asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a0) : "l"(d0));
         asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a1) : "l"(d1));
     }
-    return hsum2(a0) + hsum2(a1);
+    return sum2(a0) + sum2(a1);
 }
 template <int DP>
 __device__ __forceinline__ double dist2_f64_mem(const Params &p, const float *xg, const float *__restrict__ c) {

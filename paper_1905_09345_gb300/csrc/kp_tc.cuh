@@ -50,21 +50,9 @@ __device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *m, int c0, 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Asynchronous TMEM read of 32 columns; the registers may be used only after
-// tmem_wait32 on the same array (which names them, so that the compiler
-// cannot move their uses above the wait).
-__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
-        "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) : : "memory");
-}
-
-// Asynchronous TMEM read of 16 columns (see tmem_ld32_async)
+// Asynchronous TMEM read of 16 columns; the registers may be used only after
+// tmem_wait16 on the same array (which names them, so that the compiler cannot
+// move their uses above the wait).
 __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -110,12 +98,6 @@ __device__ __forceinline__ void split8(const float *v, uint4 &h, uint4 &l) {
     h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
     l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
-__device__ __forceinline__ unsigned long long pack_f2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-
 __device__ __forceinline__ float min3(float a, float b, float c) {
     float r;
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
@@ -138,17 +120,10 @@ struct Scan4 {
     int pend;      // the open group's slot (warp-uniform)
 
     __device__ __forceinline__ void four(const uint32_t *acc, const float4 &cn, uint32_t nib, int c) {
-        unsigned long long t01, t23;
-        const unsigned long long m2 = 0xc0000000c0000000ull;  // (-2, -2)
-        asm("fma.rn.f32x2 %0, %1, %2, %3;"
-            : "=l"(t01)
-            : "l"(pack_f2(__uint_as_float(acc[0]), __uint_as_float(acc[1]))), "l"(m2), "l"(pack_f2(cn.x, cn.y)));
-        asm("fma.rn.f32x2 %0, %1, %2, %3;"
-            : "=l"(t23)
-            : "l"(pack_f2(__uint_as_float(acc[2]), __uint_as_float(acc[3]))), "l"(m2), "l"(pack_f2(cn.z, cn.w)));
+        const f32x2 m2 = 0xc0000000c0000000ull;  // (-2, -2)
         float t[4];
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[0]), "=f"(t[1]) : "l"(t01));
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(t[2]), "=f"(t[3]) : "l"(t23));
+        unpack2(fma2(pack2(__uint_as_float(acc[0]), __uint_as_float(acc[1])), m2, pack2(cn.x, cn.y)), t[0], t[1]);
+        unpack2(fma2(pack2(__uint_as_float(acc[2]), __uint_as_float(acc[3])), m2, pack2(cn.z, cn.w)), t[2], t[3]);
         const float l0 = fminf(t[0], t[1]), h0 = fmaxf(t[0], t[1]);
         const float l1 = fminf(t[2], t[3]), h1 = fmaxf(t[2], t[3]);
         const float m = fminf(l0, l1);

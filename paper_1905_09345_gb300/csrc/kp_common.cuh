@@ -483,6 +483,19 @@ __device__ __forceinline__ void move_point(const Params &p, int64_t n, int old) 
     }
 }
 
+// The same question where pair_order leaves it open, by the FP64 distances (whole
+// warp; 0: ca, 1: cb); equal distances: b_first.  Out of line: inlined it costs
+// every launch.
+static __device__ __noinline__ int pair_order_f64(const float *x, const float *ca, const float *cb, int D,
+                                                  bool b_first) {
+    bool same = true;  // copies of one centroid need no distances
+    for (int i = threadIdx.x & 31; i < D; i += 32) same &= ca[i] == cb[i];
+    if (__all_sync(0xffffffffu, same)) return b_first;
+    const double d = dist2_f64(x, (threadIdx.x & 1) ? cb : ca, D);
+    const double da = __shfl_sync(0xffffffffu, d, 0), db = __shfl_sync(0xffffffffu, d, 1);
+    return db < da || (db == da && b_first);
+}
+
 // drift of centroid k between versions w and v (upper bound)
 __device__ __forceinline__ float drift_c(const Params &p, int v, int w, int k) {
     return v == w ? 0.0f : __fsub_ru(p.Dc[(size_t)v * p.K + k], p.Dc[(size_t)w * p.K + k]);

@@ -40,6 +40,22 @@ __device__ __forceinline__ float sqdist_gen(const float *__restrict__ x, const f
     return a0 + a1;
 }
 
+// the same for a centroid's row in global memory, 16 bytes at a time (it is
+// aligned, and zero from D up to a multiple of 4)
+__device__ __forceinline__ float sqdist_row(const float *__restrict__ x, const float *__restrict__ c, int D) {
+    float a0 = 0.f, a1 = 0.f;
+    for (int i = 0; i < D; i += 4) {
+        const float4 cv = *reinterpret_cast<const float4 *>(c + i);
+        const float t0 = x[i] - cv.x, t1 = (i + 1 < D ? x[i + 1] : 0.f) - cv.y;
+        const float t2 = (i + 2 < D ? x[i + 2] : 0.f) - cv.z, t3 = (i + 3 < D ? x[i + 3] : 0.f) - cv.w;
+        a0 = fmaf(t0, t0, a0);
+        a1 = fmaf(t1, t1, a1);
+        a0 = fmaf(t2, t2, a0);
+        a1 = fmaf(t3, t3, a1);
+    }
+    return a0 + a1;
+}
+
 // What the scan over the centroids leaves of a point.
 struct Nearest {
     float s1, s2;    // smallest and second smallest value
@@ -81,7 +97,7 @@ __device__ __forceinline__ float bound_dn(float s, const Params &p) { return s =
 // group bounds, in shared or global memory).  Near-ties are settled by the
 // whole warp, one point at a time: the lanes share the centroids out; a single
 // one that the FP32 bound cannot separate from the best is ordered by
-// pair_order, several (or what that leaves open) in FP64.
+// pair_order, several (or what that leaves open) by their FP64 distances.
 // Returns the lane's number of settled points; `changed` counts its moves.
 __device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool active, int64_t n, Nearest &t,
                                              float *row, bool bounds, int first, int v, int &changed) {
@@ -101,7 +117,7 @@ __device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool a
         float so = ref;
         for (int c0 = 0; c0 < p.K; c0 += 32) {
             const int c = c0 + lane;
-            const float s = c < p.K ? sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D) : INFINITY;
+            const float s = c < p.K ? sqdist_row(xr, p.C + (size_t)c * p.Dp, p.D) : INFINITY;
             const unsigned in = __ballot_sync(full, c < p.K && c != was && unresolved(ref, s, p));
             many += __popc(in);
             if (in) {
@@ -117,9 +133,11 @@ __device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool a
             bi = other;
             bs = so;
         } else if (o < 0) {
+            // two: a lane each, at the same time; several: the lanes share them out
             double bd = INFINITY;
-            for (int c = lane; c < p.K; c += 32) {
-                const float s = sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D);
+            const int step = many == 1 ? p.K : 32;
+            for (int c = many > 1 ? lane : (lane == 0 ? was : (lane == 1 ? other : p.K)); c < p.K; c += step) {
+                const float s = sqdist_row(xr, p.C + (size_t)c * p.Dp, p.D);
                 if (c != was && !unresolved(ref, s, p)) continue;
                 const double d = dist2_f64(xr, p.C + (size_t)c * p.Dp, p.D);
                 if (d < bd || (d == bd && tie_key(p, c) < tie_key(p, bi))) { bd = d; bi = c; bs = s; }
@@ -138,7 +156,7 @@ __device__ __forceinline__ int finish_points(const Params &p, Ctrl *ctrl, bool a
                 for (int g = lane; g < p.G; g += 32) {
                     float mn = INFINITY;
                     for (int c = p.gstart[g]; c < p.gstart[g + 1]; ++c)
-                        if (c != bi) mn = fminf(mn, sqdist_gen(xr, p.C + (size_t)c * p.Dp, p.D));
+                        if (c != bi) mn = fminf(mn, sqdist_row(xr, p.C + (size_t)c * p.Dp, p.D));
                     r[g] = bound_dn(mn, p);
                 }
                 __syncwarp();
@@ -448,7 +466,6 @@ __global__ void __launch_bounds__(256) k_apply_moves(Params p, int all_points, i
     if (respect_done && *(volatile int *)&ctrl->done) return;
     if (if_dense && !*(volatile int *)&ctrl->dense_mode) return;
     if (*(volatile int *)&ctrl->stats_full) return;  // recomputed in full instead
-    const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t count = all_points ? p.N : (int64_t)ctrl->moved_count;

@@ -321,8 +321,12 @@ __global__ void __launch_bounds__(kSettleThreads, 2) k_settle(Params p, int firs
                 int bj = a1;
                 float bsr = v1;
                 int o = -1;
-                if (v3 == INFINITY || !unresolved(v1, v3, p))
-                    o = pair_order(xg, Cb + (size_t)a1 * cst, Cb + (size_t)a2 * cst, D);
+                if (v3 == INFINITY || !unresolved(v1, v3, p)) {
+                    const float *c1 = Cb + (size_t)a1 * cst, *c2 = Cb + (size_t)a2 * cst;
+                    o = pair_order(xg, c1, c2, D);
+                    // (narrower rows: the scan below is as fast, and the call costs every launch 0.4 us)
+                    if (D > 64 && o < 0) o = pair_order_f64(xg, c1, c2, D, tie_key(p, a2) < tie_key(p, a1));
+                }
                 if (o == 1) {
                     bj = a2;
                     bsr = v2;

@@ -457,8 +457,11 @@ __global__ void __launch_bounds__(kTpThreads, DP > 64 ? 1 : 2)
             const float s1 = __shfl_sync(0xffffffffu, rc_s, src);
             const int i1 = __shfl_sync(0xffffffffu, rc_best, src);
             const int i2 = __shfl_sync(0xffffffffu, rc_sec, src);
-            const int o = i2 < 0 ? -1
-                                 : pair_order(p.X + nr * p.D, Cs + (size_t)i1 * p.Dp, Cs + (size_t)i2 * p.Dp, p.D);
+            int o = i2 < 0 ? -1 : pair_order(p.X + nr * p.D, Cs + (size_t)i1 * p.Dp, Cs + (size_t)i2 * p.Dp, p.D);
+            if constexpr (DP > 64)  // (narrower rows: the scan below is as fast, and the call costs every launch)
+                if (o < 0 && i2 >= 0)
+                    o = pair_order_f64(p.X + nr * p.D, Cs + (size_t)i1 * p.Dp, Cs + (size_t)i2 * p.Dp, p.D,
+                                       tie_key(p, i2) < tie_key(p, i1));
             if (o == 1) {
                 // the runner-up it is: every bound holds (its group's still counts
                 // it), but for those that left out i1

@@ -46,3 +46,18 @@ def test_filtered_near_ties(kp, D, together):  # noqa: F811
         C0 = np.concatenate([C0[0::2], C0[1::2]])
     st = lockstep(kp, X, C0, P, 5, check_bounds=True, dense_switch=1.0)
     assert all(s["n_recheck"] > 0 and s["path"] == kp.KM_PATH_FILTERED for s in st[1:]), st
+
+
+@pytest.mark.parametrize("D", [5, 64, 96, 128])
+@pytest.mark.parametrize("dense_switch", [0.0, 1.0])
+def test_copies_of_every_centroid(kp, D, dense_switch):  # noqa: F811
+    """Every centroid twice, in different groups, and clusters symmetric about
+    it: each point has two nearest ones in each iteration, the lower index wins."""
+    rng = np.random.default_rng(D)
+    P = 7
+    c = rng.integers(-20, 21, size=(P, D)) * 4.0
+    d = rng.integers(-3, 4, size=(P, 40, D))
+    X = np.concatenate([c[:, None] + d, c[:, None] - d], 1).reshape(-1, D).astype(np.float32)
+    C0 = np.concatenate([c, c]).astype(np.float32)
+    st = lockstep(kp, X[rng.permutation(len(X))], C0, 4, 4, check_bounds=True, dense_switch=dense_switch)
+    assert all(s["n_recheck"] == len(X) for s in st)
